@@ -148,6 +148,13 @@ struct Predictor {
     float *dcol = nullptr, *dy0 = nullptr, *dy1 = nullptr, *da5 = nullptr, *win = nullptr,
           *tgt = nullptr;
     int64_t *idx = nullptr;
+    int64_t io_cap = 0;          // rows of out, win, tgt, idx
+    // fused training path (train_tc.cu): BF16 activations and gradients of the
+    // convolutions for fcap rows, the CTAs' gradient partials
+    std::vector<uint16_t *> fy, fdz;
+    float *fpart = nullptr;
+    uint8_t *fpack = nullptr;    // the step's packed weights
+    int64_t fcap = 0;
     float *splitk = nullptr;     // partial products of the GEMMs' K splits
     int64_t splitk_n = 0;
     std::vector<float *> tiles;  // workspace of the tile engine (fully convolutional)

@@ -11,6 +11,7 @@
 #include <string>
 
 #include "cnn.h"
+#include "train_tc.h"
 
 namespace cs {
 
@@ -63,6 +64,29 @@ cs_status dalloc(cs_ctx *ctx, T **p, size_t count) {
     return dmalloc_n(ctx, p, count);
 }
 
+void free_io(cs_ctx *ctx, Predictor &P) {
+    float **fs[] = {&P.out, &P.win, &P.tgt};
+    for (float **f : fs) {
+        dfree(ctx, *f);
+        *f = nullptr;
+    }
+    dfree(ctx, P.idx);
+    P.idx = nullptr;
+    P.io_cap = 0;
+}
+
+void free_fused(cs_ctx *ctx, Predictor &P) {
+    for (uint16_t *p : P.fy) dfree(ctx, p);
+    for (uint16_t *p : P.fdz) dfree(ctx, p);
+    P.fy.clear();
+    P.fdz.clear();
+    dfree(ctx, P.fpart);
+    dfree(ctx, P.fpack);
+    P.fpart = nullptr;
+    P.fpack = nullptr;
+    P.fcap = 0;
+}
+
 void free_workspace(cs_ctx *ctx, Predictor &P) {
     for (float *p : P.col) dfree(ctx, p);
     for (float *p : P.z) dfree(ctx, p);
@@ -70,13 +94,11 @@ void free_workspace(cs_ctx *ctx, Predictor &P) {
     P.col.clear();
     P.z.clear();
     P.y.clear();
-    float **fs[] = {&P.z5, &P.a5, &P.out, &P.gout, &P.dcol, &P.dy0, &P.dy1, &P.da5, &P.win, &P.tgt};
+    float **fs[] = {&P.z5, &P.a5, &P.gout, &P.dcol, &P.dy0, &P.dy1, &P.da5};
     for (float **f : fs) {
         dfree(ctx, *f);
         *f = nullptr;
     }
-    dfree(ctx, P.idx);
-    P.idx = nullptr;
     dfree(ctx, P.splitk);
     P.splitk = nullptr;
     P.splitk_n = 0;
@@ -86,14 +108,87 @@ void free_workspace(cs_ctx *ctx, Predictor &P) {
     P.tiles_cap.clear();
 }
 
-cs_status ensure_workspace(cs_ctx *ctx, Predictor &P, int64_t B) {
-    // the error flag of the tensor-core GEMMs' bounded waits
-    if (!ctx->dev_err) {
-        cs_status rc = dalloc(ctx, &ctx->dev_err, 1);
-        if (rc) return rc;
-        if (cudaMemset(ctx->dev_err, 0, sizeof(int)) != cudaSuccess)
-            return fail(ctx, CS_ECUDA, "cudaMemset of the device error flag failed");
+// the error flag of the tensor-core kernels' bounded waits
+cs_status ensure_err(cs_ctx *ctx) {
+    if (ctx->dev_err) return CS_OK;
+    cs_status rc = dalloc(ctx, &ctx->dev_err, 1);
+    if (rc) return rc;
+    if (cudaMemset(ctx->dev_err, 0, sizeof(int)) != cudaSuccess)
+        return fail(ctx, CS_ECUDA, "cudaMemset of the device error flag failed");
+    return CS_OK;
+}
+
+// the outputs and the batch of B rows
+cs_status ensure_io(cs_ctx *ctx, Predictor &P, int64_t B) {
+    cs_status rc = ensure_err(ctx);
+    if (rc || P.io_cap >= B) return rc;
+    free_io(ctx, P);
+    const NetShape S(P.dim);
+    const int64_t win = int64_t(S.cin) * S.positions(S.S0);
+    if ((rc = dalloc(ctx, &P.out, size_t(B * S.dim))) || (rc = dalloc(ctx, &P.win, size_t(B * win))) ||
+        (rc = dalloc(ctx, &P.tgt, size_t(B * S.dim))) || (rc = dalloc(ctx, &P.idx, size_t(B))))
+        return rc;
+    P.io_cap = B;
+    return CS_OK;
+}
+
+// The fused kernels (train_tc.cu) take BF16 operands and batches whose every
+// product the tensor-core GEMM would take (tc_gemm_fits: at least 16 rows);
+// FP32 operands and smaller batches run the layer-by-layer path.
+bool fused_batch(int64_t B) { return gemm_bf16() && B >= 16; }
+
+// where the packed weights of each layer lie in Predictor::fpack
+struct FusedPack {
+    int64_t fwd[4], bwd[4], fc1, bytes;
+    explicit FusedPack(const NetShape &S) {
+        int64_t o = 0;
+        for (int l = 0; l < S.n_conv; ++l) {
+            const int64_t K = int64_t(l == 0 ? S.cin : S.ch) * S.taps();
+            fwd[l] = o;
+            o += (K + 15) / 16 * 16 * S.ch * 2;
+            bwd[l] = o;
+            o += l == 0 ? 0 : int64_t(train_packed_kw(S.dim)) * S.ch * 2;
+        }
+        fc1 = o;
+        bytes = o + int64_t(S.hidden) * S.ch * 2;
     }
+};
+
+// buffers of the fused path for batches of up to B rows
+cs_status ensure_fused(cs_ctx *ctx, Predictor &P, int64_t B, bool grad) {
+    cs_status rc = ensure_err(ctx);
+    if (rc) return rc;
+    if (P.fcap >= B && (!grad || P.fpart)) return CS_OK;
+    const int64_t cap = std::max(B, P.fcap);
+    grad = grad || P.fpart;
+    free_fused(ctx, P);
+    const NetShape S(P.dim);
+    const int64_t sm = ctx->sm_count;
+    int64_t part = std::max(sm, (cap + 127) / 128) * head_part_floats(P.dim);
+    for (int l = 0; l < S.n_conv; ++l) {
+        const ConvGeo g(P.dim, l == 0 ? S.cin : S.ch, S.S0 - 2 * l);
+        uint16_t *y = nullptr, *dz = nullptr;
+        if ((rc = dalloc(ctx, &y, size_t(cap * g.Po * S.ch)))) break;
+        P.fy.push_back(y);
+        if (grad) {
+            if ((rc = dalloc(ctx, &dz, size_t(cap * g.Po * S.ch)))) break;
+            P.fdz.push_back(dz);
+        }
+        part += sm * (int64_t(g.K) * S.ch + S.ch);
+    }
+    if (rc == CS_OK && grad) rc = dalloc(ctx, &P.fpart, size_t(part));
+    if (rc == CS_OK) rc = dalloc(ctx, &P.fpack, size_t(FusedPack(S).bytes));
+    if (rc) {
+        free_fused(ctx, P);
+        return rc;
+    }
+    P.fcap = cap;
+    return CS_OK;
+}
+
+cs_status ensure_workspace(cs_ctx *ctx, Predictor &P, int64_t B) {
+    cs_status rc0 = ensure_io(ctx, P, B);
+    if (rc0) return rc0;
     if (P.cap >= B) return CS_OK;
     free_workspace(ctx, P);
     NetShape S(P.dim);
@@ -116,14 +211,11 @@ cs_status ensure_workspace(cs_ctx *ctx, Predictor &P, int64_t B) {
         Si = So;
         C = S.ch;
     }
-    const int64_t win = int64_t(S.cin) * S.positions(S.S0);
     cs_status rc;
     if ((rc = dalloc(ctx, &P.z5, size_t(B * S.hidden))) || (rc = dalloc(ctx, &P.a5, size_t(B * S.hidden))) ||
-        (rc = dalloc(ctx, &P.out, size_t(B * S.dim))) || (rc = dalloc(ctx, &P.gout, size_t(B * S.dim))) ||
-        (rc = dalloc(ctx, &P.dcol, size_t(max_col))) || (rc = dalloc(ctx, &P.dy0, size_t(max_dy))) ||
-        (rc = dalloc(ctx, &P.dy1, size_t(max_dy))) || (rc = dalloc(ctx, &P.da5, size_t(B * S.hidden))) ||
-        (rc = dalloc(ctx, &P.win, size_t(B * win))) || (rc = dalloc(ctx, &P.tgt, size_t(B * S.dim))) ||
-        (rc = dalloc(ctx, &P.idx, size_t(B))) ||
+        (rc = dalloc(ctx, &P.gout, size_t(B * S.dim))) || (rc = dalloc(ctx, &P.dcol, size_t(max_col))) ||
+        (rc = dalloc(ctx, &P.dy0, size_t(max_dy))) || (rc = dalloc(ctx, &P.dy1, size_t(max_dy))) ||
+        (rc = dalloc(ctx, &P.da5, size_t(B * S.hidden))) ||
         (rc = dalloc(ctx, &P.splitk, size_t(tc_gemm_work_floats(ctx->sm_count)))))
         return rc;
     P.splitk_n = tc_gemm_work_floats(ctx->sm_count);
@@ -212,6 +304,90 @@ int backward(cs_ctx *ctx, Predictor &P, int64_t B, const float *tgt, float *loss
     return n;
 }
 
+// The fused path's forward pass of B windows into P.out; with targets the
+// gradients of the mean squared error into P.g as well, the loss added to
+// *loss. Every sum over the batch is one of partials in a fixed order.
+int forward_fused(cs_ctx *ctx, Predictor &P, int64_t B, const float *win, const float *tgt,
+                  cudaStream_t st) {
+    const NetShape S(P.dim);
+    const FusedPack K(S);
+    const int sm = ctx->sm_count;
+    PackSeg ps[kMaxPack];
+    for (int l = 0; l < S.n_conv; ++l)
+        ps[l] = PackSeg{P.w + S.w_off[l], (l == 0 ? S.cin : S.ch) * S.taps(), train_packed_kw(S.dim),
+                        P.fpack + K.fwd[l], tgt && l > 0 ? P.fpack + K.bwd[l] : nullptr, nullptr};
+    ps[S.n_conv] = PackSeg{P.w + S.w_off[S.n_conv], 0, 0, nullptr, nullptr, P.fpack + K.fc1};
+    int n = launch_pack_train(ps, S.n_conv + 1, st);
+    for (int l = 0; l < S.n_conv; ++l) {
+        const ConvGeo g(P.dim, l == 0 ? S.cin : S.ch, S.S0 - 2 * l);
+        n += launch_conv_fwd(g, l == 0 ? static_cast<const void *>(win) : P.fy[l - 1], l == 0, B,
+                             P.fpack + K.fwd[l], P.w + S.b_off[l], P.fy[l], 0, nullptr, ctx->dev_err,
+                             sm, st);
+    }
+    const int f1 = S.n_conv, f2 = S.n_conv + 1;
+    n += launch_train_head(P.dim, B, P.fy[S.n_conv - 1], P.fpack + K.fc1, P.w + S.b_off[f1],
+                           P.w + S.w_off[f2], P.w + S.b_off[f2], tgt, P.out,
+                           tgt ? P.fdz[S.n_conv - 1] : nullptr, P.fpart, ctx->dev_err, sm, st);
+    return n;
+}
+
+int train_fused(cs_ctx *ctx, Predictor &P, int64_t B, const float *win, const float *tgt,
+                float *loss, cudaStream_t st) {
+    const NetShape S(P.dim);
+    const int sm = ctx->sm_count;
+    const FusedPack K(S);
+    int n = forward_fused(ctx, P, B, win, tgt, st);
+    const int f1 = S.n_conv, f2 = S.n_conv + 1;
+    // the head's partials, then each convolution's
+    ReduceSeg seg[kMaxSegs];
+    int ns = 0;
+    const int hc = head_ctas(B, sm);
+    const int64_t hs = head_part_floats(P.dim);
+    float *part = P.fpart;
+    auto add = [&](const float *p, int64_t stride, int64_t count, float *out, int parts, float div) {
+        seg[ns++] = ReduceSeg{p, stride, count, out, parts, div};
+    };
+    int64_t o = 0;
+    add(part + o, hs, S.hidden * S.ch, P.g + S.w_off[f1], hc, 0.f);
+    o += S.hidden * S.ch;
+    add(part + o, hs, S.hidden, P.g + S.b_off[f1], hc, 0.f);
+    o += S.hidden;
+    add(part + o, hs, S.dim * S.hidden, P.g + S.w_off[f2], hc, 0.f);
+    o += S.dim * S.hidden;
+    add(part + o, hs, S.dim, P.g + S.b_off[f2], hc, 0.f);
+    o += S.dim;
+    add(part + o, hs, S.ch, P.g + S.b_off[S.n_conv - 1], hc, 0.f);
+    o += S.ch;
+    add(part + o, hs, 1, loss, hc, float(B * S.dim));
+    part += hs * hc;
+    for (int l = S.n_conv - 1; l >= 0; --l) {
+        const ConvGeo g(P.dim, l == 0 ? S.cin : S.ch, S.S0 - 2 * l);
+        const int ctas = conv_bwd_ctas(g, B, l == 0, sm);
+        float *wpart = part, *bpart = part + int64_t(ctas) * g.K * S.ch;
+        part = bpart + int64_t(ctas) * S.ch;
+        n += launch_conv_bwd(g, l == 0 ? static_cast<const void *>(win) : P.fy[l - 1], l == 0, B,
+                             P.fdz[l], P.fpack + K.bwd[l], wpart, l > 0 ? P.fdz[l - 1] : nullptr, 0,
+                             bpart, ctx->dev_err, sm, st);
+        add(wpart, int64_t(g.K) * S.ch, int64_t(g.K) * S.ch, P.g + S.w_off[l], ctas, 0.f);
+        if (l > 0) add(bpart, S.ch, S.ch, P.g + S.b_off[l - 1], ctas, 0.f);
+    }
+    return n + launch_reduce_parts(seg, ns, st);
+}
+
+// forward of B windows into P.out through whichever path takes the batch, and
+// the buffers of chunks of `rows` and a last one of `rest`
+int forward_any(cs_ctx *ctx, Predictor &P, int64_t B, const float *win, cudaStream_t st) {
+    return fused_batch(B) ? forward_fused(ctx, P, B, win, nullptr, st) : forward(ctx, P, B, win, st);
+}
+
+cs_status ensure_fwd(cs_ctx *ctx, Predictor &P, int64_t rows, int64_t rest) {
+    cs_status rc = CS_OK;
+    if (fused_batch(rows)) rc = ensure_fused(ctx, P, rows, false);
+    if (rc == CS_OK && !fused_batch(rows)) rc = ensure_workspace(ctx, P, rows);
+    if (rc == CS_OK && rest > 0 && !fused_batch(rest)) rc = ensure_workspace(ctx, P, rest);
+    return rc;
+}
+
 Predictor *get_pred(cs_ctx *ctx, int dim) {
     if (dim != 2 && dim != 3) return nullptr;
     return &ctx->pred[dim - 2];
@@ -264,6 +440,8 @@ namespace cs {
 
 void predictor_release(cs_ctx *ctx, Predictor &P) {
     free_workspace(ctx, P);
+    free_io(ctx, P);
+    free_fused(ctx, P);
     float **fs[] = {&P.w, &P.g, &P.m, &P.v, &P.loss};
     for (float **f : fs) {
         dfree(ctx, *f);
@@ -432,7 +610,8 @@ cs_status predict_grid_src(cs_ctx *ctx, cs::Mesh *m, const TcSource &src, double
     }
     if (m->d.dim == 3 && ctx->engine == 2) return predict_tiles(ctx, *P, m, grid, dt, dhat, st);
     const int64_t chunk = 8192;
-    cs_status rc = ensure_workspace(ctx, *P, chunk);
+    cs_status rc = ensure_io(ctx, *P, chunk);
+    if (rc == CS_OK) rc = ensure_fwd(ctx, *P, chunk, m->d.n_pasg % chunk);
     if (rc) return rc;
     const int D = m->d.dim;
     float scale[3] = {0, 0, 0};
@@ -441,7 +620,7 @@ cs_status predict_grid_src(cs_ctx *ctx, cs::Mesh *m, const TcSource &src, double
         const int64_t B = std::min(chunk, pred_view(m->d).n_asg - c0);
         ctx->launches += launch_windows(pred_view(m->d), grid, nullptr, c0, B, scale, P->win,
                                         ctx->sm_count, st);
-        ctx->launches += forward(ctx, *P, B, P->win, st);
+        ctx->launches += forward_any(ctx, *P, B, P->win, st);
         PCHK(cudaMemcpyAsync(dhat + c0 * D, P->out, size_t(B) * D * sizeof(float),
                              cudaMemcpyDeviceToDevice, st));
     }
@@ -777,16 +956,19 @@ cs_status cs_predictor_forward(cs_ctx *ctx, int dim, int64_t B, const float *win
     if (!P->loaded) return fail(ctx, CS_ENOPRED, "cs_predictor_forward: no predictor loaded");
     PCHK(cudaSetDevice(ctx->device));
     const int64_t chunk = 8192;
-    cs_status rc = ensure_workspace(ctx, *P, std::min<int64_t>(std::max<int64_t>(B, 1), chunk));
+    const int64_t rows = std::min<int64_t>(std::max<int64_t>(B, 1), chunk);
+    cs_status rc = ensure_io(ctx, *P, rows);
+    if (rc == CS_OK) rc = ensure_fwd(ctx, *P, rows, B % rows);
     if (rc) return rc;
     NetShape S(dim);
     const int64_t row = int64_t(S.cin) * S.positions(S.S0);
-    for (int64_t b0 = 0; b0 < B; b0 += P->cap) {
-        const int64_t nb = std::min(P->cap, B - b0);
-        ctx->launches += forward(ctx, *P, nb, windows + b0 * row, nullptr);
+    for (int64_t b0 = 0; b0 < B; b0 += rows) {
+        const int64_t nb = std::min(rows, B - b0);
+        ctx->launches += forward_any(ctx, *P, nb, windows + b0 * row, nullptr);
         PCHK(cudaMemcpyAsync(dhat_out + b0 * dim, P->out, size_t(nb) * dim * sizeof(float),
                              cudaMemcpyDeviceToDevice, nullptr));
     }
+    PCHK(cudaGetLastError());
     PCHK(cudaDeviceSynchronize());
     return CS_OK;
 }
@@ -815,7 +997,9 @@ cs_status cs_predictor_train(cs_ctx *ctx, int dim, const float *windows, const f
     if (!P->loaded) return fail(ctx, CS_ENOPRED, "cs_predictor_train: no predictor loaded");
     PCHK(cudaSetDevice(ctx->device));
     const int64_t B = std::min(batch, N);
-    cs_status rc = ensure_workspace(ctx, *P, B);
+    const bool fused = fused_batch(B);
+    cs_status rc = ensure_io(ctx, *P, B);
+    if (rc == CS_OK) rc = fused ? ensure_fused(ctx, *P, B, true) : ensure_workspace(ctx, *P, B);
     if (rc) return rc;
     NetShape S(dim);
     const int64_t row = int64_t(S.cin) * S.positions(S.S0);
@@ -843,14 +1027,19 @@ cs_status cs_predictor_train(cs_ctx *ctx, int dim, const float *windows, const f
         }
         ctx->launches += launch_gather_rows(windows, row, P->idx, B, P->win, ctx->sm_count, nullptr);
         ctx->launches += launch_gather_rows(targets, dim, P->idx, B, P->tgt, ctx->sm_count, nullptr);
-        ctx->launches += forward(ctx, *P, B, P->win, nullptr);
-        ctx->launches += backward(ctx, *P, B, P->tgt, losses + s, nullptr);
+        if (fused) {
+            ctx->launches += train_fused(ctx, *P, B, P->win, P->tgt, losses + s, nullptr);
+        } else {
+            ctx->launches += forward(ctx, *P, B, P->win, nullptr);
+            ctx->launches += backward(ctx, *P, B, P->tgt, losses + s, nullptr);
+        }
         P->t += 1;
         ctx->launches += launch_adam(P->w, P->g, P->m, P->v, P->n, lr, P->t, ctx->sm_count, nullptr);
         P->packed_dirty = true;
     }
     if (out == CS_OK) {
-        cudaError_t e = cudaDeviceSynchronize();
+        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaDeviceSynchronize();
         if (e == cudaSuccess && loss_out && steps > 0)
             e = cudaMemcpy(loss_out, losses, size_t(steps) * sizeof(float), cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) out = fail(ctx, CS_ECUDA, std::string("cs_predictor_train: ") +
@@ -889,11 +1078,18 @@ cs_status cs_predictor_grad(cs_ctx *ctx, int dim, int64_t B, const float *window
         return fail(ctx, CS_EINVAL, "cs_predictor_grad: bad arguments");
     if (!P->loaded) return fail(ctx, CS_ENOPRED, "cs_predictor_grad: no predictor loaded");
     PCHK(cudaSetDevice(ctx->device));
-    cs_status rc = ensure_workspace(ctx, *P, B);
+    const bool fused = fused_batch(B);
+    cs_status rc = ensure_io(ctx, *P, B);
+    if (rc == CS_OK) rc = fused ? ensure_fused(ctx, *P, B, true) : ensure_workspace(ctx, *P, B);
     if (rc) return rc;
     PCHK(cudaMemset(P->loss, 0, sizeof(float)));
-    ctx->launches += forward(ctx, *P, B, windows, nullptr);
-    ctx->launches += backward(ctx, *P, B, targets, P->loss, nullptr);
+    if (fused) {
+        ctx->launches += train_fused(ctx, *P, B, windows, targets, P->loss, nullptr);
+    } else {
+        ctx->launches += forward(ctx, *P, B, windows, nullptr);
+        ctx->launches += backward(ctx, *P, B, targets, P->loss, nullptr);
+    }
+    PCHK(cudaGetLastError());
     PCHK(cudaDeviceSynchronize());
     PCHK(cudaMemcpy(grad_out, P->g, size_t(P->n) * sizeof(float), cudaMemcpyDeviceToDevice));
     if (loss_out) PCHK(cudaMemcpy(loss_out, P->loss, sizeof(float), cudaMemcpyDeviceToHost));

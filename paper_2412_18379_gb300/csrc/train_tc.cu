@@ -1,0 +1,1106 @@
+// Training of the convolutional networks on the tensor cores: every
+// convolution's forward pass, weight gradient and input gradient as implicit
+// GEMMs (tcgen05) without an im2col copy in global memory, and the
+// regressor's head (both fully connected layers, the loss and their
+// gradients) in one kernel.
+//
+// Tiles. A CTA takes G whole inputs whose G Po output positions fill the 128
+// rows of an MMA tile (row = position of input 0, 1, ..). It keeps their
+// activations in shared memory and lays the im2col operand A[row][k] out
+// there, k = channel * taps + tap as the weights are stored. The operand
+// layout [k / 8][row][k % 8] is K-major for the forward product (K = k) and,
+// read with the transposed (MN-major) descriptor, the left operand of the
+// weight gradient (K = row), so the backward pass builds it once for both.
+//
+//   forward   z[row][o]  = sum_k A[row][k] W[o][k]        M = rows, N = 32
+//   weights   dW[k][o]   = sum_rows A[row][k] dz[row][o]  M = k,    N = 32
+//   columns   dcol[row][k] = sum_o dz[row][o] W[o][k]     M = rows, N = taps * channels
+//   col2im    dx[q][c]   = sum_t dcol[row(q, t)][c taps + t], in shared memory
+//
+// The sums over k and o run in the K order and K = 16 steps of the general
+// GEMM (tc_gemm.cu), and dx adds its taps in increasing order, so activations
+// and input gradients are that path's bits. Weight gradients accumulate over
+// a CTA's tiles in TMEM; the CTAs' partials are summed in a fixed order.
+//
+// What bounds it: not the tensor pipe but the operand build (8 two-byte
+// shared loads and one 16-byte store per 8 elements) and the col2im gather;
+// global traffic is the BF16 activations and gradients alone. At a batch of
+// 4096 the 2-D step's im2col, GEMM, col2im and ReLU kernels moved about
+// 1.2 GB through FP32 buffers.
+#include <cuda_bf16.h>
+
+#include <algorithm>
+#include <cstdint>
+
+#include "tc_common.cuh"
+#include "train_tc.h"
+
+namespace cs {
+namespace {
+
+constexpr int kPitch = 34;        // halves per position in shared memory (17 words: no conflicts)
+constexpr int kFwdThreads = 256;
+constexpr int kBwdThreads = 512;
+constexpr int kRowsT = 128;       // MMA rows
+constexpr int kChunk = kRowsT * 16;   // bytes of one 8-element K chunk of A
+
+struct ConvArgs {
+    const void *x;
+    int64_t B, tiles;
+    int G;                        // inputs per tile
+    const uint8_t *w;             // packed weights of the pass
+    // forward
+    const float *bias;
+    uint16_t *y;
+    float *z;
+    int nsplit, kc;               // K splits of the sum (kc a multiple of 64)
+    // backward
+    const uint16_t *dz;
+    float *wpart, *bpart;
+    uint16_t *dzp;
+    int ring;                     // forward: of y; backward: of x
+};
+
+// one layer's geometry: inputs of edge Si, channels first FP32 (First: the
+// network's input, D channels) or [pos][32] BF16
+template <int D, int SI, bool FIRST>
+struct Geo {
+    static constexpr int Dim = D, Si = SI, So = SI - 2;
+    static constexpr bool First = FIRST;
+    static constexpr int Pi = D == 2 ? Si * Si : Si * Si * Si;
+    static constexpr int Po = D == 2 ? So * So : So * So * So;
+    static constexpr int Taps = D == 2 ? 9 : 27;
+    static constexpr int C = FIRST ? D : kTrainCh;
+    static constexpr int K = C * Taps;
+    static constexpr int Kp = (K + 15) / 16 * 16, Chunks = Kp / 8;
+    static constexpr int GMax = kRowsT / Po;
+    static constexpr int ActHalves = FIRST ? C * Pi : Pi * kPitch;   // per input
+};
+
+// shared memory of one CTA (bytes); A first, then the activations
+struct ConvSmem {
+    int act, w, dz, tab, bar, total;
+};
+
+template <class N, bool BWD>
+struct ConvCfg {
+    static constexpr int D = N::Dim;
+    // K chunks (of 8) per operand build and buffers of them: a 2-D operand
+    // fits whole (36 chunks); a 3-D one (108) is built in pieces
+    static constexpr int CbMax = D == 2 ? 36 : BWD ? 32 : 28;
+    static constexpr int Cb = N::Chunks < CbMax ? N::Chunks : CbMax;
+    static constexpr int Nb = D == 2 || BWD || N::First ? 1 : 2;
+    // backward: channels, columns and MMA N of one dcol pass
+    static constexpr int Ch = D == 2 ? 16 : 8;
+    static constexpr int Nc = Ch * N::Taps;                  // 144, 216
+    static constexpr int Nm = (Nc + 15) / 16 * 16;           // 144, 224
+    static constexpr int Ld = Nc + 1;                        // dcol row stride (odd: no conflicts)
+    static constexpr int Passes = kTrainCh / Ch;
+    static constexpr bool Dgrad = BWD && !N::First;
+    static constexpr int Kw = D == 2 ? 288 : 872;            // rows of the dgrad weights
+    static constexpr int Dcol = Dgrad ? kRowsT * Ld * 4 : 0;
+    static constexpr int A = Nb * Cb * kChunk > Dcol ? Nb * Cb * kChunk : Dcol;
+    static constexpr int Mt = (N::K + 127) / 128;            // M-tiles of the weight gradient
+    static constexpr int WBytes = !BWD ? N::Kp * kTrainCh * 2 : Dgrad ? Kw * kTrainCh * 2 : 0;
+    static_assert((Passes - 1) * Nc + Nm <= Kw, "dgrad weight rows");
+    static_assert(256 + Nm <= 512 && 32 * Mt <= 256, "TMEM columns");
+    static_assert(Cb % 16 == 0 || Cb == N::Chunks || !BWD, "builds end on an M-tile");
+    static_assert(Cb % 2 == 0, "whole K = 16 steps per build");
+};
+
+template <class N, bool BWD>
+constexpr ConvSmem conv_smem(int G) {
+    using F = ConvCfg<N, BWD>;
+    ConvSmem s{};
+    s.act = F::A;
+    s.w = s.act + (G * N::ActHalves * 2 + 127) / 128 * 128;
+    s.dz = s.w + F::WBytes;
+    s.tab = s.dz + (BWD ? kTrainCh * kRowsT * 2 : 0);
+    s.bar = (s.tab + N::Kp * 2 + 127) / 128 * 128;
+    s.total = s.bar + 64;
+    // an M-tile of the weight gradient reads 16 chunks from its first one,
+    // past the built ones at the end (rows of no use): inside the allocation
+    const int reach = (F::Cb + 15) / 16 * 16 * kChunk;
+    if (BWD && s.total < reach) s.total = reach;
+    return s;
+}
+
+// The activations of inputs [b0, b0 + nb) on their way to shared memory:
+// start() issues the loads, finish() makes them visible to the caller (the
+// CTA still has to synchronise). BF16 activations travel as 4-byte
+// asynchronous copies into the padded rows; the network's FP32 input waits in
+// registers and is rounded as it is stored, channels first.
+template <class N, int NTH>
+struct ActLoad {
+    static constexpr int Regs = N::First ? (N::GMax * N::C * N::Pi + NTH - 1) / NTH : 1;
+    float r[Regs];
+    __device__ __forceinline__ void start(const ConvArgs &a, int64_t b0, int nb, uint8_t *act,
+                                          int tid) {
+        if constexpr (N::First) {
+            const int n = nb * N::C * N::Pi;
+            const float *src = static_cast<const float *>(a.x) + b0 * N::C * N::Pi;
+            #pragma unroll
+            for (int j = 0; j < Regs; ++j)
+                r[j] = tid + j * NTH < n ? __ldg(src + tid + j * NTH) : 0.f;
+        } else {
+            const int n = nb * N::Pi * 16;
+            const uint32_t *src = reinterpret_cast<const uint32_t *>(
+                static_cast<const uint16_t *>(a.x) + b0 * N::Pi * kTrainCh);
+            for (int i = tid; i < n; i += NTH) {
+                const uint32_t d = smem_addr(act) + ((i >> 4) * (kPitch / 2) + (i & 15)) * 4;
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src + i)
+                             : "memory");
+            }
+        }
+    }
+    __device__ __forceinline__ void finish(int nb, uint8_t *act, int tid) {
+        if constexpr (N::First) {
+            const int n = nb * N::C * N::Pi;
+            #pragma unroll
+            for (int j = 0; j < Regs; ++j)
+                if (tid + j * NTH < n)
+                    reinterpret_cast<__nv_bfloat16 *>(act)[tid + j * NTH] = __float2bfloat16_rn(r[j]);
+        } else {
+            cp_async_wait_all();
+        }
+    }
+};
+
+// offset (in halves) of operand column k from its row's base, 0xffff past K
+template <class N>
+__device__ __forceinline__ void fill_tab(uint16_t *tab, int tid, int nth) {
+    for (int k = tid; k < N::Kp; k += nth) {
+        const int i = k / N::Taps, t = k % N::Taps;
+        const int dx = t % 3, dy = (t / 3) % 3, dz = N::Dim == 3 ? t / 9 : 0;
+        const int to = (dz * N::Si + dy) * N::Si + dx;
+        tab[k] = k >= N::K ? 0xffffu : uint16_t(N::First ? i * N::Pi + to : to * kPitch + i);
+    }
+}
+
+// base (in halves) of row r's window, -1 where the row holds no output
+template <class N>
+__device__ __forceinline__ int row_base(int nb, int r) {
+    const int w = r / N::Po, p = r % N::Po;
+    if (w >= nb) return -1;
+    const int px = p % N::So, q = p / N::So;
+    const int pb = N::Dim == 2 ? q * N::Si + px : ((q / N::So) * N::Si + q % N::So) * N::Si + px;
+    return w * N::ActHalves + pb * (N::First ? 1 : kPitch);
+}
+
+// chunks [c0, c0 + nc) of the im2col operand into `dst`; a warp takes 32 rows
+// of one chunk at a time, so its loads step by one position per lane
+template <class N, int NWARPS, int CB>
+__device__ __forceinline__ void build_operand(uint8_t *dst, const uint8_t *act,
+                                              const uint16_t *tab, int base, int c0, int nc,
+                                              int warp, int lane) {
+    constexpr int Step = NWARPS / 4;
+    const int row = 32 * (warp & 3) + lane;
+    const uint16_t *s = reinterpret_cast<const uint16_t *>(act) + (base < 0 ? 0 : base);
+    const uint32_t keep = base < 0 ? 0u : 0xffffffffu;
+    #pragma unroll 3
+    for (int i = 0; i < (CB + Step - 1) / Step; ++i) {
+        const int c = (warp >> 2) + i * Step;
+        if (c >= nc) break;
+        const uint4 t = *reinterpret_cast<const uint4 *>(tab + 8 * (c0 + c));
+        const uint32_t tw[4] = {t.x, t.y, t.z, t.w};
+        uint32_t v[4];
+        if (N::K % 8 == 0 || 8 * (c0 + c) + 8 <= N::K) {
+            #pragma unroll
+            for (int j = 0; j < 4; ++j)
+                v[j] = uint32_t(s[tw[j] & 0xffffu]) | (uint32_t(s[tw[j] >> 16]) << 16);
+        } else {   // the last chunk: zero past K
+            #pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t k0 = tw[j] & 0xffffu, k1 = tw[j] >> 16;
+                v[j] = (k0 == 0xffffu ? 0u : uint32_t(s[k0])) |
+                       (k1 == 0xffffu ? 0u : uint32_t(s[k1]) << 16);
+            }
+        }
+        *reinterpret_cast<uint4 *>(dst + c * kChunk + row * 16) =
+            make_uint4(v[0] & keep, v[1] & keep, v[2] & keep, v[3] & keep);
+    }
+}
+
+__device__ __forceinline__ void tmem_alloc(uint32_t *slot, uint32_t cols) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_addr(slot)),
+                 "r"(cols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+}
+__device__ __forceinline__ void tmem_free(uint32_t tmem, uint32_t cols) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols));
+}
+
+// wait (bounded) for the CTA's MMAs in flight, then release TMEM. Every
+// thread of the CTA calls it; `bar` has no phase in use.
+__device__ __forceinline__ void mma_drain(uint64_t *bar, uint32_t tmem, uint32_t cols, int warp) {
+    if (warp == 0) {
+        if (elect_one()) {
+            mma_commit(bar);
+            for (uint32_t i = 0; i < (1u << 24) && !mbar_try_wait(bar, 0); ++i)
+                if (i > 64) __nanosleep(64);
+        }
+        __syncwarp();
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    if (warp == 0) tmem_free(tmem, cols);
+}
+
+// a BF16 value above zero: an open ReLU
+__device__ __forceinline__ bool positive(uint16_t h) { return h != 0 && h < 0x8000u; }
+
+template <class N>
+__global__ void __launch_bounds__(kFwdThreads, 2) conv_fwd_kernel(const ConvArgs a,
+                                                                  const ConvSmem L, int *err) {
+    using F = ConvCfg<N, false>;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    uint8_t *act = smem + L.act, *wop = smem + L.w;
+    uint16_t *tab = reinterpret_cast<uint16_t *>(smem + L.tab);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L.bar);   // [Nb] builds, then the drain
+    uint32_t *slot = reinterpret_cast<uint32_t *>(smem + L.bar + 32);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + L.bar + 40);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr uint32_t kCols = 128;
+    constexpr int kNw = kFwdThreads / 32;
+
+    if (tid == 0) {
+        for (int i = 0; i < 3; ++i) mbar_init(bars + i, 1u);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) tmem_alloc(slot, kCols);
+    fill_tab<N>(tab, tid, kFwdThreads);
+    // the kernel before this one wrote its inputs
+    pdl_wait();
+    for (int i = tid; i < F::WBytes / 16; i += kFwdThreads) cp_async16(wop + 16 * i, a.w + 16 * i);
+    ActLoad<N, kFwdThreads> ld;
+    int64_t t = blockIdx.x;
+    int nb = int(min(int64_t(a.G), a.B - t * a.G));
+    ld.start(a, t * a.G, nb, act, tid);
+    cp_async_wait_all();
+    fence_async_smem();
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = *slot;
+    constexpr uint32_t id = idesc_bf16(128, 32);
+    const uint64_t dw = sdesc(smem_addr(wop), kTrainCh * 16, 128);
+    const int edge = N::So + 2 * a.ring;
+    const int np = N::Dim == 2 ? edge * edge : edge * edge * edge;
+    // this thread's output row and columns
+    const int r = 32 * (warp & 3) + lane, o0 = 16 * (warp >> 2);
+    const int ow = r / N::Po, op = r % N::Po;
+    const int qx = op % N::So + a.ring, qy = (op / N::So) % N::So + a.ring;
+    const int qz = N::Dim == 3 ? op / (N::So * N::So) + a.ring : 0;
+    const int opos = (qz * edge + qy) * edge + qx;
+    bool ok = true;
+    int it = 0;
+    while (t < a.tiles) {
+        const int64_t b0 = t * a.G;
+        ld.finish(nb, act, tid);
+        const int base = row_base<N>(nb, r);
+        __syncthreads();
+        for (int c0 = 0; c0 < N::Chunks && ok; c0 += F::Cb, ++it) {
+            const int buf = F::Nb == 1 ? 0 : it % F::Nb, nc = min(F::Cb, N::Chunks - c0);
+            // the buffer's previous MMAs are complete (one build per tile: the
+            // tile before waited for them)
+            if (F::Cb < N::Chunks && it >= F::Nb)
+                ok = __syncthreads_and(
+                    mbar_wait(bars + buf, uint32_t(it / F::Nb - 1) & 1u, abort_flag, err));
+            if (!ok) break;
+            uint8_t *A = smem + buf * F::Cb * kChunk;
+            build_operand<N, kNw, F::Cb>(A, act, tab, base, c0, nc, warp, lane);
+            fence_async_smem();
+            fence_before();
+            __syncthreads();
+            fence_after();
+            if (warp == 0) {
+                if (elect_one()) {
+                    const uint64_t da = sdesc(smem_addr(A), kChunk, 128);
+                    #pragma unroll 4
+                    for (int q = 0; q < nc / 2; ++q) {
+                        const int k = 8 * c0 + 16 * q;
+                        const int s = N::K > 512 && a.nsplit > 1 ? k / a.kc : 0;
+                        mma_bf16(tmem + uint32_t(32 * s), da + uint64_t(2 * q * (kChunk >> 4)),
+                                 dw + uint64_t((c0 + 2 * q) * kTrainCh), id,
+                                 k - s * a.kc > 0 ? 1u : 0u);
+                    }
+                    mma_commit(bars + buf);
+                }
+                __syncwarp();
+            }
+        }
+        if (!ok) break;
+        // the activations are in the operand: fetch the next tile's
+        const int nb_now = nb;
+        t += gridDim.x;
+        if (t < a.tiles) {
+            nb = int(min(int64_t(a.G), a.B - t * a.G));
+            ld.start(a, t * a.G, nb, act, tid);
+        }
+        // the tile's last build completes after all others
+        ok = __syncthreads_and(mbar_wait(bars + (F::Nb == 1 ? 0 : (it - 1) % F::Nb),
+                                         uint32_t((it - 1) / F::Nb) & 1u, abort_flag, err));
+        if (!ok) break;
+        fence_after();
+        const uint32_t tq = tmem + (uint32_t(32 * (warp & 3)) << 16) + uint32_t(o0);
+        float v[16];
+        tmem_ld16(tq, v);
+        if (N::K > 512 && a.nsplit > 1) {
+            for (int s = 1; s < a.nsplit; ++s) {
+                float u[16];
+                tmem_ld16(tq + uint32_t(32 * s), u);
+                #pragma unroll
+                for (int e = 0; e < 16; ++e) v[e] += u[e];
+            }
+        }
+        fence_before();
+        if (ow < nb_now) {
+            #pragma unroll
+            for (int e = 0; e < 16; ++e) v[e] += __ldg(a.bias + o0 + e);
+            if (a.y) {
+                uint32_t h[8];
+                #pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    h[e] = pack_bf16x2(fmaxf(v[2 * e], 0.f), fmaxf(v[2 * e + 1], 0.f));
+                uint4 *d = reinterpret_cast<uint4 *>(a.y + ((b0 + ow) * np + opos) * kTrainCh + o0);
+                d[0] = make_uint4(h[0], h[1], h[2], h[3]);
+                d[1] = make_uint4(h[4], h[5], h[6], h[7]);
+            }
+            if (a.z) {
+                float4 *d = reinterpret_cast<float4 *>(a.z + ((b0 + ow) * N::Po + op) * kTrainCh + o0);
+                #pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    d[e] = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+            }
+        }
+    }
+    cp_async_wait_all();
+    mma_drain(bars + 2, tmem, kCols, warp);
+}
+
+// dx of one line of Si input positions (fixed window, channel, y and z) from
+// the tile's dcol: for every tap line (ty, tz) whose output line exists, tap
+// by tap in increasing order
+template <class N, int LD>
+__device__ __forceinline__ void col2im_line(const float *dcol, int row0, int iy, int iz,
+                                            float *s) {
+    #pragma unroll
+    for (int i = 0; i < N::Si; ++i) s[i] = 0.f;
+    #pragma unroll
+    for (int tz = 0; tz < (N::Dim == 3 ? 3 : 1); ++tz) {
+        const int z = iz - tz;
+        if (N::Dim == 3 && unsigned(z) >= unsigned(N::So)) continue;
+        #pragma unroll
+        for (int ty = 0; ty < 3; ++ty) {
+            const int y = iy - ty;
+            if (unsigned(y) >= unsigned(N::So)) continue;
+            const float *d = dcol + (row0 + ((N::Dim == 3 ? z * N::So : 0) + y) * N::So) * LD +
+                             (tz * 3 + ty) * 3;
+            #pragma unroll
+            for (int tx = 0; tx < 3; ++tx)
+                #pragma unroll
+                for (int x = 0; x < N::So; ++x) s[x + tx] += d[x * LD + tx];
+        }
+    }
+}
+
+template <class N>
+__global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs a,
+                                                                  const ConvSmem L, int *err) {
+    using F = ConvCfg<N, true>;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    uint8_t *act = smem + L.act, *wop = smem + L.w, *dzs = smem + L.dz;
+    float *dcol = reinterpret_cast<float *>(smem);          // over A once its MMAs are complete
+    uint16_t *tab = reinterpret_cast<uint16_t *>(smem + L.tab);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L.bar);   // MMAs, drain
+    uint32_t *slot = reinterpret_cast<uint32_t *>(smem + L.bar + 32);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + L.bar + 40);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr uint32_t kCols = 512, kDcol = 256;
+    constexpr int kNw = kBwdThreads / 32;
+
+    if (tid == 0) {
+        for (int i = 0; i < 2; ++i) mbar_init(bars + i, 1u);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) tmem_alloc(slot, kCols);
+    fill_tab<N>(tab, tid, kBwdThreads);
+    pdl_wait();
+    for (int i = tid; i < F::WBytes / 16; i += kBwdThreads) cp_async16(wop + 16 * i, a.w + 16 * i);
+    ActLoad<N, kBwdThreads> ld;
+    int64_t t = blockIdx.x;
+    int nb = int(min(int64_t(a.G), a.B - t * a.G));
+    // dz of a tile: one 16-byte piece (8 channels of a row) per thread, the
+    // next tile's fetched under this tile's products
+    uint4 dzr;
+    auto fetch_dz = [&]() {
+        const int i = tid, rr = i >> 2;
+        dzr = rr < nb * N::Po ? __ldg(reinterpret_cast<const uint4 *>(a.dz + t * a.G * N::Po * kTrainCh) + i)
+                              : make_uint4(0u, 0u, 0u, 0u);
+    };
+    static_assert(kRowsT * 4 == kBwdThreads, "one piece of dz per thread");
+    ld.start(a, t * a.G, nb, act, tid);
+    fetch_dz();
+    cp_async_wait_all();
+    fence_async_smem();
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = *slot;
+    constexpr uint32_t id_w = idesc_mn(idesc_bf16(128, 32), true, true);
+    constexpr uint32_t id_c = idesc_bf16(128, F::Nm);
+    // dz: K-major (K = channel) for dcol, MN-major (K = row) for the weights
+    const uint64_t dz_k = sdesc(smem_addr(dzs), kChunk, 128);
+    const uint64_t dz_mn = sdesc(smem_addr(dzs), 128, kChunk);
+    const uint64_t w_k = sdesc(smem_addr(wop), F::Kw * 16, 128);
+    float db[F::Passes];
+    #pragma unroll
+    for (int j = 0; j < F::Passes; ++j) db[j] = 0.f;
+    const int crop = N::Si - 2 * a.ring;
+    const int np = N::Dim == 2 ? crop * crop : crop * crop * crop;
+    bool ok = true, any = false;
+    uint32_t phase = 0;
+    while (t < a.tiles) {
+        const int64_t b0 = t * a.G;
+        ld.finish(nb, act, tid);
+        *reinterpret_cast<uint4 *>(dzs + (tid & 3) * kChunk + (tid >> 2) * 16) = dzr;
+        const int base = row_base<N>(nb, 32 * (warp & 3) + lane);
+        __syncthreads();
+        const int ksteps = (nb * N::Po + 15) / 16, nb_now = nb;
+        t += gridDim.x;
+        if (t < a.tiles) {
+            nb = int(min(int64_t(a.G), a.B - t * a.G));
+            fetch_dz();
+        }
+        for (int c0 = 0; c0 < N::Chunks; c0 += F::Cb) {
+            const int nc = min(F::Cb, N::Chunks - c0);
+            build_operand<N, kNw, F::Cb>(smem, act, tab, base, c0, nc, warp, lane);
+            fence_async_smem();
+            fence_before();
+            __syncthreads();
+            fence_after();
+            if (warp == 0) {
+                if (elect_one()) {
+                    for (int mt = 0; mt < (nc + 15) / 16; ++mt) {
+                        const uint64_t da = sdesc(smem_addr(smem) + mt * 16 * kChunk, 128, kChunk);
+                        #pragma unroll 4
+                        for (int q = 0; q < ksteps; ++q)
+                            mma_bf16(tmem + uint32_t(32 * (c0 / 16 + mt)), da + uint64_t(q * 16),
+                                     dz_mn + uint64_t(q * 16), id_w, any || q > 0 ? 1u : 0u);
+                    }
+                    if (F::Dgrad && c0 == 0)
+                        for (int q = 0; q < 2; ++q)
+                            mma_bf16(tmem + kDcol, dz_k + uint64_t(2 * q * (kChunk >> 4)),
+                                     w_k + uint64_t(2 * q * F::Kw), id_c, q > 0 ? 1u : 0u);
+                    mma_commit(bars + 0);
+                }
+                __syncwarp();
+            }
+            // the network's input is not read again: fetch the next tile's
+            if (N::First && t < a.tiles) ld.start(a, t * a.G, nb, act, tid);
+            ok = __syncthreads_and(mbar_wait(bars + 0, phase, abort_flag, err));
+            phase ^= 1u;
+            if (!ok) break;
+            fence_after();
+        }
+        if (!ok) break;
+        any = true;
+        if constexpr (F::Dgrad) {
+            #pragma unroll
+            for (int j = 0; j < F::Passes; ++j) {
+                // dcol of channels [Ch j, Ch j + Ch) from TMEM to shared memory
+                const uint32_t tq = tmem + kDcol + (uint32_t(32 * (warp & 3)) << 16);
+                float *drow = dcol + (32 * (warp & 3) + lane) * F::Ld;
+                #pragma unroll 1
+                for (int n0 = 16 * (warp >> 2); n0 < F::Nm; n0 += 64) {
+                    float v[16];
+                    tmem_ld16(tq + uint32_t(n0), v);
+                    #pragma unroll
+                    for (int e = 0; e < 16; ++e)
+                        if (F::Nc % 16 == 0 || n0 + e < F::Nc) drow[n0 + e] = v[e];
+                }
+                fence_before();
+                __syncthreads();
+                fence_after();
+                if (j + 1 < F::Passes && warp == 0) {
+                    // the next pass's product runs under this pass's gather
+                    if (elect_one()) {
+                        for (int q = 0; q < 2; ++q)
+                            mma_bf16(tmem + kDcol, dz_k + uint64_t(2 * q * (kChunk >> 4)),
+                                     w_k + uint64_t(2 * q * F::Kw + (j + 1) * F::Nc), id_c,
+                                     q > 0 ? 1u : 0u);
+                        mma_commit(bars + 0);
+                    }
+                    __syncwarp();
+                }
+                // a thread takes lines of one channel
+                constexpr int kLines = N::Dim == 2 ? N::Si : N::Si * N::Si;
+                const int il = tid % F::Ch, c = F::Ch * j + il;
+                float s_db = 0.f;
+                for (int q = tid / F::Ch; q < nb_now * kLines; q += kBwdThreads / F::Ch) {
+                    const int w = q / kLines, l = q % kLines;
+                    const int iy = N::Dim == 2 ? l : l % N::Si, iz = N::Dim == 2 ? 0 : l / N::Si;
+                    const int oy = iy - a.ring, oz = N::Dim == 2 ? 0 : iz - a.ring;
+                    if (unsigned(oy) >= unsigned(crop) || unsigned(oz) >= unsigned(crop)) continue;
+                    float s[N::Si];
+                    col2im_line<N, F::Ld>(dcol + il * N::Taps, w * N::Po, iy, iz, s);
+                    const uint16_t *h = reinterpret_cast<const uint16_t *>(act) +
+                                        (w * N::Pi + l * N::Si) * kPitch + c;
+                    uint16_t *out = a.dzp + ((b0 + w) * np + (oz * crop + oy) * crop) * kTrainCh + c;
+                    #pragma unroll
+                    for (int ix = 0; ix < N::Si; ++ix) {
+                        if (unsigned(ix - a.ring) >= unsigned(crop)) continue;
+                        // through the ReLU of the layer below: its output is positive
+                        const float v = positive(h[ix * kPitch]) ? s[ix] : 0.f;
+                        s_db += v;
+                        out[(ix - a.ring) * kTrainCh] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
+                    }
+                }
+                db[j] += s_db;
+                if (j + 1 < F::Passes) {
+                    ok = __syncthreads_and(mbar_wait(bars + 0, phase, abort_flag, err));
+                    phase ^= 1u;
+                    if (!ok) break;
+                    fence_after();
+                } else {
+                    __syncthreads();
+                    if (t < a.tiles) ld.start(a, t * a.G, nb, act, tid);
+                }
+            }
+            if (!ok) break;
+        }
+    }
+    cp_async_wait_all();
+    if (ok && any) {
+        // this CTA's weight gradient: rows of D are k, columns the output channel
+        float *wp = a.wpart + int64_t(blockIdx.x) * N::K * kTrainCh;
+        if ((warp >> 2) < 2) {
+            const int o0 = 16 * (warp >> 2);
+            for (int mt = 0; mt < F::Mt; ++mt) {
+                float v[16];
+                tmem_ld16(tmem + (uint32_t(32 * (warp & 3)) << 16) + uint32_t(32 * mt + o0), v);
+                const int k = 128 * mt + 32 * (warp & 3) + lane;
+                if (k < N::K) {
+                    #pragma unroll
+                    for (int e = 0; e < 16; ++e) wp[(o0 + e) * N::K + k] = v[e];
+                }
+            }
+        }
+        if constexpr (F::Dgrad) {
+            // column sums of the input gradient: threads of one channel in order
+            float *red = dcol;
+            __syncthreads();
+            #pragma unroll
+            for (int j = 0; j < F::Passes; ++j) red[j * kBwdThreads + tid] = db[j];
+            __syncthreads();
+            if (tid < kTrainCh) {
+                const float *r = red + (tid / F::Ch) * kBwdThreads + tid % F::Ch;
+                float s = 0.f;
+                for (int i = 0; i < kBwdThreads / F::Ch; ++i) s += r[i * F::Ch];
+                a.bpart[int64_t(blockIdx.x) * kTrainCh + tid] = s;
+            }
+        }
+    }
+    mma_drain(bars + 1, tmem, kCols, warp);
+}
+
+// Weights of one convolution (FP32 W[32][K]) as the operands of both passes:
+// forward bf16 [Kp / 8][32][8] and, with dgrad, backward [4][Kw][8] (zero past K).
+// Weights of fc1 (W1[256][32]) the same way: bf16 [4][256][8].
+struct PackArgs {
+    PackSeg seg[kMaxPack];
+    int n;
+};
+__global__ void __launch_bounds__(256) pack_train_kernel(const PackArgs a) {
+    const int nth = gridDim.x * 256, tid = blockIdx.x * 256 + threadIdx.x;
+    pdl_wait();
+    for (int s = 0; s < a.n; ++s) {
+        const PackSeg &g = a.seg[s];
+        const int kp = (g.K + 15) / 16 * 16;
+        __nv_bfloat16 *f = reinterpret_cast<__nv_bfloat16 *>(g.fwd);
+        if (f)
+            for (int e = tid; e < kTrainCh * kp; e += nth) {
+                const int j = e & 7, o = (e >> 3) & 31, k = (e >> 8) * 8 + j;
+                f[e] = __float2bfloat16_rn(k < g.K ? __ldg(g.W + o * g.K + k) : 0.f);
+            }
+        __nv_bfloat16 *b = reinterpret_cast<__nv_bfloat16 *>(g.bwd);
+        if (b)
+            for (int e = tid; e < kTrainCh * g.kw; e += nth) {
+                const int j = e & 7, k = (e >> 3) % g.kw, o = (e >> 3) / g.kw * 8 + j;
+                b[e] = __float2bfloat16_rn(k < g.K ? __ldg(g.W + o * g.K + k) : 0.f);
+            }
+        __nv_bfloat16 *h = reinterpret_cast<__nv_bfloat16 *>(g.fc1);
+        if (h)
+            for (int e = tid; e < kTrainCh * 256; e += nth) {
+                const int j = e & 7, n = (e >> 3) & 255, c = (e >> 11) * 8 + j;
+                h[e] = __float2bfloat16_rn(__ldg(g.W + n * kTrainCh + c));
+            }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The regressor's head. A CTA takes R (32, 64 or 128) rows; an MMA tile has
+// 128, but the row count only bounds the K = row products, and small tiles
+// spread a batch over more SMs (the two serial passes over the 256 hidden
+// units are what a CTA spends its time on).
+// ---------------------------------------------------------------------------
+constexpr int kHid = 256;
+
+struct HeadSmem {
+    static constexpr int kH = 0;                               // h: bf16 [4][128][8]
+    static constexpr int kW1 = kH + 4 * kChunk;                // W1: bf16 [4][256][8]
+    static constexpr int kA5 = kW1 + 4 * kHid * 16;            // a5: bf16 [32][128][8]
+    static constexpr int kDa = kA5 + 32 * kChunk;              // da5: the same
+    static constexpr int kGop = kDa + 32 * kChunk;             // gout: bf16 [2][128][8]
+    static constexpr int kG = kGop + 2 * kChunk;               // gout rounded to BF16: f32 [128][4]
+    static constexpr int kGf = kG + kRowsT * 16;               // gout: f32 [128][4]
+    static constexpr int kW2 = kGf + kRowsT * 16;              // W2 rounded to BF16: f32 [3][256]
+    static constexpr int kB1 = kW2 + 3 * kHid * 4;             // f32 [256]
+    static constexpr int kRed = kB1 + kHid * 4;                // f32 [128]
+    static constexpr int kBar = kRed + kRowsT * 4;
+    static constexpr int kTotal = kBar + 64;
+};
+static_assert(HeadSmem::kTotal <= 232448, "shared memory of one CTA");
+
+struct HeadArgs {
+    int64_t B;
+    int R;
+    const uint16_t *h;
+    const uint8_t *w1;            // packed W1
+    const float *b1, *W2, *b2, *tgt;
+    float *out;
+    uint16_t *dz;
+    float *part;
+};
+
+template <int DIM>
+__global__ void __launch_bounds__(256, 1) head_train_kernel(const HeadArgs a, int *err) {
+    using S = HeadSmem;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + S::kBar);
+    uint32_t *slot = reinterpret_cast<uint32_t *>(smem + S::kBar + 32);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + S::kBar + 40);
+    float *g = reinterpret_cast<float *>(smem + S::kG), *gf = reinterpret_cast<float *>(smem + S::kGf);
+    float *w2 = reinterpret_cast<float *>(smem + S::kW2);
+    float *b1 = reinterpret_cast<float *>(smem + S::kB1);
+    float *red = reinterpret_cast<float *>(smem + S::kRed);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr uint32_t kCols = 512, kDy = 256, kDw1 = 288, kDw2 = 352;
+    const int64_t r0 = int64_t(blockIdx.x) * a.R;
+    const int rows = int(min(int64_t(a.R), a.B - r0));
+    if (tid == 0) {
+        for (int i = 0; i < 3; ++i) mbar_init(bars + i, 1u);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) tmem_alloc(slot, kCols);
+    pdl_wait();
+    for (int i = tid; i < kRowsT * 4; i += 256) {
+        const int r = i >> 2, q = i & 3;
+        const uint4 *src = reinterpret_cast<const uint4 *>(a.h + r0 * kTrainCh);
+        *reinterpret_cast<uint4 *>(smem + S::kH + q * kChunk + r * 16) =
+            r < rows ? __ldg(src + i) : make_uint4(0u, 0u, 0u, 0u);
+    }
+    for (int i = tid; i < kHid * kTrainCh / 8; i += 256)
+        cp_async16(smem + S::kW1 + 16 * i, a.w1 + 16 * i);
+    for (int i = tid; i < 2 * kChunk / 16; i += 256)
+        reinterpret_cast<uint4 *>(smem + S::kGop)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = tid; i < DIM * kHid; i += 256)
+        w2[i] = __bfloat162float(__float2bfloat16_rn(__ldg(a.W2 + i)));
+    b1[tid] = __ldg(a.b1 + tid);
+    cp_async_wait_all();
+    fence_async_smem();
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = *slot;
+    const uint64_t h_k = sdesc(smem_addr(smem + S::kH), kChunk, 128);
+    const uint64_t h_mn = sdesc(smem_addr(smem + S::kH), 128, kChunk);
+    const uint64_t w1_k = sdesc(smem_addr(smem + S::kW1), kHid * 16, 128);
+    const uint64_t w1_mn = sdesc(smem_addr(smem + S::kW1), 128, kHid * 16);
+    if (warp == 0) {
+        if (elect_one()) {
+            for (int q = 0; q < 2; ++q)
+                mma_bf16(tmem, h_k + uint64_t(2 * q * (kChunk >> 4)), w1_k + uint64_t(2 * q * kHid),
+                         idesc_bf16(128, 256), q > 0 ? 1u : 0u);
+            mma_commit(bars + 0);
+        }
+        __syncwarp();
+    }
+    bool ok = __syncthreads_and(mbar_wait(bars + 0, 0u, abort_flag, err));
+    if (ok) {
+        fence_after();
+        // ---- a thread per row: a5 = ReLU(z5), the output, its gradient ----
+        float sq = 0.f;
+        if (warp < 4 && 32 * warp < a.R) {
+            const int r = tid;
+            float acc[DIM];
+            #pragma unroll
+            for (int d = 0; d < DIM; ++d) acc[d] = 0.f;
+            #pragma unroll 1
+            for (int n0 = 0; n0 < kHid; n0 += 16) {
+                float v[16];
+                tmem_ld16(tmem + (uint32_t(32 * warp) << 16) + uint32_t(n0), v);
+                uint32_t hv[8];
+                #pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float4 bb = *reinterpret_cast<const float4 *>(b1 + n0 + 4 * q);
+                    const float z[4] = {v[4 * q] + bb.x, v[4 * q + 1] + bb.y, v[4 * q + 2] + bb.z,
+                                        v[4 * q + 3] + bb.w};
+                    hv[2 * q] = pack_bf16x2(fmaxf(z[0], 0.f), fmaxf(z[1], 0.f));
+                    hv[2 * q + 1] = pack_bf16x2(fmaxf(z[2], 0.f), fmaxf(z[3], 0.f));
+                    const float hf[4] = {__uint_as_float(hv[2 * q] << 16),
+                                         __uint_as_float(hv[2 * q] & 0xffff0000u),
+                                         __uint_as_float(hv[2 * q + 1] << 16),
+                                         __uint_as_float(hv[2 * q + 1] & 0xffff0000u)};
+                    #pragma unroll
+                    for (int d = 0; d < DIM; ++d) {
+                        const float4 ww = *reinterpret_cast<const float4 *>(w2 + d * kHid + n0 + 4 * q);
+                        acc[d] = fmaf(hf[0], ww.x, acc[d]);
+                        acc[d] = fmaf(hf[1], ww.y, acc[d]);
+                        acc[d] = fmaf(hf[2], ww.z, acc[d]);
+                        acc[d] = fmaf(hf[3], ww.w, acc[d]);
+                    }
+                }
+                if (a.tgt) {
+                    uint8_t *d = smem + S::kA5 + (n0 >> 3) * kChunk + r * 16;
+                    *reinterpret_cast<uint4 *>(d) = make_uint4(hv[0], hv[1], hv[2], hv[3]);
+                    *reinterpret_cast<uint4 *>(d + kChunk) = make_uint4(hv[4], hv[5], hv[6], hv[7]);
+                }
+            }
+            fence_before();
+            #pragma unroll
+            for (int d = 0; d < DIM; ++d) {
+                const float o = acc[d] + __ldg(a.b2 + d);
+                float gd = 0.f;
+                if (r < rows) {
+                    a.out[(r0 + r) * DIM + d] = o;
+                    if (a.tgt) {
+                        const float e = o - __ldg(a.tgt + (r0 + r) * DIM + d);
+                        gd = 2.f * e / float(a.B * DIM);
+                        sq += e * e;
+                    }
+                }
+                if (a.tgt) {
+                    const __nv_bfloat16 gb = __float2bfloat16_rn(gd);
+                    gf[r * 4 + d] = gd;
+                    g[r * 4 + d] = __bfloat162float(gb);
+                    reinterpret_cast<__nv_bfloat16 *>(smem + S::kGop)[r * 8 + d] = gb;
+                }
+            }
+            red[r] = sq;
+        }
+    }
+    if (ok && a.tgt) {
+        float *part = a.part + int64_t(blockIdx.x) * (kHid * kTrainCh + kHid + DIM * kHid + DIM +
+                                                      kTrainCh + 1);
+        float *p_b1 = part + kHid * kTrainCh, *p_w2 = p_b1 + kHid, *p_b2 = p_w2 + DIM * kHid;
+        float *p_db = p_b2 + DIM, *p_loss = p_db + kTrainCh;
+        __syncthreads();
+        // ---- a thread per hidden unit: da5 = W2^T gout through the ReLU ----
+        {
+            float w[DIM], s = 0.f;
+            #pragma unroll
+            for (int d = 0; d < DIM; ++d) w[d] = w2[d * kHid + tid];
+            const uint16_t *a5 = reinterpret_cast<const uint16_t *>(smem + S::kA5) +
+                                 (tid >> 3) * (kChunk / 2) + (tid & 7);
+            __nv_bfloat16 *da = reinterpret_cast<__nv_bfloat16 *>(smem + S::kDa) +
+                                (tid >> 3) * (kChunk / 2) + (tid & 7);
+            #pragma unroll 4
+            for (int r = 0; r < a.R; ++r) {
+                float v = 0.f;
+                #pragma unroll
+                for (int d = 0; d < DIM; ++d) v = fmaf(g[r * 4 + d], w[d], v);
+                v = positive(a5[r * 8]) ? v : 0.f;
+                s += v;
+                da[r * 8] = __float2bfloat16_rn(v);
+            }
+            p_b1[tid] = s;
+            if (tid < DIM) {
+                float t = 0.f;
+                for (int r = 0; r < a.R; ++r) t += gf[r * 4 + tid];
+                p_b2[tid] = t;
+            }
+            if (tid == 32) {
+                float t = 0.f;
+                for (int r = 0; r < a.R; ++r) t += red[r];
+                *p_loss = t;
+            }
+        }
+        fence_async_smem();
+        fence_before();
+        __syncthreads();
+        fence_after();
+        if (warp == 0) {
+            if (elect_one()) {
+                const uint64_t da_k = sdesc(smem_addr(smem + S::kDa), kChunk, 128);
+                // dy[row][c] = sum_n da5[row][n] W1[n][c]
+                for (int q = 0; q < kHid / 16; ++q)
+                    mma_bf16(tmem + kDy, da_k + uint64_t(2 * q * (kChunk >> 4)),
+                             w1_mn + uint64_t(q * 16), idesc_mn(idesc_bf16(128, 32), false, true),
+                             q > 0 ? 1u : 0u);
+                for (int mt = 0; mt < 2; ++mt) {
+                    const uint64_t da_mn =
+                        sdesc(smem_addr(smem + S::kDa) + mt * 16 * kChunk, 128, kChunk);
+                    const uint64_t a5_mn =
+                        sdesc(smem_addr(smem + S::kA5) + mt * 16 * kChunk, 128, kChunk);
+                    const uint64_t g_mn = sdesc(smem_addr(smem + S::kGop), 128, kChunk);
+                    for (int q = 0; q < a.R / 16; ++q) {
+                        // dW1[n][c] = sum_rows da5[row][n] h[row][c]
+                        mma_bf16(tmem + kDw1 + uint32_t(32 * mt), da_mn + uint64_t(q * 16),
+                                 h_mn + uint64_t(q * 16), idesc_mn(idesc_bf16(128, 32), true, true),
+                                 q > 0 ? 1u : 0u);
+                        // dW2[d][n] = sum_rows gout[row][d] a5[row][n]
+                        mma_bf16(tmem + kDw2 + uint32_t(16 * mt), a5_mn + uint64_t(q * 16),
+                                 g_mn + uint64_t(q * 16), idesc_mn(idesc_bf16(128, 16), true, true),
+                                 q > 0 ? 1u : 0u);
+                    }
+                }
+                mma_commit(bars + 1);
+            }
+            __syncwarp();
+        }
+        ok = __syncthreads_and(mbar_wait(bars + 1, 0u, abort_flag, err));
+        if (ok) {
+            fence_after();
+            const uint32_t tq = tmem + (uint32_t(32 * (warp & 3)) << 16);
+            float *st = reinterpret_cast<float *>(smem + S::kA5);   // [128][33], MMAs complete
+            if (warp < 4) {
+                float v[32];
+                tmem_ld32(tq + kDy, v);
+                const int r = tid;
+                uint32_t hv[16];
+                #pragma unroll
+                for (int c = 0; c < 32; ++c) {
+                    const uint16_t hb = reinterpret_cast<const uint16_t *>(
+                        smem + S::kH + (c >> 3) * kChunk + r * 16)[c & 7];
+                    v[c] = positive(hb) && r < rows ? v[c] : 0.f;
+                    st[r * 33 + c] = v[c];
+                }
+                if (r < rows) {
+                    #pragma unroll
+                    for (int e = 0; e < 16; ++e) hv[e] = pack_bf16x2(v[2 * e], v[2 * e + 1]);
+                    uint4 *d = reinterpret_cast<uint4 *>(a.dz + (r0 + r) * kTrainCh);
+                    #pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        d[e] = make_uint4(hv[4 * e], hv[4 * e + 1], hv[4 * e + 2], hv[4 * e + 3]);
+                }
+            } else {
+                // weight gradients: lane = hidden unit
+                for (int mt = 0; mt < 2; ++mt) {
+                    const int n = 128 * mt + 32 * (warp & 3) + lane;
+                    float v[32];
+                    tmem_ld32(tq + kDw1 + uint32_t(32 * mt), v);
+                    #pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        *reinterpret_cast<float4 *>(smem + S::kDa + (n * 36 + 4 * e) * 4) =
+                            make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+                    tmem_ld16(tq + kDw2 + uint32_t(16 * mt), v);
+                    #pragma unroll
+                    for (int d = 0; d < DIM; ++d) p_w2[d * kHid + n] = v[d];
+                }
+            }
+            fence_before();
+            __syncthreads();
+            if (tid < kTrainCh) {
+                float s = 0.f;
+                for (int r = 0; r < a.R; ++r) s += st[r * 33 + tid];
+                p_db[tid] = s;
+            }
+            for (int i = tid; i < kHid * kTrainCh; i += 256)
+                part[i] = reinterpret_cast<const float *>(smem + S::kDa)[(i >> 5) * 36 + (i & 31)];
+        }
+    }
+    mma_drain(bars + 2, tmem, kCols, warp);
+}
+
+// ---------------------------------------------------------------------------
+// Sums of the CTAs' partials: 32 elements per block, eight groups of threads
+// take every eighth partial each, their sums are added in order.
+// ---------------------------------------------------------------------------
+constexpr int kRedE = 32, kRedG = 8;
+
+struct ReduceArgs {
+    ReduceSeg seg[kMaxSegs];
+    int block0[kMaxSegs + 1];
+    int n;
+};
+
+__global__ void __launch_bounds__(kRedE * kRedG) reduce_parts_kernel(const ReduceArgs a) {
+    __shared__ float red[kRedG][kRedE];
+    int s = 0;
+    while (s + 1 < a.n && int(blockIdx.x) >= a.block0[s + 1]) ++s;
+    const ReduceSeg &g = a.seg[s];
+    const int e = threadIdx.x % kRedE, grp = threadIdx.x / kRedE;
+    const int64_t i = int64_t(blockIdx.x - a.block0[s]) * kRedE + e;
+    pdl_wait();
+    float x = 0.f;
+    if (i < g.count) {
+        const float *p = g.part + i;
+        #pragma unroll 10
+        for (int q = grp; q < g.n; q += kRedG) x += __ldg(p + int64_t(q) * g.stride);
+    }
+    red[grp][e] = x;
+    __syncthreads();
+    if (grp == 0 && i < g.count) {
+        float v = red[0][e];
+        #pragma unroll
+        for (int q = 1; q < kRedG; ++q) v += red[q][e];
+        if (g.div > 0.f)
+            g.out[i] += v / g.div;
+        else
+            g.out[i] = v;
+    }
+}
+
+constexpr int kSmemMax = 232448;
+
+// the kernels' instances: f(Geo) for the layer's dimension and edge
+template <class Fn>
+void with_geo(const ConvGeo &g, bool first, Fn f) {
+    if (g.dim == 2) {
+        if (first) {
+            if (g.Si == 9) f(Geo<2, 9, true>());          // regressor
+            if (g.Si == 11) f(Geo<2, 11, true>());        // classifier, zero ring stored
+        } else {
+            if (g.Si == 11) f(Geo<2, 11, false>());
+            if (g.Si == 7) f(Geo<2, 7, false>());
+            if (g.Si == 5) f(Geo<2, 5, false>());
+            if (g.Si == 3) f(Geo<2, 3, false>());
+        }
+    } else if (first) {
+        if (g.Si == 7) f(Geo<3, 7, true>());
+    } else {
+        if (g.Si == 5) f(Geo<3, 5, false>());
+        if (g.Si == 3) f(Geo<3, 3, false>());
+    }
+}
+
+// inputs per tile: as many as fill the 128 rows and fit shared memory, but no
+// more than leaves every SM a tile
+template <class N, bool BWD>
+int tile_inputs(int64_t B, int sm_count) {
+    const int64_t even = (B + sm_count - 1) / sm_count;
+    int G = int(std::max<int64_t>(1, std::min<int64_t>(N::GMax, even)));
+    while (G > 1 && conv_smem<N, BWD>(G).total > kSmemMax) --G;
+    return G;
+}
+
+int head_rows(int64_t B, int sm_count) {
+    return B <= int64_t(32) * sm_count ? 32 : B <= int64_t(64) * sm_count ? 64 : 128;
+}
+
+}  // namespace
+
+int train_packed_kw(int dim) { return dim == 2 ? 288 : 872; }
+
+int launch_pack_train(const PackSeg *segs, int n, cudaStream_t st) {
+    PackArgs a{};
+    a.n = n;
+    for (int i = 0; i < n; ++i) a.seg[i] = segs[i];
+    launch_pdl(pack_train_kernel, dim3(76), dim3(256), 0, st, a);
+    return 1;
+}
+
+int launch_conv_fwd(const ConvGeo &g, const void *x, bool first, int64_t B, const uint8_t *packed,
+                    const float *bias, uint16_t *y, int ring, float *z, int *err, int sm_count,
+                    cudaStream_t st) {
+    ConvArgs a{};
+    a.x = x;
+    a.B = B;
+    a.w = packed;
+    a.bias = bias;
+    a.y = y;
+    a.z = z;
+    a.ring = ring;
+    // the general GEMM's K splits of this product (tc_gemm.cu): the same
+    // partial sums give the same bits
+    const int64_t chunks = (g.K + 63) / 64, tiles = (B * g.Po + 127) / 128;
+    int64_t splits = 1;
+    if (tiles < 2 * sm_count && chunks > 8)
+        splits = std::min<int64_t>(chunks / 4, (2 * sm_count + tiles - 1) / tiles);
+    a.kc = int((chunks + splits - 1) / splits * 64);
+    a.nsplit = (g.K + a.kc - 1) / a.kc;
+    with_geo(g, first, [&](auto n) {
+        using N = decltype(n);
+        a.G = tile_inputs<N, false>(B, sm_count);
+        a.tiles = (B + a.G - 1) / a.G;
+        const ConvSmem L = conv_smem<N, false>(a.G);
+        cudaFuncSetAttribute(conv_fwd_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+        const int per_sm = L.total <= 113 * 1024 ? 2 : 1;
+        const int grid = int(std::min<int64_t>(a.tiles, int64_t(sm_count) * per_sm));
+        launch_pdl(conv_fwd_kernel<N>, dim3(grid), dim3(kFwdThreads), size_t(L.total), st, a, L, err);
+    });
+    return 1;
+}
+
+int conv_bwd_ctas(const ConvGeo &g, int64_t B, bool first, int sm_count) {
+    int G = 1;
+    with_geo(g, first, [&](auto n) { G = tile_inputs<decltype(n), true>(B, sm_count); });
+    return int(std::min<int64_t>((B + G - 1) / G, sm_count));
+}
+
+int launch_conv_bwd(const ConvGeo &g, const void *x, bool first, int64_t B, const uint16_t *dz,
+                    const uint8_t *packed, float *wpart, uint16_t *dzp, int ring, float *bpart,
+                    int *err, int sm_count, cudaStream_t st) {
+    ConvArgs a{};
+    a.x = x;
+    a.B = B;
+    a.w = packed;
+    a.dz = dz;
+    a.wpart = wpart;
+    a.dzp = dzp;
+    a.bpart = bpart;
+    a.ring = ring;
+    const int grid = conv_bwd_ctas(g, B, first, sm_count);
+    with_geo(g, first, [&](auto n) {
+        using N = decltype(n);
+        a.G = tile_inputs<N, true>(B, sm_count);
+        a.tiles = (B + a.G - 1) / a.G;
+        const ConvSmem L = conv_smem<N, true>(a.G);
+        cudaFuncSetAttribute(conv_bwd_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+        launch_pdl(conv_bwd_kernel<N>, dim3(grid), dim3(kBwdThreads), size_t(L.total), st, a, L, err);
+    });
+    return 1;
+}
+
+int head_ctas(int64_t B, int sm_count) {
+    const int R = head_rows(B, sm_count);
+    return int((B + R - 1) / R);
+}
+
+int64_t head_part_floats(int dim) {
+    return kHid * kTrainCh + kHid + dim * kHid + dim + kTrainCh + 1;
+}
+
+int launch_train_head(int dim, int64_t B, const uint16_t *h, const uint8_t *packed_w1,
+                      const float *b1, const float *W2, const float *b2, const float *tgt,
+                      float *out, uint16_t *dz, float *part, int *err, int sm_count,
+                      cudaStream_t st) {
+    HeadArgs a{B, head_rows(B, sm_count), h, packed_w1, b1, W2, b2, tgt, out, dz, part};
+    const int grid = head_ctas(B, sm_count);
+    auto *k = dim == 2 ? head_train_kernel<2> : head_train_kernel<3>;
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, HeadSmem::kTotal);
+    launch_pdl(k, dim3(grid), dim3(256), size_t(HeadSmem::kTotal), st, a, err);
+    return 1;
+}
+
+int launch_reduce_parts(const ReduceSeg *segs, int n_segs, cudaStream_t st) {
+    ReduceArgs a{};
+    a.n = n_segs;
+    int blocks = 0;
+    for (int s = 0; s < n_segs; ++s) {
+        a.seg[s] = segs[s];
+        a.block0[s] = blocks;
+        blocks += int((segs[s].count + kRedE - 1) / kRedE);
+    }
+    a.block0[n_segs] = blocks;
+    launch_pdl(reduce_parts_kernel, dim3(blocks), dim3(kRedE * kRedG), 0, st, a);
+    return 1;
+}
+
+}  // namespace cs
