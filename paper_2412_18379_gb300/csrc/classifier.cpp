@@ -14,6 +14,8 @@
 
 #include "classifier.h"
 #include "cnn.h"
+#include "fc_tc.h"
+#include "train_tc.h"
 
 namespace cs {
 
@@ -70,6 +72,27 @@ struct Classifier {
     // parameters change
     uint8_t *packed = nullptr;
     bool packed_dirty = true;
+    // the tiled path (fc_tc.h): activations and gradients of the fully
+    // connected layers for fc_cap rows (the gradients' where fc_grad), and the
+    // packed weights with the tile widths they were packed for
+    std::vector<void *> fcws;
+    int64_t fc_cap = 0;
+    bool fc_grad = false;
+    uint8_t *tcat = nullptr, *tr1 = nullptr, *tru = nullptr, *tgH = nullptr, *tgu = nullptr,
+            *tgh2 = nullptr, *tgh1 = nullptr;
+    float *toff = nullptr, *tH = nullptr, *tgpool = nullptr;
+    int *tcount = nullptr;
+    int64_t *tidx = nullptr;
+    uint8_t *fcpack = nullptr;
+    int pack_bn[3] = {0, 0, 0};
+    // module 1 of a 2-D training step for tr_cap rows (train_tc.h)
+    std::vector<void *> trws;
+    int64_t tr_cap = 0;
+    float *ta0 = nullptr, *tz2 = nullptr;
+    uint16_t *ty1 = nullptr, *tdz2 = nullptr, *tdz1 = nullptr;
+    uint8_t *tcpack = nullptr;
+    float *parts = nullptr;      // partial sums of a step's gradients
+    int64_t parts_cap = 0;
 };
 
 }  // namespace cs
@@ -107,9 +130,36 @@ void free_ws(cs_ctx *ctx, Classifier &C) {
     C.cap = C.cap_conv = C.cap_grad = 0;
 }
 
+void free_list(cs_ctx *ctx, std::vector<void *> &v) {
+    for (void *p : v) dfree(ctx, p);
+    v.clear();
+}
+
+void free_fc(cs_ctx *ctx, Classifier &C) {
+    free_list(ctx, C.fcws);
+    C.tcat = C.tr1 = C.tru = C.tgH = C.tgu = C.tgh2 = C.tgh1 = nullptr;
+    C.toff = C.tH = C.tgpool = nullptr;
+    C.tcount = nullptr;
+    C.tidx = nullptr;
+    C.fc_cap = 0;
+    C.fc_grad = false;
+}
+
+void free_tr(cs_ctx *ctx, Classifier &C) {
+    free_list(ctx, C.trws);
+    C.ta0 = C.tz2 = nullptr;
+    C.ty1 = C.tdz2 = C.tdz1 = nullptr;
+    C.tcpack = nullptr;
+    C.tr_cap = 0;
+}
+
 void release(cs_ctx *ctx, Classifier *C) {
     if (!C) return;
     free_ws(ctx, *C);
+    free_fc(ctx, *C);
+    free_tr(ctx, *C);
+    dfree(ctx, C->fcpack);
+    dfree(ctx, C->parts);
     for (void *p : {static_cast<void *>(C->w), static_cast<void *>(C->g),
                     static_cast<void *>(C->m), static_cast<void *>(C->v),
                     static_cast<void *>(C->loss), static_cast<void *>(C->xp),
@@ -125,17 +175,111 @@ cs_status ws_alloc(cs_ctx *ctx, Classifier &C, T **p, int64_t count) {
     return rc;
 }
 
+// the error flag of the tensor-core kernels' bounded waits
+cs_status ensure_err(cs_ctx *ctx) {
+    if (ctx->dev_err) return CS_OK;
+    cs_status rc = dmalloc_n(ctx, &ctx->dev_err, 1);
+    if (rc) return rc;
+    if (cudaMemset(ctx->dev_err, 0, sizeof(int)) != cudaSuccess)
+        return fail(ctx, CS_ECUDA, "cudaMemset of the device error flag failed");
+    return CS_OK;
+}
+
+template <class T>
+cs_status list_alloc(cs_ctx *ctx, std::vector<void *> &v, T **p, int64_t count) {
+    cs_status rc = dmalloc_n(ctx, p, size_t(std::max<int64_t>(count, 1)));
+    if (rc == CS_OK) v.push_back(*p);
+    return rc;
+}
+
+// Packed weights of the tiled fully connected layers for products of B rows:
+// where each lies in Classifier::fcpack and its tile width. Forward W3, W4,
+// W5 (xp2, fuse, logits); backward W5^T, the two column ranges of W4^T, W3^T.
+struct FcPlan {
+    enum { W3, W4, W5, W5T, W4P, W4H, W3T, Count };
+    int rows[Count], K[Count], bn[Count];
+    int64_t off[Count], bytes;
+    FcPlan(const ClsShape &S, int64_t B, int sm) {
+        const int r[Count] = {kClsH1, kClsH2, S.n_cls, kClsH2, S.n_pool, kClsH1, kClsH1};
+        const int k[Count] = {kClsH1, S.ldc, kClsH2, S.n_cls, kClsH2, kClsH2, kClsH1};
+        bytes = 0;
+        for (int i = 0; i < Count; ++i) {
+            rows[i] = r[i];
+            K[i] = k[i];
+            bn[i] = fc_bn(B, r[i], sm);
+            off[i] = bytes;
+            // room for any tile width
+            bytes += int64_t(r[i] + 255) / 256 * 256 * fc_kp(k[i]) * 2 + fc_kp(k[i]) * 2 * 256;
+        }
+    }
+};
+
+// buffers of the tiled fully connected layers for B rows
+cs_status ensure_fc(cs_ctx *ctx, Classifier &C, int64_t B, bool grad) {
+    cs_status rc = ensure_err(ctx);
+    if (rc) return rc;
+    const ClsShape S(C.dim);
+    if (!C.fcpack) {
+        if ((rc = dmalloc_n(ctx, &C.fcpack, size_t(FcPlan(S, 1, ctx->sm_count).bytes)))) return rc;
+        C.pack_bn[0] = 0;
+    }
+    if (C.fc_cap >= B && (!grad || C.fc_grad)) return CS_OK;
+    const int64_t cap = std::max(B, C.fc_cap);
+    const bool g = grad || C.fc_grad;
+    free_fc(ctx, C);
+    auto &v = C.fcws;
+    const int np = fc_kp(S.n_cls);
+    if ((rc = list_alloc(ctx, v, &C.tcat, fc_bytes(cap, S.ldc))) ||
+        (rc = list_alloc(ctx, v, &C.tr1, fc_bytes(cap, kClsH1))) ||
+        (rc = list_alloc(ctx, v, &C.tru, fc_bytes(cap, kClsH2))) ||
+        (rc = list_alloc(ctx, v, &C.toff, cap * C.dim)) ||
+        (rc = list_alloc(ctx, v, &C.tH, cap * S.n_cls)) ||
+        (g && ((rc = list_alloc(ctx, v, &C.tgH, fc_bytes(cap, np))) ||
+               (rc = list_alloc(ctx, v, &C.tgu, fc_bytes(cap, kClsH2))) ||
+               (rc = list_alloc(ctx, v, &C.tgh2, fc_bytes(cap, kClsH1))) ||
+               (rc = list_alloc(ctx, v, &C.tgh1, fc_bytes(cap, kClsH1))) ||
+               (rc = list_alloc(ctx, v, &C.tgpool, cap * S.n_pool)) ||
+               (rc = list_alloc(ctx, v, &C.tidx, cap)) || (rc = list_alloc(ctx, v, &C.tcount, 1))))) {
+        free_fc(ctx, C);
+        return rc;
+    }
+    C.fc_cap = cap;
+    C.fc_grad = g;
+    return CS_OK;
+}
+
+// buffers of module 1 of a 2-D training step
+cs_status ensure_tr(cs_ctx *ctx, Classifier &C, int64_t B) {
+    if (C.dim != 2 || C.tr_cap >= B) return CS_OK;
+    free_tr(ctx, C);
+    const ClsShape S(2);
+    auto &v = C.trws;
+    cs_status rc;
+    if ((rc = list_alloc(ctx, v, &C.ta0, B * 2 * S.Pq)) ||
+        (rc = list_alloc(ctx, v, &C.tz2, B * S.P * kClsCh)) ||
+        (rc = list_alloc(ctx, v, &C.ty1, B * S.Pq * kClsCh)) ||
+        (rc = list_alloc(ctx, v, &C.tdz2, B * S.P * kClsCh)) ||
+        (rc = list_alloc(ctx, v, &C.tdz1, B * S.P * kClsCh)) ||
+        (rc = list_alloc(ctx, v, &C.tcpack, 64 * 1024))) {
+        free_tr(ctx, C);
+        return rc;
+    }
+    // the zero ring of conv2's input: only the interior is ever written
+    if (cudaMemset(C.ty1, 0, size_t(B) * S.Pq * kClsCh * 2) != cudaSuccess) {
+        free_tr(ctx, C);
+        return fail(ctx, CS_ECUDA, "cudaMemset of the padded activations failed");
+    }
+    C.tr_cap = B;
+    return CS_OK;
+}
+
 // workspace for B rows of the fully connected layers; `conv` adds the
 // unfused module 1's buffers, `grad` the backward pass's (which reuses
 // module 1's, so it needs `conv` too). Growing any set reallocates all of
 // them, each at its own row count.
 cs_status ensure_ws(cs_ctx *ctx, Classifier &C, int64_t B, bool conv, bool grad) {
-    if (!ctx->dev_err) {
-        cs_status rc = dmalloc_n(ctx, &ctx->dev_err, 1);
-        if (rc) return rc;
-        if (cudaMemset(ctx->dev_err, 0, sizeof(int)) != cudaSuccess)
-            return fail(ctx, CS_ECUDA, "cudaMemset of the device error flag failed");
-    }
+    cs_status rc0 = ensure_err(ctx);
+    if (rc0) return rc0;
     conv = conv || grad;
     if (C.cap >= B && (!conv || C.cap_conv >= B) && (!grad || C.cap_grad >= B)) return CS_OK;
     const int64_t rows = std::max(B, C.cap);
@@ -218,21 +362,200 @@ int forward_fc(cs_ctx *ctx, Classifier &C, int64_t B, cudaStream_t st) {
     return n;
 }
 
-// inference of B particles xp[b] into C.H: module 1 fused on the tensor cores
-// (BF16 operands), or, with FP32 operands, the training path's kernels
-int forward(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t B, const double *xp,
-            const int64_t *idx, cudaStream_t st);
-int infer(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t B, const double *xp,
+// ---------------------------------------------------------------------------
+// The tiled path: BF16 operands (fc_tc.h, train_tc.h)
+// ---------------------------------------------------------------------------
+
+// refresh the packed weights of the fully connected layers
+int pack_fc(cs_ctx *ctx, Classifier &C, const ClsShape &S, const FcPlan &P, bool grad,
+            cudaStream_t st) {
+    const float *w = C.w;
+    const float *W3 = w + S.w_off[3], *W4 = w + S.w_off[4], *W5 = w + S.w_off[5];
+    auto seg = [&](int i, const float *W, int64_t rs, int64_t ks) {
+        return FcPack{W, rs, ks, P.rows[i], P.K[i], P.bn[i], C.fcpack + P.off[i]};
+    };
+    FcPack f[FcPlan::Count] = {seg(FcPlan::W3, W3, kClsH1, 1), seg(FcPlan::W4, W4, S.ldc, 1),
+                               seg(FcPlan::W5, W5, kClsH2, 1), seg(FcPlan::W5T, W5, 1, kClsH2),
+                               seg(FcPlan::W4P, W4, 1, S.ldc), seg(FcPlan::W4H, W4 + S.n_pool, 1, S.ldc),
+                               seg(FcPlan::W3T, W3, 1, kClsH1)};
+    return launch_fc_pack(f, grad ? int(FcPlan::Count) : 3, st);
+}
+
+// module 2, fusion and logits of B rows whose pooled features (C.tcat's first
+// columns) and offsets (C.toff) are in place, into H
+int fc_forward(cs_ctx *ctx, Classifier &C, const ClsShape &S, const FcPlan &P, int64_t B, float *H,
+               cudaStream_t st) {
+    const int sm = ctx->sm_count;
+    const FcMat cat = fc_mat(C.tcat, S.ldc), r1 = fc_mat(C.tr1, kClsH1), ru = fc_mat(C.tru, kClsH2);
+    int n = launch_fc_offset(C.dim, B, C.toff, C.w + S.w_off[2], C.w + S.b_off[2], r1, sm, st);
+    FcGemm g{r1, C.fcpack + P.off[FcPlan::W3], P.bn[FcPlan::W3], kClsH1, B};
+    g.bias = C.w + S.b_off[3];
+    g.relu = true;
+    g.out = fc_cols(cat, S.n_pool, kClsH1);
+    n += launch_fc_gemm(g, ctx->dev_err, sm, st);
+    FcGemm u{cat, C.fcpack + P.off[FcPlan::W4], P.bn[FcPlan::W4], kClsH2, B};
+    u.bias = C.w + S.b_off[4];
+    u.relu = true;
+    u.out = ru;
+    fc_split_like_gemm(B, kClsH2, S.ldc, sm, &u.nsplit, &u.kc);
+    n += launch_fc_gemm(u, ctx->dev_err, sm, st);
+    FcGemm l{ru, C.fcpack + P.off[FcPlan::W5], P.bn[FcPlan::W5], S.n_cls, B};
+    l.bias = C.w + S.b_off[5];
+    l.f32 = H;
+    l.ldf = S.n_cls;
+    return n + launch_fc_gemm(l, ctx->dev_err, sm, st);
+}
+
+// inference of B particles xp[b] into H [B][n_cls]: module 1 fused on the
+// tensor cores, then the tiled fully connected layers
+int infer(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t B, const double *xp, float *H,
           cudaStream_t st) {
-    if (!gemm_bf16()) return forward(ctx, C, m, B, xp, nullptr, st);
     const ClsShape S(C.dim);
+    const FcPlan P(S, B, ctx->sm_count);
+    int n = 0;
     if (C.packed_dirty) {
         launch_cls_pack(C.dim, C.w, S.w_off[0], S.b_off[0], S.w_off[1], S.b_off[1], C.packed, st);
-        C.packed_dirty = false;
+        n += 1;
     }
-    launch_cls_conv_tc(m, m.pool_f, B, xp, C.packed, C.cat, S.ldc, C.off, ctx->dev_err,
+    if (C.packed_dirty || !std::equal(C.pack_bn, C.pack_bn + 3, P.bn)) {
+        n += pack_fc(ctx, C, S, P, false, st);
+        std::copy(P.bn, P.bn + 3, C.pack_bn);
+    }
+    C.packed_dirty = false;
+    launch_cls_conv_tc(m, m.pool_f, B, xp, C.packed, fc_mat(C.tcat, S.ldc), C.toff, ctx->dev_err,
                        ctx->sm_count, st);
-    return 2 + forward_fc(ctx, C, B, st);
+    return n + 1 + fc_forward(ctx, C, S, P, B, H, st);
+}
+
+int forward_conv(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t B, const double *xp,
+                 const int64_t *idx, float *off, cudaStream_t st);
+int backward_conv(cs_ctx *ctx, Classifier &C, int64_t B, const float *dpool, int64_t ld,
+                  cudaStream_t st);
+
+// The tiled path's training step for B rows of at least 16: gradients of the
+// cross-entropy into C.g, the loss added to *loss. In 2-D module 1 runs on the
+// implicit-GEMM convolutions as well (train_tc.h); in 3-D, whose 343 positions
+// do not fit their tile, on the layer-by-layer kernels.
+bool tiled_batch(int64_t B) { return gemm_bf16() && B >= 16; }
+
+// floats of a step's partial sums
+int64_t train_parts(cs_ctx *ctx, const ClsShape &S, int64_t B) {
+    const int sm = ctx->sm_count;
+    const int64_t mt = (B + 127) / 128;
+    int64_t n = int64_t(fc_wgrad_splits(B, S.n_cls, kClsH2, sm)) * S.n_cls * kClsH2 +
+                int64_t(fc_wgrad_splits(B, kClsH2, S.ldc, sm)) * kClsH2 * S.ldc +
+                int64_t(fc_wgrad_splits(B, kClsH1, kClsH1, sm)) * kClsH1 * kClsH1;
+    n += cls_softmax_blocks(B) * (int64_t(S.n_cls) + 1);
+    n += 4 * mt * (kClsH2 + 2 * kClsH1) + mt * kClsH1 * S.dim;
+    if (S.dim == 2)
+        n += int64_t(sm) * kClsCh * (kClsCh * S.taps + 2 * S.taps + 1) +
+             int64_t(cls_pool_back_blocks(B, sm)) * kClsCh;
+    return n;
+}
+
+cs_status ensure_train(cs_ctx *ctx, Classifier &C, int64_t B) {
+    cs_status rc = ensure_fc(ctx, C, B, true);
+    if (rc == CS_OK) rc = C.dim == 2 ? ensure_tr(ctx, C, B) : CS_OK;
+    if (rc) return rc;
+    const int64_t need = train_parts(ctx, ClsShape(C.dim), B);
+    if (C.parts_cap >= need) return CS_OK;
+    dfree(ctx, C.parts);
+    C.parts = nullptr;
+    C.parts_cap = 0;
+    if ((rc = dmalloc_n(ctx, &C.parts, size_t(need)))) return rc;
+    C.parts_cap = need;
+    return CS_OK;
+}
+
+int train_tiled(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t B, const double *xp,
+                const int32_t *labels, const int64_t *idx, float *loss, cudaStream_t st) {
+    const ClsShape S(C.dim);
+    const FcPlan P(S, B, ctx->sm_count);
+    const int sm = ctx->sm_count, d = C.dim;
+    int *err = ctx->dev_err;
+    float *g = C.g;
+    int n = pack_fc(ctx, C, S, P, true, st);
+    C.pack_bn[0] = 0;            // inference packs its own widths again
+    const FcMat cat = fc_mat(C.tcat, S.ldc), r1 = fc_mat(C.tr1, kClsH1), ru = fc_mat(C.tru, kClsH2);
+    const FcMat gH = fc_mat(C.tgH, fc_kp(S.n_cls)), gu = fc_mat(C.tgu, kClsH2);
+    const FcMat gh2 = fc_mat(C.tgh2, kClsH1), gh1 = fc_mat(C.tgh1, kClsH1);
+    const ConvGeo c1(2, 2, 11), c2(2, kClsCh, 11);
+    // 2 KB, 18 KB and 18 KB
+    uint8_t *f1 = C.tcpack, *f2 = f1 + 4 * 1024, *b2 = f2 + 20 * 1024;
+    if (d == 2) {
+        const PackSeg ps[2] = {{C.w + S.w_off[0], c1.K, 0, f1, nullptr, nullptr},
+                               {C.w + S.w_off[1], c2.K, train_packed_kw(2), f2, b2, nullptr}};
+        n += launch_pack_train(ps, 2, st);
+        launch_cls_features(m, B, xp, idx, true, C.ta0, C.toff, sm, st);
+        n += 1 + launch_conv_fwd(c1, C.ta0, true, B, f1, C.w + S.b_off[0], C.ty1, 1, nullptr, err, sm, st);
+        n += launch_conv_fwd(c2, C.ty1, false, B, f2, C.w + S.b_off[1], nullptr, 0, C.tz2, err, sm, st);
+    } else {
+        n += forward_conv(ctx, C, m, B, xp, idx, C.toff, st);
+    }
+    const float *z2 = d == 2 ? C.tz2 : C.z2;
+    launch_cls_pool_tiled(d, z2, B, cat, sm, st);
+    n += 1 + fc_forward(ctx, C, S, P, B, C.tH, st);
+
+    ReduceSeg seg[kMaxSegs];
+    int ns = 0;
+    float *part = C.parts;
+    auto sum = [&](int64_t count, int parts, float *out) {
+        float *p = part;
+        seg[ns++] = ReduceSeg{p, count, count, out, parts, 0.f};
+        part += count * parts;
+        return p;
+    };
+    auto wgrad = [&](const FcMat &Y, const FcMat &X, int N, int K, int64_t w_off) {
+        const int s = fc_wgrad_splits(B, N, K, sm);
+        n += launch_fc_wgrad(Y, X, B, N, K, s, sum(int64_t(N) * K, s, g + w_off), err, st);
+    };
+    const int mt = int((B + 127) / 128), sb = cls_softmax_blocks(B);
+    // logits
+    float *b5 = sum(S.n_cls, sb, g + S.b_off[5]);
+    float *lp = part;
+    part += sb;
+    launch_softmax_ce_tiled(C.tH, labels, idx, B, S.n_cls, gH, b5, lp, C.tcount, st);
+    launch_loss_sum(lp, sb, C.tcount, loss, st);
+    n += 3;
+    wgrad(gH, ru, S.n_cls, kClsH2, S.w_off[5]);
+    // fusion
+    FcGemm q{gH, C.fcpack + P.off[FcPlan::W5T], P.bn[FcPlan::W5T], kClsH2, B};
+    q.gate = ru;
+    q.out = gu;
+    q.colsum = sum(kClsH2, 4 * mt, g + S.b_off[4]);
+    n += launch_fc_gemm(q, err, sm, st);
+    wgrad(gu, cat, kClsH2, S.ldc, S.w_off[4]);
+    FcGemm gp{gu, C.fcpack + P.off[FcPlan::W4P], P.bn[FcPlan::W4P], S.n_pool, B};
+    gp.f32 = C.tgpool;
+    gp.ldf = S.n_pool;
+    n += launch_fc_gemm(gp, err, sm, st);
+    // module 2
+    FcGemm q2{gu, C.fcpack + P.off[FcPlan::W4H], P.bn[FcPlan::W4H], kClsH1, B};
+    q2.gate = fc_cols(cat, S.n_pool, kClsH1);
+    q2.out = gh2;
+    q2.colsum = sum(kClsH1, 4 * mt, g + S.b_off[3]);
+    n += launch_fc_gemm(q2, err, sm, st);
+    wgrad(gh2, r1, kClsH1, kClsH1, S.w_off[3]);
+    FcGemm q1{gh2, C.fcpack + P.off[FcPlan::W3T], P.bn[FcPlan::W3T], kClsH1, B};
+    q1.gate = r1;
+    q1.out = gh1;
+    q1.colsum = sum(kClsH1, 4 * mt, g + S.b_off[2]);
+    n += launch_fc_gemm(q1, err, sm, st);
+    n += launch_fc_offset_grad(d, B, C.toff, gh1, sum(int64_t(kClsH1) * d, mt, g + S.w_off[2]), st);
+    // module 1
+    if (d == 2) {
+        const int pb = cls_pool_back_blocks(B, sm);
+        launch_cls_pool_back_tiled(2, C.tgpool, z2, B, C.tdz2, sum(kClsCh, pb, g + S.b_off[1]), sm, st);
+        const int ca2 = conv_bwd_ctas(c2, B, false, sm), ca1 = conv_bwd_ctas(c1, B, true, sm);
+        float *w2 = sum(int64_t(kClsCh) * c2.K, ca2, g + S.w_off[1]);
+        float *bb1 = sum(kClsCh, ca2, g + S.b_off[0]);
+        n += 1 + launch_conv_bwd(c2, C.ty1, false, B, C.tdz2, b2, w2, C.tdz1, 1, bb1, err, sm, st);
+        float *w1 = sum(int64_t(kClsCh) * c1.K, ca1, g + S.w_off[0]);
+        n += launch_conv_bwd(c1, C.ta0, true, B, C.tdz1, nullptr, w1, nullptr, 0, nullptr, err, sm, st);
+    } else {
+        n += backward_conv(ctx, C, B, C.tgpool, S.n_pool, st);
+    }
+    return n + launch_reduce_parts(seg, ns, st);
 }
 
 // forward of B rows (particles xp[idx[b]], or xp[b]) into C.H [B][n_cls],
@@ -240,10 +563,19 @@ int infer(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t B, const double 
 int forward(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t B, const double *xp,
             const int64_t *idx, cudaStream_t st) {
     const ClsShape S(C.dim);
+    const int n = forward_conv(ctx, C, m, B, xp, idx, C.off, st);
+    launch_cls_pool(C.dim, C.z2, B, C.cat, S.ldc, ctx->sm_count, st);
+    return n + 1 + forward_fc(ctx, C, B, st);
+}
+
+// module 1 of B rows into C.z2 (before its ReLU), the offsets into `off`
+int forward_conv(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t B, const double *xp,
+                 const int64_t *idx, float *off, cudaStream_t st) {
+    const ClsShape S(C.dim);
     const int sm = ctx->sm_count, d = C.dim;
     const int64_t BP = B * S.P;
     int n = 0;
-    launch_cls_features(m, B, xp, idx, true, C.a0, C.off, sm, st);
+    launch_cls_features(m, B, xp, idx, true, C.a0, off, sm, st);
     n += 1;
     // module 1: two zero-padded 3^d convolutions with ReLU, pooling
     n += launch_im2col(d, C.a0, B, d, S.W + 2, true, C.col1, sm, st);
@@ -255,9 +587,7 @@ int forward(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t B, const doubl
     n += launch_im2col(d, C.a1, B, kClsCh, S.W + 2, false, C.col2, sm, st);
     n += gemm(ctx, C, C.col2, C.w + S.w_off[1], C.z2, C.w + S.b_off[1], BP, kClsCh,
               int64_t(kClsCh) * S.taps, false, true, st);
-    launch_cls_pool(d, C.z2, B, C.cat, S.ldc, sm, st);
-    n += 1;
-    return n + forward_fc(ctx, C, B, st);
+    return n;
 }
 
 // gradients of the cross-entropy of C.H against labels[idx[b]] into C.g;
@@ -268,7 +598,6 @@ int backward(cs_ctx *ctx, Classifier &C, int64_t B, const int32_t *labels, const
              float *loss, cudaStream_t st) {
     const ClsShape S(C.dim);
     const int sm = ctx->sm_count, d = C.dim;
-    const int64_t BP = B * S.P;
     float *g = C.g;
     const float *w = C.w;
     int n = 0;
@@ -291,8 +620,20 @@ int backward(cs_ctx *ctx, Classifier &C, int64_t B, const int32_t *labels, const
     n += launch_relu_back(C.h1, C.gh1, B * kClsH1, sm, st);
     n += gemm(ctx, C, C.gh1, C.off, g + S.w_off[2], nullptr, kClsH1, d, B, true, false, st);
     n += launch_colsum(C.gh1, B, kClsH1, g + S.b_off[2], st, C.splitk, C.splitk_n, sm);
-    // module 1: pooling, second and first convolution
-    launch_cls_pool_back(d, C.gcat, S.ldc, C.z2, B, C.gz2, sm, st);
+    return n + backward_conv(ctx, C, B, C.gcat, S.ldc, st);
+}
+
+// module 1's gradients from that of the pooled features (dpool, row stride
+// ld): pooling, second and first convolution
+int backward_conv(cs_ctx *ctx, Classifier &C, int64_t B, const float *dpool, int64_t ld,
+                  cudaStream_t st) {
+    const ClsShape S(C.dim);
+    const int sm = ctx->sm_count, d = C.dim;
+    const int64_t BP = B * S.P;
+    float *g = C.g;
+    const float *w = C.w;
+    int n = 0;
+    launch_cls_pool_back(d, dpool, ld, C.z2, B, C.gz2, sm, st);
     n += 1;
     const int64_t K2 = int64_t(kClsCh) * S.taps;
     n += gemm(ctx, C, C.gz2, C.col2, g + S.w_off[1], nullptr, kClsCh, K2, BP, true, false, st);
@@ -344,19 +685,28 @@ cs_status ensure_xp(cs_ctx *ctx, Classifier &C, int64_t n) {
     return CS_OK;
 }
 
-// logits of n particles, chunk by chunk, through the workspace; each chunk's
-// logits are copied out on the stream (or handed to `each` in place)
+// logits of n particles, chunk by chunk, into dst [n][n_cls] or, without it,
+// into a chunk's own buffer, which `each` reads before the next chunk
 template <class F>
 cs_status forward_chunks(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t n, const double *xp,
-                         cudaStream_t st, F each) {
+                         float *dst, cudaStream_t st, F each) {
     const bool fused = gemm_bf16();
+    const int ncls = cls_cells(C.dim);
     const int64_t R = std::min<int64_t>(n, chunk_rows(C.dim, fused));
-    cs_status rc = ensure_ws(ctx, C, R, !fused, false);
+    cs_status rc = fused ? ensure_fc(ctx, C, R, false) : ensure_ws(ctx, C, R, true, false);
     if (rc) return rc;
     for (int64_t r0 = 0; r0 < n; r0 += R) {
         const int64_t B = std::min(R, n - r0);
-        ctx->launches += infer(ctx, C, m, B, xp + r0 * C.dim, st);
-        if ((rc = each(r0, B))) return rc;
+        float *H = dst ? dst + r0 * ncls : fused ? C.tH : C.H;
+        if (fused) {
+            ctx->launches += infer(ctx, C, m, B, xp + r0 * C.dim, H, st);
+        } else {
+            ctx->launches += forward(ctx, C, m, B, xp + r0 * C.dim, nullptr, st);
+            if (dst && cudaMemcpyAsync(H, C.H, size_t(B) * ncls * sizeof(float),
+                                       cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+                return fail(ctx, CS_ECUDA, "copy of the logits failed");
+        }
+        if ((rc = each(r0, B, H))) return rc;
     }
     return CS_OK;
 }
@@ -471,14 +821,10 @@ cs_status cs_classifier_forward(cs_ctx *ctx, int32_t mesh_id, int64_t n, const d
     if (!C) return fail(ctx, CS_ENOPRED, "cs_classifier_forward: no classifier loaded");
     if (n == 0) return CS_OK;
     CCHK(cudaSetDevice(ctx->device));
-    const int ncls = cls_cells(C->dim);
-    cs_status rc = forward_chunks(ctx, *C, m->d, n, xp, nullptr, [&](int64_t r0, int64_t B) {
-        if (cudaMemcpyAsync(logits_out + r0 * ncls, C->H, size_t(B) * ncls * sizeof(float),
-                            cudaMemcpyDeviceToDevice, nullptr) != cudaSuccess)
-            return fail(ctx, CS_ECUDA, "cs_classifier_forward: copy of the logits failed");
-        return CS_OK;
-    });
+    cs_status rc = forward_chunks(ctx, *C, m->d, n, xp, logits_out, nullptr,
+                                  [](int64_t, int64_t, const float *) { return CS_OK; });
     if (rc) return rc;
+    CCHK(cudaGetLastError());
     CCHK(cudaDeviceSynchronize());
     return cs_device_status(ctx);
 }
@@ -542,11 +888,18 @@ cs_status cs_classifier_grad(cs_ctx *ctx, int32_t mesh_id, int64_t B, const doub
     Classifier *C = get_cls(ctx, m->d.dim);
     if (!C) return fail(ctx, CS_ENOPRED, "cs_classifier_grad: no classifier loaded");
     CCHK(cudaSetDevice(ctx->device));
-    cs_status rc = ensure_ws(ctx, *C, B, true, true);
+    const bool tiled = tiled_batch(B);
+    cs_status rc = tiled ? ensure_train(ctx, *C, B) : CS_OK;
+    if (rc == CS_OK && (!tiled || C->dim == 3)) rc = ensure_ws(ctx, *C, B, true, true);
     if (rc) return rc;
     CCHK(cudaMemset(C->loss, 0, sizeof(float)));
-    ctx->launches += forward(ctx, *C, m->d, B, xp, nullptr, nullptr);
-    ctx->launches += backward(ctx, *C, B, labels, nullptr, C->loss, nullptr);
+    if (tiled) {
+        ctx->launches += train_tiled(ctx, *C, m->d, B, xp, labels, nullptr, C->loss, nullptr);
+    } else {
+        ctx->launches += forward(ctx, *C, m->d, B, xp, nullptr, nullptr);
+        ctx->launches += backward(ctx, *C, B, labels, nullptr, C->loss, nullptr);
+    }
+    CCHK(cudaGetLastError());
     CCHK(cudaDeviceSynchronize());
     if ((rc = cs_device_status(ctx))) return rc;
     CCHK(cudaMemcpy(grad_out, C->g, size_t(C->n) * sizeof(float), cudaMemcpyDeviceToDevice));
@@ -566,7 +919,9 @@ cs_status cs_classifier_train(cs_ctx *ctx, int32_t mesh_id, const double *xp,
     if (!C) return fail(ctx, CS_ENOPRED, "cs_classifier_train: no classifier loaded");
     CCHK(cudaSetDevice(ctx->device));
     const int64_t B = std::min(batch, N);
-    cs_status rc = ensure_ws(ctx, *C, B, true, true);
+    const bool tiled = tiled_batch(B);
+    cs_status rc = tiled ? ensure_train(ctx, *C, B) : CS_OK;
+    if (rc == CS_OK && (!tiled || C->dim == 3)) rc = ensure_ws(ctx, *C, B, true, true);
     if (rc) return rc;
     float *losses = nullptr;
     if ((rc = dmalloc_n(ctx, &losses, size_t(std::max<int64_t>(steps, 1))))) return rc;
@@ -586,19 +941,25 @@ cs_status cs_classifier_train(cs_ctx *ctx, int32_t mesh_id, const double *xp,
             }
             idx[b] = perm[pos++];
         }
-        if (cudaMemcpy(C->idx, idx.data(), size_t(B) * sizeof(int64_t), cudaMemcpyHostToDevice) !=
+        int64_t *didx = tiled ? C->tidx : C->idx;
+        if (cudaMemcpy(didx, idx.data(), size_t(B) * sizeof(int64_t), cudaMemcpyHostToDevice) !=
             cudaSuccess) {
             out = fail(ctx, CS_ECUDA, "cs_classifier_train: index copy");
             break;
         }
-        ctx->launches += forward(ctx, *C, m->d, B, xp, C->idx, nullptr);
-        ctx->launches += backward(ctx, *C, B, labels, C->idx, losses + s, nullptr);
+        if (tiled) {
+            ctx->launches += train_tiled(ctx, *C, m->d, B, xp, labels, didx, losses + s, nullptr);
+        } else {
+            ctx->launches += forward(ctx, *C, m->d, B, xp, didx, nullptr);
+            ctx->launches += backward(ctx, *C, B, labels, didx, losses + s, nullptr);
+        }
         C->t += 1;
         ctx->launches += launch_adam(C->w, C->g, C->m, C->v, C->n, lr, C->t, ctx->sm_count, nullptr);
         C->packed_dirty = true;
     }
     if (out == CS_OK) {
-        cudaError_t e = cudaDeviceSynchronize();
+        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaDeviceSynchronize();
         if (e == cudaSuccess && loss_out && steps > 0)
             e = cudaMemcpy(loss_out, losses, size_t(steps) * sizeof(float), cudaMemcpyDeviceToHost);
         if (e != cudaSuccess)
@@ -652,8 +1013,8 @@ cs_status cs_track_classifier(cs_ctx *ctx, int32_t mesh_id, int64_t n, const dou
     launch_departure(n, C->dim, x, u, dt, C->xp, ctx->sm_count, st);
     ctx->launches += 1;
     const DevMesh &d = m->d;
-    rc = forward_chunks(ctx, *C, d, n, C->xp, st, [&](int64_t r0, int64_t B) {
-        launch_cls_start(d, B, C->xp + r0 * C->dim, C->H, start ? start + r0 : nullptr, r0,
+    rc = forward_chunks(ctx, *C, d, n, C->xp, nullptr, st, [&](int64_t r0, int64_t B, const float *H) {
+        launch_cls_start(d, B, C->xp + r0 * C->dim, H, start ? start + r0 : nullptr, r0,
                          C->starts + r0, nullptr, ctx->sm_count, st);
         ctx->launches += 1;
         return CS_OK;

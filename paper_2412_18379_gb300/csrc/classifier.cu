@@ -9,6 +9,7 @@
 // starts) and the FP64 feature values are those of a plain evaluation of the
 // same formulas; the network itself runs in BF16/FP32 (classifier.cpp).
 
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -292,6 +293,216 @@ __global__ void __launch_bounds__(1024) softmax_ce_kernel(const float *__restric
     }
 }
 
+// ---------------------------------------------------------------------------
+// Training on the tiled BF16 layouts of the fully connected layers (fc_tc.h)
+// ---------------------------------------------------------------------------
+
+// a thread pools one channel of a row: neighbouring threads read neighbouring
+// channels; columns of a channel are Pp consecutive ones
+template <int D>
+__global__ void __launch_bounds__(kT) pool_tiled_kernel(const float *__restrict__ z, int64_t B,
+                                                        FcMat cat) {
+    using G = Win<D>;
+    constexpr int C = kClsCh;
+    pdl_wait();
+    const int64_t rows = (B + 127) / 128 * 128;
+    for (int64_t q = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; q < rows * C;
+         q += int64_t(gridDim.x) * blockDim.x) {
+        const int c = int(q % C);
+        const int64_t b = q / C;
+        uint8_t *row = cat.p + (b >> 7) * cat.tile + int64_t(cat.chunk0) * kFcChunk + (b & 127) * 16;
+        const float *zb = z + b * G::P * C + c;
+        #pragma unroll
+        for (int p0 = 0; p0 < G::Pp; p0 += 4) {
+            float s[4] = {0.f, 0.f, 0.f, 0.f};
+            #pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int pp = p0 + u;
+                if (b >= B || pp >= G::Pp) continue;
+                const int px = pp % G::Wp, py = (pp / G::Wp) % G::Wp, pz = pp / (G::Wp * G::Wp);
+                for (int oz = 0; oz < (D == 3 ? 2 : 1); ++oz)
+                    for (int oy = 0; oy < 2; ++oy)
+                        for (int ox = 0; ox < 2; ++ox) {
+                            const int x = 2 * px + ox, y = 2 * py + oy, zz = 2 * pz + oz;
+                            const int p = D == 2 ? y * G::W + x : (zz * G::W + y) * G::W + x;
+                            s[u] += fmaxf(zb[p * C], 0.f);
+                        }
+                s[u] = s[u] / float(1 << D);
+            }
+            const int col = c * G::Pp + p0;
+            uint8_t *o = row + int64_t(col >> 3) * kFcChunk + (col & 7) * 2;
+            if constexpr (G::Pp % 4 == 0) {
+                const __nv_bfloat162 lo = __floats2bfloat162_rn(s[0], s[1]);
+                const __nv_bfloat162 hi = __floats2bfloat162_rn(s[2], s[3]);
+                *reinterpret_cast<uint2 *>(o) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo),
+                                                           *reinterpret_cast<const uint32_t *>(&hi));
+            } else {
+                #pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int cu = col + u;
+                    if (p0 + u < G::Pp)
+                        *reinterpret_cast<__nv_bfloat16 *>(row + int64_t(cu >> 3) * kFcChunk +
+                                                           (cu & 7) * 2) = __float2bfloat16_rn(s[u]);
+                }
+            }
+        }
+    }
+}
+
+// a block takes whole rows: the row's pooled gradient goes through shared
+// memory (read along the pooled positions, used along the channels); a thread
+// keeps one channel, whose column sum it carries
+template <int D>
+__global__ void __launch_bounds__(kT) pool_back_tiled_kernel(const float *__restrict__ dpool,
+                                                             const float *__restrict__ z,
+                                                             int64_t B, uint16_t *__restrict__ dz,
+                                                             float *__restrict__ part) {
+    using G = Win<D>;
+    constexpr int C = kClsCh, Ld = G::Pp | 1;      // odd stride: no bank conflicts
+    __shared__ float sg[C * Ld];
+    __shared__ float red[kT];
+    pdl_wait();
+    const int c = threadIdx.x % C;
+    float sum = 0.f;
+    for (int64_t b = blockIdx.x; b < B; b += gridDim.x) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < C * G::Pp; i += kT)
+            sg[i / G::Pp * Ld + i % G::Pp] = dpool[b * (C * G::Pp) + i];
+        __syncthreads();
+        for (int p = threadIdx.x / C; p < G::P; p += kT / C) {
+            const int px = p % G::W, py = (p / G::W) % G::W, pz = D == 3 ? p / (G::W * G::W) : 0;
+            float g = 0.f;
+            if (px < 2 * G::Wp && py < 2 * G::Wp && (D == 2 || pz < 2 * G::Wp) &&
+                z[(b * G::P + p) * C + c] > 0.f) {
+                const int pp = D == 2 ? (py / 2) * G::Wp + px / 2
+                                      : ((pz / 2) * G::Wp + py / 2) * G::Wp + px / 2;
+                g = sg[c * Ld + pp] / float(1 << D);
+            }
+            sum += g;
+            dz[(b * G::P + p) * C + c] = __bfloat16_as_ushort(__float2bfloat16_rn(g));
+        }
+    }
+    red[threadIdx.x] = sum;
+    __syncthreads();
+    if (threadIdx.x < C) {
+        float s = 0.f;
+        for (int i = 0; i < kT / C; ++i) s += red[i * C + c];
+        part[int64_t(blockIdx.x) * C + c] = s;
+    }
+}
+
+constexpr int kSmRows = 32;      // rows per block of the tiled softmax
+
+// rows with a label in [0, n_cls)
+__global__ void __launch_bounds__(1024) count_labels_kernel(const int32_t *__restrict__ labels,
+                                                            const int64_t *__restrict__ idx,
+                                                            int64_t B, int n_cls,
+                                                            int *__restrict__ count) {
+    __shared__ int cnt[32];
+    pdl_wait();
+    int c = 0;
+    for (int64_t b = threadIdx.x; b < B; b += blockDim.x) {
+        const int32_t l = labels[idx ? idx[b] : b];
+        c += l >= 0 && l < n_cls;
+    }
+    c = __reduce_add_sync(kFull, c);
+    if ((threadIdx.x & 31) == 0) cnt[threadIdx.x >> 5] = c;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int n = 0;
+        for (int w = 0; w < 32; ++w) n += cnt[w];
+        *count = n;
+    }
+}
+
+// softmax_ce_kernel's rows (the same arithmetic, a warp per row), spread over
+// blocks of kSmRows rows. NJ: columns per lane.
+template <int NJ>
+__global__ void __launch_bounds__(kT) softmax_ce_tiled_kernel(const float *__restrict__ H,
+                                                              const int32_t *__restrict__ labels,
+                                                              const int64_t *__restrict__ idx,
+                                                              int64_t B, int n_cls, FcMat gH,
+                                                              float *__restrict__ part,
+                                                              float *__restrict__ loss_part,
+                                                              const int *__restrict__ count) {
+    extern __shared__ float sred[];                 // [8][32 NJ]
+    __shared__ float lred[8];
+    pdl_wait();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n_valid = *count;
+    const float inv = n_valid > 0 ? 1.f / float(n_valid) : 0.f;
+    float col[NJ], lsum = 0.f;
+    #pragma unroll
+    for (int j = 0; j < NJ; ++j) col[j] = 0.f;
+    const int64_t b0 = int64_t(blockIdx.x) * kSmRows;
+    for (int r = warp; r < kSmRows; r += 8) {
+        const int64_t b = b0 + r;                   // rows past B up to a tile's end are zero
+        uint8_t *row = gH.p + (b >> 7) * gH.tile + int64_t(gH.chunk0) * kFcChunk + (b & 127) * 16;
+        float g[NJ];
+        #pragma unroll
+        for (int j = 0; j < NJ; ++j) g[j] = 0.f;
+        if (b < B) {
+            const int32_t l = labels[idx ? idx[b] : b];
+            const bool valid = l >= 0 && l < n_cls;
+            const float *h = H + b * n_cls;
+            float v[NJ], mx = -INFINITY;
+            #pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                v[j] = lane + 32 * j < n_cls ? h[lane + 32 * j] : -INFINITY;
+                if (lane + 32 * j < n_cls) mx = fmaxf(mx, v[j]);
+            }
+            mx = warp_max(mx);
+            float e[NJ], se = 0.f;
+            #pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                e[j] = expf(v[j] - mx);
+                if (lane + 32 * j < n_cls) se += e[j];
+            }
+            se = warp_sum(se);
+            const float rse = 1.f / se;
+            #pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                const int k = lane + 32 * j;
+                g[j] = valid && k < n_cls ? (e[j] * rse - (k == l ? 1.f : 0.f)) * inv : 0.f;
+            }
+            if (valid && lane == 0) lsum += logf(se) - (h[l] - mx);
+        }
+        #pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+            const int k = lane + 32 * j;
+            col[j] += g[j];
+            if (k < gH.chunks * 8)
+                *reinterpret_cast<__nv_bfloat16 *>(row + int64_t(k >> 3) * kFcChunk + (k & 7) * 2) =
+                    __float2bfloat16_rn(g[j]);
+        }
+    }
+    #pragma unroll
+    for (int j = 0; j < NJ; ++j) sred[warp * (32 * NJ) + lane + 32 * j] = col[j];
+    if (lane == 0) lred[warp] = lsum;
+    __syncthreads();
+    for (int k = threadIdx.x; k < n_cls; k += kT) {
+        float s = 0.f;
+        for (int w = 0; w < 8; ++w) s += sred[w * (32 * NJ) + k];
+        part[int64_t(blockIdx.x) * n_cls + k] = s;
+    }
+    if (threadIdx.x == 0) {
+        float s = 0.f;
+        for (int w = 0; w < 8; ++w) s += lred[w];
+        loss_part[blockIdx.x] = s;
+    }
+}
+
+__global__ void __launch_bounds__(32) loss_sum_kernel(const float *__restrict__ loss_part, int n,
+                                                      const int *__restrict__ count,
+                                                      float *__restrict__ loss) {
+    pdl_wait();
+    float s = 0.f;
+    for (int i = threadIdx.x; i < n; i += 32) s += loss_part[i];
+    s = warp_sum(s);
+    const int n_valid = *count;
+    if (threadIdx.x == 0) *loss += s * (n_valid > 0 ? 1.f / float(n_valid) : 0.f);
+}
+
 // label = window cell (x fastest) holding the centroid of the host element,
 // the cell coordinates clamped into the window around x_p's ASG cell (label
 // may be host: each row is read before it is written)
@@ -469,6 +680,42 @@ void launch_cls_uncat_relu_back(const float *dcat, int64_t ldc, int64_t off, con
 void launch_softmax_ce(const float *H, const int32_t *labels, const int64_t *idx, int64_t B,
                        int n_cls, float *dH, float *loss, cudaStream_t st) {
     softmax_ce_kernel<<<1, 1024, 0, st>>>(H, labels, idx, B, n_cls, dH, loss);
+}
+
+void launch_cls_pool_tiled(int dim, const float *z, int64_t B, const FcMat &cat, int sm_count,
+                           cudaStream_t st) {
+    const int g = blocks_for((B + 127) / 128 * 128 * kClsCh, sm_count, 8);
+    launch_pdl(dim == 2 ? pool_tiled_kernel<2> : pool_tiled_kernel<3>, dim3(g), dim3(kT), 0, st, z, B,
+               cat);
+}
+
+int cls_pool_back_blocks(int64_t B, int sm_count) {
+    return int(std::min<int64_t>(B, int64_t(sm_count) * 4));
+}
+
+void launch_cls_pool_back_tiled(int dim, const float *dpool, const float *z, int64_t B,
+                                uint16_t *dz, float *part, int sm_count, cudaStream_t st) {
+    launch_pdl(dim == 2 ? pool_back_tiled_kernel<2> : pool_back_tiled_kernel<3>,
+               dim3(cls_pool_back_blocks(B, sm_count)), dim3(kT), 0, st, dpool, z, B, dz, part);
+}
+
+int cls_softmax_blocks(int64_t B) { return int((B + 127) / 128 * (128 / kSmRows)); }
+
+void launch_softmax_ce_tiled(const float *H, const int32_t *labels, const int64_t *idx, int64_t B,
+                             int n_cls, const FcMat &gH, float *part, float *loss_part, int *count,
+                             cudaStream_t st) {
+    launch_pdl(count_labels_kernel, dim3(1), dim3(1024), 0, st, labels, idx, B, n_cls, count);
+    const int g = cls_softmax_blocks(B);
+    if (n_cls <= 96)
+        launch_pdl(softmax_ce_tiled_kernel<3>, dim3(g), dim3(kT), 8 * 96 * 4, st, H, labels, idx, B,
+                   n_cls, gH, part, loss_part, count);
+    else
+        launch_pdl(softmax_ce_tiled_kernel<11>, dim3(g), dim3(kT), 8 * 352 * 4, st, H, labels, idx, B,
+                   n_cls, gH, part, loss_part, count);
+}
+
+void launch_loss_sum(const float *loss_part, int n, const int *count, float *loss, cudaStream_t st) {
+    launch_pdl(loss_sum_kernel, dim3(1), dim3(32), 0, st, loss_part, n, count, loss);
 }
 
 void launch_cls_labels(const DevMesh &m, int64_t n, const double *xp, const int32_t *host,

@@ -6,6 +6,7 @@
 
 #include <cstdint>
 
+#include "fc_tc.h"
 #include "internal.h"
 
 namespace cs {
@@ -55,13 +56,34 @@ void launch_cls_start(const DevMesh &m, int64_t n, const double *xp, const float
 // module 1 fused on the tensor cores (classifier_tc.cu): conv1 and conv2
 // weights packed for the kernel (bytes, and the packing from the FP32
 // parameters), then per particle the window inputs, both convolutions and the
-// pooling into cat[b][0, 32 (W/2)^dim) (row stride ldc) and the offset into
-// off[b][dim]. pool_f: the mesh's pooled centroids as float hi + lo.
+// pooling into the first 32 (W/2)^dim columns of cat (BF16 tiled, fc_tc.h) and
+// the offset into off[b][dim]. pool_f: the mesh's pooled centroids as float hi + lo.
 int64_t cls_packed_bytes(int dim);
 void launch_cls_pack(int dim, const float *w, int64_t off_w1, int64_t off_b1, int64_t off_w2,
                      int64_t off_b2, uint8_t *packed, cudaStream_t st);
 void launch_cls_conv_tc(const DevMesh &m, const float *pool_f, int64_t B, const double *xp,
-                        const uint8_t *packed, float *cat, int64_t ldc, float *off, int *err,
+                        const uint8_t *packed, const FcMat &cat, float *off, int *err,
                         int sm_count, cudaStream_t st);
+
+// Training on the tiled layouts (classifier.cu).
+// The pooled ReLU(z) of pool_relu as BF16 into cat's first columns (zero rows past B)
+void launch_cls_pool_tiled(int dim, const float *z, int64_t B, const FcMat &cat, int sm_count,
+                           cudaStream_t st);
+// the pooling's gradient through the second ReLU: dz[b][p][c] BF16 from
+// dpool [B][32 (W/2)^dim], and its column sums part[block][32], blocks =
+// cls_pool_back_blocks
+int cls_pool_back_blocks(int64_t B, int sm_count);
+void launch_cls_pool_back_tiled(int dim, const float *dpool, const float *z, int64_t B,
+                                uint16_t *dz, float *part, int sm_count, cudaStream_t st);
+// softmax and cross-entropy gradient (softmax_ce) into the tiled gH (n_cls
+// columns rounded up to 16, zero padding), column sums and loss sums per block:
+// part[block][n_cls], loss_part[block], blocks = cls_softmax_blocks(B); the
+// loss is the sum over n_valid, a count left in *count
+int cls_softmax_blocks(int64_t B);
+void launch_softmax_ce_tiled(const float *H, const int32_t *labels, const int64_t *idx, int64_t B,
+                             int n_cls, const FcMat &gH, float *part, float *loss_part, int *count,
+                             cudaStream_t st);
+// *loss += sum of n loss_part / max(*count, 1)
+void launch_loss_sum(const float *loss_part, int n, const int *count, float *loss, cudaStream_t st);
 
 }  // namespace cs

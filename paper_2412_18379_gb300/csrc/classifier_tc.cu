@@ -202,8 +202,7 @@ __device__ __forceinline__ void cls_inputs(const DevMesh &m, const float *__rest
 template <int D>
 __global__ void __launch_bounds__(kThreadsC, D == 2 ? 4 : 1) cls_conv_tc_kernel(
     const DevMesh m, const float *__restrict__ pool_f, int64_t B, const double *__restrict__ xp,
-    const uint8_t *__restrict__ packed, float *__restrict__ cat, int64_t ldc,
-    float *__restrict__ off_out, int *err) {
+    const uint8_t *__restrict__ packed, const FcMat cat, float *__restrict__ off_out, int *err) {
     using G = ClsGeo<D>;
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t *in = smem + G::kSmIn;
@@ -348,18 +347,34 @@ __global__ void __launch_bounds__(kThreadsC, D == 2 ? 4 : 1) cls_conv_tc_kernel(
             }
             fence_before();
             epi_sync();
-            for (int i = tid; i < 32 * G::Pp; i += kEpiC * 32) {
-                const int c = i % 32, pp = i / 32;
-                const int px = pp % G::Wp, py = (pp / G::Wp) % G::Wp, pz = D == 3 ? pp / (G::Wp * G::Wp) : 0;
-                float s = 0.f;
-                for (int oz = 0; oz < (D == 3 ? 2 : 1); ++oz)
-                    for (int oy = 0; oy < 2; ++oy)
-                        for (int ox = 0; ox < 2; ++ox) {
-                            const int r = D == 2 ? (2 * py + oy) * G::E + 2 * px + ox
-                                                 : ((2 * pz + oz) * G::E + 2 * py + oy) * G::E + 2 * px + ox;
-                            s += stage[r * G::Ld + c];
-                        }
-                cat[b * ldc + int64_t(c) * G::Pp + pp] = s / float(1 << D);
+            // BF16 into the tiled feature matrix (fc_tc.h), row b: column
+            // c Pp + pp. 2-D: four neighbouring columns per thread
+            uint8_t *crow = cat.p + (b >> 7) * cat.tile + int64_t(cat.chunk0) * kFcChunk + (b & 127) * 16;
+            constexpr int kPer = G::Pp % 4 == 0 ? 4 : 1;
+            for (int i = tid; i < 32 * G::Pp / kPer; i += kEpiC * 32) {
+                const int c = i % 32, p0 = i / 32 * kPer;
+                float s[kPer];
+                #pragma unroll
+                for (int u = 0; u < kPer; ++u) {
+                    const int pp = p0 + u;
+                    const int px = pp % G::Wp, py = (pp / G::Wp) % G::Wp, pz = D == 3 ? pp / (G::Wp * G::Wp) : 0;
+                    s[u] = 0.f;
+                    for (int oz = 0; oz < (D == 3 ? 2 : 1); ++oz)
+                        for (int oy = 0; oy < 2; ++oy)
+                            for (int ox = 0; ox < 2; ++ox) {
+                                const int r = D == 2 ? (2 * py + oy) * G::E + 2 * px + ox
+                                                     : ((2 * pz + oz) * G::E + 2 * py + oy) * G::E + 2 * px + ox;
+                                s[u] += stage[r * G::Ld + c];
+                            }
+                    s[u] = s[u] / float(1 << D);
+                }
+                const int col = c * G::Pp + p0;
+                uint8_t *o = crow + int64_t(col >> 3) * kFcChunk + (col & 7) * 2;
+                if constexpr (kPer == 4)
+                    *reinterpret_cast<uint2 *>(o) =
+                        make_uint2(pack_bf16x2(s[0], s[1]), pack_bf16x2(s[2], s[3]));
+                else
+                    *reinterpret_cast<__nv_bfloat16 *>(o) = __float2bfloat16_rn(s[0]);
             }
             epi_sync();
         }
@@ -408,8 +423,8 @@ __global__ void cls_pack_kernel(const float *__restrict__ w, int64_t off_w1, int
 
 template <int D>
 void launch_conv(const DevMesh &m, const float *pool_f, int64_t B, const double *xp,
-                 const uint8_t *packed, float *cat, int64_t ldc, float *off, int *err,
-                 int sm_count, cudaStream_t st) {
+                 const uint8_t *packed, const FcMat &cat, float *off, int *err, int sm_count,
+                 cudaStream_t st) {
     using G = ClsGeo<D>;
     static bool attr = false;
     if (!attr) {
@@ -419,8 +434,8 @@ void launch_conv(const DevMesh &m, const float *pool_f, int64_t B, const double 
     }
     const int per_sm = D == 2 ? 4 : 1;
     const int grid = int(std::min<int64_t>(B, int64_t(sm_count) * per_sm));
-    cls_conv_tc_kernel<D><<<grid, kThreadsC, G::kSmTotal, st>>>(m, pool_f, B, xp, packed, cat, ldc,
-                                                                off, err);
+    cls_conv_tc_kernel<D><<<grid, kThreadsC, G::kSmTotal, st>>>(m, pool_f, B, xp, packed, cat, off,
+                                                                err);
 }
 
 }  // namespace
@@ -436,13 +451,13 @@ void launch_cls_pack(int dim, const float *w, int64_t off_w1, int64_t off_b1, in
 }
 
 void launch_cls_conv_tc(const DevMesh &m, const float *pool_f, int64_t B, const double *xp,
-                        const uint8_t *packed, float *cat, int64_t ldc, float *off, int *err,
+                        const uint8_t *packed, const FcMat &cat, float *off, int *err,
                         int sm_count, cudaStream_t st) {
     if (B <= 0) return;
     if (m.dim == 2)
-        launch_conv<2>(m, pool_f, B, xp, packed, cat, ldc, off, err, sm_count, st);
+        launch_conv<2>(m, pool_f, B, xp, packed, cat, off, err, sm_count, st);
     else
-        launch_conv<3>(m, pool_f, B, xp, packed, cat, ldc, off, err, sm_count, st);
+        launch_conv<3>(m, pool_f, B, xp, packed, cat, off, err, sm_count, st);
 }
 
 }  // namespace cs
