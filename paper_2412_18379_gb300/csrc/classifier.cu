@@ -48,67 +48,115 @@ __global__ void departure_kernel(int64_t n, const double *__restrict__ x,
         xp[i] = __dsub_rn(x[i], __dmul_rn(u[i], dt));
 }
 
+// float(a / s) with the quotient rounded to FP64 first, without the FP64
+// division (some 25 instructions of the pipe that every FP64 instruction
+// holds for ~56 cycles per warp): a * (1 / s) is within 2 ulp of it, so both
+// round to the same float unless a rounding boundary (the midpoint of two
+// floats: the 29 dropped bits at 2^28) lies that close; those values, and
+// those outside the normal floats, take the division.
+__device__ __forceinline__ float quotient_to_float(double a, double s, double inv) {
+    const double q = __dmul_rn(a, inv);
+    uint32_t lo, hi;
+    dbits(q, lo, hi);
+    const int E = int((hi >> 20) & 0x7ffu) - 1023;
+    const int tail = int(lo & 0x1fffffffu) - 0x10000000;
+    if (((hi << 1) | lo) == 0 || (E >= -126 && E < 127 && (tail > 16 || tail < -16)))
+        return __double2float_rn(q);
+    return __double2float_rn(__ddiv_rn(a, s));
+}
+
+// Cell of one axis: the FP64 formula's, certified in FP32 (grid_cell_cert's
+// test) where the rounding bound cannot move the quotient across an integer.
+__device__ __forceinline__ int cell_axis_cert(const DevMesh &m, int k, double x, float xh, float xl) {
+    const float df = (xh - m.lo_h[k]) + (xl - m.lo_l[k]);
+    const float ed = delta_bound(df, xh, m.lo_h[k]);
+    const float q = df * m.inv_sa[k];
+    const float bnd = fmaf(2.0f * ed, m.inv_sa[k], fmaf(k8U, fabsf(q), kTiny));
+    const int a = __float2int_rd(q - bnd), b = __float2int_rd(q + bnd);
+    if (a == b && fabsf(q) < 4.0e6f) return a < 0 ? 0 : (a > m.ga[k] - 1 ? m.ga[k] - 1 : a);
+    return int(cell_axis64(x, m.lo[k], m.sa[k], m.ga[k]));
+}
+
 // Inputs of row b (particle idx[b], or b): the window of dim channels at
-// every (padded, if pad) window position, channels first, and the offset.
+// every (padded, if PAD) window position, channels first, and the offset.
 // Window cell o (x fastest) of a particle whose ASG cell is c is cell
 // c - W/2 + o; its point is the pooled centroid of that cell if the cell is
-// in the grid and holds one, else its centre lo + (cell + 1/2) s.
-template <int D>
+// in the grid and holds one, else its centre lo + (cell + 1/2) s. A warp takes
+// a particle: its cell and offset once, then 32 window positions at a time.
+template <int D, int PAD>
 __global__ void __launch_bounds__(kT) features_kernel(const DevMesh m, int64_t B,
                                                       const double *__restrict__ xp,
-                                                      const int64_t *__restrict__ idx, int pad,
+                                                      const int64_t *__restrict__ idx,
                                                       float *__restrict__ win,
                                                       float *__restrict__ offset) {
     using G = Win<D>;
-    const int E = G::W + 2 * pad;                    // stored edge
-    const int PE = D == 2 ? E * E : E * E * E;
-    const int64_t total = B * PE;
-    for (int64_t q = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; q < total;
-         q += int64_t(gridDim.x) * blockDim.x) {
-        const int64_t b = q / PE;
-        const int pe = int(q % PE);
-        int e[3] = {pe % E, (pe / E) % E, D == 3 ? pe / (E * E) : 0};
-        bool ring = false;
-        #pragma unroll
-        for (int k = 0; k < D; ++k) {
-            e[k] -= pad;
-            ring |= e[k] < 0 || e[k] >= G::W;
-        }
-        float *out = win + b * D * PE + pe;
-        if (ring) {
-            #pragma unroll
-            for (int k = 0; k < D; ++k) out[int64_t(k) * PE] = 0.f;
-            continue;
-        }
+    constexpr int E = G::W + 2 * PAD;                // stored edge
+    constexpr int PE = D == 2 ? E * E : E * E * E;
+    __shared__ double inv_s[3];
+    if (threadIdx.x < D) inv_s[threadIdx.x] = __ddiv_rn(1.0, m.sa[threadIdx.x]);
+    __syncthreads();
+    double inv[D];
+    #pragma unroll
+    for (int k = 0; k < D; ++k) inv[k] = inv_s[k];
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = int64_t(gridDim.x) * (blockDim.x >> 5);
+    for (int64_t b = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; b < B; b += warps) {
         const int64_t r = idx ? idx[b] : b;
         double x[D];
-        int64_t c0[D], cc[D];
-        bool inside = true;
+        int c0[D];
         #pragma unroll
         for (int k = 0; k < D; ++k) {
             x[k] = xp[r * D + k];
-            c0[k] = cell_axis64(x[k], m.lo[k], m.sa[k], m.ga[k]);
-            cc[k] = c0[k] - G::W / 2 + e[k];
-            inside &= cc[k] >= 0 && cc[k] < m.ga[k];
+            float xh, xl;
+            split_double(x[k], xh, xl);
+            c0[k] = cell_axis_cert(m, k, x[k], xh, xl);
         }
-        int64_t flat = 0;
-        #pragma unroll
-        for (int k = D - 1; k >= 0; --k) {
-            const int64_t ck = cc[k] < 0 ? 0 : (cc[k] > m.ga[k] - 1 ? m.ga[k] - 1 : cc[k]);
-            flat = flat * m.ga[k] + ck;
+        if (lane < D) {
+            double xv = x[0], s = m.sa[0], lo = m.lo[0];
+            int c = c0[0];
+            #pragma unroll
+            for (int k = 1; k < D; ++k)
+                if (lane == k) {
+                    xv = x[k];
+                    s = m.sa[k];
+                    lo = m.lo[k];
+                    c = c0[k];
+                }
+            offset[b * D + lane] = float(__dsub_rn(__ddiv_rn(__dsub_rn(xv, lo), s), double(c) + 0.5));
         }
-        const bool has = inside && !isnan(m.pool[flat * D]);
-        #pragma unroll
-        for (int k = 0; k < D; ++k) {
-            const double pt = has ? m.pool[flat * D + k]
-                                  : __dadd_rn(m.lo[k], __dmul_rn(double(cc[k]) + 0.5, m.sa[k]));
-            out[int64_t(k) * PE] = float(__ddiv_rn(__dsub_rn(pt, x[k]), m.sa[k]));
-        }
-        if (e[0] == 0 && e[1] == 0 && e[2] == 0) {
+        float *out = win + b * D * PE;
+        #pragma unroll 2
+        for (int pe = lane; pe < PE; pe += 32) {
+            int e[3] = {pe % E - PAD, (pe / E) % E - PAD, D == 3 ? pe / (E * E) - PAD : 0};
+            bool ring = false, inside = true;
+            int64_t flat = 0;
+            #pragma unroll
+            for (int k = D - 1; k >= 0; --k) {
+                ring |= e[k] < 0 || e[k] >= G::W;
+                const int cc = c0[k] - G::W / 2 + e[k];
+                inside &= cc >= 0 && cc < m.ga[k];
+                flat = flat * m.ga[k] + (cc < 0 ? 0 : (cc > m.ga[k] - 1 ? m.ga[k] - 1 : cc));
+            }
+            if (ring) {
+                #pragma unroll
+                for (int k = 0; k < D; ++k) out[int64_t(k) * PE + pe] = 0.f;
+                continue;
+            }
+            double pt[D];
+            #pragma unroll
+            for (int k = 0; k < D; ++k) pt[k] = __ldg(m.pool + flat * D + k);
+            uint32_t nl, nh;
+            dbits(pt[0], nl, nh);
+            const bool nan = (nh & 0x7ff00000u) == 0x7ff00000u && ((nh & 0xfffffu) | nl) != 0;
+            if (!inside || nan) {
+                #pragma unroll
+                for (int k = 0; k < D; ++k)
+                    pt[k] = __dadd_rn(m.lo[k], __dmul_rn(double(c0[k] - G::W / 2 + e[k]) + 0.5, m.sa[k]));
+            }
             #pragma unroll
             for (int k = 0; k < D; ++k)
-                offset[b * D + k] = float(__dsub_rn(__ddiv_rn(__dsub_rn(x[k], m.lo[k]), m.sa[k]),
-                                                    double(c0[k]) + 0.5));
+                out[int64_t(k) * PE + pe] =
+                    quotient_to_float(__dsub_rn(pt[k], x[k]), m.sa[k], inv[k]);
         }
     }
 }
@@ -618,13 +666,15 @@ void launch_departure(int64_t n, int dim, const double *x, const double *u, doub
 
 void launch_cls_features(const DevMesh &m, int64_t B, const double *xp, const int64_t *idx,
                          bool pad, float *win, float *offset, int sm_count, cudaStream_t st) {
-    const int E = cls_window(m.dim) + (pad ? 2 : 0);
-    const int64_t total = B * (m.dim == 2 ? E * E : E * E * E);
-    const int g = blocks_for(total, sm_count);
-    if (m.dim == 2)
-        features_kernel<2><<<g, kT, 0, st>>>(m, B, xp, idx, pad ? 1 : 0, win, offset);
+    const int g = int(std::max<int64_t>(1, std::min<int64_t>((B + 7) / 8, int64_t(sm_count) * 16)));
+    if (m.dim == 2 && pad)
+        features_kernel<2, 1><<<g, kT, 0, st>>>(m, B, xp, idx, win, offset);
+    else if (m.dim == 2)
+        features_kernel<2, 0><<<g, kT, 0, st>>>(m, B, xp, idx, win, offset);
+    else if (pad)
+        features_kernel<3, 1><<<g, kT, 0, st>>>(m, B, xp, idx, win, offset);
     else
-        features_kernel<3><<<g, kT, 0, st>>>(m, B, xp, idx, pad ? 1 : 0, win, offset);
+        features_kernel<3, 0><<<g, kT, 0, st>>>(m, B, xp, idx, win, offset);
 }
 
 void launch_cls_pad(int dim, const float *y, int64_t B, int C, float *a, int sm_count,
