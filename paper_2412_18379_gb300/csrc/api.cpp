@@ -287,6 +287,8 @@ cs_status cs_mesh_upload(cs_ctx *ctx, int dim, int64_t n_v, const double *xyz, i
     d.centroid = cent;
     d.iperm = iperm;
     d.node_elem = node;
+    d.xyz = xyzd;
+    d.vhost = nullptr;
     d.seed = seed;
     d.pool = pool;
     d.pool_f = pool_f;
@@ -325,6 +327,13 @@ cs_status cs_mesh_upload(cs_ctx *ctx, int dim, int64_t n_v, const double *xyz, i
     d.pseed = seed;
 
     ctx->launches += cs::launch_seed_grid(d, seed, ctx->sm_count, nullptr);
+    // hosts of the vertices, where memory (or the budget) has room for them:
+    // the walk does without, only slower at nodes at rest
+    int2 *vhost = nullptr;
+    if (dev_copy<int2>(ctx, m, nullptr, size_t(n_v), &vhost) == CS_OK) {
+        ctx->launches += cs::launch_vertex_hosts(d, vhost, ctx->sm_count, nullptr);
+        d.vhost = vhost;
+    }
     cudaError_t e = cudaDeviceSynchronize();
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {

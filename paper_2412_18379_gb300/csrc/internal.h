@@ -63,6 +63,10 @@ struct DevMesh {
     const double *centroid;   // [n_e][dim], internal order
     const int32_t *iperm;     // user id -> internal id
     const int32_t *node_elem; // [n_v] internal id of the plain-SNS start
+    const double *xyz;        // [n_v][dim] the uploaded vertices, user order
+    const int2 *vhost;        // [n_v] host (user id, or -1) of every point within (float
+                              // bits) .y of the vertex on each axis; .y < 0: unknown.
+                              // null: not resident (the walk searches instead)
     const int32_t *seed;      // [n_asg] internal id of the host of each cell centre, or -1
     const double *pool;       // [n_asg][dim] mean element centroid per ASG cell, NaN if none
     const float *pool_f;      // [n_asg][dim][2] the same as float hi + lo (NaN hi if none)
@@ -251,6 +255,7 @@ struct Profiler {
 int launch_track(const DevMesh &m, const TrackArgs &a, Scratch &s, int sm_count,
                  cudaStream_t st, Profiler *prof = nullptr);
 int launch_seed_grid(const DevMesh &m, int32_t *seed, int sm_count, cudaStream_t st);
+int launch_vertex_hosts(const DevMesh &m, int2 *vhost, int sm_count, cudaStream_t st);
 int launch_stats(int64_t n, const int32_t *path, const uint8_t *status, int64_t *out,
                  int sm_count, cudaStream_t st);
 int launch_error_stats(const DevMesh &m, int64_t n, const int32_t *start, const int32_t *host,

