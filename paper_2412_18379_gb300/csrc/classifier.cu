@@ -580,12 +580,6 @@ __global__ void __launch_bounds__(kT) labels_kernel(const DevMesh m, int64_t n,
     }
 }
 
-template <int D>
-__device__ __forceinline__ int32_t rec_uid(const DevMesh &m, int32_t internal) {
-    if (D == 2) return static_cast<const WalkRec2 *>(m.recw)[internal].uid;
-    return static_cast<const WalkRec3 *>(m.recw)[internal].uid;
-}
-
 // K_p (Eq. 8): one warp per particle takes the class of the largest logit
 // (the lowest among equal ones; NaN never wins), then the ASG seed of that
 // window cell (user id), else the fallback start (fallback[i], or the plain
@@ -640,7 +634,7 @@ __global__ void __launch_bounds__(kT) start_kernel(const DevMesh m, int64_t n,
                 #pragma unroll
                 for (int k = D - 1; k >= 0; --k) flat = flat * m.ga[k] + cc[k];
                 const int32_t seed = m.seed[flat];
-                if (seed >= 0) s = rec_uid<D>(m, seed);
+                if (seed >= 0) s = walk_uid<D>(m.recw, seed);
             }
         }
         if (s < 0) {
@@ -648,7 +642,7 @@ __global__ void __launch_bounds__(kT) start_kernel(const DevMesh m, int64_t n,
                 s = fallback[i];
             } else {
                 const int32_t e = m.node_elem[row0 + i];
-                s = e < 0 ? -1 : rec_uid<D>(m, e);
+                s = e < 0 ? -1 : walk_uid<D>(m.recw, e);
             }
         }
         start[i] = s;

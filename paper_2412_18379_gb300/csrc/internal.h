@@ -23,7 +23,13 @@ struct Server;   // serve.cpp
 // needs: the origin vertex v0 split into float hi + lo parts, the inverse-
 // affine matrix M rounded to float, the neighbour across face i (internal id,
 // -1 on the boundary) and the caller's id of the element. 48 bytes (2-D, two
-// 32-byte sectors) / 80 bytes (3-D, three sectors).
+// 32-byte sectors) / 80 bytes (3-D, three sectors). A step's lanes read records
+// on as many lines, so what a step costs the L1 is one lookup per lane and
+// load: records are stored in pairs so that each is one (3-D: two) aligned
+// 32-byte load and one 16-byte load, where 16-byte loads took three (five):
+//   2-D, 96 bytes:  [main 0: 32][tail 0: 16][tail 1: 16][main 1: 32]
+//   3-D, 160 bytes: [main 0: 64][tail 0: 16][tail 1: 16][main 1: 64]
+// main: all but the struct's last 16 bytes, which are the tail.
 //
 // The exact record holds v0 and M in FP64 (row k of M gives
 // lambda_{k+1} = M[k] . (x_p - v0)); it is read only when the FP32 filter
@@ -53,11 +59,25 @@ static_assert(sizeof(WalkRec3) == 80, "WalkRec3 is 80 bytes");
 static_assert(sizeof(ExactRec2) == 48, "ExactRec2 is 48 bytes");
 static_assert(sizeof(ExactRec3) == 96, "ExactRec3 is 96 bytes");
 
+// byte offsets of record e's parts in the paired layout, and its size
+#ifdef __CUDACC__
+#define CS_HD __host__ __device__
+#else
+#define CS_HD
+#endif
+CS_HD inline int64_t walk_main(int dim, int64_t e) {
+    return dim == 2 ? (e >> 1) * 96 + (e & 1) * 64 : (e >> 1) * 160 + (e & 1) * 96;
+}
+CS_HD inline int64_t walk_tail(int dim, int64_t e) {
+    return dim == 2 ? (e >> 1) * 96 + 32 + (e & 1) * 16 : (e >> 1) * 160 + 64 + (e & 1) * 16;
+}
+CS_HD inline int64_t walk_bytes(int dim, int64_t n_e) { return (n_e + 1) / 2 * (dim == 2 ? 96 : 160); }
+
 // Everything a kernel needs to know about a resident mesh (passed by value).
 struct DevMesh {
     int32_t dim;
     int64_t n_v, n_e;
-    const void *recw;         // WalkRec2 / WalkRec3 [n_e], Hilbert (internal) order
+    const void *recw;         // WalkRec2 / WalkRec3 [n_e] in pairs, Hilbert (internal) order
     const void *recx;         // ExactRec2 / ExactRec3 [n_e], same order
     const int32_t *conn;      // [n_e][dim+1] vertex ids, internal order
     const double *centroid;   // [n_e][dim], internal order

@@ -328,15 +328,19 @@ cs_status build_host_mesh(int dim, int64_t n_v, const double *xyz, int64_t n_e,
     // ---- records, connectivity and centroids in internal order ----
     // walk record: v0 as float hi + lo (hi = v0 rounded to float, lo = the
     // remainder v0 - hi rounded to float), M rounded to float
-    const size_t wb = dim == 2 ? sizeof(WalkRec2) : sizeof(WalkRec3);
     const size_t xb = dim == 2 ? sizeof(ExactRec2) : sizeof(ExactRec3);
-    H.recw.assign(size_t(n_e) * wb, 0);
+    H.recw.assign(size_t(walk_bytes(dim, n_e)), 0);
     H.recx.assign(size_t(n_e) * xb, 0);
     H.conn.resize(size_t(n_e) * nv);
     H.centroid.resize(size_t(n_e) * dim);
     auto split = [](double v, float &hi, float &lo) {
         hi = static_cast<float>(v);
         lo = static_cast<float>(v - static_cast<double>(hi));
+    };
+    // a record into its two places of the paired layout
+    auto put = [&](int64_t i, const void *w, size_t main) {
+        std::memcpy(&H.recw[size_t(walk_main(dim, i))], w, main);
+        std::memcpy(&H.recw[size_t(walk_tail(dim, i))], static_cast<const char *>(w) + main, 16);
     };
     for (int64_t i = 0; i < n_e; ++i) {
         const int64_t l = H.order[i];
@@ -352,7 +356,7 @@ cs_status build_host_mesh(int dim, int64_t n_v, const double *xyz, int64_t n_e,
                 w.nbr[f] = n < 0 ? -1 : H.iperm[n];
             }
             w.uid = int32_t(l);
-            std::memcpy(&H.recw[size_t(i) * wb], &w, wb);
+            put(i, &w, sizeof(w) - 16);
             std::memcpy(&H.recx[size_t(i) * xb], &x, xb);
         } else {
             WalkRec3 w{};
@@ -366,7 +370,7 @@ cs_status build_host_mesh(int dim, int64_t n_v, const double *xyz, int64_t n_e,
                 w.nbr[f] = n < 0 ? -1 : H.iperm[n];
             }
             w.uid = int32_t(l);
-            std::memcpy(&H.recw[size_t(i) * wb], &w, wb);
+            put(i, &w, sizeof(w) - 16);
             std::memcpy(&H.recx[size_t(i) * xb], &x, xb);
         }
         for (int k = 0; k < nv; ++k) H.conn[i * nv + k] = conn_user[l * nv + k];

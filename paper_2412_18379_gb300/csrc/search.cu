@@ -57,7 +57,6 @@ __global__ void __launch_bounds__(256) seed_kernel(const DevMesh m, int32_t *see
 // end their walk at such a point.
 template <int D>
 __global__ void __launch_bounds__(256) vertex_host_kernel(const DevMesh m, int2 *vhost) {
-    using WR = typename Recs<D>::W;
     using XR = typename Recs<D>::X;
     const int lane = threadIdx.x & 31;
     const int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
@@ -96,7 +95,7 @@ __global__ void __launch_bounds__(256) vertex_host_kernel(const DevMesh m, int2 
                 const double slack = in ? lo + CS_EPS : -CS_EPS - lo;
                 r = fmin(r, (0.5 * slack - 1e-14 * (1.0 + S)) / N);
                 if (!(slack >= 0.0)) r = -1.0;     // NaN
-                if (in) best = min(best, unsigned(static_cast<const WR *>(m.recw)[e].uid));
+                if (in) best = min(best, unsigned(walk_uid<D>(m.recw, e)));
             }
         }
         best = __reduce_min_sync(kFull, best);

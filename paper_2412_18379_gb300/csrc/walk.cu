@@ -207,13 +207,12 @@ __device__ __forceinline__ int32_t vertex_host(const DevMesh &m, int32_t cur, co
 template <int D>
 __global__ void __launch_bounds__(256, D == 2 ? 4 : 3) walk_kernel(const DevMesh m, const TrackArgs a,
                                                    int32_t *cursor, int32_t *next_cursor) {
-    using WR = typename Recs<D>::W;
     using XR = typename Recs<D>::X;
     __shared__ Queue<D> queues[kWarps];
     __shared__ Prefetch<D> prefetched[kPrefetch<D> ? kWarps : 1];
     Queue<D> &q = queues[threadIdx.x >> 5];
     Prefetch<D> &f = prefetched[kPrefetch<D> ? threadIdx.x >> 5 : 0];
-    const WR *__restrict__ rw = static_cast<const WR *>(m.recw);
+    const uint8_t *__restrict__ rw = static_cast<const uint8_t *>(m.recw);
     const XR *__restrict__ rx = static_cast<const XR *>(m.recx);
     const int lane = threadIdx.x & 31;
     const int64_t n = a.n;

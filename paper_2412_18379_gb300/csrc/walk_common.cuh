@@ -61,8 +61,8 @@ constexpr float kNegEpsIn = -0.99e-12f;      // certain: lambda >= -eps
 constexpr float kNegEpsOut = -1.01e-12f;     // certain: lambda <  -eps
 
 template <int D> struct Recs;
-template <> struct Recs<2> { using W = WalkRec2; using X = ExactRec2; };
-template <> struct Recs<3> { using W = WalkRec3; using X = ExactRec3; };
+template <> struct Recs<2> { using X = ExactRec2; };
+template <> struct Recs<3> { using X = ExactRec3; };
 
 // walk record fields in registers
 template <int D> struct WalkE {
@@ -71,33 +71,42 @@ template <int D> struct WalkE {
     int32_t uid;
 };
 
-// walk record fields from its 16-byte words
-__device__ __forceinline__ void decode_walk(const float4 a, const float4 b, const float4 c,
-                                            WalkE<2> &o) {
-    o.vh[0] = a.x; o.vh[1] = a.y; o.vl[0] = a.z; o.vl[1] = a.w;
-    o.m[0] = b.x; o.m[1] = b.y; o.m[2] = b.z; o.m[3] = b.w;
-    o.nbr[0] = __float_as_int(c.x); o.nbr[1] = __float_as_int(c.y);
-    o.nbr[2] = __float_as_int(c.z); o.uid = __float_as_int(c.w);
-}
-__device__ __forceinline__ void decode_walk(const float4 a, const float4 b, const float4 c,
-                                            const float4 d, const float4 n, WalkE<3> &o) {
-    o.vh[0] = a.x; o.vh[1] = a.y; o.vh[2] = a.z; o.vl[0] = a.w;
-    o.vl[1] = b.x; o.vl[2] = b.y; o.m[0] = b.z; o.m[1] = b.w;
-    o.m[2] = c.x; o.m[3] = c.y; o.m[4] = c.z; o.m[5] = c.w;
-    o.m[6] = d.x; o.m[7] = d.y; o.m[8] = d.z; o.uid = __float_as_int(d.w);
-    o.nbr[0] = __float_as_int(n.x); o.nbr[1] = __float_as_int(n.y);
-    o.nbr[2] = __float_as_int(n.z); o.nbr[3] = __float_as_int(n.w);
+// 32 bytes of read-only global memory (32-byte aligned) in one load
+__device__ __forceinline__ void ldg32(const uint8_t *p, float *v) {
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]),
+          "=f"(v[7])
+        : "l"(p));
 }
 
-__device__ __forceinline__ void load_walk(const WalkRec2 *__restrict__ r, int32_t e,
-                                          WalkE<2> &o) {
-    const float4 *p = reinterpret_cast<const float4 *>(r + e);
-    decode_walk(__ldg(p + 0), __ldg(p + 1), __ldg(p + 2), o);
+__device__ __forceinline__ void load_walk(const uint8_t *__restrict__ r, int32_t e, WalkE<2> &o) {
+    float a[8];
+    ldg32(r + walk_main(2, e), a);
+    const int4 t = __ldg(reinterpret_cast<const int4 *>(r + walk_tail(2, e)));
+    o.vh[0] = a[0]; o.vh[1] = a[1]; o.vl[0] = a[2]; o.vl[1] = a[3];
+    o.m[0] = a[4]; o.m[1] = a[5]; o.m[2] = a[6]; o.m[3] = a[7];
+    o.nbr[0] = t.x; o.nbr[1] = t.y; o.nbr[2] = t.z; o.uid = t.w;
 }
-__device__ __forceinline__ void load_walk(const WalkRec3 *__restrict__ r, int32_t e,
-                                          WalkE<3> &o) {
-    const float4 *p = reinterpret_cast<const float4 *>(r + e);
-    decode_walk(__ldg(p + 0), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3), __ldg(p + 4), o);
+__device__ __forceinline__ void load_walk(const uint8_t *__restrict__ r, int32_t e, WalkE<3> &o) {
+    float a[16];
+    ldg32(r + walk_main(3, e), a);
+    ldg32(r + walk_main(3, e) + 32, a + 8);
+    const int4 t = __ldg(reinterpret_cast<const int4 *>(r + walk_tail(3, e)));
+    #pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        o.vh[k] = a[k];
+        o.vl[k] = a[3 + k];
+    }
+    #pragma unroll
+    for (int k = 0; k < 9; ++k) o.m[k] = a[6 + k];
+    o.uid = __float_as_int(a[15]);
+    o.nbr[0] = t.x; o.nbr[1] = t.y; o.nbr[2] = t.z; o.nbr[3] = t.w;
+}
+// the caller's id of element e
+template <int D>
+__device__ __forceinline__ int32_t walk_uid(const void *recw, int32_t e) {
+    return __ldg(reinterpret_cast<const int32_t *>(static_cast<const uint8_t *>(recw) +
+                                                   (D == 2 ? walk_tail(2, e) + 12 : walk_main(3, e) + 60)));
 }
 // FP64 coordinates from the exact record (the arbiter).
 __device__ __forceinline__ void bary64(const ExactRec2 *__restrict__ r, int32_t e,
@@ -310,9 +319,8 @@ template <int D>
 __device__ __forceinline__ int32_t exact_search_lane(const DevMesh &m, const double *xp,
                                                      const float *xh, const float *xl, int j,
                                                      int lane) {
-    using WR = typename Recs<D>::W;
     using XR = typename Recs<D>::X;
-    const WR *__restrict__ rw = static_cast<const WR *>(m.recw);
+    const uint8_t *__restrict__ rw = static_cast<const uint8_t *>(m.recw);
     const XR *__restrict__ rx = static_cast<const XR *>(m.recx);
     double q[D];
     float qh[D], ql[D];
