@@ -7,7 +7,7 @@
 // transposed descriptor the same tiles are the operands of the weight
 // gradients (K = row).
 //
-// fc_gemm: one producer thread, one MMA-issuing warp, four epilogue warps;
+// fc_gemm: one producer thread, one MMA-issuing warp, eight epilogue warps;
 // four stages of K = 64; two accumulators, so the epilogue of a tile (bias,
 // ReLU or its gate, BF16, column sums) runs under the next tile's products.
 // The sums run in K order in K = 16 steps, as the general GEMM's
@@ -24,7 +24,9 @@
 namespace cs {
 namespace {
 
-constexpr int kFcThreads = 192;      // producer, MMA, four epilogue warps
+constexpr int kFcEpi = 8;            // epilogue warps: two per TMEM lane quarter
+constexpr int kFcThreads = (2 + kFcEpi) * 32;   // producer, MMA, epilogue
+constexpr int kFcBiasMax = 512;
 constexpr int kStages = 4, kStageChunks = 8;
 constexpr int kCh = int(kFcChunk);   // bytes of one 8-column chunk of a row tile
 
@@ -72,8 +74,9 @@ struct FcGeo {
     static constexpr int kA = kStageChunks * kCh;
     static constexpr int kB = kStageChunks * BN * 16;
     static constexpr int kStage = kA + kB;
-    static constexpr int kTile = kStages * kStage;                  // f32 [4][32 * 17]
-    static constexpr int kBar = kTile + 4 * 32 * 17 * 4;            // full, empty, tfull, tempty
+    static constexpr int kTile = kStages * kStage;                  // f32 [kFcEpi][32 * 17]
+    static constexpr int kBias = kTile + kFcEpi * 32 * 17 * 4;      // f32 [kFcBiasMax]
+    static constexpr int kBar = kBias + kFcBiasMax * 4;             // full, empty, tfull, tempty
     static constexpr int kSlot = kBar + (2 * kStages + 5) * 8;
     static constexpr int kTotal = kSlot + 16;
     static_assert(kTotal <= 232448 && kStage % 128 == 0, "shared memory of one CTA");
@@ -95,7 +98,7 @@ __global__ void __launch_bounds__(kFcThreads, 1) fc_gemm_kernel(const FcArgs a, 
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(tfull + i, 1u);
-            mbar_init(tempty + i, 4u);
+            mbar_init(tempty + i, uint32_t(kFcEpi));
         }
         mbar_init(last, 1u);
         *abort_flag = 0;
@@ -179,8 +182,14 @@ __global__ void __launch_bounds__(kFcThreads, 1) fc_gemm_kernel(const FcArgs a, 
         }
         __syncwarp();
     } else {
-        const int quarter = warp & 3;
-        float *tile = reinterpret_cast<float *>(smem + G::kTile) + quarter * (32 * 17);
+        // warps w and w + 4 share a lane quarter and take alternate 16-column pieces
+        const int quarter = warp & 3, half = (warp - 2) >> 2;
+        float *tile = reinterpret_cast<float *>(smem + G::kTile) + (warp - 2) * (32 * 17);
+        float *bias = reinterpret_cast<float *>(smem + G::kBias);
+        if (a.bias) {
+            for (int j = tid - 64; j < a.N; j += kFcEpi * 32) bias[j] = __ldg(a.bias + j);
+            asm volatile("bar.sync 1, %0;" ::"n"(kFcEpi * 32) : "memory");
+        }
         uint32_t i = 0;
         for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++i) {
             const uint32_t buf = i % nbuf;
@@ -192,7 +201,7 @@ __global__ void __launch_bounds__(kFcThreads, 1) fc_gemm_kernel(const FcArgs a, 
             const bool in = row < a.M;
             const uint32_t tq = tmem + buf * (a.cols / 2) + (uint32_t(32 * quarter) << 16);
             #pragma unroll 1
-            for (int c = 0; c < BN; c += 16) {
+            for (int c = 16 * half; c < BN; c += 32) {
                 if (n0 + c >= a.N) break;
                 float v[16];
                 tmem_ld16(tq + uint32_t(c), v);
@@ -204,8 +213,13 @@ __global__ void __launch_bounds__(kFcThreads, 1) fc_gemm_kernel(const FcArgs a, 
                 }
                 if (a.bias) {
                     #pragma unroll
-                    for (int e = 0; e < 16; ++e)
-                        if (n0 + c + e < a.N) v[e] += __ldg(a.bias + n0 + c + e);
+                    for (int e = 0; e < 4; ++e) {
+                        const float4 b = *reinterpret_cast<const float4 *>(bias + n0 + c + 4 * e);
+                        v[4 * e] += b.x;
+                        v[4 * e + 1] += b.y;
+                        v[4 * e + 2] += b.z;
+                        v[4 * e + 3] += b.w;
+                    }
                 }
                 if (a.relu) {
                     #pragma unroll
@@ -286,7 +300,7 @@ struct FcWgGeo {
     static constexpr int kY = 16 * kCh, kX = (BK / 8) * kCh, kStage = kY + kX;
     static constexpr int kStagesW = 2;
     static constexpr int kTile = kStagesW * kStage;
-    static constexpr int kBar = kTile + 4 * 32 * 17 * 4;
+    static constexpr int kBar = kTile + kFcEpi * 32 * 17 * 4;
     static constexpr int kSlot = kBar + 8 * (2 * kStagesW + 1);
     static constexpr int kTotal = kSlot + 16;
     static_assert(kTotal <= 232448, "shared memory of one CTA");
@@ -370,14 +384,14 @@ __global__ void __launch_bounds__(kFcThreads, 1) fc_wgrad_kernel(const FcWgArgs 
         }
         __syncwarp();
     } else if (t0 < t1) {
-        const int quarter = warp & 3;
-        float *tile = reinterpret_cast<float *>(smem + G::kTile) + quarter * (32 * 17);
+        const int quarter = warp & 3, half = (warp - 2) >> 2;
+        float *tile = reinterpret_cast<float *>(smem + G::kTile) + (warp - 2) * (32 * 17);
         if (warp_wait(done, 0, abort_flag, err)) {
             fence_after();
             float *dst = a.part + int64_t(blockIdx.z) * a.N * a.K;
             const uint32_t tq = tmem + (uint32_t(32 * quarter) << 16);
             #pragma unroll 1
-            for (int c = 0; c < G::BK; c += 16) {
+            for (int c = 16 * half; c < G::BK; c += 32) {
                 if (k0 + c >= a.K) break;
                 float v[16];
                 tmem_ld16(tq + uint32_t(c), v);
@@ -553,6 +567,7 @@ int launch_fc_pack(const FcPack *segs, int n, cudaStream_t st) {
 }
 
 int launch_fc_gemm(const FcGemm &g, int *err, int sm_count, cudaStream_t st) {
+    static_assert(kFcBiasMax % 16 == 0, "whole pieces of the bias");
     FcArgs a{};
     a.A = g.A;
     a.gate = g.gate;
