@@ -3,27 +3,35 @@
 // convolutions of 32 channels with ReLU and the 2^D average pooling, in one
 // CTA, with no im2col copy and no activation leaving shared memory.
 //
-// Layout. A particle's zero-padded window (edge E = W + 2) sits on a flat
-// index q = (z E + y) E + x. A convolution output is computed at the row
-// r = q - (E + 1) (2-D; q - (E^2 + E + 1) in 3-D) of the window position q it
-// belongs to, and reads its input at r + shift(tap), shift = (dz E + dy) E + dx:
-// a tap is a row offset of the shared-memory operand, so each convolution is
-// an implicit GEMM. Output rows whose position lies outside the window (the
-// wrap-around columns) are garbage and are never stored or pooled.
+// Layout. A particle's window with its zero padding sits on a flat index
+// q = (z E + y) E + x of pitch E = W + 1: the ring's cells before a line are
+// the ring's cells after the line before it (and so for planes, and for the
+// next particle of a group), so one zero column and row serve both. A
+// convolution output is computed at the row r = q - (E + 1) (2-D;
+// q - (E^2 + E + 1) in 3-D) of the window position q it belongs to, and reads
+// its input at r + shift(tap), shift = (dz E + dy) E + dx: a tap is a row
+// offset of the shared-memory operand, so each convolution is an implicit
+// GEMM. Output rows whose position lies outside the window (the ring's
+// columns) are garbage and are never stored or pooled. In 2-D a group of NP = 5
+// particles (100 rows each) fills four M-tiles of 128 rows, where a particle
+// on its own takes one; in 3-D a particle takes four (five at pitch W + 2).
 //
 //   input  [rows][8] BF16: the D window channels and 8 - D zero channels;
 //          the ring and the rows past the window stay zero
 //   conv1  tcgen05.mma kind::f16, M = 128 rows, N = 32, K = 16 = two taps of
 //          8 channels: the A descriptor's leading byte offset is the row
 //          distance of the two taps (5 MMAs per M-tile in 2-D, 14 in 3-D; the
-//          last pair's second tap has zero weights)
+//          last pair's first tap has zero weights)
 //   conv2  K = 32 channels of one tap in two K = 16 steps: 2 MMAs per tap
 //   act    [4 chunks][rows][8] BF16: ReLU(conv1 + b1), written at the window
 //          position of each valid output row (its padded layout is conv2's
 //          operand, ring zero)
-//   stage  [output rows][33] FP32: ReLU(conv2 + b2), read by the pooling
+//   stage  [pooled positions][33] FP32: ReLU(conv2 + b2), read by the pooling
 //   FP32 accumulation in TMEM: conv1 in columns [0, 32 MT), conv2 in
-//   [32 MT, 64 MT), MT the M-tiles of a particle (1 in 2-D, 5 in 3-D).
+//   [32 MT, 64 MT), MT the M-tiles of a group.
+// An MMA of M = 128, N = 32, K = 16 takes 42 cycles whatever its row offset,
+// if it is issued as fast: the taps are unrolled, so that issuing one is a
+// few additions to a descriptor (with the taps in a loop it took 58).
 //
 // Inputs. Each window cell holds (p - x_p) / s: p is the cell's pooled
 // element centroid, given as float hi + lo parts, so the difference is taken
@@ -33,11 +41,12 @@
 // FP64 formula as arbiter: the same cell as the labels and the start rule);
 // its offset from the cell centre is taken in FP32.
 //
-// Warps. Warps 0-3 compute the inputs, run both epilogues and the pooling
-// (warp w reads TMEM lanes 32 w .. 32 w + 31); warp 4 issues the MMAs. A CTA
-// takes particles blockIdx.x, blockIdx.x + gridDim.x, ...; the inputs of
-// particle k + 1 are computed while particle k's conv2 runs, and its conv1
-// runs while particle k's conv2 epilogue and pooling run. Every wait is
+// Warps. Warps 0-7 compute the inputs, run both epilogues and the pooling
+// (warp w reads TMEM lanes 32 (w % 4) .. and 16 of the 32 channels); warp 8
+// issues the MMAs. A CTA
+// takes groups blockIdx.x, blockIdx.x + gridDim.x, ...; the inputs of
+// group k + 1 are computed while group k's conv2 runs, and its conv1
+// runs while group k's conv2 epilogue and pooling run. Every wait is
 // bounded; one that gives up raises the CTA's abort flag and the device
 // error flag.
 #include <cuda_bf16.h>
@@ -51,26 +60,32 @@
 namespace cs {
 namespace {
 
-constexpr int kEpiC = 4;                    // epilogue warps 0..3
-constexpr int kMmaC = 4;                    // the MMA-issuing warp
+constexpr int kEpiC = 8;                    // epilogue warps 0..7
+constexpr int kMmaC = kEpiC;                // the MMA-issuing warp
 constexpr int kThreadsC = (kEpiC + 1) * 32;
 
-template <int D>
+template <int D, int NP_>
 struct ClsGeo {
+    static constexpr int NP = NP_;                                   // particles of a group
+    static_assert(D == 2 || NP == 1, "groups of particles in 2-D only");
     static constexpr int W = D == 2 ? 9 : 7;
-    static constexpr int E = W + 2;                                  // padded edge
+    static constexpr int E = W + 1;                                  // pitch
     static constexpr int P = D == 2 ? W * W : W * W * W;             // window cells
+    static constexpr int Pitch = D == 2 ? E * E : E * E * E;         // rows of a particle
     static constexpr int S = D == 2 ? 2 * E + 2 : (2 * E + 2) * E + 2;   // largest tap shift
-    static constexpr int Ro = D == 2 ? (W - 1) * E + W : ((W - 1) * E + W - 1) * E + W;
-    static constexpr int MT = (Ro + 127) / 128;                      // M-tiles per particle
+    static constexpr int Ro = (NP - 1) * Pitch +
+                              (D == 2 ? (W - 1) * E + W : ((W - 1) * E + W - 1) * E + W);
+    static constexpr int MT = (Ro + 127) / 128;                      // M-tiles per group
     static constexpr int Rows = (128 * MT + S + 8 + 7) / 8 * 8;      // operand rows
     static constexpr int Coff = D == 2 ? E + 1 : (E + 1) * E + 1;    // output row -> position
     static constexpr int Taps = D == 2 ? 9 : 27;
     static constexpr int Pairs = (Taps + 1) / 2;
     static constexpr int Wp = W / 2;
     static constexpr int Pp = D == 2 ? Wp * Wp : Wp * Wp * Wp;
+    static constexpr int Ws = 2 * Wp;                                // edge that is pooled
+    static constexpr int Ps = D == 2 ? Ws * Ws : Ws * Ws * Ws;
     static constexpr int Ld = 33;                                    // stage row stride (floats)
-    static constexpr uint32_t Cols = D == 2 ? 64 : 512;              // TMEM columns allocated
+    static constexpr uint32_t Cols = 64 * MT <= 64 ? 64 : 64 * MT <= 128 ? 128 : 64 * MT <= 256 ? 256 : 512;
     // packed weights
     static constexpr int kW1 = 0;                                    // bf16 [Pairs][2][32][8]
     static constexpr int kB1 = kW1 + Pairs * 1024;                   // f32 [32]
@@ -82,23 +97,24 @@ struct ClsGeo {
     static constexpr int kSmAct = kSmIn + Rows * 16;
     static constexpr int kSmW = kSmAct + 4 * Rows * 16;
     static constexpr int kSmStage = kSmW + kPacked;
-    static constexpr int kSmBar = (kSmStage + Ro * Ld * 4 + 7) / 8 * 8;   // mbarriers [3]
+    static constexpr int kSmBar = (kSmStage + NP * Ps * Ld * 4 + 7) / 8 * 8;   // mbarriers [3]
     static constexpr int kSmCnt = kSmBar + 3 * 8;                    // u32 in_ready, act_ready
-    static constexpr int kSmPart = kSmCnt + 8;                       // int c0[3], float off[3], x hi/lo [6]
-    static constexpr int kSmSlot = kSmPart + 12 * 4;                 // TMEM address, abort flag
+    // per particle: int c0[3], float off[3], x hi/lo [6]
+    static constexpr int kSmPart = kSmCnt + 8;
+    static constexpr int kSmSlot = kSmPart + NP * 12 * 4;            // TMEM address, abort flag
     static constexpr int kSmTotal = kSmSlot + 16;
 
     static_assert(64 * MT <= int(Cols), "TMEM columns");
     static_assert(128 * MT + S < Rows, "operand reads in bounds (the zero tap included)");
-    static_assert(Ro - 1 + Coff < (D == 2 ? E * E : E * E * E), "outputs land in the window");
+    static_assert(Ro - 1 + Coff < Rows, "outputs land in the window");
     static_assert(kSmTotal <= 232448, "shared memory of one CTA");
     static_assert(kSmW % 128 == 0 && kSmAct % 128 == 0, "operand alignment");
 };
 
 template <int D>
 __device__ __forceinline__ constexpr int cls_shift(int t) {
-    using G = ClsGeo<D>;
-    return D == 2 ? (t / 3) * G::E + t % 3 : ((t / 9) * G::E + (t / 3) % 3) * G::E + t % 3;
+    constexpr int E = ClsGeo<D, 1>::E;
+    return D == 2 ? (t / 3) * E + t % 3 : ((t / 9) * E + (t / 3) % 3) * E + t % 3;
 }
 
 // named barrier 1 over the epilogue warps
@@ -140,37 +156,43 @@ __device__ __forceinline__ void cell_offset(const DevMesh &m, int k, double x, f
     off = q - (float(i) + 0.5f);
 }
 
-// The inputs of particle b into the operand rows (epilogue warps): thread
-// tid < D first computes axis tid's cell, offset and the hi/lo split of x_p;
-// then every window cell is one 16-byte row.
-template <int D>
+// The inputs of particles [b0, b0 + nb) into the operand rows (epilogue
+// warps): thread tid < nb D first computes an axis's cell, offset and the
+// hi/lo split of x_p; then every window cell is one 16-byte row.
+template <int D, int NP>
 __device__ __forceinline__ void cls_inputs(const DevMesh &m, const float *__restrict__ pool_f,
-                                           const double *__restrict__ xp, int64_t b,
-                                           uint8_t *in, int *sc0, float *soff, float *sxh,
-                                           float *sxl, float *__restrict__ off_out, int tid) {
-    using G = ClsGeo<D>;
-    if (tid < D) {
-        const double x = xp[b * D + tid];
+                                           const double *__restrict__ xp, int64_t b0, int nb,
+                                           uint8_t *in, float *part, float *__restrict__ off_out,
+                                           int tid) {
+    using G = ClsGeo<D, NP>;
+    if (tid < nb * D) {
+        const int w = tid / D, k = tid % D;
+        float *sp = part + 12 * w;
+        const double x = xp[b0 * D + tid];
         const float h = __double2float_rn(x);
         const float l = __double2float_rn(__dsub_rn(x, double(h)));
-        int c0;
-        float o;
-        cell_offset(m, tid, x, h, l, c0, o);
-        sc0[tid] = c0;
-        soff[tid] = o;
-        off_out[b * D + tid] = o;
-        sxh[tid] = h;
-        sxl[tid] = l;
+        int c0 = 0;
+        float o = 0.f;
+        #pragma unroll
+        for (int q = 0; q < D; ++q)
+            if (k == q) cell_offset(m, q, x, h, l, c0, o);
+        reinterpret_cast<int *>(sp)[k] = c0;
+        sp[3 + k] = o;
+        off_out[b0 * D + tid] = o;
+        sp[6 + k] = h;
+        sp[9 + k] = l;
     }
     epi_sync();
-    for (int e = tid; e < G::P; e += kEpiC * 32) {
+    for (int i = tid; i < nb * G::P; i += kEpiC * 32) {
+        const int w = i / G::P, e = i % G::P;
+        const float *sp = part + 12 * w;
         int ek[3] = {e % G::W, (e / G::W) % G::W, D == 3 ? e / (G::W * G::W) : 0};
         bool inside = true;
         int64_t flat = 0;
         int cc[3];
         #pragma unroll
         for (int k = 0; k < D; ++k) {
-            cc[k] = sc0[k] - G::W / 2 + ek[k];
+            cc[k] = reinterpret_cast<const int *>(sp)[k] - G::W / 2 + ek[k];
             inside &= cc[k] >= 0 && cc[k] < m.ga[k];
         }
         #pragma unroll
@@ -179,31 +201,41 @@ __device__ __forceinline__ void cls_inputs(const DevMesh &m, const float *__rest
         bool has = false;
         float ph[3], pl[3];
         if (inside) {
-            #pragma unroll
-            for (int k = 0; k < D; ++k) {
-                ph[k] = __ldg(pool_f + flat * 2 * D + 2 * k);
-                pl[k] = __ldg(pool_f + flat * 2 * D + 2 * k + 1);
+            if constexpr (D == 2) {
+                const float4 q = __ldg(reinterpret_cast<const float4 *>(pool_f) + flat);
+                ph[0] = q.x;
+                pl[0] = q.y;
+                ph[1] = q.z;
+                pl[1] = q.w;
+            } else {
+                #pragma unroll
+                for (int k = 0; k < D; ++k) {
+                    const float2 q = __ldg(reinterpret_cast<const float2 *>(pool_f) + flat * D + k);
+                    ph[k] = q.x;
+                    pl[k] = q.y;
+                }
             }
             has = !isnan(ph[0]);
         }
         #pragma unroll
         for (int k = 0; k < D; ++k) {
             const float inv = m.inv_sa[k];
-            v[k] = has ? __fmul_rn(__fadd_rn(__fsub_rn(ph[k], sxh[k]), __fsub_rn(pl[k], sxl[k])), inv)
-                       : __fsub_rn(float(ek[k] - G::W / 2), soff[k]);
+            v[k] = has ? __fmul_rn(__fadd_rn(__fsub_rn(ph[k], sp[6 + k]), __fsub_rn(pl[k], sp[9 + k])),
+                                   inv)
+                       : __fsub_rn(float(ek[k] - G::W / 2), sp[3 + k]);
         }
-        const int q = D == 2 ? (ek[1] + 1) * G::E + ek[0] + 1
-                             : ((ek[2] + 1) * G::E + ek[1] + 1) * G::E + ek[0] + 1;
+        const int q = w * G::Pitch + (D == 2 ? (ek[1] + 1) * G::E + ek[0] + 1
+                                             : ((ek[2] + 1) * G::E + ek[1] + 1) * G::E + ek[0] + 1);
         *reinterpret_cast<uint4 *>(in + 16 * q) =
             make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], 0.f), 0u, 0u);
     }
 }
 
-template <int D>
-__global__ void __launch_bounds__(kThreadsC, D == 2 ? 4 : 1) cls_conv_tc_kernel(
+template <int D, int NP>
+__global__ void __launch_bounds__(kThreadsC, D == 3 ? 1 : NP == 1 ? 3 : 2) cls_conv_tc_kernel(
     const DevMesh m, const float *__restrict__ pool_f, int64_t B, const double *__restrict__ xp,
     const uint8_t *__restrict__ packed, const FcMat cat, float *__restrict__ off_out, int *err) {
-    using G = ClsGeo<D>;
+    using G = ClsGeo<D, NP>;
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t *in = smem + G::kSmIn;
     uint8_t *act = smem + G::kSmAct;
@@ -212,9 +244,7 @@ __global__ void __launch_bounds__(kThreadsC, D == 2 ? 4 : 1) cls_conv_tc_kernel(
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + G::kSmBar);   // conv1, conv2, final
     uint32_t *in_ready = reinterpret_cast<uint32_t *>(smem + G::kSmCnt);
     uint32_t *act_ready = in_ready + 1;
-    int *sc0 = reinterpret_cast<int *>(smem + G::kSmPart);
-    float *soff = reinterpret_cast<float *>(smem + G::kSmPart) + 3;
-    float *sxh = soff + 3, *sxl = soff + 6;
+    float *part = reinterpret_cast<float *>(smem + G::kSmPart);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + G::kSmSlot);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + G::kSmSlot + 4);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -242,7 +272,8 @@ __global__ void __launch_bounds__(kThreadsC, D == 2 ? 4 : 1) cls_conv_tc_kernel(
     __syncthreads();
     fence_after();
     const uint32_t tmem = *tmem_slot;
-    const int64_t n_mine = B > blockIdx.x ? (B - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+    const int64_t groups = (B + NP - 1) / NP;
+    const int64_t n_mine = groups > blockIdx.x ? (groups - 1 - blockIdx.x) / gridDim.x + 1 : 0;
 
     if (warp == kMmaC) {
         const bool leader = elect_one();
@@ -252,33 +283,37 @@ __global__ void __launch_bounds__(kThreadsC, D == 2 ? 4 : 1) cls_conv_tc_kernel(
         const uint64_t d_w2 = sdesc(smem_addr(wsm + G::kW2), 32 * 16, 128);
         constexpr uint32_t id32 = idesc_bf16(128, 32);
         for (int64_t k = 0; k < n_mine; ++k) {
-            // conv1 of particle k, once its inputs are in place
+            // conv1 of group k, once its inputs are in place
             if (!wait_count(in_ready, uint32_t(k + 1), abort_flag, err)) break;
             fence_after();
             if (leader) {
+                #pragma unroll 1
                 for (int mt = 0; mt < G::MT; ++mt) {
                     const uint32_t dcol = tmem + uint32_t(32 * mt);
                     const int r0 = 128 * mt;
                     #pragma unroll
                     for (int i = 0; i < G::Pairs; ++i) {
-                        const int t0 = 2 * i, t1 = 2 * i + 1 < G::Taps ? 2 * i + 1 : 2 * i;
+                        // the last step's first tap has zero weights: it reads the
+                        // tap before, rows of the same particle
+                        const int t0 = min(2 * i, G::Taps - 2), t1 = t0 + 1;
                         const int sh0 = cls_shift<D>(t0), sh1 = cls_shift<D>(t1);
                         const uint64_t a = (d_in & ~(uint64_t(0x3fff) << 16)) + uint64_t(r0 + sh0) +
-                                           (uint64_t(sh1 - sh0 > 0 ? sh1 - sh0 : 1) << 16);
+                                           (uint64_t(sh1 - sh0) << 16);
                         mma_bf16(dcol, a, d_w1 + uint64_t(i * 64), id32, i > 0 ? 1u : 0u);
                     }
                 }
                 mma_commit(bars + 0);
             }
             __syncwarp();
-            // conv2 of particle k, once conv1's activations are in place
+            // conv2 of group k, once conv1's activations are in place
             if (!wait_count(act_ready, uint32_t(k + 1), abort_flag, err)) break;
             fence_after();
             if (leader) {
+                #pragma unroll 1
                 for (int mt = 0; mt < G::MT; ++mt) {
                     const uint32_t dcol = tmem + uint32_t(32 * (G::MT + mt));
                     const int r0 = 128 * mt;
-                    #pragma unroll 3
+                    #pragma unroll
                     for (int t = 0; t < G::Taps; ++t) {
                         const int sh = cls_shift<D>(t);
                         #pragma unroll
@@ -296,38 +331,47 @@ __global__ void __launch_bounds__(kThreadsC, D == 2 ? 4 : 1) cls_conv_tc_kernel(
     } else {
         const float *b1 = reinterpret_cast<const float *>(wsm + G::kB1);
         const float *b2 = reinterpret_cast<const float *>(wsm + G::kB2);
-        const uint32_t tq = tmem + (uint32_t(32 * warp) << 16);
+        const int c0 = 16 * (warp >> 2);                 // this warp's channels
+        const uint32_t tq = tmem + (uint32_t(32 * (warp & 3)) << 16) + uint32_t(c0);
         bool ok = true;
         if (n_mine > 0) {
-            cls_inputs<D>(m, pool_f, xp, blockIdx.x, in, sc0, soff, sxh, sxl, off_out, tid);
+            const int64_t b0 = int64_t(blockIdx.x) * NP;
+            cls_inputs<D, NP>(m, pool_f, xp, b0, int(min(int64_t(NP), B - b0)), in, part, off_out, tid);
             fence_async_smem();
             epi_sync();
             if (tid == 0) red_release_add(in_ready, 1u);
         }
         for (int64_t k = 0; k < n_mine && ok; ++k) {
-            const int64_t b = blockIdx.x + k * gridDim.x;
+            const int64_t b0 = (blockIdx.x + k * gridDim.x) * NP;
+            const int nb = int(min(int64_t(NP), B - b0));
             const uint32_t par = uint32_t(k & 1);
             // ---- conv1 epilogue: ReLU(z + b1) in BF16 at each valid row's window position ----
             ok = __all_sync(kFull, mbar_wait(bars + 0, par, abort_flag, err)) != 0;
             if (epi_or(!ok)) break;
             fence_after();
             for (int mt = 0; mt < G::MT; ++mt) {
-                float v[32];
-                tmem_ld32(tq + uint32_t(32 * mt), v);
-                uint32_t hv[16];
-                bias_relu_bf16(v, b1, hv);
-                const int r = 128 * mt + 32 * warp + lane;
-                const int x = r % G::E, y = (r / G::E) % G::E, z = D == 3 ? r / (G::E * G::E) : 0;
-                if (r < G::Ro && x < G::W && y < G::W && z < G::W)
-                    store_act<G::Rows>(act, r + G::Coff, hv);
+                float v[16];
+                tmem_ld16(tq + uint32_t(32 * mt), v);
+                uint32_t hv[8];
+                bias_relu_bf16_16(v, b1 + c0, hv);
+                const int r = 128 * mt + 32 * (warp & 3) + lane;
+                const int rr = r % G::Pitch;
+                const int x = rr % G::E, y = (rr / G::E) % G::E, z = D == 3 ? rr / (G::E * G::E) : 0;
+                if (r < G::Ro && x < G::W && y < G::W && z < G::W) {
+                    uint8_t *o = act + (size_t(c0 >> 3) * G::Rows + r + G::Coff) * 16;
+                    *reinterpret_cast<uint4 *>(o) = make_uint4(hv[0], hv[1], hv[2], hv[3]);
+                    *reinterpret_cast<uint4 *>(o + G::Rows * 16) = make_uint4(hv[4], hv[5], hv[6], hv[7]);
+                }
             }
             fence_before();
             fence_async_smem();
             epi_sync();
             if (tid == 0) red_release_add(act_ready, 1u);
-            // ---- inputs of the next particle (its conv1 read of `in` is over) ----
+            // ---- inputs of the next group (this one's conv1 has read `in`) ----
             if (k + 1 < n_mine) {
-                cls_inputs<D>(m, pool_f, xp, b + gridDim.x, in, sc0, soff, sxh, sxl, off_out, tid);
+                const int64_t b1n = b0 + int64_t(gridDim.x) * NP;
+                cls_inputs<D, NP>(m, pool_f, xp, b1n, int(min(int64_t(NP), B - b1n)), in, part, off_out,
+                                  tid);
                 fence_async_smem();
                 epi_sync();
                 if (tid == 0) red_release_add(in_ready, 1u);
@@ -337,39 +381,49 @@ __global__ void __launch_bounds__(kThreadsC, D == 2 ? 4 : 1) cls_conv_tc_kernel(
             if (epi_or(!ok)) break;
             fence_after();
             for (int mt = 0; mt < G::MT; ++mt) {
-                float v[32];
-                tmem_ld32(tq + uint32_t(32 * (G::MT + mt)), v);
-                const int r = 128 * mt + 32 * warp + lane;
-                if (r < G::Ro) {
+                float v[16];
+                tmem_ld16(tq + uint32_t(32 * (G::MT + mt)), v);
+                const int r = 128 * mt + 32 * (warp & 3) + lane, w = r / G::Pitch, rr = r % G::Pitch;
+                const int x = rr % G::E, y = (rr / G::E) % G::E, z = D == 3 ? rr / (G::E * G::E) : 0;
+                if (r < G::Ro && x < G::Ws && y < G::Ws && z < G::Ws) {
+                    float *st = stage + (w * G::Ps + (z * G::Ws + y) * G::Ws + x) * G::Ld + c0;
                     #pragma unroll
-                    for (int c = 0; c < 32; ++c) stage[r * G::Ld + c] = fmaxf(v[c] + b2[c], 0.f);
+                    for (int e = 0; e < 4; ++e) {
+                        const float4 b = *reinterpret_cast<const float4 *>(b2 + c0 + 4 * e);
+                        st[4 * e] = fmaxf(v[4 * e] + b.x, 0.f);
+                        st[4 * e + 1] = fmaxf(v[4 * e + 1] + b.y, 0.f);
+                        st[4 * e + 2] = fmaxf(v[4 * e + 2] + b.z, 0.f);
+                        st[4 * e + 3] = fmaxf(v[4 * e + 3] + b.w, 0.f);
+                    }
                 }
             }
             fence_before();
             epi_sync();
-            // BF16 into the tiled feature matrix (fc_tc.h), row b: column
-            // c Pp + pp. 2-D: four neighbouring columns per thread
-            uint8_t *crow = cat.p + (b >> 7) * cat.tile + int64_t(cat.chunk0) * kFcChunk + (b & 127) * 16;
-            constexpr int kPer = G::Pp % 4 == 0 ? 4 : 1;
-            for (int i = tid; i < 32 * G::Pp / kPer; i += kEpiC * 32) {
-                const int c = i % 32, p0 = i / 32 * kPer;
+            // BF16 into the tiled feature matrix (fc_tc.h): column c Pp + pp of
+            // the particle's row. 2-D: four neighbouring columns per thread
+            constexpr int kPer = G::Pp % 4 == 0 ? 4 : 1, kUnits = 32 * G::Pp / kPer;
+            for (int i = tid; i < nb * kUnits; i += kEpiC * 32) {
+                const int w = i / kUnits, u0 = i % kUnits, c = u0 % 32, p0 = u0 / 32 * kPer;
+                const float *st = stage + w * G::Ps * G::Ld + c;
                 float s[kPer];
                 #pragma unroll
                 for (int u = 0; u < kPer; ++u) {
                     const int pp = p0 + u;
                     const int px = pp % G::Wp, py = (pp / G::Wp) % G::Wp, pz = D == 3 ? pp / (G::Wp * G::Wp) : 0;
                     s[u] = 0.f;
+                    #pragma unroll
                     for (int oz = 0; oz < (D == 3 ? 2 : 1); ++oz)
+                        #pragma unroll
                         for (int oy = 0; oy < 2; ++oy)
-                            for (int ox = 0; ox < 2; ++ox) {
-                                const int r = D == 2 ? (2 * py + oy) * G::E + 2 * px + ox
-                                                     : ((2 * pz + oz) * G::E + 2 * py + oy) * G::E + 2 * px + ox;
-                                s[u] += stage[r * G::Ld + c];
-                            }
+                            #pragma unroll
+                            for (int ox = 0; ox < 2; ++ox)
+                                s[u] += st[(((2 * pz + oz) * G::Ws + 2 * py + oy) * G::Ws + 2 * px + ox) * G::Ld];
                     s[u] = s[u] / float(1 << D);
                 }
                 const int col = c * G::Pp + p0;
-                uint8_t *o = crow + int64_t(col >> 3) * kFcChunk + (col & 7) * 2;
+                const int64_t b = b0 + w;
+                uint8_t *o = cat.p + (b >> 7) * cat.tile + int64_t(cat.chunk0 + (col >> 3)) * kFcChunk +
+                             (b & 127) * 16 + (col & 7) * 2;
                 if constexpr (kPer == 4)
                     *reinterpret_cast<uint2 *>(o) =
                         make_uint2(pack_bf16x2(s[0], s[1]), pack_bf16x2(s[2], s[3]));
@@ -396,18 +450,19 @@ __global__ void __launch_bounds__(kThreadsC, D == 2 ? 4 : 1) cls_conv_tc_kernel(
 }
 
 // conv1 W[o][i][t] (i < D) -> [pair p][half h][o][8] (tap 2p + h, channel j;
-// zero for j >= D and past the last tap); conv2 W[o][i][t] -> [t][q][o][8]
+// zero for j >= D; the last pair is a zero tap and the last tap); conv2 W[o][i][t] -> [t][q][o][8]
 // with i = 8 q + j; biases as FP32.
 template <int D>
 __global__ void cls_pack_kernel(const float *__restrict__ w, int64_t off_w1, int64_t off_b1,
                                 int64_t off_w2, int64_t off_b2, uint8_t *__restrict__ out) {
-    using G = ClsGeo<D>;
+    using G = ClsGeo<D, 1>;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
     __nv_bfloat16 *w1 = reinterpret_cast<__nv_bfloat16 *>(out + G::kW1);
     for (int e = tid; e < G::Pairs * 2 * 32 * 8; e += nth) {
         const int j = e % 8, o = (e / 8) % 32, h = (e / 256) % 2, p = e / 512;
-        const int t = 2 * p + h;
-        w1[e] = __float2bfloat16_rn(t < G::Taps && j < D ? w[off_w1 + (o * D + j) * G::Taps + t] : 0.f);
+        // the odd last tap is the second of its step
+        const int t = p < G::Pairs - 1 ? 2 * p + h : h == 1 ? G::Taps - 1 : -1;
+        w1[e] = __float2bfloat16_rn(t >= 0 && j < D ? w[off_w1 + (o * D + j) * G::Taps + t] : 0.f);
     }
     __nv_bfloat16 *w2 = reinterpret_cast<__nv_bfloat16 *>(out + G::kW2);
     for (int e = tid; e < G::Taps * 32 * 32; e += nth) {
@@ -421,26 +476,26 @@ __global__ void cls_pack_kernel(const float *__restrict__ w, int64_t off_w1, int
     }
 }
 
-template <int D>
+template <int D, int NP>
 void launch_conv(const DevMesh &m, const float *pool_f, int64_t B, const double *xp,
                  const uint8_t *packed, const FcMat &cat, float *off, int *err, int sm_count,
                  cudaStream_t st) {
-    using G = ClsGeo<D>;
+    using G = ClsGeo<D, NP>;
     static bool attr = false;
     if (!attr) {
-        cudaFuncSetAttribute(cls_conv_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(cls_conv_tc_kernel<D, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              G::kSmTotal);
         attr = true;
     }
-    const int per_sm = D == 2 ? 4 : 1;
-    const int grid = int(std::min<int64_t>(B, int64_t(sm_count) * per_sm));
-    cls_conv_tc_kernel<D><<<grid, kThreadsC, G::kSmTotal, st>>>(m, pool_f, B, xp, packed, cat, off,
-                                                                err);
+    const int per_sm = D == 3 ? 1 : NP == 1 ? 3 : 2;
+    const int grid = int(std::min<int64_t>((B + NP - 1) / NP, int64_t(sm_count) * per_sm));
+    cls_conv_tc_kernel<D, NP><<<grid, kThreadsC, G::kSmTotal, st>>>(m, pool_f, B, xp, packed, cat,
+                                                                    off, err);
 }
 
 }  // namespace
 
-int64_t cls_packed_bytes(int dim) { return dim == 2 ? ClsGeo<2>::kPacked : ClsGeo<3>::kPacked; }
+int64_t cls_packed_bytes(int dim) { return dim == 2 ? ClsGeo<2, 1>::kPacked : ClsGeo<3, 1>::kPacked; }
 
 void launch_cls_pack(int dim, const float *w, int64_t off_w1, int64_t off_b1, int64_t off_w2,
                      int64_t off_b2, uint8_t *packed, cudaStream_t st) {
@@ -454,10 +509,14 @@ void launch_cls_conv_tc(const DevMesh &m, const float *pool_f, int64_t B, const 
                         const uint8_t *packed, const FcMat &cat, float *off, int *err,
                         int sm_count, cudaStream_t st) {
     if (B <= 0) return;
-    if (m.dim == 2)
-        launch_conv<2>(m, pool_f, B, xp, packed, cat, off, err, sm_count, st);
+    // groups of five once they fill two CTAs per SM a few times over; a particle
+    // per CTA pass spreads fewer particles over more CTAs
+    if (m.dim == 2 && B >= int64_t(20) * sm_count)
+        launch_conv<2, 5>(m, pool_f, B, xp, packed, cat, off, err, sm_count, st);
+    else if (m.dim == 2)
+        launch_conv<2, 1>(m, pool_f, B, xp, packed, cat, off, err, sm_count, st);
     else
-        launch_conv<3>(m, pool_f, B, xp, packed, cat, off, err, sm_count, st);
+        launch_conv<3, 1>(m, pool_f, B, xp, packed, cat, off, err, sm_count, st);
 }
 
 }  // namespace cs

@@ -226,6 +226,21 @@ __device__ __forceinline__ void bias_relu_bf16(const float *v, const float *bias
     }
 }
 
+// the same over 16 channels
+__device__ __forceinline__ void bias_relu_bf16_16(const float *v, const float *bias, uint32_t *hv) {
+    const __nv_bfloat162 zero = __float2bfloat162_rn(0.f);
+    #pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float4 b = reinterpret_cast<const float4 *>(bias)[e];
+        const float2 s0 = __fadd2_rn(make_float2(v[4 * e], v[4 * e + 1]), make_float2(b.x, b.y));
+        const float2 s1 = __fadd2_rn(make_float2(v[4 * e + 2], v[4 * e + 3]), make_float2(b.z, b.w));
+        const __nv_bfloat162 h0 = __hmax2(__floats2bfloat162_rn(s0.x, s0.y), zero);
+        const __nv_bfloat162 h1 = __hmax2(__floats2bfloat162_rn(s1.x, s1.y), zero);
+        hv[2 * e] = *reinterpret_cast<const uint32_t *>(&h0);
+        hv[2 * e + 1] = *reinterpret_cast<const uint32_t *>(&h1);
+    }
+}
+
 // Bounded wait until the device-memory flag *flag is non-zero (an acquire
 // load per poll, at most `polls` polls ~256 ns apart). Gives up (false) when
 // the CTA's abort flag is raised, or at the limit, raising the abort flag and
