@@ -433,7 +433,7 @@ int backward_conv(cs_ctx *ctx, Classifier &C, int64_t B, const float *dpool, int
                   cudaStream_t st);
 
 // The tiled path's training step for B rows of at least 16: gradients of the
-// cross-entropy into C.g, the loss added to *loss. In 2-D module 1 runs on the
+// cross-entropy into C.g, and *loss. In 2-D module 1 runs on the
 // implicit-GEMM convolutions as well (train_tc.h); in 3-D, whose 343 positions
 // do not fit their tile, on the layer-by-layer kernels.
 bool tiled_batch(int64_t B) { return gemm_bf16() && B >= 16; }
@@ -448,7 +448,7 @@ int64_t train_parts(cs_ctx *ctx, const ClsShape &S, int64_t B) {
     n += cls_softmax_blocks(B) * (int64_t(S.n_cls) + 1);
     n += 4 * mt * (kClsH2 + 2 * kClsH1) + mt * kClsH1 * S.dim;
     if (S.dim == 2)
-        n += int64_t(sm) * kClsCh * (kClsCh * S.taps + 2 * S.taps + 1) +
+        n += 2 * int64_t(sm) * kClsCh * (kClsCh * S.taps + 2 * S.taps + 1) +
              int64_t(cls_pool_back_blocks(B, sm)) * kClsCh;
     return n;
 }
@@ -825,8 +825,7 @@ cs_status cs_classifier_forward(cs_ctx *ctx, int32_t mesh_id, int64_t n, const d
                                   [](int64_t, int64_t, const float *) { return CS_OK; });
     if (rc) return rc;
     CCHK(cudaGetLastError());
-    CCHK(cudaDeviceSynchronize());
-    return cs_device_status(ctx);
+    return cs_device_status(ctx);     // synchronises
 }
 
 cs_status cs_classifier_labels(cs_ctx *ctx, int32_t mesh_id, int64_t n, const double *xp,
@@ -892,18 +891,21 @@ cs_status cs_classifier_grad(cs_ctx *ctx, int32_t mesh_id, int64_t B, const doub
     cs_status rc = tiled ? ensure_train(ctx, *C, B) : CS_OK;
     if (rc == CS_OK && (!tiled || C->dim == 3)) rc = ensure_ws(ctx, *C, B, true, true);
     if (rc) return rc;
-    CCHK(cudaMemset(C->loss, 0, sizeof(float)));
     if (tiled) {
         ctx->launches += train_tiled(ctx, *C, m->d, B, xp, labels, nullptr, C->loss, nullptr);
     } else {
+        CCHK(cudaMemset(C->loss, 0, sizeof(float)));
         ctx->launches += forward(ctx, *C, m->d, B, xp, nullptr, nullptr);
         ctx->launches += backward(ctx, *C, B, labels, nullptr, C->loss, nullptr);
     }
     CCHK(cudaGetLastError());
-    CCHK(cudaDeviceSynchronize());
-    if ((rc = cs_device_status(ctx))) return rc;
-    CCHK(cudaMemcpy(grad_out, C->g, size_t(C->n) * sizeof(float), cudaMemcpyDeviceToDevice));
-    if (loss_out) CCHK(cudaMemcpy(loss_out, C->loss, sizeof(float), cudaMemcpyDeviceToHost));
+    if ((rc = cs_device_status(ctx))) return rc;     // synchronises
+    CCHK(cudaMemcpyAsync(grad_out, C->g, size_t(C->n) * sizeof(float), cudaMemcpyDeviceToDevice,
+                         nullptr));
+    if (loss_out)
+        CCHK(cudaMemcpy(loss_out, C->loss, sizeof(float), cudaMemcpyDeviceToHost));
+    else
+        CCHK(cudaDeviceSynchronize());
     return CS_OK;
 }
 

@@ -412,16 +412,26 @@ __global__ void __launch_bounds__(kT) pool_back_tiled_kernel(const float *__rest
     pdl_wait();
     const int c = threadIdx.x % C;
     float sum = 0.f;
+    constexpr int kZ = (G::P + kT / C - 1) / (kT / C);       // positions of a thread
     for (int64_t b = blockIdx.x; b < B; b += gridDim.x) {
+        // the row's pre-activations travel with its pooled gradient
+        float zv[kZ];
+        #pragma unroll
+        for (int j = 0; j < kZ; ++j) {
+            const int p = threadIdx.x / C + j * (kT / C);
+            zv[j] = p < G::P ? __ldg(z + (b * G::P + p) * C + c) : 0.f;
+        }
         __syncthreads();
         for (int i = threadIdx.x; i < C * G::Pp; i += kT)
-            sg[i / G::Pp * Ld + i % G::Pp] = dpool[b * (C * G::Pp) + i];
+            sg[i / G::Pp * Ld + i % G::Pp] = __ldg(dpool + b * (C * G::Pp) + i);
         __syncthreads();
-        for (int p = threadIdx.x / C; p < G::P; p += kT / C) {
+        #pragma unroll
+        for (int j = 0; j < kZ; ++j) {
+            const int p = threadIdx.x / C + j * (kT / C);
+            if (p >= G::P) continue;
             const int px = p % G::W, py = (p / G::W) % G::W, pz = D == 3 ? p / (G::W * G::W) : 0;
             float g = 0.f;
-            if (px < 2 * G::Wp && py < 2 * G::Wp && (D == 2 || pz < 2 * G::Wp) &&
-                z[(b * G::P + p) * C + c] > 0.f) {
+            if (px < 2 * G::Wp && py < 2 * G::Wp && (D == 2 || pz < 2 * G::Wp) && zv[j] > 0.f) {
                 const int pp = D == 2 ? (py / 2) * G::Wp + px / 2
                                       : ((pz / 2) * G::Wp + py / 2) * G::Wp + px / 2;
                 g = sg[c * Ld + pp] / float(1 << D);
@@ -548,7 +558,7 @@ __global__ void __launch_bounds__(32) loss_sum_kernel(const float *__restrict__ 
     for (int i = threadIdx.x; i < n; i += 32) s += loss_part[i];
     s = warp_sum(s);
     const int n_valid = *count;
-    if (threadIdx.x == 0) *loss += s * (n_valid > 0 ? 1.f / float(n_valid) : 0.f);
+    if (threadIdx.x == 0) *loss = s * (n_valid > 0 ? 1.f / float(n_valid) : 0.f);
 }
 
 // label = window cell (x fastest) holding the centroid of the host element,
@@ -734,7 +744,7 @@ void launch_cls_pool_tiled(int dim, const float *z, int64_t B, const FcMat &cat,
 }
 
 int cls_pool_back_blocks(int64_t B, int sm_count) {
-    return int(std::min<int64_t>(B, int64_t(sm_count) * 4));
+    return int(std::min<int64_t>(B, int64_t(sm_count) * 6));
 }
 
 void launch_cls_pool_back_tiled(int dim, const float *dpool, const float *z, int64_t B,

@@ -83,7 +83,7 @@ int cls_softmax_blocks(int64_t B);
 void launch_softmax_ce_tiled(const float *H, const int32_t *labels, const int64_t *idx, int64_t B,
                              int n_cls, const FcMat &gH, float *part, float *loss_part, int *count,
                              cudaStream_t st);
-// *loss += sum of n loss_part / max(*count, 1)
+// *loss = sum of n loss_part / *count (0 where that is 0)
 void launch_loss_sum(const float *loss_part, int n, const int *count, float *loss, cudaStream_t st);
 
 }  // namespace cs

@@ -304,9 +304,8 @@ int backward(cs_ctx *ctx, Predictor &P, int64_t B, const float *tgt, float *loss
     return n;
 }
 
-// The fused path's forward pass of B windows into P.out; with targets the
-// gradients of the mean squared error into P.g as well, the loss added to
-// *loss. Every sum over the batch is one of partials in a fixed order.
+// The fused path's forward pass of B windows into P.out; train_fused adds the
+// gradients of the mean squared error into P.g, and *loss. Every sum over the batch is one of partials in a fixed order.
 int forward_fused(cs_ctx *ctx, Predictor &P, int64_t B, const float *win, const float *tgt,
                   cudaStream_t st) {
     const NetShape S(P.dim);
@@ -1082,13 +1081,21 @@ cs_status cs_predictor_grad(cs_ctx *ctx, int dim, int64_t B, const float *window
     cs_status rc = ensure_io(ctx, *P, B);
     if (rc == CS_OK) rc = fused ? ensure_fused(ctx, *P, B, true) : ensure_workspace(ctx, *P, B);
     if (rc) return rc;
-    PCHK(cudaMemset(P->loss, 0, sizeof(float)));
     if (fused) {
         ctx->launches += train_fused(ctx, *P, B, windows, targets, P->loss, nullptr);
-    } else {
-        ctx->launches += forward(ctx, *P, B, windows, nullptr);
-        ctx->launches += backward(ctx, *P, B, targets, P->loss, nullptr);
+        PCHK(cudaGetLastError());
+        // in the stream's order; the copy of the loss waits for everything
+        PCHK(cudaMemcpyAsync(grad_out, P->g, size_t(P->n) * sizeof(float), cudaMemcpyDeviceToDevice,
+                             nullptr));
+        if (loss_out)
+            PCHK(cudaMemcpy(loss_out, P->loss, sizeof(float), cudaMemcpyDeviceToHost));
+        else
+            PCHK(cudaDeviceSynchronize());
+        return CS_OK;
     }
+    PCHK(cudaMemset(P->loss, 0, sizeof(float)));
+    ctx->launches += forward(ctx, *P, B, windows, nullptr);
+    ctx->launches += backward(ctx, *P, B, targets, P->loss, nullptr);
     PCHK(cudaGetLastError());
     PCHK(cudaDeviceSynchronize());
     PCHK(cudaMemcpy(grad_out, P->g, size_t(P->n) * sizeof(float), cudaMemcpyDeviceToDevice));

@@ -38,7 +38,7 @@
 namespace cs {
 namespace {
 
-constexpr int kPitch = 34;        // halves per position in shared memory (17 words: no conflicts)
+constexpr int kPitch = 40;        // halves per position in shared memory (5 x 16 bytes: no conflicts)
 constexpr int kFwdThreads = 256;
 constexpr int kBwdThreads = 512;
 constexpr int kRowsT = 128;       // MMA rows
@@ -77,19 +77,24 @@ struct Geo {
     static constexpr int ActHalves = FIRST ? C * Pi : Pi * kPitch;   // per input
 };
 
-// shared memory of one CTA (bytes); A first, then the activations
+// shared memory of one CTA (bytes); A first, then the activations (act2: the
+// second buffer of a backward pass, the first one where it does not fit)
 struct ConvSmem {
-    int act, w, dz, tab, bar, total;
+    int act, act2, w, dz, tab, bar, total;
 };
 
 template <class N, bool BWD>
 struct ConvCfg {
     static constexpr int D = N::Dim;
-    // K chunks (of 8) per operand build and buffers of them: a 2-D operand
-    // fits whole (36 chunks); a 3-D one (108) is built in pieces
-    static constexpr int CbMax = D == 2 ? 36 : BWD ? 32 : 28;
-    static constexpr int Cb = N::Chunks < CbMax ? N::Chunks : CbMax;
-    static constexpr int Nb = D == 2 || BWD || N::First ? 1 : 2;
+    // The operand is built in groups of 8 channels (Taps chunks of 8 columns;
+    // the FP32 input's few columns all at once). A 2-D operand fits whole (four
+    // groups); a 3-D one is built two groups at a time (an even number of
+    // chunks: whole K = 16 steps).
+    static constexpr int Groups = N::First ? 1 : 4;
+    static constexpr int GroupChunks = N::First ? N::Chunks : N::Taps;
+    static constexpr int Gb = N::First ? 1 : D == 2 ? 4 : 2;   // groups per build
+    static constexpr int Cb = Gb * GroupChunks;
+    static constexpr int Builds = Groups / Gb;
     // backward: channels, columns and MMA N of one dcol pass
     static constexpr int Ch = D == 2 ? 16 : 8;
     static constexpr int Nc = Ch * N::Taps;                  // 144, 216
@@ -99,35 +104,53 @@ struct ConvCfg {
     static constexpr bool Dgrad = BWD && !N::First;
     static constexpr int Kw = D == 2 ? 288 : 872;            // rows of the dgrad weights
     static constexpr int Dcol = Dgrad ? kRowsT * Ld * 4 : 0;
-    static constexpr int A = Nb * Cb * kChunk > Dcol ? Nb * Cb * kChunk : Dcol;
-    static constexpr int Mt = (N::K + 127) / 128;            // M-tiles of the weight gradient
+    static constexpr int A = Cb * kChunk > Dcol ? Cb * kChunk : Dcol;
+    static constexpr int MtB = (Cb + 15) / 16;               // weight-gradient M-tiles per build
+    static constexpr int Mt = MtB * Builds;
+    static constexpr uint32_t ColD = 32 * Mt;                // TMEM column of dcol
+    static constexpr uint32_t Cols = !Dgrad ? 128 : ColD + Nm <= 256 ? 256 : 512;
     static constexpr int WBytes = !BWD ? N::Kp * kTrainCh * 2 : Dgrad ? Kw * kTrainCh * 2 : 0;
+    // the classifier's layer, one input of 81 rows per tile, leaves room for a
+    // second CTA per SM
+    static constexpr int PerSm = BWD && N::Si == 11 ? 2 : 1;
     static_assert((Passes - 1) * Nc + Nm <= Kw, "dgrad weight rows");
-    static_assert(256 + Nm <= 512 && 32 * Mt <= 256, "TMEM columns");
-    static_assert(Cb % 16 == 0 || Cb == N::Chunks || !BWD, "builds end on an M-tile");
-    static_assert(Cb % 2 == 0, "whole K = 16 steps per build");
+    static_assert(!BWD || ColD + (Dgrad ? Nm : 0) <= Cols, "TMEM columns");
+    static_assert(BWD || Cb % 2 == 0, "whole K = 16 steps per build");
 };
 
+constexpr int kSmemMax = 232448, kSmemHalf = 113 * 1024;
+
 template <class N, bool BWD>
-constexpr ConvSmem conv_smem(int G) {
+constexpr ConvSmem conv_smem_of(int G, int buffers) {
     using F = ConvCfg<N, BWD>;
     ConvSmem s{};
     s.act = F::A;
-    s.w = s.act + (G * N::ActHalves * 2 + 127) / 128 * 128;
+    const int act = (G * N::ActHalves * 2 + 127) / 128 * 128;
+    s.act2 = s.act + (buffers - 1) * act;
+    s.w = s.act2 + act;
     s.dz = s.w + F::WBytes;
     s.tab = s.dz + (BWD ? kTrainCh * kRowsT * 2 : 0);
-    s.bar = (s.tab + N::Kp * 2 + 127) / 128 * 128;
+    s.bar = (s.tab + (N::First ? N::Kp * 2 : 0) + 127) / 128 * 128;
     s.total = s.bar + 64;
     // an M-tile of the weight gradient reads 16 chunks from its first one,
     // past the built ones at the end (rows of no use): inside the allocation
-    const int reach = (F::Cb + 15) / 16 * 16 * kChunk;
+    const int reach = F::MtB * 16 * kChunk;
     if (BWD && s.total < reach) s.total = reach;
     return s;
 }
 
+template <class N, bool BWD>
+constexpr ConvSmem conv_smem(int G) {
+    if (BWD && !N::First) {
+        const ConvSmem s = conv_smem_of<N, BWD>(G, 2);
+        if (s.total <= (ConvCfg<N, BWD>::PerSm > 1 ? kSmemHalf : kSmemMax)) return s;
+    }
+    return conv_smem_of<N, BWD>(G, 1);
+}
+
 // The activations of inputs [b0, b0 + nb) on their way to shared memory:
 // start() issues the loads, finish() makes them visible to the caller (the
-// CTA still has to synchronise). BF16 activations travel as 4-byte
+// CTA still has to synchronise). BF16 activations travel as
 // asynchronous copies into the padded rows; the network's FP32 input waits in
 // registers and is rounded as it is stored, channels first.
 template <class N, int NTH>
@@ -143,14 +166,11 @@ struct ActLoad {
             for (int j = 0; j < Regs; ++j)
                 r[j] = tid + j * NTH < n ? __ldg(src + tid + j * NTH) : 0.f;
         } else {
-            const int n = nb * N::Pi * 16;
-            const uint32_t *src = reinterpret_cast<const uint32_t *>(
-                static_cast<const uint16_t *>(a.x) + b0 * N::Pi * kTrainCh);
-            for (int i = tid; i < n; i += NTH) {
-                const uint32_t d = smem_addr(act) + ((i >> 4) * (kPitch / 2) + (i & 15)) * 4;
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src + i)
-                             : "memory");
-            }
+            const int n = nb * N::Pi * 4;
+            const uint4 *src = reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(a.x) +
+                                                               b0 * N::Pi * kTrainCh);
+            for (int i = tid; i < n; i += NTH)
+                cp_async16(act + (i >> 2) * (kPitch * 2) + (i & 3) * 16, src + i);
         }
     }
     __device__ __forceinline__ void finish(int nb, uint8_t *act, int tid) {
@@ -166,15 +186,16 @@ struct ActLoad {
     }
 };
 
-// offset (in halves) of operand column k from its row's base, 0xffff past K
+// offset (in halves) of operand column k of the network's input from its
+// row's base, 0xffff past K
 template <class N>
 __device__ __forceinline__ void fill_tab(uint16_t *tab, int tid, int nth) {
-    for (int k = tid; k < N::Kp; k += nth) {
-        const int i = k / N::Taps, t = k % N::Taps;
-        const int dx = t % 3, dy = (t / 3) % 3, dz = N::Dim == 3 ? t / 9 : 0;
-        const int to = (dz * N::Si + dy) * N::Si + dx;
-        tab[k] = k >= N::K ? 0xffffu : uint16_t(N::First ? i * N::Pi + to : to * kPitch + i);
-    }
+    if constexpr (N::First)
+        for (int k = tid; k < N::Kp; k += nth) {
+            const int i = k / N::Taps, t = k % N::Taps;
+            const int dx = t % 3, dy = (t / 3) % 3, dz = N::Dim == 3 ? t / 9 : 0;
+            tab[k] = k >= N::K ? 0xffffu : uint16_t(i * N::Pi + (dz * N::Si + dy) * N::Si + dx);
+        }
 }
 
 // base (in halves) of row r's window, -1 where the row holds no output
@@ -187,37 +208,118 @@ __device__ __forceinline__ int row_base(int nb, int r) {
     return w * N::ActHalves + pb * (N::First ? 1 : kPitch);
 }
 
-// chunks [c0, c0 + nc) of the im2col operand into `dst`; a warp takes 32 rows
-// of one chunk at a time, so its loads step by one position per lane
-template <class N, int NWARPS, int CB>
-__device__ __forceinline__ void build_operand(uint8_t *dst, const uint8_t *act,
-                                              const uint16_t *tab, int base, int c0, int nc,
-                                              int warp, int lane) {
+// The im2col operand of the network's input into `dst`: a warp takes 32 rows
+// of one chunk at a time, so its loads step by one position per lane.
+template <class N, int NWARPS>
+__device__ __forceinline__ void build_first(uint8_t *dst, const uint8_t *act, const uint16_t *tab,
+                                            int base, int warp, int lane) {
     constexpr int Step = NWARPS / 4;
     const int row = 32 * (warp & 3) + lane;
     const uint16_t *s = reinterpret_cast<const uint16_t *>(act) + (base < 0 ? 0 : base);
     const uint32_t keep = base < 0 ? 0u : 0xffffffffu;
     #pragma unroll 3
-    for (int i = 0; i < (CB + Step - 1) / Step; ++i) {
+    for (int i = 0; i < (N::Chunks + Step - 1) / Step; ++i) {
         const int c = (warp >> 2) + i * Step;
-        if (c >= nc) break;
-        const uint4 t = *reinterpret_cast<const uint4 *>(tab + 8 * (c0 + c));
+        if (c >= N::Chunks) break;
+        const uint4 t = *reinterpret_cast<const uint4 *>(tab + 8 * c);
         const uint32_t tw[4] = {t.x, t.y, t.z, t.w};
         uint32_t v[4];
-        if (N::K % 8 == 0 || 8 * (c0 + c) + 8 <= N::K) {
-            #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                v[j] = uint32_t(s[tw[j] & 0xffffu]) | (uint32_t(s[tw[j] >> 16]) << 16);
-        } else {   // the last chunk: zero past K
-            #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uint32_t k0 = tw[j] & 0xffffu, k1 = tw[j] >> 16;
-                v[j] = (k0 == 0xffffu ? 0u : uint32_t(s[k0])) |
-                       (k1 == 0xffffu ? 0u : uint32_t(s[k1]) << 16);
-            }
+        #pragma unroll
+        for (int j = 0; j < 4; ++j) {   // zero past K
+            const uint32_t k0 = tw[j] & 0xffffu, k1 = tw[j] >> 16;
+            v[j] = (k0 == 0xffffu ? 0u : uint32_t(s[k0])) | (k1 == 0xffffu ? 0u : uint32_t(s[k1]) << 16);
         }
         *reinterpret_cast<uint4 *>(dst + c * kChunk + row * 16) =
             make_uint4(v[0] & keep, v[1] & keep, v[2] & keep, v[3] & keep);
+    }
+}
+
+// tap t's offset in bytes from a row's base
+template <class N>
+__device__ __forceinline__ constexpr int tap_bytes(int t) {
+    return (((N::Dim == 3 ? t / 9 : 0) * N::Si + (t / 3) % 3) * N::Si + t % 3) * kPitch * 2;
+}
+
+// halves i0 of a and i1 of b as one word
+__device__ __forceinline__ uint32_t halves(uint32_t a, int i0, uint32_t b, int i1) {
+    return __byte_perm(a, b, (i0 ? 0x32u : 0x10u) | ((i1 ? 0x76u : 0x54u) << 8));
+}
+
+// Part of a group of 8 channels of one row of the operand: column k = channel
+// * Taps + tap of the group at chunk k / 8. 2-D: all of it; every tap's 8
+// channels are one 16-byte load, transposed to (channel, tap) order in
+// registers, and a chunk is one 16-byte store, conflict-free like the loads.
+// 3-D: the group's channels 4 p .. 4 p + 3 (8-byte loads; 27 taps of 8 channels
+// would not fit the registers), that is columns 108 p .. 108 p + 107: 13 chunks
+// and half of the one in the middle. dst: the group's first chunk at the row;
+// s: the row's window at the group's channels.
+template <class N>
+__device__ __forceinline__ void build_part(uint8_t *dst, const uint8_t *s, uint32_t keep, int p) {
+    if constexpr (N::Dim == 2) {
+        uint32_t v[9][4];
+        #pragma unroll
+        for (int t = 0; t < 9; ++t) {
+            const uint4 q = *reinterpret_cast<const uint4 *>(s + tap_bytes<N>(t));
+            v[t][0] = q.x & keep;
+            v[t][1] = q.y & keep;
+            v[t][2] = q.z & keep;
+            v[t][3] = q.w & keep;
+        }
+        #pragma unroll
+        for (int c = 0; c < 9; ++c) {
+            uint32_t w[4];
+            #pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int k0 = 8 * c + 2 * j, k1 = k0 + 1;
+                w[j] = halves(v[k0 % 9][k0 / 9 / 2], (k0 / 9) & 1, v[k1 % 9][k1 / 9 / 2], (k1 / 9) & 1);
+            }
+            *reinterpret_cast<uint4 *>(dst + c * kChunk) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    } else {
+        uint32_t v[27][2];
+        #pragma unroll
+        for (int t = 0; t < 27; ++t) {
+            const uint2 q = *reinterpret_cast<const uint2 *>(s + tap_bytes<N>(t) + 8 * p);
+            v[t][0] = q.x & keep;
+            v[t][1] = q.y & keep;
+        }
+        auto word = [&](int k) {    // columns k, k + 1 of the part
+            return halves(v[k % 27][k / 27 / 2], (k / 27) & 1, v[(k + 1) % 27][(k + 1) / 27 / 2],
+                          ((k + 1) / 27) & 1);
+        };
+        if (p == 0) {
+            #pragma unroll
+            for (int c = 0; c < 13; ++c)
+                *reinterpret_cast<uint4 *>(dst + c * kChunk) =
+                    make_uint4(word(8 * c), word(8 * c + 2), word(8 * c + 4), word(8 * c + 6));
+            *reinterpret_cast<uint2 *>(dst + 13 * kChunk) = make_uint2(word(104), word(106));
+        } else {
+            *reinterpret_cast<uint2 *>(dst + 13 * kChunk + 8) = make_uint2(word(0), word(2));
+            #pragma unroll
+            for (int c = 14; c < 27; ++c)
+                *reinterpret_cast<uint4 *>(dst + c * kChunk) = make_uint4(
+                    word(8 * c - 108), word(8 * c - 106), word(8 * c - 104), word(8 * c - 102));
+        }
+    }
+}
+
+// build j of the operand into `dst`
+template <class N, bool BWD, int NWARPS>
+__device__ __forceinline__ void build_operand(uint8_t *dst, const uint8_t *act, const uint16_t *tab,
+                                              int base, int j, int warp, int lane) {
+    using F = ConvCfg<N, BWD>;
+    if constexpr (N::First) {
+        build_first<N, NWARPS>(dst, act, tab, base, warp, lane);
+    } else {
+        const int row = 32 * (warp & 3) + lane;
+        const uint8_t *s = act + (base < 0 ? 0 : base) * 2;
+        constexpr int Parts = N::Dim == 2 ? 1 : 2;
+        #pragma unroll 1
+        for (int i = warp >> 2; i < F::Gb * Parts; i += NWARPS / 4) {
+            const int g = i / Parts;
+            build_part<N>(dst + g * F::GroupChunks * kChunk + row * 16, s + (j * F::Gb + g) * 16,
+                          base < 0 ? 0u : 0xffffffffu, i % Parts);
+        }
     }
 }
 
@@ -258,7 +360,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) conv_fwd_kernel(const ConvArgs
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t *act = smem + L.act, *wop = smem + L.w;
     uint16_t *tab = reinterpret_cast<uint16_t *>(smem + L.tab);
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L.bar);   // [Nb] builds, then the drain
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L.bar);   // MMAs, [2] the drain
     uint32_t *slot = reinterpret_cast<uint32_t *>(smem + L.bar + 32);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + L.bar + 40);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -301,33 +403,34 @@ __global__ void __launch_bounds__(kFwdThreads, 2) conv_fwd_kernel(const ConvArgs
         const int64_t b0 = t * a.G;
         ld.finish(nb, act, tid);
         const int base = row_base<N>(nb, r);
+        fence_before();
         __syncthreads();
-        for (int c0 = 0; c0 < N::Chunks && ok; c0 += F::Cb, ++it) {
-            const int buf = F::Nb == 1 ? 0 : it % F::Nb, nc = min(F::Cb, N::Chunks - c0);
-            // the buffer's previous MMAs are complete (one build per tile: the
-            // tile before waited for them)
-            if (F::Cb < N::Chunks && it >= F::Nb)
-                ok = __syncthreads_and(
-                    mbar_wait(bars + buf, uint32_t(it / F::Nb - 1) & 1u, abort_flag, err));
+        fence_after();
+        for (int j = 0; j < F::Builds && ok; ++j, ++it) {
+            // the operand's previous MMAs are complete (with one build per tile
+            // the tile before waited for them)
+            if (F::Builds > 1 && it >= 1)
+                ok = __syncthreads_and(mbar_wait(bars + 0, uint32_t(it - 1) & 1u, abort_flag, err));
             if (!ok) break;
-            uint8_t *A = smem + buf * F::Cb * kChunk;
-            build_operand<N, kNw, F::Cb>(A, act, tab, base, c0, nc, warp, lane);
+            build_operand<N, false, kNw>(smem, act, tab, base, j, warp, lane);
             fence_async_smem();
             fence_before();
             __syncthreads();
             fence_after();
             if (warp == 0) {
                 if (elect_one()) {
-                    const uint64_t da = sdesc(smem_addr(A), kChunk, 128);
-                    #pragma unroll 4
-                    for (int q = 0; q < nc / 2; ++q) {
+                    const uint64_t da = sdesc(smem_addr(smem), kChunk, 128);
+                    const int c0 = j * F::Cb;
+                    #pragma unroll
+                    for (int q = 0; q < F::Cb / 2; ++q) {
                         const int k = 8 * c0 + 16 * q;
-                        const int s = N::K > 512 && a.nsplit > 1 ? k / a.kc : 0;
+                        // at most three splits (kc >= K without any)
+                        const int s = N::K > 512 ? (k >= a.kc) + (k >= 2 * a.kc) : 0;
                         mma_bf16(tmem + uint32_t(32 * s), da + uint64_t(2 * q * (kChunk >> 4)),
                                  dw + uint64_t((c0 + 2 * q) * kTrainCh), id,
                                  k - s * a.kc > 0 ? 1u : 0u);
                     }
-                    mma_commit(bars + buf);
+                    mma_commit(bars + 0);
                 }
                 __syncwarp();
             }
@@ -341,8 +444,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) conv_fwd_kernel(const ConvArgs
             ld.start(a, t * a.G, nb, act, tid);
         }
         // the tile's last build completes after all others
-        ok = __syncthreads_and(mbar_wait(bars + (F::Nb == 1 ? 0 : (it - 1) % F::Nb),
-                                         uint32_t((it - 1) / F::Nb) & 1u, abort_flag, err));
+        ok = __syncthreads_and(mbar_wait(bars + 0, uint32_t(it - 1) & 1u, abort_flag, err));
         if (!ok) break;
         fence_after();
         const uint32_t tq = tmem + (uint32_t(32 * (warp & 3)) << 16) + uint32_t(o0);
@@ -408,22 +510,23 @@ __device__ __forceinline__ void col2im_line(const float *dcol, int row0, int iy,
 }
 
 template <class N>
-__global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs a,
+__global__ void __launch_bounds__(kBwdThreads, ConvCfg<N, true>::PerSm) conv_bwd_kernel(const ConvArgs a,
                                                                   const ConvSmem L, int *err) {
     using F = ConvCfg<N, true>;
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t *act = smem + L.act, *wop = smem + L.w, *dzs = smem + L.dz;
+    uint8_t *act = smem + L.act, *next = smem + L.act2, *wop = smem + L.w, *dzs = smem + L.dz;
+    const bool two = L.act2 != L.act;
     float *dcol = reinterpret_cast<float *>(smem);          // over A once its MMAs are complete
     uint16_t *tab = reinterpret_cast<uint16_t *>(smem + L.tab);
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L.bar);   // MMAs, drain
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L.bar);   // builds, dcol, drain
     uint32_t *slot = reinterpret_cast<uint32_t *>(smem + L.bar + 32);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + L.bar + 40);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    constexpr uint32_t kCols = 512, kDcol = 256;
+    constexpr uint32_t kCols = F::Cols, kDcol = F::ColD;
     constexpr int kNw = kBwdThreads / 32;
 
     if (tid == 0) {
-        for (int i = 0; i < 2; ++i) mbar_init(bars + i, 1u);
+        for (int i = 0; i < 3; ++i) mbar_init(bars + i, 1u);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -463,36 +566,47 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
     const int crop = N::Si - 2 * a.ring;
     const int np = N::Dim == 2 ? crop * crop : crop * crop * crop;
     bool ok = true, any = false;
-    uint32_t phase = 0;
+    uint32_t phase = 0;          // of the dcol products
+    int it = 0;                  // builds so far
     while (t < a.tiles) {
         const int64_t b0 = t * a.G;
         ld.finish(nb, act, tid);
         *reinterpret_cast<uint4 *>(dzs + (tid & 3) * kChunk + (tid >> 2) * 16) = dzr;
         const int base = row_base<N>(nb, 32 * (warp & 3) + lane);
+        fence_before();
         __syncthreads();
+        fence_after();
         const int ksteps = (nb * N::Po + 15) / 16, nb_now = nb;
         t += gridDim.x;
         if (t < a.tiles) {
             nb = int(min(int64_t(a.G), a.B - t * a.G));
             fetch_dz();
+            if (two) ld.start(a, t * a.G, nb, next, tid);
         }
-        for (int c0 = 0; c0 < N::Chunks; c0 += F::Cb) {
-            const int nc = min(F::Cb, N::Chunks - c0);
-            build_operand<N, kNw, F::Cb>(smem, act, tab, base, c0, nc, warp, lane);
+        #pragma unroll 1
+        for (int j = 0; j < F::Builds; ++j, ++it) {
+            // the operand's MMAs of the build before (each tile ends with all of
+            // its builds complete)
+            if (j > 0)
+                ok = __syncthreads_and(mbar_wait(bars + 0, uint32_t(it - 1) & 1u, abort_flag, err));
+            if (!ok) break;
+            build_operand<N, true, kNw>(smem, act, tab, base, j, warp, lane);
             fence_async_smem();
             fence_before();
             __syncthreads();
             fence_after();
             if (warp == 0) {
                 if (elect_one()) {
-                    for (int mt = 0; mt < (nc + 15) / 16; ++mt) {
+                    #pragma unroll 1
+                    for (int mt = 0; mt < F::MtB; ++mt) {
                         const uint64_t da = sdesc(smem_addr(smem) + mt * 16 * kChunk, 128, kChunk);
-                        #pragma unroll 4
-                        for (int q = 0; q < ksteps; ++q)
-                            mma_bf16(tmem + uint32_t(32 * (c0 / 16 + mt)), da + uint64_t(q * 16),
-                                     dz_mn + uint64_t(q * 16), id_w, any || q > 0 ? 1u : 0u);
+                        #pragma unroll
+                        for (int q = 0; q < kRowsT / 16; ++q)
+                            if (q < ksteps)
+                                mma_bf16(tmem + uint32_t(32 * (F::MtB * j + mt)), da + uint64_t(q * 16),
+                                         dz_mn + uint64_t(q * 16), id_w, any || q > 0 ? 1u : 0u);
                     }
-                    if (F::Dgrad && c0 == 0)
+                    if (F::Dgrad && j == F::Builds - 1)
                         for (int q = 0; q < 2; ++q)
                             mma_bf16(tmem + kDcol, dz_k + uint64_t(2 * q * (kChunk >> 4)),
                                      w_k + uint64_t(2 * q * F::Kw), id_c, q > 0 ? 1u : 0u);
@@ -502,11 +616,11 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
             }
             // the network's input is not read again: fetch the next tile's
             if (N::First && t < a.tiles) ld.start(a, t * a.G, nb, act, tid);
-            ok = __syncthreads_and(mbar_wait(bars + 0, phase, abort_flag, err));
-            phase ^= 1u;
-            if (!ok) break;
-            fence_after();
         }
+        // the last build's MMAs complete after all others
+        if (ok)
+            ok = __syncthreads_and(mbar_wait(bars + 0, uint32_t(it - 1) & 1u, abort_flag, err));
+        fence_after();
         if (!ok) break;
         any = true;
         if constexpr (F::Dgrad) {
@@ -533,7 +647,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
                             mma_bf16(tmem + kDcol, dz_k + uint64_t(2 * q * (kChunk >> 4)),
                                      w_k + uint64_t(2 * q * F::Kw + (j + 1) * F::Nc), id_c,
                                      q > 0 ? 1u : 0u);
-                        mma_commit(bars + 0);
+                        mma_commit(bars + 1);
                     }
                     __syncwarp();
                 }
@@ -562,17 +676,20 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
                 }
                 db[j] += s_db;
                 if (j + 1 < F::Passes) {
-                    ok = __syncthreads_and(mbar_wait(bars + 0, phase, abort_flag, err));
+                    ok = __syncthreads_and(mbar_wait(bars + 1, phase, abort_flag, err));
                     phase ^= 1u;
                     if (!ok) break;
                     fence_after();
                 } else {
                     __syncthreads();
-                    if (t < a.tiles) ld.start(a, t * a.G, nb, act, tid);
+                    if (t < a.tiles && !two) ld.start(a, t * a.G, nb, act, tid);
                 }
             }
             if (!ok) break;
         }
+        uint8_t *q = act;
+        act = next;
+        next = q;
     }
     cp_async_wait_all();
     if (ok && any) {
@@ -583,8 +700,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
             for (int mt = 0; mt < F::Mt; ++mt) {
                 float v[16];
                 tmem_ld16(tmem + (uint32_t(32 * (warp & 3)) << 16) + uint32_t(32 * mt + o0), v);
-                const int k = 128 * mt + 32 * (warp & 3) + lane;
-                if (k < N::K) {
+                // M-tile mt: columns from 8 Cb (mt / MtB) + 128 (mt % MtB) of A
+                const int kl = 128 * (mt % F::MtB) + 32 * (warp & 3) + lane;
+                const int k = 8 * F::Cb * (mt / F::MtB) + kl;
+                if (kl < 8 * F::Cb && k < N::K) {
                     #pragma unroll
                     for (int e = 0; e < 16; ++e) wp[(o0 + e) * N::K + k] = v[e];
                 }
@@ -605,7 +724,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
             }
         }
     }
-    mma_drain(bars + 1, tmem, kCols, warp);
+    mma_drain(bars + 2, tmem, kCols, warp);
 }
 
 // Weights of one convolution (FP32 W[32][K]) as the operands of both passes:
@@ -919,30 +1038,77 @@ __global__ void __launch_bounds__(256, 1) head_train_kernel(const HeadArgs a, in
 }
 
 // ---------------------------------------------------------------------------
-// Sums of the CTAs' partials: 32 elements per block, eight groups of threads
-// take every eighth partial each, their sums are added in order.
+// Sums of the CTAs' partials in a fixed order. Few partials (up to kRedFew):
+// a thread adds them all, four neighbouring elements at a time where the
+// alignment allows. Many: 32 elements per block, eight groups of threads take
+// every eighth partial each and their sums are added in order (a long chain of
+// loads per thread would be latency alone).
 // ---------------------------------------------------------------------------
-constexpr int kRedE = 32, kRedG = 8;
+constexpr int kRedE = 32, kRedG = 8, kRedFew = 48, kRedT = kRedE * kRedG;
 
 struct ReduceArgs {
     ReduceSeg seg[kMaxSegs];
     int block0[kMaxSegs + 1];
+    int vec[kMaxSegs];            // elements per thread of a segment of few, else 0
     int n;
 };
 
-__global__ void __launch_bounds__(kRedE * kRedG) reduce_parts_kernel(const ReduceArgs a) {
+__device__ __forceinline__ void reduce_store(const ReduceSeg &g, int64_t i, float v) {
+    g.out[i] = g.div > 0.f ? v / g.div : v;
+}
+
+__global__ void __launch_bounds__(kRedT) reduce_parts_kernel(const ReduceArgs a) {
     __shared__ float red[kRedG][kRedE];
     int s = 0;
     while (s + 1 < a.n && int(blockIdx.x) >= a.block0[s + 1]) ++s;
     const ReduceSeg &g = a.seg[s];
-    const int e = threadIdx.x % kRedE, grp = threadIdx.x / kRedE;
-    const int64_t i = int64_t(blockIdx.x - a.block0[s]) * kRedE + e;
+    const int64_t blk = blockIdx.x - a.block0[s];
     pdl_wait();
+    // batches of loads in flight together, then added in order
+    constexpr int kBatch = 8;
+    if (a.vec[s] == 4) {
+        const int64_t i = (blk * kRedT + threadIdx.x) * 4;
+        if (i >= g.count) return;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int q0 = 0; q0 < g.n; q0 += kBatch) {
+            float4 v[kBatch];
+            #pragma unroll
+            for (int j = 0; j < kBatch; ++j)
+                v[j] = q0 + j < g.n ? __ldg(reinterpret_cast<const float4 *>(
+                                          g.part + int64_t(q0 + j) * g.stride + i))
+                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+            #pragma unroll
+            for (int j = 0; j < kBatch; ++j) {
+                x.x += v[j].x;
+                x.y += v[j].y;
+                x.z += v[j].z;
+                x.w += v[j].w;
+            }
+        }
+        reduce_store(g, i, x.x);
+        reduce_store(g, i + 1, x.y);
+        reduce_store(g, i + 2, x.z);
+        reduce_store(g, i + 3, x.w);
+        return;
+    }
+    const bool few = a.vec[s] == 1;
+    const int e = threadIdx.x % kRedE, grp = threadIdx.x / kRedE;
+    const int64_t i = few ? blk * kRedT + threadIdx.x : blk * kRedE + e;
     float x = 0.f;
     if (i < g.count) {
-        const float *p = g.part + i;
-        #pragma unroll 10
-        for (int q = grp; q < g.n; q += kRedG) x += __ldg(p + int64_t(q) * g.stride);
+        const int step = few ? 1 : kRedG;
+        for (int q0 = few ? 0 : grp; q0 < g.n; q0 += step * kBatch) {
+            float v[kBatch];
+            #pragma unroll
+            for (int j = 0; j < kBatch; ++j)
+                v[j] = q0 + j * step < g.n ? __ldg(g.part + int64_t(q0 + j * step) * g.stride + i) : 0.f;
+            #pragma unroll
+            for (int j = 0; j < kBatch; ++j) x += v[j];
+        }
+    }
+    if (few) {
+        if (i < g.count) reduce_store(g, i, x);
+        return;
     }
     red[grp][e] = x;
     __syncthreads();
@@ -950,14 +1116,9 @@ __global__ void __launch_bounds__(kRedE * kRedG) reduce_parts_kernel(const Reduc
         float v = red[0][e];
         #pragma unroll
         for (int q = 1; q < kRedG; ++q) v += red[q][e];
-        if (g.div > 0.f)
-            g.out[i] += v / g.div;
-        else
-            g.out[i] = v;
+        reduce_store(g, i, v);
     }
 }
-
-constexpr int kSmemMax = 232448;
 
 // the kernels' instances: f(Geo) for the layer's dimension and edge
 template <class Fn>
@@ -986,7 +1147,7 @@ template <class N, bool BWD>
 int tile_inputs(int64_t B, int sm_count) {
     const int64_t even = (B + sm_count - 1) / sm_count;
     int G = int(std::max<int64_t>(1, std::min<int64_t>(N::GMax, even)));
-    while (G > 1 && conv_smem<N, BWD>(G).total > kSmemMax) --G;
+    while (G > 1 && conv_smem_of<N, BWD>(G, 1).total > kSmemMax) --G;
     return G;
 }
 
@@ -1031,7 +1192,7 @@ int launch_conv_fwd(const ConvGeo &g, const void *x, bool first, int64_t B, cons
         a.tiles = (B + a.G - 1) / a.G;
         const ConvSmem L = conv_smem<N, false>(a.G);
         cudaFuncSetAttribute(conv_fwd_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-        const int per_sm = L.total <= 113 * 1024 ? 2 : 1;
+        const int per_sm = L.total <= kSmemHalf ? 2 : 1;
         const int grid = int(std::min<int64_t>(a.tiles, int64_t(sm_count) * per_sm));
         launch_pdl(conv_fwd_kernel<N>, dim3(grid), dim3(kFwdThreads), size_t(L.total), st, a, L, err);
     });
@@ -1040,8 +1201,12 @@ int launch_conv_fwd(const ConvGeo &g, const void *x, bool first, int64_t B, cons
 
 int conv_bwd_ctas(const ConvGeo &g, int64_t B, bool first, int sm_count) {
     int G = 1;
-    with_geo(g, first, [&](auto n) { G = tile_inputs<decltype(n), true>(B, sm_count); });
-    return int(std::min<int64_t>((B + G - 1) / G, sm_count));
+    int per_sm = 1;
+    with_geo(g, first, [&](auto n) {
+        G = tile_inputs<decltype(n), true>(B, sm_count);
+        per_sm = ConvCfg<decltype(n), true>::PerSm;
+    });
+    return int(std::min<int64_t>((B + G - 1) / G, int64_t(sm_count) * per_sm));
 }
 
 int launch_conv_bwd(const ConvGeo &g, const void *x, bool first, int64_t B, const uint16_t *dz,
@@ -1062,6 +1227,8 @@ int launch_conv_bwd(const ConvGeo &g, const void *x, bool first, int64_t B, cons
         a.G = tile_inputs<N, true>(B, sm_count);
         a.tiles = (B + a.G - 1) / a.G;
         const ConvSmem L = conv_smem<N, true>(a.G);
+        static_assert(ConvCfg<N, true>::PerSm == 1 || conv_smem<N, true>(1).total <= kSmemHalf,
+                      "two CTAs per SM");
         cudaFuncSetAttribute(conv_bwd_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
         launch_pdl(conv_bwd_kernel<N>, dim3(grid), dim3(kBwdThreads), size_t(L.total), st, a, L, err);
     });
@@ -1094,12 +1261,16 @@ int launch_reduce_parts(const ReduceSeg *segs, int n_segs, cudaStream_t st) {
     a.n = n_segs;
     int blocks = 0;
     for (int s = 0; s < n_segs; ++s) {
-        a.seg[s] = segs[s];
+        const ReduceSeg &g = a.seg[s] = segs[s];
+        const bool four = g.count % 4 == 0 && g.stride % 4 == 0 &&
+                          (reinterpret_cast<uintptr_t>(g.part) & 15u) == 0;
+        a.vec[s] = g.n > kRedFew ? 0 : four ? 4 : 1;
         a.block0[s] = blocks;
-        blocks += int((segs[s].count + kRedE - 1) / kRedE);
+        const int per = a.vec[s] ? kRedT * a.vec[s] : kRedE;
+        blocks += int((g.count + per - 1) / per);
     }
     a.block0[n_segs] = blocks;
-    launch_pdl(reduce_parts_kernel, dim3(blocks), dim3(kRedE * kRedG), 0, st, a);
+    launch_pdl(reduce_parts_kernel, dim3(blocks), dim3(kRedT), 0, st, a);
     return 1;
 }
 

@@ -65,8 +65,8 @@ int launch_train_head(int dim, int64_t B, const uint16_t *h, const uint8_t *pack
                       float *out, uint16_t *dz, float *part, int *err, int sm_count,
                       cudaStream_t st);
 
-// out[i] = sum over p < n, in a fixed order, of part[p stride + i] for i < count;
-// with `div` > 0 the sum over `div` is added to out instead
+// out[i] = sum over p < n, in a fixed order, of part[p stride + i] for i < count,
+// divided by `div` where that is > 0
 struct ReduceSeg {
     const float *part;
     int64_t stride, count;
