@@ -27,8 +27,8 @@
 //          position of each valid output row (its padded layout is conv2's
 //          operand, ring zero)
 //   stage  [pooled positions][33] FP32: ReLU(conv2 + b2), read by the pooling
-//   FP32 accumulation in TMEM: conv1 in columns [0, 32 MT), conv2 in
-//   [32 MT, 64 MT), MT the M-tiles of a group.
+//   FP32 accumulation in TMEM: conv1 in columns [0, 32 MT), conv2 in the next
+//   range of 32 MT (or two, by turns), MT the M-tiles of a group.
 // An MMA of M = 128, N = 32, K = 16 takes 42 cycles whatever its row offset,
 // if it is issued as fast: the taps are unrolled, so that issuing one is a
 // few additions to a descriptor (with the taps in a loop it took 58).
@@ -41,14 +41,25 @@
 // FP64 formula as arbiter: the same cell as the labels and the start rule);
 // its offset from the cell centre is taken in FP32.
 //
-// Warps. Warps 0-7 compute the inputs, run both epilogues and the pooling
-// (warp w reads TMEM lanes 32 (w % 4) .. and 16 of the 32 channels); warp 8
-// issues the MMAs. A CTA
-// takes groups blockIdx.x, blockIdx.x + gridDim.x, ...; the inputs of
-// group k + 1 are computed while group k's conv2 runs, and its conv1
-// runs while group k's conv2 epilogue and pooling run. Every wait is
-// bounded; one that gives up raises the CTA's abort flag and the device
+// Pipeline. Warps 0-7 compute the inputs and run conv1's epilogue, warps 8-15
+// in 3-D (the same warps in 2-D) conv2's epilogue and the pooling: warp w reads
+// TMEM lanes 32 (w % 4) .. and 16 of the 32 channels. One more warp issues the
+// MMAs. A CTA takes groups blockIdx.x, blockIdx.x + gridDim.x, ... In 3-D
+// inputs, activations and conv2's accumulators have two buffers (NB), and conv1
+// of group k + 1 is issued before conv2 of group k: while conv2(k) holds the
+// tensor pipe, conv1(k + 1)'s epilogue, the inputs of k + 3 and conv2(k - 1)'s
+// epilogue run. In 2-D, where a group's inputs and epilogues take about as long
+// as its products, two CTAs per SM with one buffer each overlap better. Every
+// wait is bounded; one that gives up raises the CTA's abort flag and the device
 // error flag.
+//
+// Bound by the tensor pipe's rate at N = 32 in 3-D (272 MMAs of 42 cycles a
+// particle: 648 us per chunk of 16384 at 152 SMs and 1.9 GHz), by the epilogues
+// and inputs in 2-D (92 MMAs a group of five: 88 us per chunk of 32768).
+// Measured: 662 us and 127 us. One set of warps for both epilogues and one
+// buffer: 807 us in 3-D; two buffers and one CTA per SM: 158 us in 2-D, two
+// sets and two CTAs 131 us. Padded by W + 2, one particle a group, with taps in a
+// loop: 1045 us and 182 us.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -60,13 +71,16 @@
 namespace cs {
 namespace {
 
-constexpr int kEpiC = 8;                    // epilogue warps 0..7
-constexpr int kMmaC = kEpiC;                // the MMA-issuing warp
-constexpr int kThreadsC = (kEpiC + 1) * 32;
+constexpr int kEpiC = 8;                    // warps of an epilogue set
 
 template <int D, int NP_>
 struct ClsGeo {
     static constexpr int NP = NP_;                                   // particles of a group
+    static constexpr int NB = D == 3 ? 2 : 1;                        // buffers
+    static constexpr int Sets = D == 3 ? 2 : 1;                      // epilogue sets
+    static constexpr int PerSm = D == 3 ? 1 : NP_ > 1 ? 2 : 3;       // CTAs per SM
+    static constexpr int MmaWarp = Sets * kEpiC;                     // issues the MMAs
+    static constexpr int Threads = (MmaWarp + 1) * 32;
     static_assert(D == 2 || NP == 1, "groups of particles in 2-D only");
     static constexpr int W = D == 2 ? 9 : 7;
     static constexpr int E = W + 1;                                  // pitch
@@ -85,7 +99,8 @@ struct ClsGeo {
     static constexpr int Ws = 2 * Wp;                                // edge that is pooled
     static constexpr int Ps = D == 2 ? Ws * Ws : Ws * Ws * Ws;
     static constexpr int Ld = 33;                                    // stage row stride (floats)
-    static constexpr uint32_t Cols = 64 * MT <= 64 ? 64 : 64 * MT <= 128 ? 128 : 64 * MT <= 256 ? 256 : 512;
+    static constexpr int NeedCols = 32 * MT * (1 + NB);
+    static constexpr uint32_t Cols = NeedCols <= 64 ? 64 : NeedCols <= 128 ? 128 : NeedCols <= 256 ? 256 : 512;
     // packed weights
     static constexpr int kW1 = 0;                                    // bf16 [Pairs][2][32][8]
     static constexpr int kB1 = kW1 + Pairs * 1024;                   // f32 [32]
@@ -94,20 +109,20 @@ struct ClsGeo {
     static constexpr int kPacked = kB2 + 128;
     // shared memory
     static constexpr int kSmIn = 0;
-    static constexpr int kSmAct = kSmIn + Rows * 16;
-    static constexpr int kSmW = kSmAct + 4 * Rows * 16;
+    static constexpr int kSmAct = kSmIn + NB * Rows * 16;
+    static constexpr int kSmW = kSmAct + NB * 4 * Rows * 16;
     static constexpr int kSmStage = kSmW + kPacked;
-    static constexpr int kSmBar = (kSmStage + NP * Ps * Ld * 4 + 7) / 8 * 8;   // mbarriers [3]
-    static constexpr int kSmCnt = kSmBar + 3 * 8;                    // u32 in_ready, act_ready
+    static constexpr int kSmBar = (kSmStage + NP * Ps * Ld * 4 + 7) / 8 * 8;   // mbarriers [4]
+    static constexpr int kSmCnt = kSmBar + 4 * 8;                    // u32 in_ready, act_ready, out_free
     // per particle: int c0[3], float off[3], x hi/lo [6]
-    static constexpr int kSmPart = kSmCnt + 8;
+    static constexpr int kSmPart = kSmCnt + 16;
     static constexpr int kSmSlot = kSmPart + NP * 12 * 4;            // TMEM address, abort flag
     static constexpr int kSmTotal = kSmSlot + 16;
 
-    static_assert(64 * MT <= int(Cols), "TMEM columns");
+    static_assert(NeedCols <= int(Cols) && int(Cols) * PerSm <= 512, "TMEM columns");
     static_assert(128 * MT + S < Rows, "operand reads in bounds (the zero tap included)");
     static_assert(Ro - 1 + Coff < Rows, "outputs land in the window");
-    static_assert(kSmTotal <= 232448, "shared memory of one CTA");
+    static_assert(kSmTotal <= (PerSm == 1 ? 232448 : PerSm == 2 ? 113 * 1024 : 75 * 1024), "shared memory of one CTA");
     static_assert(kSmW % 128 == 0 && kSmAct % 128 == 0, "operand alignment");
 };
 
@@ -117,19 +132,19 @@ __device__ __forceinline__ constexpr int cls_shift(int t) {
     return D == 2 ? (t / 3) * E + t % 3 : ((t / 9) * E + (t / 3) % 3) * E + t % 3;
 }
 
-// named barrier 1 over the epilogue warps
-__device__ __forceinline__ void epi_sync() {
-    asm volatile("bar.sync 1, %0;" ::"n"(kEpiC * 32) : "memory");
+// named barrier `id` (1, 2) over a set of epilogue warps
+__device__ __forceinline__ void epi_sync(int id) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kEpiC * 32) : "memory");
 }
-__device__ __forceinline__ bool epi_or(bool flag) {
+__device__ __forceinline__ bool epi_or(int id, bool flag) {
     uint32_t r;
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.u32 q, %1, 0;\n\t"
-        "bar.red.or.pred p, 1, %2, q;\n\t"
+        "bar.red.or.pred p, %3, %2, q;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}\n"
         : "=r"(r)
-        : "r"(uint32_t(flag)), "n"(kEpiC * 32)
+        : "r"(uint32_t(flag)), "n"(kEpiC * 32), "r"(id)
         : "memory");
     return r != 0;
 }
@@ -182,7 +197,7 @@ __device__ __forceinline__ void cls_inputs(const DevMesh &m, const float *__rest
         sp[6 + k] = h;
         sp[9 + k] = l;
     }
-    epi_sync();
+    epi_sync(1);
     for (int i = tid; i < nb * G::P; i += kEpiC * 32) {
         const int w = i / G::P, e = i % G::P;
         const float *sp = part + 12 * w;
@@ -232,7 +247,7 @@ __device__ __forceinline__ void cls_inputs(const DevMesh &m, const float *__rest
 }
 
 template <int D, int NP>
-__global__ void __launch_bounds__(kThreadsC, D == 3 ? 1 : NP == 1 ? 3 : 2) cls_conv_tc_kernel(
+__global__ void __launch_bounds__(ClsGeo<D, NP>::Threads, ClsGeo<D, NP>::PerSm) cls_conv_tc_kernel(
     const DevMesh m, const float *__restrict__ pool_f, int64_t B, const double *__restrict__ xp,
     const uint8_t *__restrict__ packed, const FcMat cat, float *__restrict__ off_out, int *err) {
     using G = ClsGeo<D, NP>;
@@ -241,21 +256,25 @@ __global__ void __launch_bounds__(kThreadsC, D == 3 ? 1 : NP == 1 ? 3 : 2) cls_c
     uint8_t *act = smem + G::kSmAct;
     uint8_t *wsm = smem + G::kSmW;
     float *stage = reinterpret_cast<float *>(smem + G::kSmStage);
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + G::kSmBar);   // conv1, conv2, final
+    // conv1; conv2, one per buffer; final
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + G::kSmBar);
+    // groups whose inputs are in place; whose conv1 epilogue is done; whose conv2
+    // accumulators are read
     uint32_t *in_ready = reinterpret_cast<uint32_t *>(smem + G::kSmCnt);
-    uint32_t *act_ready = in_ready + 1;
+    uint32_t *act_ready = in_ready + 1, *out_free = in_ready + 2;
     float *part = reinterpret_cast<float *>(smem + G::kSmPart);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + G::kSmSlot);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + G::kSmSlot + 4);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     // operands zero (ring, padding channels, rows past the window), barriers, TMEM
-    for (int i = tid; i < G::kSmW / 16; i += kThreadsC)
+    for (int i = tid; i < G::kSmW / 16; i += G::Threads)
         reinterpret_cast<uint4 *>(smem)[i] = make_uint4(0, 0, 0, 0);
     if (tid == 0) {
-        for (int i = 0; i < 3; ++i) mbar_init(bars + i, 1u);
+        for (int i = 0; i < 4; ++i) mbar_init(bars + i, 1u);
         *in_ready = 0;
         *act_ready = 0;
+        *out_free = 0;
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -265,7 +284,7 @@ __global__ void __launch_bounds__(kThreadsC, D == 3 ? 1 : NP == 1 ? 3 : 2) cls_c
                      "r"(G::Cols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    for (int i = tid; i < G::kPacked / 16; i += kThreadsC) cp_async16(wsm + 16 * i, packed + 16 * i);
+    for (int i = tid; i < G::kPacked / 16; i += G::Threads) cp_async16(wsm + 16 * i, packed + 16 * i);
     cp_async_wait_all();
     fence_async_smem();
     fence_before();
@@ -273,117 +292,135 @@ __global__ void __launch_bounds__(kThreadsC, D == 3 ? 1 : NP == 1 ? 3 : 2) cls_c
     fence_after();
     const uint32_t tmem = *tmem_slot;
     const int64_t groups = (B + NP - 1) / NP;
-    const int64_t n_mine = groups > blockIdx.x ? (groups - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+    const int n_mine = groups > blockIdx.x ? int((groups - 1 - blockIdx.x) / gridDim.x + 1) : 0;
+    const int wq = warp & 3, c0 = 16 * ((warp & 7) >> 2);     // lane quarter, first channel
+    const uint32_t tq = tmem + (uint32_t(32 * wq) << 16) + uint32_t(c0);
 
-    if (warp == kMmaC) {
+    if (warp == G::MmaWarp) {
         const bool leader = elect_one();
-        const uint64_t d_in = sdesc(smem_addr(in), 16, 128);
-        const uint64_t d_act = sdesc(smem_addr(act), G::Rows * 16, 128);
         const uint64_t d_w1 = sdesc(smem_addr(wsm + G::kW1), 32 * 16, 128);
         const uint64_t d_w2 = sdesc(smem_addr(wsm + G::kW2), 32 * 16, 128);
         constexpr uint32_t id32 = idesc_bf16(128, 32);
-        for (int64_t k = 0; k < n_mine; ++k) {
-            // conv1 of group k, once its inputs are in place
-            if (!wait_count(in_ready, uint32_t(k + 1), abort_flag, err)) break;
-            fence_after();
-            if (leader) {
-                #pragma unroll 1
-                for (int mt = 0; mt < G::MT; ++mt) {
-                    const uint32_t dcol = tmem + uint32_t(32 * mt);
-                    const int r0 = 128 * mt;
-                    #pragma unroll
-                    for (int i = 0; i < G::Pairs; ++i) {
-                        // the last step's first tap has zero weights: it reads the
-                        // tap before, rows of the same particle
-                        const int t0 = min(2 * i, G::Taps - 2), t1 = t0 + 1;
-                        const int sh0 = cls_shift<D>(t0), sh1 = cls_shift<D>(t1);
-                        const uint64_t a = (d_in & ~(uint64_t(0x3fff) << 16)) + uint64_t(r0 + sh0) +
-                                           (uint64_t(sh1 - sh0) << 16);
-                        mma_bf16(dcol, a, d_w1 + uint64_t(i * 64), id32, i > 0 ? 1u : 0u);
-                    }
+        auto conv1 = [&](int k) {
+            const uint64_t d_in = sdesc(smem_addr(in + (k % G::NB) * G::Rows * 16), 0, 128);
+            #pragma unroll 1
+            for (int mt = 0; mt < G::MT; ++mt) {
+                const uint32_t dcol = tmem + uint32_t(32 * mt);
+                #pragma unroll
+                for (int i = 0; i < G::Pairs; ++i) {
+                    // the last step's first tap has zero weights: it reads the
+                    // tap before, rows of the same particle
+                    const int t0 = min(2 * i, G::Taps - 2), t1 = t0 + 1;
+                    const int sh0 = cls_shift<D>(t0), sh1 = cls_shift<D>(t1);
+                    const uint64_t a = d_in + uint64_t(128 * mt + sh0) + (uint64_t(sh1 - sh0) << 16);
+                    mma_bf16(dcol, a, d_w1 + uint64_t(i * 64), id32, i > 0 ? 1u : 0u);
                 }
-                mma_commit(bars + 0);
             }
-            __syncwarp();
-            // conv2 of group k, once conv1's activations are in place
-            if (!wait_count(act_ready, uint32_t(k + 1), abort_flag, err)) break;
-            fence_after();
-            if (leader) {
+            mma_commit(bars + 0);
+        };
+        auto conv2 = [&](int k) {
+            const uint64_t d_act = sdesc(smem_addr(act + (k % G::NB) * 4 * G::Rows * 16), G::Rows * 16, 128);
+            #pragma unroll 1
+            for (int mt = 0; mt < G::MT; ++mt) {
+                const uint32_t dcol = tmem + uint32_t(32 * (G::MT * (1 + k % G::NB) + mt));
+                // nine taps unrolled, a plane (3-D) at a time: more of them hold
+                // their offsets in more registers than there are
                 #pragma unroll 1
-                for (int mt = 0; mt < G::MT; ++mt) {
-                    const uint32_t dcol = tmem + uint32_t(32 * (G::MT + mt));
-                    const int r0 = 128 * mt;
+                for (int tz = 0; tz < G::Taps / 9; ++tz) {
+                    const uint64_t az = d_act + uint64_t(128 * mt + tz * G::E * G::E);
+                    const uint64_t wz = d_w2 + uint64_t(tz * 9 * 4 * 32);
                     #pragma unroll
-                    for (int t = 0; t < G::Taps; ++t) {
-                        const int sh = cls_shift<D>(t);
+                    for (int t = 0; t < 9; ++t)
                         #pragma unroll
-                        for (int kk = 0; kk < 2; ++kk) {
-                            const uint64_t a = d_act + uint64_t(2 * kk * G::Rows + r0 + sh);
-                            const uint64_t bw = d_w2 + uint64_t((t * 4 + 2 * kk) * 32);
-                            mma_bf16(dcol, a, bw, id32, (t | kk) != 0 ? 1u : 0u);
-                        }
-                    }
+                        for (int kk = 0; kk < 2; ++kk)
+                            mma_bf16(dcol, az + uint64_t(2 * kk * G::Rows + (t / 3) * G::E + t % 3),
+                                     wz + uint64_t((t * 4 + 2 * kk) * 32), id32,
+                                     (tz | t | kk) != 0 ? 1u : 0u);
                 }
-                mma_commit(bars + 1);
+            }
+            mma_commit(bars + 1 + k % G::NB);
+        };
+        bool ok = n_mine == 0 || wait_count(in_ready, 1u, abort_flag, err);
+        fence_after();
+        if (ok && n_mine > 0 && leader) conv1(0);
+        __syncwarp();
+        for (int k = 0; k < n_mine && ok; ++k) {
+            // conv1's accumulators are read and its activations written; the
+            // accumulators that conv2 takes are read
+            ok = wait_count(act_ready, uint32_t(k + 1), abort_flag, err);
+            if (G::Sets == 2 && ok && k >= G::NB) ok = wait_count(out_free, uint32_t(k - G::NB + 1), abort_flag, err);
+            if (ok && G::NB == 2 && k + 1 < n_mine)
+                ok = wait_count(in_ready, uint32_t(k + 2), abort_flag, err);
+            if (!ok) break;
+            fence_after();
+            if (leader) {
+                if (G::NB == 2 && k + 1 < n_mine) conv1(k + 1);
+                conv2(k);
             }
             __syncwarp();
+            if (G::NB == 1 && k + 1 < n_mine) {
+                ok = wait_count(in_ready, uint32_t(k + 2), abort_flag, err);
+                if (!ok) break;
+                fence_after();
+                if (leader) conv1(k + 1);
+                __syncwarp();
+            }
         }
     } else {
         const float *b1 = reinterpret_cast<const float *>(wsm + G::kB1);
         const float *b2 = reinterpret_cast<const float *>(wsm + G::kB2);
-        const int c0 = 16 * (warp >> 2);                 // this warp's channels
-        const uint32_t tq = tmem + (uint32_t(32 * (warp & 3)) << 16) + uint32_t(c0);
-        bool ok = true;
-        if (n_mine > 0) {
-            const int64_t b0 = int64_t(blockIdx.x) * NP;
-            cls_inputs<D, NP>(m, pool_f, xp, b0, int(min(int64_t(NP), B - b0)), in, part, off_out, tid);
+        auto inputs = [&](int k) {
+            const int64_t b0 = (blockIdx.x + int64_t(k) * gridDim.x) * NP;
+            cls_inputs<D, NP>(m, pool_f, xp, b0, int(min(int64_t(NP), B - b0)),
+                              in + (k % G::NB) * G::Rows * 16, part, off_out, tid);
             fence_async_smem();
-            epi_sync();
+            epi_sync(1);
             if (tid == 0) red_release_add(in_ready, 1u);
-        }
-        for (int64_t k = 0; k < n_mine && ok; ++k) {
-            const int64_t b0 = (blockIdx.x + k * gridDim.x) * NP;
-            const int nb = int(min(int64_t(NP), B - b0));
-            const uint32_t par = uint32_t(k & 1);
-            // ---- conv1 epilogue: ReLU(z + b1) in BF16 at each valid row's window position ----
-            ok = __all_sync(kFull, mbar_wait(bars + 0, par, abort_flag, err)) != 0;
-            if (epi_or(!ok)) break;
+        };
+        auto epilogue1 = [&](int k) {
+            // ---- conv1 epilogue: ReLU(z + b1) in BF16 at each valid row's window
+            //      position, once conv2(k - NB) has read that buffer ----
+            bool ok = __all_sync(kFull, mbar_wait(bars + 0, uint32_t(k & 1), abort_flag, err)) != 0;
+            if (ok && k >= G::NB)
+                ok = __all_sync(kFull, mbar_wait(bars + 1 + k % G::NB, uint32_t(k / G::NB - 1) & 1u,
+                                                 abort_flag, err)) != 0;
+            if (epi_or(1, !ok)) return false;
             fence_after();
+            uint8_t *ak = act + (k % G::NB) * 4 * G::Rows * 16 + (size_t(c0 >> 3) * G::Rows + G::Coff) * 16;
             for (int mt = 0; mt < G::MT; ++mt) {
                 float v[16];
                 tmem_ld16(tq + uint32_t(32 * mt), v);
                 uint32_t hv[8];
                 bias_relu_bf16_16(v, b1 + c0, hv);
-                const int r = 128 * mt + 32 * (warp & 3) + lane;
+                const int r = 128 * mt + 32 * wq + lane;
                 const int rr = r % G::Pitch;
                 const int x = rr % G::E, y = (rr / G::E) % G::E, z = D == 3 ? rr / (G::E * G::E) : 0;
                 if (r < G::Ro && x < G::W && y < G::W && z < G::W) {
-                    uint8_t *o = act + (size_t(c0 >> 3) * G::Rows + r + G::Coff) * 16;
+                    uint8_t *o = ak + r * 16;
                     *reinterpret_cast<uint4 *>(o) = make_uint4(hv[0], hv[1], hv[2], hv[3]);
                     *reinterpret_cast<uint4 *>(o + G::Rows * 16) = make_uint4(hv[4], hv[5], hv[6], hv[7]);
                 }
             }
             fence_before();
             fence_async_smem();
-            epi_sync();
+            epi_sync(1);
             if (tid == 0) red_release_add(act_ready, 1u);
-            // ---- inputs of the next group (this one's conv1 has read `in`) ----
-            if (k + 1 < n_mine) {
-                const int64_t b1n = b0 + int64_t(gridDim.x) * NP;
-                cls_inputs<D, NP>(m, pool_f, xp, b1n, int(min(int64_t(NP), B - b1n)), in, part, off_out,
-                                  tid);
-                fence_async_smem();
-                epi_sync();
-                if (tid == 0) red_release_add(in_ready, 1u);
-            }
+            return true;
+        };
+        constexpr int kBar2 = G::Sets;
+        const int t2 = tid - (G::Sets - 1) * kEpiC * 32;
+        auto epilogue2 = [&](int k) {
+            const int64_t b0 = (blockIdx.x + int64_t(k) * gridDim.x) * NP;
+            const int nb = int(min(int64_t(NP), B - b0));
             // ---- conv2 epilogue: ReLU(z + b2) in FP32 to the stage, then pooling ----
-            ok = __all_sync(kFull, mbar_wait(bars + 1, par, abort_flag, err)) != 0;
-            if (epi_or(!ok)) break;
+            const bool ok = __all_sync(kFull, mbar_wait(bars + 1 + k % G::NB, uint32_t(k / G::NB) & 1u,
+                                                        abort_flag, err)) != 0;
+            if (epi_or(kBar2, !ok)) return false;
             fence_after();
             for (int mt = 0; mt < G::MT; ++mt) {
                 float v[16];
-                tmem_ld16(tq + uint32_t(32 * (G::MT + mt)), v);
-                const int r = 128 * mt + 32 * (warp & 3) + lane, w = r / G::Pitch, rr = r % G::Pitch;
+                tmem_ld16(tq + uint32_t(32 * (G::MT * (1 + k % G::NB) + mt)), v);
+                const int r = 128 * mt + 32 * wq + lane, w = r / G::Pitch, rr = r % G::Pitch;
                 const int x = rr % G::E, y = (rr / G::E) % G::E, z = D == 3 ? rr / (G::E * G::E) : 0;
                 if (r < G::Ro && x < G::Ws && y < G::Ws && z < G::Ws) {
                     float *st = stage + (w * G::Ps + (z * G::Ws + y) * G::Ws + x) * G::Ld + c0;
@@ -398,11 +435,12 @@ __global__ void __launch_bounds__(kThreadsC, D == 3 ? 1 : NP == 1 ? 3 : 2) cls_c
                 }
             }
             fence_before();
-            epi_sync();
+            epi_sync(kBar2);
+            if (G::Sets == 2 && t2 == 0) red_release_add(out_free, 1u);
             // BF16 into the tiled feature matrix (fc_tc.h): column c Pp + pp of
             // the particle's row. 2-D: four neighbouring columns per thread
             constexpr int kPer = G::Pp % 4 == 0 ? 4 : 1, kUnits = 32 * G::Pp / kPer;
-            for (int i = tid; i < nb * kUnits; i += kEpiC * 32) {
+            for (int i = t2; i < nb * kUnits; i += kEpiC * 32) {
                 const int w = i / kUnits, u0 = i % kUnits, c = u0 % 32, p0 = u0 / 32 * kPer;
                 const float *st = stage + w * G::Ps * G::Ld + c;
                 float s[kPer];
@@ -430,14 +468,25 @@ __global__ void __launch_bounds__(kThreadsC, D == 3 ? 1 : NP == 1 ? 3 : 2) cls_c
                 else
                     *reinterpret_cast<__nv_bfloat16 *>(o) = __float2bfloat16_rn(s[0]);
             }
-            epi_sync();
+            epi_sync(kBar2);      // the stage is free
+            return true;
+        };
+        if (warp < kEpiC) {
+            for (int k = 0; k < G::NB && k < n_mine; ++k) inputs(k);
+            for (int k = 0; k < n_mine && epilogue1(k); ++k) {
+                // conv1(k) has read its inputs' buffer
+                if (k + G::NB < n_mine) inputs(k + G::NB);
+                if (G::Sets == 1 && !epilogue2(k)) break;
+            }
+        } else {
+            for (int k = 0; k < n_mine && epilogue2(k); ++k) {}
         }
     }
     // wait (bounded) for this CTA's MMAs in flight before TMEM is released
-    if (warp == kMmaC) {
+    if (warp == G::MmaWarp) {
         if (elect_one()) {
-            mma_commit(bars + 2);
-            for (uint32_t i = 0; i < (1u << 24) && !mbar_try_wait(bars + 2, 0); ++i)
+            mma_commit(bars + 3);
+            for (uint32_t i = 0; i < (1u << 24) && !mbar_try_wait(bars + 3, 0); ++i)
                 if (i > 64) __nanosleep(64);
         }
         __syncwarp();
@@ -487,9 +536,8 @@ void launch_conv(const DevMesh &m, const float *pool_f, int64_t B, const double 
                              G::kSmTotal);
         attr = true;
     }
-    const int per_sm = D == 3 ? 1 : NP == 1 ? 3 : 2;
-    const int grid = int(std::min<int64_t>((B + NP - 1) / NP, int64_t(sm_count) * per_sm));
-    cls_conv_tc_kernel<D, NP><<<grid, kThreadsC, G::kSmTotal, st>>>(m, pool_f, B, xp, packed, cat,
+    const int grid = int(std::min<int64_t>((B + NP - 1) / NP, int64_t(sm_count) * G::PerSm));
+    cls_conv_tc_kernel<D, NP><<<grid, G::Threads, G::kSmTotal, st>>>(m, pool_f, B, xp, packed, cat,
                                                                     off, err);
 }
 
@@ -509,9 +557,10 @@ void launch_cls_conv_tc(const DevMesh &m, const float *pool_f, int64_t B, const 
                         const uint8_t *packed, const FcMat &cat, float *off, int *err,
                         int sm_count, cudaStream_t st) {
     if (B <= 0) return;
-    // groups of five once they fill two CTAs per SM a few times over; a particle
-    // per CTA pass spreads fewer particles over more CTAs
-    if (m.dim == 2 && B >= int64_t(20) * sm_count)
+    // groups of five once every CTA gets more than one; a particle per CTA pass
+    // spreads fewer particles over more CTAs (a forward pass of 2279 particles by
+    // ones 83.0 us, of 2281 by fives 79.4 us)
+    if (m.dim == 2 && B >= int64_t(15) * sm_count)
         launch_conv<2, 5>(m, pool_f, B, xp, packed, cat, off, err, sm_count, st);
     else if (m.dim == 2)
         launch_conv<2, 1>(m, pool_f, B, xp, packed, cat, off, err, sm_count, st);
