@@ -549,9 +549,9 @@ int train_tiled(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t B, const d
         const int ca2 = conv_bwd_ctas(c2, B, false, sm), ca1 = conv_bwd_ctas(c1, B, true, sm);
         float *w2 = sum(int64_t(kClsCh) * c2.K, ca2, g + S.w_off[1]);
         float *bb1 = sum(kClsCh, ca2, g + S.b_off[0]);
-        n += 1 + launch_conv_bwd(c2, C.ty1, false, B, C.tdz2, b2, w2, C.tdz1, 1, bb1, err, sm, st);
+        n += 1 + launch_conv_bwd(c2, C.ty1, false, B, C.tdz2, b2, w2, C.tdz1, bb1, err, sm, st);
         float *w1 = sum(int64_t(kClsCh) * c1.K, ca1, g + S.w_off[0]);
-        n += launch_conv_bwd(c1, C.ta0, true, B, C.tdz1, nullptr, w1, nullptr, 0, nullptr, err, sm, st);
+        n += launch_conv_bwd(c1, C.ta0, true, B, C.tdz1, nullptr, w1, nullptr, nullptr, err, sm, st);
     } else {
         n += backward_conv(ctx, C, B, C.tgpool, S.n_pool, st);
     }

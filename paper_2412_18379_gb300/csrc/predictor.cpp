@@ -365,8 +365,8 @@ int train_fused(cs_ctx *ctx, Predictor &P, int64_t B, const float *win, const fl
         float *wpart = part, *bpart = part + int64_t(ctas) * g.K * S.ch;
         part = bpart + int64_t(ctas) * S.ch;
         n += launch_conv_bwd(g, l == 0 ? static_cast<const void *>(win) : P.fy[l - 1], l == 0, B,
-                             P.fdz[l], P.fpack + K.bwd[l], wpart, l > 0 ? P.fdz[l - 1] : nullptr, 0,
-                             bpart, ctx->dev_err, sm, st);
+                             P.fdz[l], P.fpack + K.bwd[l], wpart, l > 0 ? P.fdz[l - 1] : nullptr, bpart,
+                             ctx->dev_err, sm, st);
         add(wpart, int64_t(g.K) * S.ch, int64_t(g.K) * S.ch, P.g + S.w_off[l], ctas, 0.f);
         if (l > 0) add(bpart, S.ch, S.ch, P.g + S.b_off[l - 1], ctas, 0.f);
     }

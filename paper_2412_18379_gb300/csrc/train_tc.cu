@@ -9,24 +9,25 @@
 // activations in shared memory and lays the im2col operand A[row][k] out
 // there, k = channel * taps + tap as the weights are stored. The operand
 // layout [k / 8][row][k % 8] is K-major for the forward product (K = k) and,
-// read with the transposed (MN-major) descriptor, the left operand of the
-// weight gradient (K = row), so the backward pass builds it once for both.
+// read with the transposed (MN-major) descriptor, the left operand of the first
+// layer's weight gradient (K = row). The other layers' backward pass needs no
+// im2col operand (conv_bwd_kernel below).
 //
 //   forward   z[row][o]  = sum_k A[row][k] W[o][k]        M = rows, N = 32
-//   weights   dW[k][o]   = sum_rows A[row][k] dz[row][o]  M = k,    N = 32
-//   columns   dcol[row][k] = sum_o dz[row][o] W[o][k]     M = rows, N = taps * channels
-//   col2im    dx[q][c]   = sum_t dcol[row(q, t)][c taps + t], in shared memory
+//   first     dW[k][o]   = sum_rows A[row][k] dz[row][o]  M = k,    N = 32
 //
-// The sums over k and o run in the K order and K = 16 steps of the general
-// GEMM (tc_gemm.cu), and dx adds its taps in increasing order, so activations
-// and input gradients are that path's bits. Weight gradients accumulate over
-// a CTA's tiles in TMEM; the CTAs' partials are summed in a fixed order.
+// The sums over k run in the K order and K = 16 steps of the general GEMM
+// (tc_gemm.cu), those of the input gradient over the output channels and then
+// the taps, in increasing order, so activations and input gradients are that
+// path's bits. Weight gradients accumulate over a CTA's tiles in TMEM; the CTAs'
+// partials are summed in a fixed order.
 //
-// What bounds it: not the tensor pipe but the operand build (8 two-byte
-// shared loads and one 16-byte store per 8 elements) and the col2im gather;
-// global traffic is the BF16 activations and gradients alone. At a batch of
-// 4096 the 2-D step's im2col, GEMM, col2im and ReLU kernels moved about
-// 1.2 GB through FP32 buffers.
+// What bounds the forward pass is not the tensor pipe but the operand build (a
+// 16-byte shared load per tap and 8 channels, transposed in registers); global
+// traffic is the BF16 activations and gradients alone. At a batch of 4096 the
+// 2-D step's im2col, GEMM, col2im and ReLU kernels moved about 1.2 GB through
+// FP32 buffers: a gradient call took 1102 us there and 1594 us for 2048 rows in
+// 3-D, now 143 us and 212 us.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -40,7 +41,7 @@ namespace {
 
 constexpr int kPitch = 40;        // halves per position in shared memory (5 x 16 bytes: no conflicts)
 constexpr int kFwdThreads = 256;
-constexpr int kBwdThreads = 512;
+constexpr int kWgThreads = 512;
 constexpr int kRowsT = 128;       // MMA rows
 constexpr int kChunk = kRowsT * 16;   // bytes of one 8-element K chunk of A
 
@@ -58,7 +59,7 @@ struct ConvArgs {
     const uint16_t *dz;
     float *wpart, *bpart;
     uint16_t *dzp;
-    int ring;                     // forward: of y; backward: of x
+    int ring;                     // of y
 };
 
 // one layer's geometry: inputs of edge Si, channels first FP32 (First: the
@@ -77,10 +78,9 @@ struct Geo {
     static constexpr int ActHalves = FIRST ? C * Pi : Pi * kPitch;   // per input
 };
 
-// shared memory of one CTA (bytes); A first, then the activations (act2: the
-// second buffer of a backward pass, the first one where it does not fit)
+// shared memory of one CTA (bytes); the operand first
 struct ConvSmem {
-    int act, act2, w, dz, tab, bar, total;
+    int act, w, dz, tab, bar, total;
 };
 
 template <class N, bool BWD>
@@ -95,57 +95,35 @@ struct ConvCfg {
     static constexpr int Gb = N::First ? 1 : D == 2 ? 4 : 2;   // groups per build
     static constexpr int Cb = Gb * GroupChunks;
     static constexpr int Builds = Groups / Gb;
-    // backward: channels, columns and MMA N of one dcol pass
-    static constexpr int Ch = D == 2 ? 16 : 8;
-    static constexpr int Nc = Ch * N::Taps;                  // 144, 216
-    static constexpr int Nm = (Nc + 15) / 16 * 16;           // 144, 224
-    static constexpr int Ld = Nc + 1;                        // dcol row stride (odd: no conflicts)
-    static constexpr int Passes = kTrainCh / Ch;
-    static constexpr bool Dgrad = BWD && !N::First;
-    static constexpr int Kw = D == 2 ? 288 : 872;            // rows of the dgrad weights
-    static constexpr int Dcol = Dgrad ? kRowsT * Ld * 4 : 0;
-    static constexpr int A = Cb * kChunk > Dcol ? Cb * kChunk : Dcol;
-    static constexpr int MtB = (Cb + 15) / 16;               // weight-gradient M-tiles per build
-    static constexpr int Mt = MtB * Builds;
-    static constexpr uint32_t ColD = 32 * Mt;                // TMEM column of dcol
-    static constexpr uint32_t Cols = !Dgrad ? 128 : ColD + Nm <= 256 ? 256 : 512;
-    static constexpr int WBytes = !BWD ? N::Kp * kTrainCh * 2 : Dgrad ? Kw * kTrainCh * 2 : 0;
+    static constexpr int Mt = (Cb + 15) / 16;                // weight-gradient M-tiles (first layer)
+    static constexpr uint32_t Cols = 128;
+    static constexpr int WBytes = !BWD ? N::Kp * kTrainCh * 2 : 0;
     // the classifier's layer, one input of 81 rows per tile, leaves room for a
     // second CTA per SM
     static constexpr int PerSm = BWD && N::Si == 11 ? 2 : 1;
-    static_assert((Passes - 1) * Nc + Nm <= Kw, "dgrad weight rows");
-    static_assert(!BWD || ColD + (Dgrad ? Nm : 0) <= Cols, "TMEM columns");
+    static_assert(!BWD || N::First, "weight gradient of the first layer alone");
     static_assert(BWD || Cb % 2 == 0, "whole K = 16 steps per build");
+    static_assert(Builds * Gb == Groups && PerSm * Cols <= 512 && 32 * (BWD ? Mt : 1) <= int(Cols),
+                  "whole builds, TMEM columns");
 };
 
 constexpr int kSmemMax = 232448, kSmemHalf = 113 * 1024;
 
 template <class N, bool BWD>
-constexpr ConvSmem conv_smem_of(int G, int buffers) {
+constexpr ConvSmem conv_smem(int G) {
     using F = ConvCfg<N, BWD>;
     ConvSmem s{};
-    s.act = F::A;
-    const int act = (G * N::ActHalves * 2 + 127) / 128 * 128;
-    s.act2 = s.act + (buffers - 1) * act;
-    s.w = s.act2 + act;
+    s.act = F::Cb * kChunk;
+    s.w = s.act + (G * N::ActHalves * 2 + 127) / 128 * 128;
     s.dz = s.w + F::WBytes;
     s.tab = s.dz + (BWD ? kTrainCh * kRowsT * 2 : 0);
     s.bar = (s.tab + (N::First ? N::Kp * 2 : 0) + 127) / 128 * 128;
     s.total = s.bar + 64;
     // an M-tile of the weight gradient reads 16 chunks from its first one,
     // past the built ones at the end (rows of no use): inside the allocation
-    const int reach = F::MtB * 16 * kChunk;
+    const int reach = F::Mt * 16 * kChunk;
     if (BWD && s.total < reach) s.total = reach;
     return s;
-}
-
-template <class N, bool BWD>
-constexpr ConvSmem conv_smem(int G) {
-    if (BWD && !N::First) {
-        const ConvSmem s = conv_smem_of<N, BWD>(G, 2);
-        if (s.total <= (ConvCfg<N, BWD>::PerSm > 1 ? kSmemHalf : kSmemMax)) return s;
-    }
-    return conv_smem_of<N, BWD>(G, 1);
 }
 
 // The activations of inputs [b0, b0 + nb) on their way to shared memory:
@@ -483,58 +461,30 @@ __global__ void __launch_bounds__(kFwdThreads, 2) conv_fwd_kernel(const ConvArgs
     mma_drain(bars + 2, tmem, kCols, warp);
 }
 
-// dx of one line of Si input positions (fixed window, channel, y and z) from
-// the tile's dcol: for every tap line (ty, tz) whose output line exists, tap
-// by tap in increasing order
-template <class N, int LD>
-__device__ __forceinline__ void col2im_line(const float *dcol, int row0, int iy, int iz,
-                                            float *s) {
-    #pragma unroll
-    for (int i = 0; i < N::Si; ++i) s[i] = 0.f;
-    #pragma unroll
-    for (int tz = 0; tz < (N::Dim == 3 ? 3 : 1); ++tz) {
-        const int z = iz - tz;
-        if (N::Dim == 3 && unsigned(z) >= unsigned(N::So)) continue;
-        #pragma unroll
-        for (int ty = 0; ty < 3; ++ty) {
-            const int y = iy - ty;
-            if (unsigned(y) >= unsigned(N::So)) continue;
-            const float *d = dcol + (row0 + ((N::Dim == 3 ? z * N::So : 0) + y) * N::So) * LD +
-                             (tz * 3 + ty) * 3;
-            #pragma unroll
-            for (int tx = 0; tx < 3; ++tx)
-                #pragma unroll
-                for (int x = 0; x < N::So; ++x) s[x + tx] += d[x * LD + tx];
-        }
-    }
-}
-
+// Weight gradient of the first layer (its input's gradient is not wanted): the
+// im2col operand of a tile is built as in the forward pass and read with the
+// transposed descriptor; the sum over all of a CTA's tiles stays in TMEM.
 template <class N>
-__global__ void __launch_bounds__(kBwdThreads, ConvCfg<N, true>::PerSm) conv_bwd_kernel(const ConvArgs a,
-                                                                  const ConvSmem L, int *err) {
+__global__ void __launch_bounds__(kWgThreads, ConvCfg<N, true>::PerSm) first_wgrad_kernel(
+    const ConvArgs a, const ConvSmem L, int *err) {
     using F = ConvCfg<N, true>;
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t *act = smem + L.act, *next = smem + L.act2, *wop = smem + L.w, *dzs = smem + L.dz;
-    const bool two = L.act2 != L.act;
-    float *dcol = reinterpret_cast<float *>(smem);          // over A once its MMAs are complete
+    uint8_t *act = smem + L.act, *dzs = smem + L.dz;
     uint16_t *tab = reinterpret_cast<uint16_t *>(smem + L.tab);
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L.bar);   // builds, dcol, drain
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L.bar);   // products, -, drain
     uint32_t *slot = reinterpret_cast<uint32_t *>(smem + L.bar + 32);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + L.bar + 40);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    constexpr uint32_t kCols = F::Cols, kDcol = F::ColD;
-    constexpr int kNw = kBwdThreads / 32;
 
     if (tid == 0) {
         for (int i = 0; i < 3; ++i) mbar_init(bars + i, 1u);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) tmem_alloc(slot, kCols);
-    fill_tab<N>(tab, tid, kBwdThreads);
+    if (warp == 0) tmem_alloc(slot, F::Cols);
+    fill_tab<N>(tab, tid, kWgThreads);
     pdl_wait();
-    for (int i = tid; i < F::WBytes / 16; i += kBwdThreads) cp_async16(wop + 16 * i, a.w + 16 * i);
-    ActLoad<N, kBwdThreads> ld;
+    ActLoad<N, kWgThreads> ld;
     int64_t t = blockIdx.x;
     int nb = int(min(int64_t(a.G), a.B - t * a.G));
     // dz of a tile: one 16-byte piece (8 channels of a row) per thread, the
@@ -545,190 +495,485 @@ __global__ void __launch_bounds__(kBwdThreads, ConvCfg<N, true>::PerSm) conv_bwd
         dzr = rr < nb * N::Po ? __ldg(reinterpret_cast<const uint4 *>(a.dz + t * a.G * N::Po * kTrainCh) + i)
                               : make_uint4(0u, 0u, 0u, 0u);
     };
-    static_assert(kRowsT * 4 == kBwdThreads, "one piece of dz per thread");
+    static_assert(kRowsT * 4 == kWgThreads, "one piece of dz per thread");
     ld.start(a, t * a.G, nb, act, tid);
     fetch_dz();
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = *slot;
+    constexpr uint32_t id_w = idesc_mn(idesc_bf16(128, 32), true, true);
+    const uint64_t dz_mn = sdesc(smem_addr(dzs), 128, kChunk);
+    bool ok = true, any = false;
+    uint32_t phase = 0;
+    while (t < a.tiles) {
+        ld.finish(nb, act, tid);
+        *reinterpret_cast<uint4 *>(dzs + (tid & 3) * kChunk + (tid >> 2) * 16) = dzr;
+        const int base = row_base<N>(nb, 32 * (warp & 3) + lane);
+        __syncthreads();
+        const int ksteps = (nb * N::Po + 15) / 16;
+        t += gridDim.x;
+        if (t < a.tiles) {
+            nb = int(min(int64_t(a.G), a.B - t * a.G));
+            fetch_dz();
+        }
+        build_first<N, kWgThreads / 32>(smem, act, tab, base, warp, lane);
+        fence_async_smem();
+        fence_before();
+        __syncthreads();
+        fence_after();
+        if (warp == 0) {
+            if (elect_one()) {
+                #pragma unroll 1
+                for (int mt = 0; mt < F::Mt; ++mt) {
+                    const uint64_t da = sdesc(smem_addr(smem) + mt * 16 * kChunk, 128, kChunk);
+                    #pragma unroll
+                    for (int q = 0; q < kRowsT / 16; ++q)
+                        if (q < ksteps)
+                            mma_bf16(tmem + uint32_t(32 * mt), da + uint64_t(q * 16),
+                                     dz_mn + uint64_t(q * 16), id_w, any || q > 0 ? 1u : 0u);
+                }
+                mma_commit(bars + 0);
+            }
+            __syncwarp();
+        }
+        // the input is not read again: fetch the next tile's
+        if (t < a.tiles) ld.start(a, t * a.G, nb, act, tid);
+        ok = __syncthreads_and(mbar_wait(bars + 0, phase, abort_flag, err));
+        phase ^= 1u;
+        fence_after();
+        if (!ok) break;
+        any = true;
+    }
+    if (ok && any && (warp >> 2) < 2) {
+        // this CTA's weight gradient: rows of D are k, columns the output channel
+        float *wp = a.wpart + int64_t(blockIdx.x) * N::K * kTrainCh;
+        const int o0 = 16 * (warp >> 2);
+        for (int mt = 0; mt < F::Mt; ++mt) {
+            float v[16];
+            tmem_ld16(tmem + (uint32_t(32 * (warp & 3)) << 16) + uint32_t(32 * mt + o0), v);
+            const int k = 128 * mt + 32 * (warp & 3) + lane;
+            if (k < N::K) {
+                #pragma unroll
+                for (int e = 0; e < 16; ++e) wp[(o0 + e) * N::K + k] = v[e];
+            }
+        }
+    }
+    mma_drain(bars + 2, tmem, F::Cols, warp);
+}
+
+// ---------------------------------------------------------------------------
+// Backward pass of the other layers, without an im2col operand. dz is laid out
+// on the flat index of its input's positions, q = (z Si + y) Si + x of every
+// input in turn, with zeros where no output position is: output position p of
+// tap t then meets input position p + shift(t), shift = (dz Si + dy) Si + dx, and
+// a tap is a row offset of an operand in shared memory.
+//
+//   columns  T_t[q][c] = sum_o dz[q - shift(t)][o] W[o][c][t]: M = 128 positions,
+//            N = 32, K = 32, one product per tap into TMEM columns of its own.
+//            dx[q][c] is the sum of the T_t in increasing t, each thread adding
+//            its position's in registers: the same sums in the same order as
+//            with the columns gradient in memory, with no gather (where the tap
+//            leaves the output the product is 0).
+//   weights  dW[(dy, o)][(dx, c)] += sum_q dz[q - Si dy][o] act[q + dx + Si^2 dz][c]:
+//            M = 128 (3 x 32 used), N = 96, K = positions. Both operands are kept
+//            in three copies, shifted by Si dy and by dx, so that the copies
+//            continue the 8-channel chunks at one stride; 3-D adds dz by a row
+//            offset, in TMEM columns of its own.
+//
+// Warps 0-7 add up T and mask it by the ReLU (warp w: positions 32 (w % 4) .. of
+// the M-tile, 16 channels), warps 8-11 load, warp 12 issues the MMAs. Two buffers
+// of operands; the epilogue follows the tensor pipe three taps behind, and a
+// slice of the weights' steps keeps the pipe busy until it has read a unit's last.
+// Every wait is bounded (abort flag and device error flag).
+//
+// The tensor pipe needs 42 cycles for an MMA of N = 32 and 58 for N = 96, per tile
+// of 250 positions 36 and 16 of them in 2-D (2.4k cycles), 54 and 24 per 125 in
+// 3-D (3.7k). The kernel takes about twice that: a unit's products may not start
+// before the unit before is read, and a commit is seen 250 cycles after the
+// products, a part is read and added in 70. Measured: Si = 11 (4096 inputs) 39 us,
+// Si = 7 21, 5 14, 3 9.6; 3-D (2048) Si = 5 55, Si = 3 23. With the im2col operand,
+// dcol in shared memory and a gather from it: 108, 40, 18, 9.3; 72, 17.
+// ---------------------------------------------------------------------------
+constexpr int kBwdEpi = 8, kBwdLoad = 4, kBwdMma = kBwdEpi + kBwdLoad;
+constexpr int kBwdThreads = (kBwdMma + 1) * 32;
+
+template <class N>
+struct BwdCfg {
+    static constexpr int D = N::Dim, Si = N::Si;
+    static constexpr int RowsMax = D == 2 ? 256 : 128;        // positions of a tile
+    static constexpr int GMax = RowsMax / N::Pi;
+    // positions whose gradient leaves: the classifier's second layer has its
+    // input's zero ring stored, which has none
+    static constexpr int Ring = Si == 11 ? 1 : 0;
+    static constexpr int Crop = Si - 2 * Ring;
+    static constexpr int Np = D == 2 ? Crop * Crop : Crop * Crop * Crop;
+    static constexpr int Planes = D == 2 ? 1 : 3;
+    // T is computed a unit of taps at a time (the last one of 3-D shorter), and
+    // UnitSteps steps of the weights' product follow each unit
+    static constexpr int UnitTaps = D == 2 ? 9 : 7, Units = (N::Taps + UnitTaps - 1) / UnitTaps;
+    static constexpr int Parts = (UnitTaps + 2) / 3, UnitSteps = 8 * Planes / Units;
+    static_assert(UnitSteps * Units == 8 * Planes && UnitTaps % 3 <= 1, "whole slices, parts of three or one");
+    static constexpr int Front = D == 2 ? 2 : 2 * Si * Si + 2;     // zero rows before dz
+    // rows of a chunk: 2 mod 8, so that four chunks' stores meet no bank twice
+    static constexpr int RowsA = (RowsMax + (D == 2 ? 0 : 2 * Si * Si) + 5) / 8 * 8 + 2;
+    static constexpr int RowsZ = (Front + 2 * Si + RowsMax + 5) / 8 * 8 + 2;
+    static constexpr int Kw = kTrainCh * N::Taps;             // rows of the weights
+    static constexpr int ActB = 12 * RowsA * 16, DzB = 12 * RowsZ * 16;   // bytes of a buffer
+    static constexpr int kAct = 2 * DzB;
+    static constexpr int kW = kAct + 2 * ActB;
+    static constexpr int kBar = kW + Kw * kTrainCh * 2;       // mbarriers: parts, 2 buffers, drain
+    static constexpr int kCnt = kBar + (Parts + 3) * 8;       // u32 full [2], hdone [2], freed
+    static constexpr uint32_t ColT = 96 * Planes;             // TMEM: weights, then a unit's T
+    static constexpr int kSlot = kCnt + 5 * 4;                // TMEM address, abort flag
+    static constexpr int kRed = (kSlot + 8 + 15) / 16 * 16;   // f32 [8][16]
+    static constexpr int kTotal = kRed + kBwdEpi * 16 * 4;
+    static constexpr int PieceA = (GMax * N::Pi * 4 + kBwdLoad * 32 - 1) / (kBwdLoad * 32);
+    static constexpr int PieceZ = (GMax * N::Po * 4 + kBwdLoad * 32 - 1) / (kBwdLoad * 32);
+    static_assert(ColT + 32 * UnitTaps <= 512, "TMEM columns");
+    static_assert(kTotal <= 232448, "shared memory of one CTA");
+    // the last rows of M (a fourth copy of dz, never stored) are read from what
+    // follows the buffer
+    static_assert(DzB + 16 * RowsZ * 16 <= kTotal, "operand reads inside the allocation");
+    static_assert(kTrainCh * (N::K + 1) * 4 <= kW, "the weight gradient's stage");
+};
+
+// Warp-uniform bounded wait for a phase that is a few hundred cycles away: polls
+// without the suspension of try_wait (104 cycles a poll of a warp, 215 with it).
+__device__ __forceinline__ bool spin_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
+                                          int *err) {
+    const uint32_t addr = smem_addr(bar);
+    for (uint32_t i = 0; i < (1u << 24); ++i) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}\n"
+            : "=r"(ok)
+            : "r"(addr), "r"(parity)
+            : "memory");
+        if (__all_sync(0xffffffffu, ok)) return true;
+        if ((i & 255) == 255 && __any_sync(0xffffffffu, *abort_flag)) return false;
+    }
+    *abort_flag = 1;
+    atomicExch(err, 1);
+    return false;
+}
+
+// bounded wait for a phase that may be far away: sparse polls
+__device__ __forceinline__ bool idle_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
+                                          int *err) {
+    for (uint32_t i = 0; i < (1u << 22); ++i) {
+        const bool ok = (threadIdx.x & 31) != 0 || mbar_try_wait(bar, parity);
+        if (__all_sync(0xffffffffu, ok)) return true;
+        if (__any_sync(0xffffffffu, *abort_flag)) return false;
+        __nanosleep(128);
+    }
+    *abort_flag = 1;
+    atomicExch(err, 1);
+    return false;
+}
+
+// 3 x 16 columns of FP32 from TMEM, 32 columns apart
+__device__ __forceinline__ void tmem_ld16x3(uint32_t taddr, float (&v)[3][16]) {
+    uint32_t r[48];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+        "%11, %12, %13, %14, %15}, [%48];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, "
+        "%26, %27, %28, %29, %30, %31}, [%49];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, "
+        "%42, %43, %44, %45, %46, %47}, [%50];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
+          "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
+          "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
+          "=r"(r[31]), "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]),
+          "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]), "=r"(r[42]),
+          "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47])
+        : "r"(taddr), "r"(taddr + 32u), "r"(taddr + 64u)
+        : "memory");
+    #pragma unroll
+    for (int i = 0; i < 48; ++i) v[i / 16][i % 16] = __uint_as_float(r[i]);
+}
+
+template <class N>
+__global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs a, int *err) {
+    using F = BwdCfg<N>;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    uint8_t *dzs = smem, *acts = smem + F::kAct, *wop = smem + F::kW;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + F::kBar);
+    uint64_t *done = bars + F::Parts, *drain = done + 2;
+    // running counts (a warp is never a use ahead in one): loader warps that have
+    // filled a buffer, epilogue warps that have read its activations, that have
+    // read a unit's T
+    uint32_t *full = reinterpret_cast<uint32_t *>(smem + F::kCnt);
+    uint32_t *hdone = full + 2, *freed = full + 4;
+    uint32_t *slot = reinterpret_cast<uint32_t *>(smem + F::kSlot);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + F::kSlot + 4);
+    float *red = reinterpret_cast<float *>(smem + F::kRed);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+    if (tid == 0) {
+        for (int i = 0; i < F::Parts + 3; ++i) mbar_init(bars + i, 1u);
+        for (int i = 0; i < 5; ++i) full[i] = 0;
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) tmem_alloc(slot, 512);
+    for (int i = tid; i < F::kW / 16; i += kBwdThreads)
+        reinterpret_cast<uint4 *>(smem)[i] = make_uint4(0u, 0u, 0u, 0u);
+    pdl_wait();
+    for (int i = tid; i < F::Kw * kTrainCh * 2 / 16; i += kBwdThreads) cp_async16(wop + 16 * i, a.w + 16 * i);
     cp_async_wait_all();
     fence_async_smem();
     fence_before();
     __syncthreads();
     fence_after();
     const uint32_t tmem = *slot;
-    constexpr uint32_t id_w = idesc_mn(idesc_bf16(128, 32), true, true);
-    constexpr uint32_t id_c = idesc_bf16(128, F::Nm);
-    // dz: K-major (K = channel) for dcol, MN-major (K = row) for the weights
-    const uint64_t dz_k = sdesc(smem_addr(dzs), kChunk, 128);
-    const uint64_t dz_mn = sdesc(smem_addr(dzs), 128, kChunk);
-    const uint64_t w_k = sdesc(smem_addr(wop), F::Kw * 16, 128);
-    float db[F::Passes];
-    #pragma unroll
-    for (int j = 0; j < F::Passes; ++j) db[j] = 0.f;
-    const int crop = N::Si - 2 * a.ring;
-    const int np = N::Dim == 2 ? crop * crop : crop * crop * crop;
-    bool ok = true, any = false;
-    uint32_t phase = 0;          // of the dcol products
-    int it = 0;                  // builds so far
-    while (t < a.tiles) {
-        const int64_t b0 = t * a.G;
-        ld.finish(nb, act, tid);
-        *reinterpret_cast<uint4 *>(dzs + (tid & 3) * kChunk + (tid >> 2) * 16) = dzr;
-        const int base = row_base<N>(nb, 32 * (warp & 3) + lane);
-        fence_before();
-        __syncthreads();
-        fence_after();
-        const int ksteps = (nb * N::Po + 15) / 16, nb_now = nb;
-        t += gridDim.x;
-        if (t < a.tiles) {
-            nb = int(min(int64_t(a.G), a.B - t * a.G));
-            fetch_dz();
-            if (two) ld.start(a, t * a.G, nb, next, tid);
-        }
-        #pragma unroll 1
-        for (int j = 0; j < F::Builds; ++j, ++it) {
-            // the operand's MMAs of the build before (each tile ends with all of
-            // its builds complete)
-            if (j > 0)
-                ok = __syncthreads_and(mbar_wait(bars + 0, uint32_t(it - 1) & 1u, abort_flag, err));
+    const int n_mine = int((a.tiles - 1 - blockIdx.x) / gridDim.x + 1);
+    auto tile_b0 = [&](int k) { return (blockIdx.x + int64_t(k) * gridDim.x) * a.G; };
+    auto tile_nb = [&](int k) { return int(min(int64_t(a.G), a.B - tile_b0(k))); };
+    bool ok = true;
+
+    if (warp == kBwdMma) {
+        constexpr uint32_t id_c = idesc_bf16(128, 32);
+        constexpr uint32_t id_w = idesc_mn(idesc_bf16(128, 96), true, true);
+        const bool leader = elect_one();
+        const uint64_t w_k = sdesc(smem_addr(wop), F::Kw * 16, 128);
+        uint32_t n = 0;                                  // units so far
+        for (int k = 0; k < n_mine && ok; ++k) {
+            ok = wait_count(full + (k & 1), uint32_t(kBwdLoad * (k / 2 + 1)), abort_flag, err);
             if (!ok) break;
-            build_operand<N, true, kNw>(smem, act, tab, base, j, warp, lane);
-            fence_async_smem();
-            fence_before();
-            __syncthreads();
             fence_after();
-            if (warp == 0) {
-                if (elect_one()) {
-                    #pragma unroll 1
-                    for (int mt = 0; mt < F::MtB; ++mt) {
-                        const uint64_t da = sdesc(smem_addr(smem) + mt * 16 * kChunk, 128, kChunk);
+            const uint32_t zb = smem_addr(dzs + (k & 1) * F::DzB);
+            // dz for T: the copy shifted by 2 Si; row q - shift is Front + 2 Si further on
+            const uint64_t z_k = sdesc(zb + 8 * F::RowsZ * 16, F::RowsZ * 16, 128) + uint64_t(F::Front + 2 * N::Si);
+            const uint64_t z_mn = sdesc(zb, 128, F::RowsZ * 16) + uint64_t(F::Front);
+            const uint64_t a_mn = sdesc(smem_addr(acts + (k & 1) * F::ActB), 128, F::RowsA * 16);
+            const int rows = tile_nb(k) * N::Pi, mts = (rows + 127) / 128, ksteps = (rows + 15) / 16;
+            #pragma unroll 1
+            for (int mt = 0; mt < mts && ok; ++mt) {
+                #pragma unroll
+                for (int u = 0; u < F::Units; ++u, ++n) {
+                    // the unit before is read
+                    ok = ok && wait_count(freed, kBwdEpi * n, abort_flag, err);
+                    fence_after();
+                    if (ok && leader) {
+                        // a value of its own, or the taps' descriptors are kept in
+                        // registers over the tiles
+                        uint64_t wt = w_k;
+                        asm volatile("" : "+l"(wt));
                         #pragma unroll
-                        for (int q = 0; q < kRowsT / 16; ++q)
+                        for (int i = 0; i < F::UnitTaps && u * F::UnitTaps + i < N::Taps; ++i) {
+                            const int t = u * F::UnitTaps + i;
+                            const int sh = ((N::Dim == 3 ? t / 9 : 0) * N::Si + t / 3 % 3) * N::Si + t % 3;
+                            #pragma unroll
+                            for (int q = 0; q < 2; ++q)
+                                mma_bf16(tmem + F::ColT + uint32_t(32 * i),
+                                         z_k + uint64_t(128 * mt) + uint64_t(2 * q * F::RowsZ - sh),
+                                         wt + uint64_t(32 * t + 2 * q * F::Kw), id_c, q > 0 ? 1u : 0u);
+                            // the epilogue takes three taps at a time
+                            if (i % 3 == 2 || i + 1 == F::UnitTaps) mma_commit(bars + i / 3);
+                        }
+                        #pragma unroll
+                        for (int i = 0; i < F::UnitSteps; ++i) {
+                            const int j = u * F::UnitSteps + i, pl = N::Dim == 2 ? 0 : j / 8;
+                            const int q = N::Dim == 2 ? 8 * mt + j : j % 8;
                             if (q < ksteps)
-                                mma_bf16(tmem + uint32_t(32 * (F::MtB * j + mt)), da + uint64_t(q * 16),
-                                         dz_mn + uint64_t(q * 16), id_w, any || q > 0 ? 1u : 0u);
-                    }
-                    if (F::Dgrad && j == F::Builds - 1)
-                        for (int q = 0; q < 2; ++q)
-                            mma_bf16(tmem + kDcol, dz_k + uint64_t(2 * q * (kChunk >> 4)),
-                                     w_k + uint64_t(2 * q * F::Kw), id_c, q > 0 ? 1u : 0u);
-                    mma_commit(bars + 0);
-                }
-                __syncwarp();
-            }
-            // the network's input is not read again: fetch the next tile's
-            if (N::First && t < a.tiles) ld.start(a, t * a.G, nb, act, tid);
-        }
-        // the last build's MMAs complete after all others
-        if (ok)
-            ok = __syncthreads_and(mbar_wait(bars + 0, uint32_t(it - 1) & 1u, abort_flag, err));
-        fence_after();
-        if (!ok) break;
-        any = true;
-        if constexpr (F::Dgrad) {
-            #pragma unroll
-            for (int j = 0; j < F::Passes; ++j) {
-                // dcol of channels [Ch j, Ch j + Ch) from TMEM to shared memory
-                const uint32_t tq = tmem + kDcol + (uint32_t(32 * (warp & 3)) << 16);
-                float *drow = dcol + (32 * (warp & 3) + lane) * F::Ld;
-                #pragma unroll 1
-                for (int n0 = 16 * (warp >> 2); n0 < F::Nm; n0 += 64) {
-                    float v[16];
-                    tmem_ld16(tq + uint32_t(n0), v);
-                    #pragma unroll
-                    for (int e = 0; e < 16; ++e)
-                        if (F::Nc % 16 == 0 || n0 + e < F::Nc) drow[n0 + e] = v[e];
-                }
-                fence_before();
-                __syncthreads();
-                fence_after();
-                if (j + 1 < F::Passes && warp == 0) {
-                    // the next pass's product runs under this pass's gather
-                    if (elect_one()) {
-                        for (int q = 0; q < 2; ++q)
-                            mma_bf16(tmem + kDcol, dz_k + uint64_t(2 * q * (kChunk >> 4)),
-                                     w_k + uint64_t(2 * q * F::Kw + (j + 1) * F::Nc), id_c,
-                                     q > 0 ? 1u : 0u);
-                        mma_commit(bars + 1);
+                                mma_bf16(tmem + uint32_t(96 * pl), z_mn + uint64_t(16 * q),
+                                         a_mn + uint64_t(16 * q + pl * N::Si * N::Si), id_w,
+                                         (k | q) != 0 ? 1u : 0u);
+                        }
+                        if (u + 1 == F::Units && mt + 1 == mts) mma_commit(done + (k & 1));
                     }
                     __syncwarp();
                 }
-                // a thread takes lines of one channel
-                constexpr int kLines = N::Dim == 2 ? N::Si : N::Si * N::Si;
-                const int il = tid % F::Ch, c = F::Ch * j + il;
-                float s_db = 0.f;
-                for (int q = tid / F::Ch; q < nb_now * kLines; q += kBwdThreads / F::Ch) {
-                    const int w = q / kLines, l = q % kLines;
-                    const int iy = N::Dim == 2 ? l : l % N::Si, iz = N::Dim == 2 ? 0 : l / N::Si;
-                    const int oy = iy - a.ring, oz = N::Dim == 2 ? 0 : iz - a.ring;
-                    if (unsigned(oy) >= unsigned(crop) || unsigned(oz) >= unsigned(crop)) continue;
-                    float s[N::Si];
-                    col2im_line<N, F::Ld>(dcol + il * N::Taps, w * N::Po, iy, iz, s);
-                    const uint16_t *h = reinterpret_cast<const uint16_t *>(act) +
-                                        (w * N::Pi + l * N::Si) * kPitch + c;
-                    uint16_t *out = a.dzp + ((b0 + w) * np + (oz * crop + oy) * crop) * kTrainCh + c;
+            }
+        }
+    } else if (warp >= kBwdEpi) {
+        const int lt = tid - kBwdEpi * 32;
+        for (int k = 0; k < n_mine; ++k) {
+            const int64_t b0 = tile_b0(k);
+            const int nb = tile_nb(k);
+            const uint4 *xa = reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(a.x) + b0 * N::Pi * kTrainCh);
+            const uint4 *xz = reinterpret_cast<const uint4 *>(a.dz + b0 * N::Po * kTrainCh);
+            uint4 va[F::PieceA], vz[F::PieceZ];
+            #pragma unroll
+            for (int j = 0; j < F::PieceZ; ++j) {
+                const int i = lt + j * kBwdLoad * 32;
+                vz[j] = i < nb * N::Po * 4 ? __ldg(xz + i) : make_uint4(0u, 0u, 0u, 0u);
+            }
+            #pragma unroll
+            for (int j = 0; j < F::PieceA; ++j) {
+                const int i = lt + j * kBwdLoad * 32;
+                va[j] = i < nb * N::Pi * 4 ? __ldg(xa + i) : make_uint4(0u, 0u, 0u, 0u);
+            }
+            // the tile before last is done with this buffer
+            if (k >= 2)
+                ok = idle_wait(done + (k & 1), uint32_t(k / 2 - 1) & 1u, abort_flag, err) &&
+                     wait_count(hdone + (k & 1), uint32_t(kBwdEpi * (k / 2)), abort_flag, err);
+            if (!ok) break;
+            uint8_t *zb = dzs + (k & 1) * F::DzB, *ab = acts + (k & 1) * F::ActB;
+            #pragma unroll
+            for (int j = 0; j < F::PieceZ; ++j) {
+                const int i = lt + j * kBwdLoad * 32;
+                if (i >= a.G * N::Po * 4) break;          // inputs past the batch: zeros
+                const int p = i >> 2, w = p / N::Po, o = p % N::Po;
+                const int q = w * N::Pi + (N::Dim == 2 ? o / N::So * N::Si + o % N::So
+                                                       : (o / (N::So * N::So) * N::Si + o / N::So % N::So) * N::Si + o % N::So);
+                #pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    *reinterpret_cast<uint4 *>(zb + ((4 * c + (i & 3)) * F::RowsZ + F::Front + q + c * N::Si) * 16) = vz[j];
+            }
+            #pragma unroll
+            for (int j = 0; j < F::PieceA; ++j) {
+                const int i = lt + j * kBwdLoad * 32, q = i >> 2;
+                if (i >= a.G * N::Pi * 4) break;
+                #pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    if (q >= c) *reinterpret_cast<uint4 *>(ab + ((4 * c + (i & 3)) * F::RowsA + q - c) * 16) = va[j];
+            }
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) red_release_add(full + (k & 1), 1u);
+        }
+    } else {
+        const int wq = warp & 3, ch = 2 * (warp >> 2);   // lane quarter, first 8-channel chunk
+        const uint32_t tq = tmem + F::ColT + (uint32_t(32 * wq) << 16) + uint32_t(8 * ch);
+        float db[16];
+        #pragma unroll
+        for (int e = 0; e < 16; ++e) db[e] = 0.f;
+        uint32_t ph = 0;                                 // phases of the parts' barriers
+        for (int k = 0; k < n_mine && ok; ++k) {
+            const int64_t b0 = tile_b0(k);
+            const int rows = tile_nb(k) * N::Pi, mts = (rows + 127) / 128;
+            const uint8_t *h = acts + (k & 1) * F::ActB + ch * F::RowsA * 16;
+            for (int mt = 0; mt < mts && ok; ++mt) {
+                float s[16];
+                #pragma unroll
+                for (int e = 0; e < 16; ++e) s[e] = 0.f;
+                #pragma unroll 1
+                for (int u = 0; u < F::Units && ok; ++u) {
+                    const int taps = min(F::UnitTaps, N::Taps - u * F::UnitTaps);
                     #pragma unroll
-                    for (int ix = 0; ix < N::Si; ++ix) {
-                        if (unsigned(ix - a.ring) >= unsigned(crop)) continue;
-                        // through the ReLU of the layer below: its output is positive
-                        const float v = positive(h[ix * kPitch]) ? s[ix] : 0.f;
-                        s_db += v;
-                        out[(ix - a.ring) * kTrainCh] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
+                    for (int g = 0; g < F::Parts; ++g) {
+                        // (the last unit may have a part less)
+                        if (3 * g >= taps) break;
+                        ok = spin_wait(bars + g, (ph >> g) & 1u, abort_flag, err);
+                        if (!ok) break;
+                        ph ^= 1u << g;
+                        fence_after();
+                        if (F::UnitTaps - 3 * g >= 3) {
+                            float v[3][16];
+                            tmem_ld16x3(tq + uint32_t(96 * g), v);
+                            #pragma unroll
+                            for (int i = 0; i < 3; ++i)
+                                #pragma unroll
+                                for (int e = 0; e < 16; ++e) s[e] += v[i][e];
+                        } else {
+                            float v[16];
+                            tmem_ld16(tq + uint32_t(96 * g), v);
+                            #pragma unroll
+                            for (int e = 0; e < 16; ++e) s[e] += v[e];
+                        }
+                    }
+                    fence_before();
+                    __syncwarp();
+                    if (lane == 0) red_release_add(freed, 1u);
+                }
+                if (!ok) break;
+                const int p = 128 * mt + 32 * wq + lane, w = p / N::Pi, o = p % N::Pi;
+                const int x = o % N::Si - F::Ring, y = (o / N::Si) % N::Si - F::Ring;
+                bool in = p < rows;
+                int64_t op = b0 * N::Pi + p;
+                if (F::Ring) {
+                    in = in && unsigned(x) < unsigned(F::Crop) && unsigned(y) < unsigned(F::Crop);
+                    op = (b0 + w) * F::Np + y * F::Crop + x;
+                }
+                // the activations are in place (the loaders' stores, seen through `full`)
+                if (mt == 0) ok = wait_count(full + (k & 1), uint32_t(kBwdLoad * (k / 2 + 1)), abort_flag, err);
+                if (!ok) break;
+                if (in) {
+                    uint4 *out = reinterpret_cast<uint4 *>(a.dzp + op * kTrainCh + 8 * ch);
+                    #pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        const uint4 hq = *reinterpret_cast<const uint4 *>(h + (c * F::RowsA + p) * 16);
+                        const uint32_t hw[4] = {hq.x, hq.y, hq.z, hq.w};
+                        uint32_t r[4];
+                        #pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            // through the ReLU of the layer below: its output is positive
+                            const float v0 = positive(uint16_t(hw[e])) ? s[8 * c + 2 * e] : 0.f;
+                            const float v1 = positive(uint16_t(hw[e] >> 16)) ? s[8 * c + 2 * e + 1] : 0.f;
+                            db[8 * c + 2 * e] += v0;
+                            db[8 * c + 2 * e + 1] += v1;
+                            r[e] = pack_bf16x2(v0, v1);
+                        }
+                        out[c] = make_uint4(r[0], r[1], r[2], r[3]);
                     }
                 }
-                db[j] += s_db;
-                if (j + 1 < F::Passes) {
-                    ok = __syncthreads_and(mbar_wait(bars + 1, phase, abort_flag, err));
-                    phase ^= 1u;
-                    if (!ok) break;
-                    fence_after();
-                } else {
-                    __syncthreads();
-                    if (t < a.tiles && !two) ld.start(a, t * a.G, nb, act, tid);
-                }
             }
-            if (!ok) break;
+            __syncwarp();
+            if (lane == 0) red_release_add(hdone + (k & 1), 1u);
         }
-        uint8_t *q = act;
-        act = next;
-        next = q;
-    }
-    cp_async_wait_all();
-    if (ok && any) {
-        // this CTA's weight gradient: rows of D are k, columns the output channel
-        float *wp = a.wpart + int64_t(blockIdx.x) * N::K * kTrainCh;
-        if ((warp >> 2) < 2) {
-            const int o0 = 16 * (warp >> 2);
-            for (int mt = 0; mt < F::Mt; ++mt) {
-                float v[16];
-                tmem_ld16(tmem + (uint32_t(32 * (warp & 3)) << 16) + uint32_t(32 * mt + o0), v);
-                // M-tile mt: columns from 8 Cb (mt / MtB) + 128 (mt % MtB) of A
-                const int kl = 128 * (mt % F::MtB) + 32 * (warp & 3) + lane;
-                const int k = 8 * F::Cb * (mt / F::MtB) + kl;
-                if (kl < 8 * F::Cb && k < N::K) {
-                    #pragma unroll
-                    for (int e = 0; e < 16; ++e) wp[(o0 + e) * N::K + k] = v[e];
-                }
-            }
-        }
-        if constexpr (F::Dgrad) {
-            // column sums of the input gradient: threads of one channel in order
-            float *red = dcol;
-            __syncthreads();
+        // column sums of the input gradient: a warp's lanes, then the warps in order
+        #pragma unroll
+        for (int e = 0; e < 16; ++e) {
             #pragma unroll
-            for (int j = 0; j < F::Passes; ++j) red[j * kBwdThreads + tid] = db[j];
-            __syncthreads();
-            if (tid < kTrainCh) {
-                const float *r = red + (tid / F::Ch) * kBwdThreads + tid % F::Ch;
-                float s = 0.f;
-                for (int i = 0; i < kBwdThreads / F::Ch; ++i) s += r[i * F::Ch];
-                a.bpart[int64_t(blockIdx.x) * kTrainCh + tid] = s;
-            }
+            for (int m = 16; m > 0; m >>= 1) db[e] += __shfl_xor_sync(0xffffffffu, db[e], m);
+            if (lane == 0) red[warp * 16 + e] = db[e];
         }
     }
-    mma_drain(bars + 2, tmem, kCols, warp);
+    // wait (bounded) for the MMAs in flight; the weight gradient is complete
+    if (warp == kBwdMma) {
+        if (elect_one()) {
+            mma_commit(drain);
+            for (uint32_t i = 0; i < (1u << 24) && !mbar_try_wait(drain, 0); ++i)
+                if (i > 64) __nanosleep(64);
+        }
+        __syncwarp();
+    }
+    fence_before();
+    const bool good = __syncthreads_and(ok && !*abort_flag) != 0;
+    fence_after();
+    if (good) {
+        // this CTA's weight gradient through shared memory in the weights' layout:
+        // D's lanes are (line dy, output channel), columns (dx, input channel)
+        float *stage = reinterpret_cast<float *>(smem);
+        const int dy = warp & 3;
+        if (warp < kBwdEpi && dy < 3) {
+            const int c0 = 16 * (warp >> 2);
+            #pragma unroll 1
+            for (int pl = 0; pl < F::Planes; ++pl) {
+                float v[3][16];
+                tmem_ld16x3(tmem + (uint32_t(32 * dy) << 16) + uint32_t(96 * pl + c0), v);
+                float *st = stage + lane * (N::K + 1) + (3 * pl + dy) * 3;
+                #pragma unroll
+                for (int e = 0; e < 16; ++e)
+                    #pragma unroll
+                    for (int dx = 0; dx < 3; ++dx) st[(c0 + e) * N::Taps + dx] = v[dx][e];
+            }
+        }
+        __syncthreads();
+        float *wp = a.wpart + int64_t(blockIdx.x) * N::K * kTrainCh;
+        for (int i = tid; i < N::K * kTrainCh; i += kBwdThreads) wp[i] = stage[i / N::K * (N::K + 1) + i % N::K];
+        if (tid < kTrainCh) {
+            const float *r = red + (tid / 16) * 64 + tid % 16;
+            a.bpart[int64_t(blockIdx.x) * kTrainCh + tid] = ((r[0] + r[16]) + r[32]) + r[48];
+        }
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    if (warp == 0) tmem_free(tmem, 512);
 }
 
 // Weights of one convolution (FP32 W[32][K]) as the operands of both passes:
-// forward bf16 [Kp / 8][32][8] and, with dgrad, backward [4][Kw][8] (zero past K).
+// forward bf16 [Kp / 8][32][8] (zero past K) and, with dgrad, backward [4][Kw][8],
+// row 32 tap + channel.
 // Weights of fc1 (W1[256][32]) the same way: bf16 [4][256][8].
 struct PackArgs {
     PackSeg seg[kMaxPack];
@@ -750,7 +995,8 @@ __global__ void __launch_bounds__(256) pack_train_kernel(const PackArgs a) {
         if (b)
             for (int e = tid; e < kTrainCh * g.kw; e += nth) {
                 const int j = e & 7, k = (e >> 3) % g.kw, o = (e >> 3) / g.kw * 8 + j;
-                b[e] = __float2bfloat16_rn(k < g.K ? __ldg(g.W + o * g.K + k) : 0.f);
+                // row k: tap k / 32, channel k % 32
+                b[e] = __float2bfloat16_rn(__ldg(g.W + o * g.K + k % kTrainCh * (g.K / kTrainCh) + k / kTrainCh));
             }
         __nv_bfloat16 *h = reinterpret_cast<__nv_bfloat16 *>(g.fc1);
         if (h)
@@ -1141,14 +1387,21 @@ void with_geo(const ConvGeo &g, bool first, Fn f) {
     }
 }
 
-// inputs per tile: as many as fill the 128 rows and fit shared memory, but no
-// more than leaves every SM a tile
+// inputs per tile of the im2col kernels: as many as fill the 128 rows and fit
+// shared memory, but no more than leaves every SM a tile
 template <class N, bool BWD>
 int tile_inputs(int64_t B, int sm_count) {
     const int64_t even = (B + sm_count - 1) / sm_count;
     int G = int(std::max<int64_t>(1, std::min<int64_t>(N::GMax, even)));
-    while (G > 1 && conv_smem_of<N, BWD>(G, 1).total > kSmemMax) --G;
+    while (G > 1 && conv_smem<N, BWD>(G).total > kSmemMax) --G;
     return G;
+}
+
+// inputs per tile of the backward pass: the same number of tiles for every SM
+template <class N>
+int bwd_inputs(int64_t B, int sm_count) {
+    const int64_t each = int64_t(sm_count) * BwdCfg<N>::GMax, rounds = (B + each - 1) / each;
+    return int((B + sm_count * rounds - 1) / (sm_count * rounds));
 }
 
 int head_rows(int64_t B, int sm_count) {
@@ -1157,7 +1410,7 @@ int head_rows(int64_t B, int sm_count) {
 
 }  // namespace
 
-int train_packed_kw(int dim) { return dim == 2 ? 288 : 872; }
+int train_packed_kw(int dim) { return kTrainCh * (dim == 2 ? 9 : 27); }
 
 int launch_pack_train(const PackSeg *segs, int n, cudaStream_t st) {
     PackArgs a{};
@@ -1200,18 +1453,23 @@ int launch_conv_fwd(const ConvGeo &g, const void *x, bool first, int64_t B, cons
 }
 
 int conv_bwd_ctas(const ConvGeo &g, int64_t B, bool first, int sm_count) {
-    int G = 1;
-    int per_sm = 1;
+    int64_t ctas = 1;
     with_geo(g, first, [&](auto n) {
-        G = tile_inputs<decltype(n), true>(B, sm_count);
-        per_sm = ConvCfg<decltype(n), true>::PerSm;
+        using N = decltype(n);
+        if constexpr (N::First) {
+            const int G = tile_inputs<N, true>(B, sm_count);
+            ctas = std::min<int64_t>((B + G - 1) / G, int64_t(sm_count) * ConvCfg<N, true>::PerSm);
+        } else {
+            const int G = bwd_inputs<N>(B, sm_count);
+            ctas = std::min<int64_t>((B + G - 1) / G, sm_count);
+        }
     });
-    return int(std::min<int64_t>((B + G - 1) / G, int64_t(sm_count) * per_sm));
+    return int(ctas);
 }
 
 int launch_conv_bwd(const ConvGeo &g, const void *x, bool first, int64_t B, const uint16_t *dz,
-                    const uint8_t *packed, float *wpart, uint16_t *dzp, int ring, float *bpart,
-                    int *err, int sm_count, cudaStream_t st) {
+                    const uint8_t *packed, float *wpart, uint16_t *dzp, float *bpart, int *err,
+                    int sm_count, cudaStream_t st) {
     ConvArgs a{};
     a.x = x;
     a.B = B;
@@ -1220,17 +1478,24 @@ int launch_conv_bwd(const ConvGeo &g, const void *x, bool first, int64_t B, cons
     a.wpart = wpart;
     a.dzp = dzp;
     a.bpart = bpart;
-    a.ring = ring;
     const int grid = conv_bwd_ctas(g, B, first, sm_count);
     with_geo(g, first, [&](auto n) {
         using N = decltype(n);
-        a.G = tile_inputs<N, true>(B, sm_count);
-        a.tiles = (B + a.G - 1) / a.G;
-        const ConvSmem L = conv_smem<N, true>(a.G);
-        static_assert(ConvCfg<N, true>::PerSm == 1 || conv_smem<N, true>(1).total <= kSmemHalf,
-                      "two CTAs per SM");
-        cudaFuncSetAttribute(conv_bwd_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-        launch_pdl(conv_bwd_kernel<N>, dim3(grid), dim3(kBwdThreads), size_t(L.total), st, a, L, err);
+        if constexpr (N::First) {
+            a.G = tile_inputs<N, true>(B, sm_count);
+            a.tiles = (B + a.G - 1) / a.G;
+            const ConvSmem L = conv_smem<N, true>(a.G);
+            static_assert(ConvCfg<N, true>::PerSm == 1 || conv_smem<N, true>(1).total <= kSmemHalf,
+                          "two CTAs per SM");
+            cudaFuncSetAttribute(first_wgrad_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+            launch_pdl(first_wgrad_kernel<N>, dim3(grid), dim3(kWgThreads), size_t(L.total), st, a, L, err);
+        } else {
+            using F = BwdCfg<N>;
+            a.G = bwd_inputs<N>(B, sm_count);
+            a.tiles = (B + a.G - 1) / a.G;
+            cudaFuncSetAttribute(conv_bwd_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, F::kTotal);
+            launch_pdl(conv_bwd_kernel<N>, dim3(grid), dim3(kBwdThreads), size_t(F::kTotal), st, a, err);
+        }
     });
     return 1;
 }

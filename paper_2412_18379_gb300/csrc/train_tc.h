@@ -22,8 +22,8 @@ struct ConvGeo {
 };
 
 // Packed weights of a training step: per convolution W[32][K] -> fwd (BF16
-// [Kp / 8][32][8], Kp = K rounded up to 16) and bwd (BF16 [4][kw][8]); fc1's
-// W1[256][32] -> fc1 (BF16 [4][256][8]). Null outputs are skipped.
+// [Kp / 8][32][8], Kp = K rounded up to 16) and bwd (BF16 [4][kw][8], row 32 tap +
+// channel); fc1's W1[256][32] -> fc1 (BF16 [4][256][8]). Null outputs are skipped.
 struct PackSeg {
     const float *W;
     int K, kw;
@@ -46,12 +46,12 @@ int conv_bwd_ctas(const ConvGeo &g, int64_t B, bool first, int sm_count);
 // Weight gradient partials of one convolution, wpart[cta][32 K] (the weights'
 // layout), from its input x (as in launch_conv_fwd) and its output gradient dz
 // (BF16 [B][Po][32]); and, except for the first layer, its input's gradient
-// through the ReLU (x > 0): dzp BF16 [B][(Si - 2 ring)^D][32] (the positions
-// `ring` away from the border), and the column sums of its FP32 values
+// through the ReLU (x > 0): dzp BF16 [B][Pi][32] (Si = 11: x has a zero ring that
+// dzp leaves out, [B][81][32]), and the column sums of its FP32 values
 // bpart[cta][32]. packed: PackSeg::bwd.
 int launch_conv_bwd(const ConvGeo &g, const void *x, bool first, int64_t B, const uint16_t *dz,
-                    const uint8_t *packed, float *wpart, uint16_t *dzp, int ring, float *bpart,
-                    int *err, int sm_count, cudaStream_t st);
+                    const uint8_t *packed, float *wpart, uint16_t *dzp, float *bpart, int *err,
+                    int sm_count, cudaStream_t st);
 
 // The regressor's head on h [B][32] (BF16): out = W2 ReLU(W1 h + b1) + b2 (FP32
 // [B][dim]). With targets also the mean squared error's gradients: dz [B][32]

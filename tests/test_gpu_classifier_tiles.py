@@ -80,3 +80,11 @@ def test_permuted_batch_gradient(ctx, dim, B):
     again, _ = ctx.classifier_grad(mesh, xp, lab)
     assert np.array_equal(again.cpu().numpy().view(np.uint32), g.cpu().numpy().view(np.uint32))
     mesh.release()
+
+
+@pytest.mark.parametrize("B", [152, 153, 305, 609])
+def test_permuted_gradient_of_paired_windows(ctx, B):
+    """The second layer's backward pass takes two windows a tile once every SM has
+    one (152 SMs): one tile more, an odd window left over, a second tile per CTA.
+    The bound is the permuted batch's above."""
+    test_permuted_batch_gradient(ctx, 2, B)
