@@ -27,7 +27,7 @@
 // traffic is the BF16 activations and gradients alone. At a batch of 4096 the
 // 2-D step's im2col, GEMM, col2im and ReLU kernels moved about 1.2 GB through
 // FP32 buffers: a gradient call took 1102 us there and 1594 us for 2048 rows in
-// 3-D, now 143 us and 212 us.
+// 3-D, now 142 us and 212 us.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -582,8 +582,8 @@ __global__ void __launch_bounds__(kWgThreads, ConvCfg<N, true>::PerSm) first_wgr
 //            offset, in TMEM columns of its own.
 //
 // Warps 0-7 add up T and mask it by the ReLU (warp w: positions 32 (w % 4) .. of
-// the M-tile, 16 channels), warps 8-11 load, warp 12 issues the MMAs. Two buffers
-// of operands; the epilogue follows the tensor pipe three taps behind, and a
+// the M-tile, 16 channels), warps 8-11 load, warp 12 issues the MMAs, handed over
+// unit by unit by warp 13, which does its waiting. Two buffers of operands; the epilogue follows the tensor pipe three taps behind, and a
 // slice of the weights' steps keeps the pipe busy until it has read a unit's last.
 // Every wait is bounded (abort flag and device error flag).
 //
@@ -591,12 +591,15 @@ __global__ void __launch_bounds__(kWgThreads, ConvCfg<N, true>::PerSm) first_wgr
 // of 250 positions 36 and 16 of them in 2-D (2.4k cycles), 54 and 24 per 125 in
 // 3-D (3.7k). The kernel takes about twice that: a unit's products may not start
 // before the unit before is read, and a commit is seen 250 cycles after the
-// products, a part is read and added in 70. Measured: Si = 11 (4096 inputs) 39 us,
-// Si = 7 21, 5 14, 3 9.6; 3-D (2048) Si = 5 55, Si = 3 23. With the im2col operand,
-// dcol in shared memory and a gather from it: 108, 40, 18, 9.3; 72, 17.
+// products, a part is read and added in 70. Measured: Si = 11 (4096 inputs) 36 us,
+// Si = 7 20, 5 13.5, 3 9.8; 3-D (2048) Si = 5 56, Si = 3 23. With the im2col
+// operand, dcol in shared memory and a gather from it: 108, 40, 18, 9.3; 72, 17.
+// With the MMA warp waiting itself: 39, 21, 14, 9.6; 56, 23. T in two regions by
+// turns, a hand-back per part, two M-tiles by turns, or one lane polling: 3-D
+// Si = 5 63, 62, 74, 77.
 // ---------------------------------------------------------------------------
-constexpr int kBwdEpi = 8, kBwdLoad = 4, kBwdMma = kBwdEpi + kBwdLoad;
-constexpr int kBwdThreads = (kBwdMma + 1) * 32;
+constexpr int kBwdEpi = 8, kBwdLoad = 4, kBwdMma = kBwdEpi + kBwdLoad, kBwdSched = kBwdMma + 1;
+constexpr int kBwdThreads = (kBwdSched + 1) * 32;
 
 template <class N>
 struct BwdCfg {
@@ -658,6 +661,22 @@ __device__ __forceinline__ bool spin_wait(uint64_t *bar, uint32_t parity, volati
     *abort_flag = 1;
     atomicExch(err, 1);
     return false;
+}
+
+// The scheduler warp hands a unit to the MMA warp on a named barrier; false for
+// both where either's ok is. (A shared-memory load of the MMA warp itself returns
+// only once its queued MMAs have drained.)
+__device__ __forceinline__ bool handover(bool ok) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "barrier.cta.red.and.pred q, 1, 64, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}\n"
+        : "=r"(r)
+        : "r"(uint32_t(ok))
+        : "memory");
+    return r != 0;
 }
 
 // bounded wait for a phase that may be far away: sparse polls
@@ -743,11 +762,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
         constexpr uint32_t id_w = idesc_mn(idesc_bf16(128, 96), true, true);
         const bool leader = elect_one();
         const uint64_t w_k = sdesc(smem_addr(wop), F::Kw * 16, 128);
-        uint32_t n = 0;                                  // units so far
         for (int k = 0; k < n_mine && ok; ++k) {
-            ok = wait_count(full + (k & 1), uint32_t(kBwdLoad * (k / 2 + 1)), abort_flag, err);
-            if (!ok) break;
-            fence_after();
             const uint32_t zb = smem_addr(dzs + (k & 1) * F::DzB);
             // dz for T: the copy shifted by 2 Si; row q - shift is Front + 2 Si further on
             const uint64_t z_k = sdesc(zb + 8 * F::RowsZ * 16, F::RowsZ * 16, 128) + uint64_t(F::Front + 2 * N::Si);
@@ -757,9 +772,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
             #pragma unroll 1
             for (int mt = 0; mt < mts && ok; ++mt) {
                 #pragma unroll
-                for (int u = 0; u < F::Units; ++u, ++n) {
-                    // the unit before is read
-                    ok = ok && wait_count(freed, kBwdEpi * n, abort_flag, err);
+                for (int u = 0; u < F::Units; ++u) {
+                    ok = ok && handover(true);
                     fence_after();
                     if (ok && leader) {
                         // a value of its own, or the taps' descriptors are kept in
@@ -791,6 +805,17 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
                     }
                     __syncwarp();
                 }
+            }
+        }
+    } else if (warp == kBwdSched) {
+        uint32_t n = 0;                                  // units so far
+        for (int k = 0; k < n_mine && ok; ++k) {
+            const int units = (tile_nb(k) * N::Pi + 127) / 128 * F::Units;
+            for (int u = 0; u < units && ok; ++u, ++n) {
+                // the operands are in place; the unit before is read
+                ok = (u > 0 || wait_count(full + (k & 1), uint32_t(kBwdLoad * (k / 2 + 1)), abort_flag, err)) &&
+                     wait_count(freed, kBwdEpi * n, abort_flag, err);
+                ok = handover(ok);
             }
         }
     } else if (warp >= kBwdEpi) {
