@@ -327,10 +327,11 @@ cs_status cs_mesh_upload(cs_ctx *ctx, int dim, int64_t n_v, const double *xyz, i
     d.pseed = seed;
 
     ctx->launches += cs::launch_seed_grid(d, seed, ctx->sm_count, nullptr);
-    // hosts of the vertices, where memory (or the budget) has room for them:
-    // the walk does without, only slower at nodes at rest
+    // 3-D: hosts of the vertices, where memory (or the budget) has room for them;
+    // the walk does without, only slower at nodes at rest. In 2-D, where few
+    // elements meet at a node, reading them costs the walk more than it saves.
     int2 *vhost = nullptr;
-    if (dev_copy<int2>(ctx, m, nullptr, size_t(n_v), &vhost) == CS_OK) {
+    if (dim == 3 && dev_copy<int2>(ctx, m, nullptr, size_t(n_v), &vhost) == CS_OK) {
         ctx->launches += cs::launch_vertex_hosts(d, vhost, ctx->sm_count, nullptr);
         d.vhost = vhost;
     }

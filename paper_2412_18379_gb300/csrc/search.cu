@@ -243,10 +243,7 @@ int launch_seed_grid(const DevMesh &m, int32_t *seed, int sm_count, cudaStream_t
 
 int launch_vertex_hosts(const DevMesh &m, int2 *vhost, int sm_count, cudaStream_t st) {
     const int grid = sm_count * 8;
-    if (m.dim == 2)
-        vertex_host_kernel<2><<<grid, 256, 0, st>>>(m, vhost);
-    else
-        vertex_host_kernel<3><<<grid, 256, 0, st>>>(m, vhost);
+    vertex_host_kernel<3><<<grid, 256, 0, st>>>(m, vhost);
     return 1;
 }
 
