@@ -545,7 +545,7 @@ int train_tiled(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t B, const d
     // module 1
     if (d == 2) {
         const int pb = cls_pool_back_blocks(B, sm);
-        launch_cls_pool_back_tiled(2, C.tgpool, z2, B, C.tdz2, sum(kClsCh, pb, g + S.b_off[1]), sm, st);
+        launch_cls_pool_back_tiled(C.tgpool, z2, B, C.tdz2, sum(kClsCh, pb, g + S.b_off[1]), sm, st);
         const int ca2 = conv_bwd_ctas(c2, B, false, sm), ca1 = conv_bwd_ctas(c1, B, true, sm);
         float *w2 = sum(int64_t(kClsCh) * c2.K, ca2, g + S.w_off[1]);
         float *bb1 = sum(kClsCh, ca2, g + S.b_off[0]);

@@ -747,10 +747,9 @@ int cls_pool_back_blocks(int64_t B, int sm_count) {
     return int(std::min<int64_t>(B, int64_t(sm_count) * 6));
 }
 
-void launch_cls_pool_back_tiled(int dim, const float *dpool, const float *z, int64_t B,
-                                uint16_t *dz, float *part, int sm_count, cudaStream_t st) {
-    launch_pdl(dim == 2 ? pool_back_tiled_kernel<2> : pool_back_tiled_kernel<3>,
-               dim3(cls_pool_back_blocks(B, sm_count)), dim3(kT), 0, st, dpool, z, B, dz, part);
+void launch_cls_pool_back_tiled(const float *dpool, const float *z, int64_t B, uint16_t *dz,
+                                float *part, int sm_count, cudaStream_t st) {
+    launch_pdl(pool_back_tiled_kernel<2>, dim3(cls_pool_back_blocks(B, sm_count)), dim3(kT), 0, st, dpool, z, B, dz, part);
 }
 
 int cls_softmax_blocks(int64_t B) { return int((B + 127) / 128 * (128 / kSmRows)); }

@@ -73,8 +73,8 @@ void launch_cls_pool_tiled(int dim, const float *z, int64_t B, const FcMat &cat,
 // dpool [B][32 (W/2)^dim], and its column sums part[block][32], blocks =
 // cls_pool_back_blocks
 int cls_pool_back_blocks(int64_t B, int sm_count);
-void launch_cls_pool_back_tiled(int dim, const float *dpool, const float *z, int64_t B,
-                                uint16_t *dz, float *part, int sm_count, cudaStream_t st);
+void launch_cls_pool_back_tiled(const float *dpool, const float *z, int64_t B, uint16_t *dz,
+                                float *part, int sm_count, cudaStream_t st);
 // softmax and cross-entropy gradient (softmax_ce) into the tiled gH (n_cls
 // columns rounded up to 16, zero padding), column sums and loss sums per block:
 // part[block][n_cls], loss_part[block], blocks = cls_softmax_blocks(B); the
