@@ -583,8 +583,9 @@ __global__ void __launch_bounds__(kWgThreads, ConvCfg<N, true>::PerSm) first_wgr
 //
 // Warps 0-7 add up T and mask it by the ReLU (warp w: positions 32 (w % 4) .. of
 // the M-tile, 16 channels), warps 8-11 load, warp 12 issues the MMAs, handed over
-// unit by unit by warp 13, which does its waiting. Two buffers of operands; the epilogue follows the tensor pipe three taps behind, and a
-// slice of the weights' steps keeps the pipe busy until it has read a unit's last.
+// unit by unit by warp 13, which does its waiting. Two buffers of operands; the
+// epilogue follows the tensor pipe three taps behind, and a slice of the weights'
+// steps keeps the pipe busy until it has read a unit's last.
 // Every wait is bounded (abort flag and device error flag).
 //
 // The tensor pipe needs 42 cycles for an MMA of N = 32 and 58 for N = 96, per tile
