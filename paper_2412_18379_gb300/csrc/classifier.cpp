@@ -435,7 +435,9 @@ int backward_conv(cs_ctx *ctx, Classifier &C, int64_t B, const float *dpool, int
 // The tiled path's training step for B rows of at least 16: gradients of the
 // cross-entropy into C.g, and *loss. In 2-D module 1 runs on the
 // implicit-GEMM convolutions as well (train_tc.h); in 3-D, whose 343 positions
-// do not fit their tile, on the layer-by-layer kernels.
+// do not fit their tile, on the layer-by-layer kernels. (Below 16 rows the GEMM's
+// products do not run on the tensor cores, and their bits differ. A gradient call
+// of 15 rows takes 576 us in 2-D and 720 in 3-D, one of 16 206 and 423.)
 bool tiled_batch(int64_t B) { return gemm_bf16() && B >= 16; }
 
 // floats of a step's partial sums

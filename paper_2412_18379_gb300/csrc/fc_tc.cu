@@ -13,6 +13,12 @@
 // The sums run in K order in K = 16 steps, as the general GEMM's
 // (tc_gemm.cu), which staged FP32 operands through the threads and needed a
 // separate pass for every bias, ReLU and layout change.
+//
+// Bound by the copies' latency and the epilogues (these layers' K is short), not
+// by the tensor pipe. A chunk of 32768 particles in 2-D: xp2 11 us, fusion 26 us,
+// logits 15 us; with four epilogue warps and the bias read from global memory 25,
+// 48 and 20 us. A forward pass of 160801 particles took 3016 us with these layers
+// on the general GEMM, 1420 us with them here and module 1 as it was.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -540,6 +546,10 @@ void launch_bn(const FcArgs &a, int sm_count, int *err, cudaStream_t st) {
 
 }  // namespace
 
+// Columns of a tile: one tile for up to 96 (81 classes) and two for up to 352
+// (343 classes: 176 each, 3% padding, where 256 + 87 would compute half as much
+// again); otherwise the widest that still gives every SM a tile, as an MMA of 256
+// columns takes 130 cycles and four of 64 take 200.
 int fc_bn(int64_t M, int N, int sm_count) {
     if (N <= 96) return 96;
     if (N > 256 && N <= 352) return 176;

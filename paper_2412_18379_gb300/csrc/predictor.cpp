@@ -133,8 +133,10 @@ cs_status ensure_io(cs_ctx *ctx, Predictor &P, int64_t B) {
 }
 
 // The fused kernels (train_tc.cu) take BF16 operands and batches whose every
-// product the tensor-core GEMM would take (tc_gemm_fits: at least 16 rows);
-// FP32 operands and smaller batches run the layer-by-layer path.
+// product the tensor-core GEMM would take (tc_gemm_fits: at least 16 rows), so
+// that they give its bits; FP32 operands and smaller batches run the
+// layer-by-layer path. A gradient call of 15 rows there 360 us (2-D) and 347
+// (3-D), of 16 rows here 85 and 98; a forward call 132 and 142, 44 and 48.
 bool fused_batch(int64_t B) { return gemm_bf16() && B >= 16; }
 
 // where the packed weights of each layer lie in Predictor::fpack

@@ -183,8 +183,8 @@ __device__ __forceinline__ void prepare(const DevMesh &m, const TrackArgs &a, in
 // rest at a node (no-slip walls, stagnation points) end there, where many
 // elements meet. A line of wall nodes ends 32 walks of one warp so, each of
 // which took the whole warp through a search: on the 75^3 nodes of a cube, the
-// 884 on its edges alone took 243 us (58 now), and the CNN-SNS step 248 us
-// (104 now).
+// 884 on its edges alone took 243 us (58 now), and the CNN-SNS step 250 us
+// (116 now).
 constexpr int32_t kNoVertex = INT32_MIN;
 template <int D>
 __device__ __forceinline__ int32_t vertex_host(const DevMesh &m, int32_t cur, const double *xp) {
