@@ -350,7 +350,8 @@ cs_status cs_windows(cs_ctx *ctx, int32_t mesh_id, const float *grid, double dt,
                      const int64_t *cells, int64_t B, float *out, void *stream);
 
 /* Predictor forward on explicit windows (DEVICE pointers): windows
- * [B][dim][S^dim] -> dhat [B][dim] (cell units). Synchronous. */
+ * [B][dim][S^dim] -> dhat [B][dim] (cell units). Synchronous; CS_EDEVICE if a
+ * bounded device wait gave up (the outputs are of no use then). */
 cs_status cs_predictor_forward(cs_ctx *ctx, int dim, int64_t B, const float *windows,
                                float *dhat_out);
 
@@ -364,7 +365,9 @@ cs_status cs_predict(cs_ctx *ctx, int32_t mesh_id, double dt, float *dhat_out, v
  * (lr, beta1 0.9, beta2 0.999, eps 1e-8) on the mean squared error, for
  * `steps` batches of `batch` pairs drawn without replacement per epoch from a
  * generator seeded by `seed`. loss_out (HOST, may be NULL) receives the loss
- * of every step. Synchronous. CS_ENOPRED if no predictor is loaded. */
+ * of every step. Synchronous. CS_ENOPRED if no predictor is loaded;
+ * CS_EDEVICE if a bounded device wait gave up, in this call or unreported
+ * before it: the weights are then those before the first step it touched. */
 cs_status cs_predictor_train(cs_ctx *ctx, int dim, const float *windows, const float *targets,
                              int64_t N, int64_t batch, int64_t steps, float lr, uint64_t seed,
                              float *loss_out);
@@ -382,7 +385,8 @@ cs_status cs_training_pairs(cs_ctx *ctx, int32_t mesh_id, int64_t n, const doubl
 /* Gradient of the mean squared error of the predictor of dimension dim on B
  * (window, target) pairs (DEVICE pointers; grad_out [cs_predictor_size],
  * same layout as the weights) without updating the weights; loss_out (HOST,
- * may be NULL). Synchronous. */
+ * may be NULL). Synchronous; CS_EDEVICE if a bounded device wait gave up (the
+ * outputs are of no use then). */
 cs_status cs_predictor_grad(cs_ctx *ctx, int dim, int64_t B, const float *windows,
                             const float *targets, float *grad_out, float *loss_out);
 

@@ -167,6 +167,7 @@ void cs_destroy(cs_ctx *ctx) {
     for (auto &p : ctx->pred) cs::predictor_release(ctx, p);
     cs::classifier_release_all(ctx);
     cs::dfree(ctx, ctx->dev_err);
+    if (ctx->host_err) cudaFreeHost(ctx->host_err);
     cs::dfree(ctx, ctx->hold_flag);
     cs::dfree(ctx, ctx->scratch.counters);
     cs::dfree(ctx, ctx->scratch.stats);

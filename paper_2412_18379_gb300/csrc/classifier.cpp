@@ -958,7 +958,8 @@ cs_status cs_classifier_train(cs_ctx *ctx, int32_t mesh_id, const double *xp,
             ctx->launches += backward(ctx, *C, B, labels, didx, losses + s, nullptr);
         }
         C->t += 1;
-        ctx->launches += launch_adam(C->w, C->g, C->m, C->v, C->n, lr, C->t, ctx->sm_count, nullptr);
+        ctx->launches += launch_adam(C->w, C->g, C->m, C->v, C->n, lr, C->t, ctx->dev_err,
+                                     ctx->sm_count, nullptr);
         C->packed_dirty = true;
     }
     if (out == CS_OK) {

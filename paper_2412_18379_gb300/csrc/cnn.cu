@@ -462,10 +462,13 @@ __global__ void mse_grad_kernel(const float *__restrict__ out, const float *__re
 
 // Adam on the FP32 master weights (Sec. 2.3 names Adam; constants are the
 // customary ones): m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2,
-// w -= lr * m/(1-b1^t) / (sqrt(v/(1-b2^t)) + eps).
+// w -= lr * m/(1-b1^t) / (sqrt(v/(1-b2^t)) + eps). Nothing is updated once the
+// device error flag is up: the gradients are not this step's then.
 __global__ void adam_kernel(float *__restrict__ w, const float *__restrict__ g,
                             float *__restrict__ mo, float *__restrict__ ve, int64_t n, float lr,
-                            float b1, float b2, float eps, float c1, float c2) {
+                            float b1, float b2, float eps, float c1, float c2,
+                            const int *__restrict__ err) {
+    if (err && __ldg(err)) return;
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
          i += int64_t(gridDim.x) * blockDim.x) {
         const float gi = g[i];
@@ -999,12 +1002,12 @@ int launch_mse_grad(const float *out, const float *tgt, int64_t n, float *g, flo
 }
 
 int launch_adam(float *w, const float *g, float *m, float *v, int64_t n, float lr, int64_t t,
-                int sm_count, cudaStream_t st) {
+                const int *err, int sm_count, cudaStream_t st) {
     const double b1 = 0.9, b2 = 0.999;
     const float c1 = float(1.0 - std::pow(b1, double(t)));
     const float c2 = float(1.0 - std::pow(b2, double(t)));
     adam_kernel<<<grid_for(n, sm_count, 4), kThreads, 0, st>>>(w, g, m, v, n, lr, float(b1),
-                                                                float(b2), 1e-8f, c1, c2);
+                                                                float(b2), 1e-8f, c1, c2, err);
     return 1;
 }
 

@@ -77,8 +77,9 @@ int launch_colsum(const float *x, int64_t M, int64_t N, float *out, cudaStream_t
                   float *work = nullptr, int64_t work_floats = 0, int sm_count = 0);
 int launch_mse_grad(const float *out, const float *tgt, int64_t n, float *g, float *loss,
                     int sm_count, cudaStream_t st);
+// err (may be null): the device error flag; where it is up nothing is updated
 int launch_adam(float *w, const float *g, float *m, float *v, int64_t n, float lr, int64_t t,
-                int sm_count, cudaStream_t st);
+                const int *err, int sm_count, cudaStream_t st);
 // Test hook of the tensor-core predictor kernels: when flag is not null, the
 // kernel first waits (bounded, `polls` polls) for *flag != 0 before any MMA;
 // nothing sets the flag, so the wait runs out and the kernel ends through its

@@ -118,6 +118,24 @@ cs_status ensure_err(cs_ctx *ctx) {
     return CS_OK;
 }
 
+// The device error flag at the end of a synchronous call: fetch_err enqueues
+// its copy to the host behind the call's kernels (a blocking read of its own
+// would cost a gradient call of 143 us another 8), and check_err reads it once
+// they have completed. A kernel whose wait gave up leaves no results, and what an
+// earlier call left in their place must not pass for them.
+cs_status fetch_err(cs_ctx *ctx) {
+    if (!ctx->dev_err) return CS_OK;
+    if (!ctx->host_err) PCHK(cudaHostAlloc(&ctx->host_err, sizeof(int), cudaHostAllocDefault));
+    *ctx->host_err = 0;
+    PCHK(cudaMemcpyAsync(ctx->host_err, ctx->dev_err, sizeof(int), cudaMemcpyDeviceToHost, nullptr));
+    return CS_OK;
+}
+
+cs_status check_err(cs_ctx *ctx) {
+    // raised: report it as cs_device_status does, which also clears it
+    return ctx->dev_err && *ctx->host_err ? cs_device_status(ctx) : CS_OK;
+}
+
 // the outputs and the batch of B rows
 cs_status ensure_io(cs_ctx *ctx, Predictor &P, int64_t B) {
     cs_status rc = ensure_err(ctx);
@@ -970,8 +988,9 @@ cs_status cs_predictor_forward(cs_ctx *ctx, int dim, int64_t B, const float *win
                              cudaMemcpyDeviceToDevice, nullptr));
     }
     PCHK(cudaGetLastError());
+    if ((rc = fetch_err(ctx))) return rc;
     PCHK(cudaDeviceSynchronize());
-    return CS_OK;
+    return check_err(ctx);
 }
 
 cs_status cs_predict(cs_ctx *ctx, int32_t mesh_id, double dt, float *dhat_out, void *stream) {
@@ -1035,7 +1054,8 @@ cs_status cs_predictor_train(cs_ctx *ctx, int dim, const float *windows, const f
             ctx->launches += backward(ctx, *P, B, P->tgt, losses + s, nullptr);
         }
         P->t += 1;
-        ctx->launches += launch_adam(P->w, P->g, P->m, P->v, P->n, lr, P->t, ctx->sm_count, nullptr);
+        ctx->launches += launch_adam(P->w, P->g, P->m, P->v, P->n, lr, P->t, ctx->dev_err,
+                                     ctx->sm_count, nullptr);
         P->packed_dirty = true;
     }
     if (out == CS_OK) {
@@ -1043,8 +1063,10 @@ cs_status cs_predictor_train(cs_ctx *ctx, int dim, const float *windows, const f
         if (e == cudaSuccess) e = cudaDeviceSynchronize();
         if (e == cudaSuccess && loss_out && steps > 0)
             e = cudaMemcpy(loss_out, losses, size_t(steps) * sizeof(float), cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) out = fail(ctx, CS_ECUDA, std::string("cs_predictor_train: ") +
-                                                            cudaGetErrorString(e));
+        if (e == cudaSuccess)
+            out = cs_device_status(ctx);
+        else
+            out = fail(ctx, CS_ECUDA, std::string("cs_predictor_train: ") + cudaGetErrorString(e));
     }
     dfree(ctx, losses);
     return out;
@@ -1085,24 +1107,21 @@ cs_status cs_predictor_grad(cs_ctx *ctx, int dim, int64_t B, const float *window
     if (rc) return rc;
     if (fused) {
         ctx->launches += train_fused(ctx, *P, B, windows, targets, P->loss, nullptr);
-        PCHK(cudaGetLastError());
-        // in the stream's order; the copy of the loss waits for everything
-        PCHK(cudaMemcpyAsync(grad_out, P->g, size_t(P->n) * sizeof(float), cudaMemcpyDeviceToDevice,
-                             nullptr));
-        if (loss_out)
-            PCHK(cudaMemcpy(loss_out, P->loss, sizeof(float), cudaMemcpyDeviceToHost));
-        else
-            PCHK(cudaDeviceSynchronize());
-        return CS_OK;
+    } else {
+        PCHK(cudaMemset(P->loss, 0, sizeof(float)));
+        ctx->launches += forward(ctx, *P, B, windows, nullptr);
+        ctx->launches += backward(ctx, *P, B, targets, P->loss, nullptr);
     }
-    PCHK(cudaMemset(P->loss, 0, sizeof(float)));
-    ctx->launches += forward(ctx, *P, B, windows, nullptr);
-    ctx->launches += backward(ctx, *P, B, targets, P->loss, nullptr);
     PCHK(cudaGetLastError());
-    PCHK(cudaDeviceSynchronize());
-    PCHK(cudaMemcpy(grad_out, P->g, size_t(P->n) * sizeof(float), cudaMemcpyDeviceToDevice));
-    if (loss_out) PCHK(cudaMemcpy(loss_out, P->loss, sizeof(float), cudaMemcpyDeviceToHost));
-    return CS_OK;
+    if ((rc = fetch_err(ctx))) return rc;
+    // in the stream's order; the copy of the loss waits for everything
+    PCHK(cudaMemcpyAsync(grad_out, P->g, size_t(P->n) * sizeof(float), cudaMemcpyDeviceToDevice,
+                         nullptr));
+    if (loss_out)
+        PCHK(cudaMemcpy(loss_out, P->loss, sizeof(float), cudaMemcpyDeviceToHost));
+    else
+        PCHK(cudaDeviceSynchronize());
+    return check_err(ctx);
 }
 
 cs_status cs_track_dhat(cs_ctx *ctx, int32_t mesh_id, int64_t n, const double *x, const double *u,
