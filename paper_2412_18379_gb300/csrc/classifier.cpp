@@ -274,9 +274,10 @@ cs_status ensure_tr(cs_ctx *ctx, Classifier &C, int64_t B) {
 }
 
 // workspace for B rows of the fully connected layers; `conv` adds the
-// unfused module 1's buffers, `grad` the backward pass's (which reuses
-// module 1's, so it needs `conv` too). Growing any set reallocates all of
-// them, each at its own row count.
+// unfused module 1's buffers and the GEMMs' K splits (no product of the fully
+// connected layers alone splits its K off the tensor cores), `grad` the backward
+// pass's (which reuses module 1's, so it needs `conv` too). Growing any set
+// reallocates all of them, each at its own row count.
 cs_status ensure_ws(cs_ctx *ctx, Classifier &C, int64_t B, bool conv, bool grad) {
     cs_status rc0 = ensure_err(ctx);
     if (rc0) return rc0;
@@ -295,14 +296,14 @@ cs_status ensure_ws(cs_ctx *ctx, Classifier &C, int64_t B, bool conv, bool grad)
         (rc = ws_alloc(ctx, C, &C.h2, rows * kClsH1)) ||
         (rc = ws_alloc(ctx, C, &C.u, rows * kClsH2)) ||
         (rc = ws_alloc(ctx, C, &C.ru, rows * kClsH2)) ||
-        (rc = ws_alloc(ctx, C, &C.H, rows * S.n_cls)) ||
-        (rc = ws_alloc(ctx, C, &C.splitk, tc_gemm_work_floats(ctx->sm_count)))) {
+        (rc = ws_alloc(ctx, C, &C.H, rows * S.n_cls))) {
         free_ws(ctx, C);
         return rc;
     }
     const int64_t rv = rows_conv;
     if (rv > 0 &&
-        ((rc = ws_alloc(ctx, C, &C.a0, rv * d * S.Pq)) ||
+        ((rc = ws_alloc(ctx, C, &C.splitk, tc_gemm_work_floats(ctx->sm_count))) ||
+         (rc = ws_alloc(ctx, C, &C.a0, rv * d * S.Pq)) ||
          (rc = ws_alloc(ctx, C, &C.col1, rv * S.P * K1)) ||
          (rc = ws_alloc(ctx, C, &C.z1, rv * S.P * kClsCh)) ||
          (rc = ws_alloc(ctx, C, &C.y1, rv * S.P * kClsCh)) ||
@@ -322,7 +323,7 @@ cs_status ensure_ws(cs_ctx *ctx, Classifier &C, int64_t B, bool conv, bool grad)
         free_ws(ctx, C);
         return rc;
     }
-    C.splitk_n = tc_gemm_work_floats(ctx->sm_count);
+    C.splitk_n = rv > 0 ? tc_gemm_work_floats(ctx->sm_count) : 0;
     C.cap = rows;
     C.cap_conv = rows_conv;
     C.cap_grad = rows_grad;
@@ -406,8 +407,17 @@ int fc_forward(cs_ctx *ctx, Classifier &C, const ClsShape &S, const FcPlan &P, i
     return n + launch_fc_gemm(l, ctx->dev_err, sm, st);
 }
 
+// Batches that the tiled path takes: BF16 operands and at least 16 rows. Below
+// 16 the GEMM's products do not run on the tensor cores, and their sums round
+// differently; such a batch or chunk keeps those layers, so that its results do
+// not depend on which kernels the larger ones use. (A gradient call of 15 rows
+// takes 576 us in 2-D and 720 in 3-D, one of 16 206 and 423.)
+bool tiled_batch(int64_t B) { return gemm_bf16() && B >= 16; }
+
 // inference of B particles xp[b] into H [B][n_cls]: module 1 fused on the
-// tensor cores, then the tiled fully connected layers
+// tensor cores, then the tiled fully connected layers or, for less than a tiled
+// batch, those of the training path (its BF16 features widened to FP32 lose
+// nothing: that path rounds its operands to BF16 itself)
 int infer(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t B, const double *xp, float *H,
           cudaStream_t st) {
     const ClsShape S(C.dim);
@@ -417,14 +427,23 @@ int infer(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t B, const double 
         launch_cls_pack(C.dim, C.w, S.w_off[0], S.b_off[0], S.w_off[1], S.b_off[1], C.packed, st);
         n += 1;
     }
-    if (C.packed_dirty || !std::equal(C.pack_bn, C.pack_bn + 3, P.bn)) {
+    const bool tiled = tiled_batch(B);
+    if (C.packed_dirty) C.pack_bn[0] = 0;
+    if (tiled && !std::equal(C.pack_bn, C.pack_bn + 3, P.bn)) {
         n += pack_fc(ctx, C, S, P, false, st);
         std::copy(P.bn, P.bn + 3, C.pack_bn);
     }
     C.packed_dirty = false;
-    launch_cls_conv_tc(m, m.pool_f, B, xp, C.packed, fc_mat(C.tcat, S.ldc), C.toff, ctx->dev_err,
+    const FcMat cat = fc_mat(C.tcat, S.ldc);
+    launch_cls_conv_tc(m, m.pool_f, B, xp, C.packed, cat, tiled ? C.toff : C.off, ctx->dev_err,
                        ctx->sm_count, st);
-    return n + 1 + fc_forward(ctx, C, S, P, B, H, st);
+    n += 1;
+    if (tiled) return n + fc_forward(ctx, C, S, P, B, H, st);
+    n += launch_fc_widen(fc_cols(cat, 0, S.n_pool), B, C.cat, S.ldc, st);
+    n += forward_fc(ctx, C, B, st);
+    if (H != C.H)
+        cudaMemcpyAsync(H, C.H, size_t(B) * S.n_cls * sizeof(float), cudaMemcpyDeviceToDevice, st);
+    return n;
 }
 
 int forward_conv(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t B, const double *xp,
@@ -432,13 +451,10 @@ int forward_conv(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t B, const 
 int backward_conv(cs_ctx *ctx, Classifier &C, int64_t B, const float *dpool, int64_t ld,
                   cudaStream_t st);
 
-// The tiled path's training step for B rows of at least 16: gradients of the
+// The tiled path's training step for B rows (tiled_batch): gradients of the
 // cross-entropy into C.g, and *loss. In 2-D module 1 runs on the
 // implicit-GEMM convolutions as well (train_tc.h); in 3-D, whose 343 positions
-// do not fit their tile, on the layer-by-layer kernels. (Below 16 rows the GEMM's
-// products do not run on the tensor cores, and their bits differ. A gradient call
-// of 15 rows takes 576 us in 2-D and 720 in 3-D, one of 16 206 and 423.)
-bool tiled_batch(int64_t B) { return gemm_bf16() && B >= 16; }
+// do not fit their tile, on the layer-by-layer kernels.
 
 // floats of a step's partial sums
 int64_t train_parts(cs_ctx *ctx, const ClsShape &S, int64_t B) {
@@ -696,10 +712,13 @@ cs_status forward_chunks(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t n
     const int ncls = cls_cells(C.dim);
     const int64_t R = std::min<int64_t>(n, chunk_rows(C.dim, fused));
     cs_status rc = fused ? ensure_fc(ctx, C, R, false) : ensure_ws(ctx, C, R, true, false);
+    // a chunk, the last one, of less than a tiled batch
+    const int64_t rest = n % R > 0 ? n % R : R;
+    if (rc == CS_OK && fused && !tiled_batch(rest)) rc = ensure_ws(ctx, C, rest, false, false);
     if (rc) return rc;
     for (int64_t r0 = 0; r0 < n; r0 += R) {
         const int64_t B = std::min(R, n - r0);
-        float *H = dst ? dst + r0 * ncls : fused ? C.tH : C.H;
+        float *H = dst ? dst + r0 * ncls : fused && tiled_batch(B) ? C.tH : C.H;
         if (fused) {
             ctx->launches += infer(ctx, C, m, B, xp + r0 * C.dim, H, st);
         } else {

@@ -536,6 +536,19 @@ __global__ void __launch_bounds__(256) fc_offset_grad_kernel(int64_t M,
     }
 }
 
+// a few rows of a tiled matrix as row-major FP32 (fewer than an MMA's 16; larger
+// products read the tiles)
+__global__ void __launch_bounds__(256) fc_widen_kernel(FcMat A, int64_t M, float *__restrict__ out,
+                                                       int64_t ld) {
+    pdl_wait();
+    const int64_t cols = int64_t(A.chunks) * 8;
+    for (int64_t i = int64_t(blockIdx.x) * 256 + threadIdx.x; i < M * cols; i += int64_t(gridDim.x) * 256) {
+        const int64_t b = i / cols, c = i % cols;
+        out[b * ld + c] = __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(
+            A.p + (b >> 7) * A.tile + (A.chunk0 + (c >> 3)) * kFcChunk + (b & 127) * 16 + (c & 7) * 2));
+    }
+}
+
 template <int BN>
 void launch_bn(const FcArgs &a, int sm_count, int *err, cudaStream_t st) {
     using G = FcGeo<BN>;
@@ -629,6 +642,13 @@ int launch_fc_wgrad(const FcMat &Y, const FcMat &X, int64_t M, int N, int K, int
     launch_pdl(fc_wgrad_kernel,
                dim3((N + 127) / 128, (K + FcWgGeo::BK - 1) / FcWgGeo::BK, splits), dim3(kFcThreads),
                size_t(FcWgGeo::kTotal), st, a, err);
+    return 1;
+}
+
+int launch_fc_widen(const FcMat &A, int64_t M, float *out, int64_t ld, cudaStream_t st) {
+    const int64_t n = M * A.chunks * 8;
+    launch_pdl(fc_widen_kernel, dim3(unsigned(std::min<int64_t>((n + 255) / 256, 64))), dim3(256), 0, st,
+               A, M, out, ld);
     return 1;
 }
 

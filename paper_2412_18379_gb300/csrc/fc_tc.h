@@ -76,6 +76,9 @@ int fc_wgrad_splits(int64_t M, int N, int K, int sm_count);
 int launch_fc_wgrad(const FcMat &Y, const FcMat &X, int64_t M, int N, int K, int splits,
                     float *part, int *err, cudaStream_t st);
 
+// out[i][c] = FP32 of A(i, c), row-major with row stride ld, i < M
+int launch_fc_widen(const FcMat &A, int64_t M, float *out, int64_t ld, cudaStream_t st);
+
 // r[i][n] = BF16 of ReLU(sum_d BF16(off[i][d]) BF16(W[n][d]) + b[n]), n < 256, tiled
 int launch_fc_offset(int dim, int64_t M, const float *off, const float *W, const float *b,
                      const FcMat &r, int sm_count, cudaStream_t st);
