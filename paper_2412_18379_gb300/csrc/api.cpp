@@ -136,6 +136,24 @@ void cs::dfree(cs_ctx *ctx, void *p) {
     cudaFree(p);
 }
 
+cs_status cs::ensure_err(cs_ctx *ctx) {
+    if (ctx->dev_err) return CS_OK;
+    int *h = nullptr, *d = nullptr;
+    if (cudaHostAlloc(&h, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(ctx, CS_ENOMEM, "host memory of the device error flag");
+    }
+    *h = 0;
+    const cudaError_t e = cudaHostGetDevicePointer(&d, h, 0);
+    if (e != cudaSuccess) {
+        cudaFreeHost(h);
+        return cuda_fail(ctx, e, "device address of the error flag");
+    }
+    ctx->host_err = h;
+    ctx->dev_err = d;
+    return CS_OK;
+}
+
 extern "C" {
 
 cs_status cs_create(cs_ctx **out, int cuda_device, size_t hbm_budget_bytes) {
@@ -166,8 +184,7 @@ void cs_destroy(cs_ctx *ctx) {
     for (auto &kv : ctx->meshes) free_mesh(ctx, kv.second);
     for (auto &p : ctx->pred) cs::predictor_release(ctx, p);
     cs::classifier_release_all(ctx);
-    cs::dfree(ctx, ctx->dev_err);
-    if (ctx->host_err) cudaFreeHost(ctx->host_err);
+    if (ctx->host_err) cudaFreeHost(const_cast<int *>(ctx->host_err));
     cs::dfree(ctx, ctx->hold_flag);
     cs::dfree(ctx, ctx->scratch.counters);
     cs::dfree(ctx, ctx->scratch.stats);

@@ -175,16 +175,6 @@ cs_status ws_alloc(cs_ctx *ctx, Classifier &C, T **p, int64_t count) {
     return rc;
 }
 
-// the error flag of the tensor-core kernels' bounded waits
-cs_status ensure_err(cs_ctx *ctx) {
-    if (ctx->dev_err) return CS_OK;
-    cs_status rc = dmalloc_n(ctx, &ctx->dev_err, 1);
-    if (rc) return rc;
-    if (cudaMemset(ctx->dev_err, 0, sizeof(int)) != cudaSuccess)
-        return fail(ctx, CS_ECUDA, "cudaMemset of the device error flag failed");
-    return CS_OK;
-}
-
 template <class T>
 cs_status list_alloc(cs_ctx *ctx, std::vector<void *> &v, T **p, int64_t count) {
     cs_status rc = dmalloc_n(ctx, p, size_t(std::max<int64_t>(count, 1)));

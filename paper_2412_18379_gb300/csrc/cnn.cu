@@ -468,7 +468,10 @@ __global__ void adam_kernel(float *__restrict__ w, const float *__restrict__ g,
                             float *__restrict__ mo, float *__restrict__ ve, int64_t n, float lr,
                             float b1, float b2, float eps, float c1, float c2,
                             const int *__restrict__ err) {
-    if (err && __ldg(err)) return;
+    __shared__ int raised;
+    if (threadIdx.x == 0) raised = err ? *reinterpret_cast<const volatile int *>(err) : 0;
+    __syncthreads();
+    if (raised) return;
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
          i += int64_t(gridDim.x) * blockDim.x) {
         const float gi = g[i];

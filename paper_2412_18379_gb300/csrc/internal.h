@@ -308,8 +308,12 @@ struct cs_ctx {
     int engine = 1;          // grid prediction: 1 tensor cores, 0 window GEMMs, 2 CUDA-core tiles (3-D)
     int tc_tile_rows = 0;    // 2-D tensor-core predictor tile height, 0 = automatic
     int tc3_tile = 0;        // 3-D tensor-core predictor tile side, 0 = automatic
-    int *dev_err = nullptr;  // device error flag of bounded waits
-    int *host_err = nullptr; // its copy in pinned host memory, as a synchronous call ends
+    // the error flag of bounded waits, in mapped host memory: a kernel writes it only
+    // when it gives up, and a call that has waited for its kernels reads it without
+    // a copy (a blocking one or one behind the kernels takes 8 us, of a gradient
+    // call's 145). Its two addresses.
+    int *dev_err = nullptr;
+    volatile int *host_err = nullptr;
     int *hold_flag = nullptr;  // test hook: a device flag nothing sets (cs_debug_hold_predictor)
     cs::Server *server = nullptr;   // serving loop (serve.cpp), if started
     // cs_track_host: copy-in, compute and copy-out streams, and its events
@@ -332,6 +336,12 @@ cs_status dmalloc_n(cs_ctx *ctx, T **p, size_t count) {
     *p = static_cast<T *>(q);
     return rc;
 }
+// The error flag of the tensor-core kernels' bounded waits (api.cpp): made once,
+// before the first kernel that may raise it; read and cleared once those launched
+// have completed.
+cs_status ensure_err(cs_ctx *ctx);
+inline bool err_raised(const cs_ctx *ctx) { return ctx->host_err && *ctx->host_err != 0; }
+inline void clear_err(cs_ctx *ctx) { *ctx->host_err = 0; }
 // The grid velocity of a field on its mesh's current predictor grid,
 // resampled (allocating) if the predictor grid changed since (predictor.cpp).
 cs_status field_grid(cs_ctx *ctx, Mesh *m, Field *f, cudaStream_t st, const float **grid_out);

@@ -108,33 +108,10 @@ void free_workspace(cs_ctx *ctx, Predictor &P) {
     P.tiles_cap.clear();
 }
 
-// the error flag of the tensor-core kernels' bounded waits
-cs_status ensure_err(cs_ctx *ctx) {
-    if (ctx->dev_err) return CS_OK;
-    cs_status rc = dalloc(ctx, &ctx->dev_err, 1);
-    if (rc) return rc;
-    if (cudaMemset(ctx->dev_err, 0, sizeof(int)) != cudaSuccess)
-        return fail(ctx, CS_ECUDA, "cudaMemset of the device error flag failed");
-    return CS_OK;
-}
-
-// The device error flag at the end of a synchronous call: fetch_err enqueues
-// its copy to the host behind the call's kernels (a blocking read of its own
-// would cost a gradient call of 143 us another 8), and check_err reads it once
-// they have completed. A kernel whose wait gave up leaves no results, and what an
-// earlier call left in their place must not pass for them.
-cs_status fetch_err(cs_ctx *ctx) {
-    if (!ctx->dev_err) return CS_OK;
-    if (!ctx->host_err) PCHK(cudaHostAlloc(&ctx->host_err, sizeof(int), cudaHostAllocDefault));
-    *ctx->host_err = 0;
-    PCHK(cudaMemcpyAsync(ctx->host_err, ctx->dev_err, sizeof(int), cudaMemcpyDeviceToHost, nullptr));
-    return CS_OK;
-}
-
-cs_status check_err(cs_ctx *ctx) {
-    // raised: report it as cs_device_status does, which also clears it
-    return ctx->dev_err && *ctx->host_err ? cs_device_status(ctx) : CS_OK;
-}
+// the end of a synchronous call, whose kernels have completed: a kernel whose
+// wait gave up leaves no results, and what an earlier call left in their place
+// must not pass for them (raised, it is reported as cs_device_status does)
+cs_status check_err(cs_ctx *ctx) { return err_raised(ctx) ? cs_device_status(ctx) : CS_OK; }
 
 // the outputs and the batch of B rows
 cs_status ensure_io(cs_ctx *ctx, Predictor &P, int64_t B) {
@@ -603,11 +580,7 @@ cs_status predict_grid_src(cs_ctx *ctx, cs::Mesh *m, const TcSource &src, double
             cs_status rc = dalloc(ctx, &P->packed, size_t(bytes));
             if (rc) return rc;
         }
-        if (!ctx->dev_err) {
-            cs_status rc = dalloc(ctx, &ctx->dev_err, 1);
-            if (rc) return rc;
-            PCHK(cudaMemset(ctx->dev_err, 0, sizeof(int)));
-        }
+        if (cs_status rc = ensure_err(ctx)) return rc;
         if (P->packed_dirty) {
             ctx->launches += m->d.dim == 2 ? launch_pack_tc(P->w, NetShape(2), P->packed, st)
                                            : launch_pack_tc3(P->w, NetShape(3), P->packed, st);
@@ -677,11 +650,7 @@ cs_status prepare_serving(cs_ctx *ctx) {
                 cs_status rc = dalloc(ctx, &P.packed, size_t(bytes));
                 if (rc) return rc;
             }
-            if (!ctx->dev_err) {
-                cs_status rc = dalloc(ctx, &ctx->dev_err, 1);
-                if (rc) return rc;
-                PCHK(cudaMemset(ctx->dev_err, 0, sizeof(int)));
-            }
+            if (cs_status rc = ensure_err(ctx)) return rc;
             if (P.packed_dirty) {
                 ctx->launches += dim == 2 ? launch_pack_tc(P.w, NetShape(2), P.packed, nullptr)
                                           : launch_pack_tc3(P.w, NetShape(3), P.packed, nullptr);
@@ -815,11 +784,8 @@ cs_status cs_device_status(cs_ctx *ctx) {
     if (!ctx) return CS_EINVAL;
     PCHK(cudaSetDevice(ctx->device));
     PCHK(cudaDeviceSynchronize());
-    if (!ctx->dev_err) return CS_OK;
-    int e = 0;
-    PCHK(cudaMemcpy(&e, ctx->dev_err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (e) {
-        PCHK(cudaMemset(ctx->dev_err, 0, sizeof(int)));
+    if (err_raised(ctx)) {
+        clear_err(ctx);
         return fail(ctx, CS_EDEVICE, "a bounded device wait gave up (tensor-core kernel)");
     }
     return CS_OK;
@@ -988,7 +954,6 @@ cs_status cs_predictor_forward(cs_ctx *ctx, int dim, int64_t B, const float *win
                              cudaMemcpyDeviceToDevice, nullptr));
     }
     PCHK(cudaGetLastError());
-    if ((rc = fetch_err(ctx))) return rc;
     PCHK(cudaDeviceSynchronize());
     return check_err(ctx);
 }
@@ -1113,7 +1078,6 @@ cs_status cs_predictor_grad(cs_ctx *ctx, int dim, int64_t B, const float *window
         ctx->launches += backward(ctx, *P, B, targets, P->loss, nullptr);
     }
     PCHK(cudaGetLastError());
-    if ((rc = fetch_err(ctx))) return rc;
     // in the stream's order; the copy of the loss waits for everything
     PCHK(cudaMemcpyAsync(grad_out, P->g, size_t(P->n) * sizeof(float), cudaMemcpyDeviceToDevice,
                          nullptr));
