@@ -32,6 +32,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "tc_common.cuh"
 #include "train_tc.h"
@@ -574,12 +575,19 @@ __global__ void __launch_bounds__(kWgThreads, ConvCfg<N, true>::PerSm) first_wgr
 //            dx[q][c] is the sum of the T_t in increasing t, each thread adding
 //            its position's in registers: the same sums in the same order as
 //            with the columns gradient in memory, with no gather (where the tap
-//            leaves the output the product is 0).
+//            leaves the output the product is 0: of finite weights).
 //   weights  dW[(dy, o)][(dx, c)] += sum_q dz[q - Si dy][o] act[q + dx + Si^2 dz][c]:
 //            M = 128 (3 x 32 used), N = 96, K = positions. Both operands are kept
 //            in three copies, shifted by Si dy and by dx, so that the copies
 //            continue the 8-channel chunks at one stride; 3-D adds dz by a row
 //            offset, in TMEM columns of its own.
+//
+// Zero times a value that is not finite is no zero, so the products that no output
+// position takes part in must not meet one. With weights that are not finite the
+// epilogue adds only the taps that meet an output. An activation that is not finite
+// is 1 in the operand, and the CTA adds its true products to its weight gradient
+// at the end (add_nonfinite). Both are looked for as the operands are loaded; finite
+// ones take the same path as before.
 //
 // Warps 0-7 add up T and mask it by the ReLU (warp w: positions 32 (w % 4) .. of
 // the M-tile, 16 channels), warps 8-11 load, warp 12 issues the MMAs, handed over
@@ -629,8 +637,9 @@ struct BwdCfg {
     static constexpr int kBar = kW + Kw * kTrainCh * 2;       // mbarriers: parts, 2 buffers, drain
     static constexpr int kCnt = kBar + (Parts + 3) * 8;       // u32 full [2], hdone [2], freed
     static constexpr uint32_t ColT = 96 * Planes;             // TMEM: weights, then a unit's T
-    static constexpr int kSlot = kCnt + 5 * 4;                // TMEM address, abort flag
-    static constexpr int kRed = (kSlot + 8 + 15) / 16 * 16;   // f32 [8][16]
+    static constexpr int kSlot = kCnt + 5 * 4;                // TMEM address, abort flag, an
+                                                              // activation that is not finite
+    static constexpr int kRed = (kSlot + 12 + 15) / 16 * 16;  // f32 [8][16]
     static constexpr int kTotal = kRed + kBwdEpi * 16 * 4;
     static constexpr int PieceA = (GMax * N::Pi * 4 + kBwdLoad * 32 - 1) / (kBwdLoad * 32);
     static constexpr int PieceZ = (GMax * N::Po * 4 + kBwdLoad * 32 - 1) / (kBwdLoad * 32);
@@ -640,7 +649,77 @@ struct BwdCfg {
     // follows the buffer
     static_assert(DzB + 16 * RowsZ * 16 <= kTotal, "operand reads inside the allocation");
     static_assert(kTrainCh * (N::K + 1) * 4 <= kW, "the weight gradient's stage");
+    static_assert(N::K * 3 * 4 <= kW, "add_nonfinite's masks");
 };
+
+// non-zero where a half of w is a BF16 infinity or NaN
+__device__ __forceinline__ uint32_t nonfinite2(uint32_t w) {
+    return ((w & 0x7fff7fffu) + 0x00800080u) & 0x80008000u;
+}
+__device__ __forceinline__ uint32_t nonfinite8(const uint4 v) {
+    return nonfinite2(v.x) | nonfinite2(v.y) | nonfinite2(v.z) | nonfinite2(v.w);
+}
+// the halves of w that are not finite replaced by 1 of their sign
+__device__ __forceinline__ uint32_t ones_for_nonfinite2(uint32_t w) {
+    const uint32_t m = (nonfinite2(w) >> 15) * 0x7fffu;
+    return (w & ~m) | (0x3f803f80u & m);
+}
+
+// The products of this CTA's activations that are not finite, into its weight
+// gradient wp[o][K]: a warp takes an activation and a tap that meets an output,
+// lane o its product with dz[o], an infinity or (with zero or NaN) a NaN. A sum of
+// such terms and finite ones only depends on which of them occur, so each is one
+// bit: mask [K][+Inf, -Inf, NaN], bit o. Runs only where the loader has met one.
+template <class N>
+__device__ __noinline__ void add_nonfinite(const uint16_t *act, const uint16_t *dz, int64_t B, int G,
+                                           int n_mine, uint32_t *mask, float *wp) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    for (int i = tid; i < N::K * 3; i += kBwdThreads) mask[i] = 0;
+    __syncthreads();
+    for (int k = 0; k < n_mine; ++k) {
+        const int64_t b0 = (blockIdx.x + int64_t(k) * gridDim.x) * G;
+        const int n = int(min(int64_t(G), B - b0)) * N::Pi;
+        const uint16_t *x = act + b0 * N::Pi * kTrainCh;
+        for (int q = warp; q < n; q += kBwdThreads / 32) {
+            const uint16_t mine = x[q * kTrainCh + lane];
+            uint32_t bad = __ballot_sync(kFull, (mine & 0x7f80u) == 0x7f80u);
+            const int w = q / N::Pi, p = q % N::Pi;
+            const int px = p % N::Si, py = p / N::Si % N::Si, pz = N::Dim == 3 ? p / (N::Si * N::Si) : 0;
+            for (; bad; bad &= bad - 1) {
+                const int c = __ffs(bad) - 1;
+                const float v = __uint_as_float(uint32_t(__shfl_sync(kFull, uint32_t(mine), c)) << 16);
+                for (int t = 0; t < N::Taps; ++t) {
+                    const int ox = px - t % 3, oy = py - t / 3 % 3, oz = N::Dim == 3 ? pz - t / 9 : 0;
+                    if (unsigned(ox) >= unsigned(N::So) || unsigned(oy) >= unsigned(N::So) ||
+                        unsigned(oz) >= unsigned(N::Dim == 3 ? N::So : 1))
+                        continue;
+                    uint32_t *m = mask + 3 * (c * N::Taps + t);
+                    if (*static_cast<volatile uint32_t *>(m + 2) == 0xffffffffu) continue;
+                    const int64_t r = (b0 + w) * N::Po + (oz * N::So + oy) * N::So + ox;
+                    const float s = v * __uint_as_float(uint32_t(dz[r * kTrainCh + lane]) << 16);
+                    const uint32_t pos = __ballot_sync(kFull, s > 0.f), neg = __ballot_sync(kFull, s < 0.f);
+                    if (lane == 0) {
+                        if (pos) atomicOr(m, pos);
+                        if (neg) atomicOr(m + 1, neg);
+                        if (~(pos | neg)) atomicOr(m + 2, ~(pos | neg));
+                    }
+                    __syncwarp();
+                }
+            }
+        }
+    }
+    __syncthreads();
+    for (int i = tid; i < N::K * kTrainCh; i += kBwdThreads) {
+        const uint32_t *m = mask + 3 * (i % N::K);
+        const int o = i / N::K;
+        const bool pos = (m[0] >> o) & 1u, neg = (m[1] >> o) & 1u, nan = (m[2] >> o) & 1u;
+        const float inf = __int_as_float(0x7f800000);
+        if (nan || (pos && neg))
+            wp[i] += inf - inf;
+        else if (pos || neg)
+            wp[i] += pos ? inf : -inf;
+    }
+}
 
 // Warp-uniform bounded wait for a phase that is a few hundred cycles away: polls
 // without the suspension of try_wait (104 cycles a poll of a warp, 215 with it).
@@ -733,6 +812,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
     uint32_t *hdone = full + 2, *freed = full + 4;
     uint32_t *slot = reinterpret_cast<uint32_t *>(smem + F::kSlot);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + F::kSlot + 4);
+    volatile int *bad_act = abort_flag + 1;
     float *red = reinterpret_cast<float *>(smem + F::kRed);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -740,6 +820,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
         for (int i = 0; i < F::Parts + 3; ++i) mbar_init(bars + i, 1u);
         for (int i = 0; i < 5; ++i) full[i] = 0;
         *abort_flag = 0;
+        *bad_act = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) tmem_alloc(slot, 512);
@@ -748,9 +829,13 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
     pdl_wait();
     for (int i = tid; i < F::Kw * kTrainCh * 2 / 16; i += kBwdThreads) cp_async16(wop + 16 * i, a.w + 16 * i);
     cp_async_wait_all();
+    // weights that are not finite (each thread looks at those it copied)
+    uint32_t bad = 0;
+    for (int i = tid; i < F::Kw * kTrainCh * 2 / 16; i += kBwdThreads)
+        bad |= nonfinite8(reinterpret_cast<const uint4 *>(wop)[i]);
     fence_async_smem();
     fence_before();
-    __syncthreads();
+    const bool bad_w = __syncthreads_or(bad != 0) != 0;
     fence_after();
     const uint32_t tmem = *slot;
     const int n_mine = int((a.tiles - 1 - blockIdx.x) / gridDim.x + 1);
@@ -854,6 +939,18 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
                 for (int c = 0; c < 3; ++c)
                     *reinterpret_cast<uint4 *>(zb + ((4 * c + (i & 3)) * F::RowsZ + F::Front + q + c * N::Si) * 16) = vz[j];
             }
+            // the largest half (activations come from a ReLU: none is negative)
+            uint32_t top = 0;
+            #pragma unroll
+            for (int j = 0; j < F::PieceA; ++j)
+                top = __vmaxu2(top, __vmaxu2(__vmaxu2(va[j].x, va[j].y), __vmaxu2(va[j].z, va[j].w)));
+            if (nonfinite2(top)) {
+                *bad_act = 1;
+                #pragma unroll
+                for (int j = 0; j < F::PieceA; ++j)
+                    va[j] = make_uint4(ones_for_nonfinite2(va[j].x), ones_for_nonfinite2(va[j].y),
+                                       ones_for_nonfinite2(va[j].z), ones_for_nonfinite2(va[j].w));
+            }
             #pragma unroll
             for (int j = 0; j < F::PieceA; ++j) {
                 const int i = lt + j * kBwdLoad * 32, q = i >> 2;
@@ -881,35 +978,55 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
                 float s[16];
                 #pragma unroll
                 for (int e = 0; e < 16; ++e) s[e] = 0.f;
-                #pragma unroll 1
-                for (int u = 0; u < F::Units && ok; ++u) {
-                    const int taps = min(F::UnitTaps, N::Taps - u * F::UnitTaps);
-                    #pragma unroll
-                    for (int g = 0; g < F::Parts; ++g) {
-                        // (the last unit may have a part less)
-                        if (3 * g >= taps) break;
-                        ok = spin_wait(bars + g, (ph >> g) & 1u, abort_flag, err);
-                        if (!ok) break;
-                        ph ^= 1u << g;
-                        fence_after();
-                        if (F::UnitTaps - 3 * g >= 3) {
-                            float v[3][16];
-                            tmem_ld16x3(tq + uint32_t(96 * g), v);
-                            #pragma unroll
-                            for (int i = 0; i < 3; ++i)
-                                #pragma unroll
-                                for (int e = 0; e < 16; ++e) s[e] += v[i][e];
-                        } else {
-                            float v[16];
-                            tmem_ld16(tq + uint32_t(96 * g), v);
-                            #pragma unroll
-                            for (int e = 0; e < 16; ++e) s[e] += v[e];
-                        }
+                // the sum of a position's T_t; masked: of the taps that meet an output
+                auto sum_taps = [&](auto m) {
+                    constexpr bool masked = decltype(m)::value;
+                    uint32_t meets = 0xffffffffu;        // bit t: tap t
+                    if (masked) {
+                        const int o = (128 * mt + 32 * wq + lane) % N::Pi;
+                        const int x = o % N::Si, y = o / N::Si % N::Si, z = o / (N::Si * N::Si);
+                        #pragma unroll
+                        for (int t = 0; t < N::Taps; ++t)
+                            if (unsigned(x - t % 3) >= unsigned(N::So) || unsigned(y - t / 3 % 3) >= unsigned(N::So) ||
+                                (N::Dim == 3 && unsigned(z - t / 9) >= unsigned(N::So)))
+                                meets &= ~(1u << t);
                     }
-                    fence_before();
-                    __syncwarp();
-                    if (lane == 0) red_release_add(freed, 1u);
-                }
+                    #pragma unroll 1
+                    for (int u = 0; u < F::Units && ok; ++u) {
+                        const int taps = min(F::UnitTaps, N::Taps - u * F::UnitTaps);
+                        #pragma unroll
+                        for (int g = 0; g < F::Parts; ++g) {
+                            // (the last unit may have a part less)
+                            if (3 * g >= taps) break;
+                            ok = spin_wait(bars + g, (ph >> g) & 1u, abort_flag, err);
+                            if (!ok) break;
+                            ph ^= 1u << g;
+                            fence_after();
+                            const uint32_t part = meets >> (u * F::UnitTaps + 3 * g);
+                            if (F::UnitTaps - 3 * g >= 3) {
+                                float v[3][16];
+                                tmem_ld16x3(tq + uint32_t(96 * g), v);
+                                #pragma unroll
+                                for (int i = 0; i < 3; ++i)
+                                    #pragma unroll
+                                    for (int e = 0; e < 16; ++e)
+                                        s[e] += !masked || ((part >> i) & 1u) ? v[i][e] : 0.f;
+                            } else {
+                                float v[16];
+                                tmem_ld16(tq + uint32_t(96 * g), v);
+                                #pragma unroll
+                                for (int e = 0; e < 16; ++e) s[e] += !masked || (part & 1u) ? v[e] : 0.f;
+                            }
+                        }
+                        fence_before();
+                        __syncwarp();
+                        if (lane == 0) red_release_add(freed, 1u);
+                    }
+                };
+                if (bad_w)
+                    sum_taps(std::true_type());
+                else
+                    sum_taps(std::false_type());
                 if (!ok) break;
                 const int p = 128 * mt + 32 * wq + lane, w = p / N::Pi, o = p % N::Pi;
                 const int x = o % N::Si - F::Ring, y = (o / N::Si) % N::Si - F::Ring;
@@ -989,6 +1106,11 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
         if (tid < kTrainCh) {
             const float *r = red + (tid / 16) * 64 + tid % 16;
             a.bpart[int64_t(blockIdx.x) * kTrainCh + tid] = ((r[0] + r[16]) + r[32]) + r[48];
+        }
+        if (*bad_act) {
+            __syncthreads();                             // the stage is read
+            add_nonfinite<N>(static_cast<const uint16_t *>(a.x), a.dz, a.B, a.G, n_mine,
+                             reinterpret_cast<uint32_t *>(smem), wp);
         }
     }
     fence_before();
@@ -1158,9 +1280,14 @@ __global__ void __launch_bounds__(256, 1) head_train_kernel(const HeadArgs a, in
                     }
                 }
                 if (a.tgt) {
+                    // rows past the batch are zero: they meet zeros, and
+                    // ReLU(b1) need not be finite
+                    const uint32_t keep = r < rows ? 0xffffffffu : 0u;
                     uint8_t *d = smem + S::kA5 + (n0 >> 3) * kChunk + r * 16;
-                    *reinterpret_cast<uint4 *>(d) = make_uint4(hv[0], hv[1], hv[2], hv[3]);
-                    *reinterpret_cast<uint4 *>(d + kChunk) = make_uint4(hv[4], hv[5], hv[6], hv[7]);
+                    *reinterpret_cast<uint4 *>(d) =
+                        make_uint4(hv[0] & keep, hv[1] & keep, hv[2] & keep, hv[3] & keep);
+                    *reinterpret_cast<uint4 *>(d + kChunk) =
+                        make_uint4(hv[4] & keep, hv[5] & keep, hv[6] & keep, hv[7] & keep);
                 }
             }
             fence_before();
