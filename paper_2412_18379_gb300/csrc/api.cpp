@@ -306,7 +306,6 @@ cs_status cs_mesh_upload(cs_ctx *ctx, int dim, int64_t n_v, const double *xyz, i
     d.iperm = iperm;
     d.node_elem = node;
     d.xyz = xyzd;
-    d.vhost = nullptr;
     d.seed = seed;
     d.pool = pool;
     d.pool_f = pool_f;
@@ -330,6 +329,7 @@ cs_status cs_mesh_upload(cs_ctx *ctx, int dim, int64_t n_v, const double *xyz, i
         d.hi_m[k] = d.hi[k] + d.margin;
     }
     d.tau = H.tau;
+    d.rest = H.rest;
     d.cap = H.cap;
     d.n_asg = n_asg;
     d.n_bucket = n_b;
@@ -345,19 +345,14 @@ cs_status cs_mesh_upload(cs_ctx *ctx, int dim, int64_t n_v, const double *xyz, i
     d.pseed = seed;
 
     ctx->launches += cs::launch_seed_grid(d, seed, ctx->sm_count, nullptr);
-    // 3-D: hosts of the vertices, where memory (or the budget) has room for them;
-    // the walk does without, only slower at nodes at rest. In 2-D, where few
-    // elements meet at a node, reading them costs the walk more than it saves.
-    int2 *vhost = nullptr;
-    if (dim == 3 && dev_copy<int2>(ctx, m, nullptr, size_t(n_v), &vhost) == CS_OK) {
-        ctx->launches += cs::launch_vertex_hosts(d, vhost, ctx->sm_count, nullptr);
-        d.vhost = vhost;
-    }
+    // In 2-D, where few elements meet at a node, looking there costs the walk more
+    // than the searches it saves.
+    if (dim == 3) ctx->launches += cs::launch_settle_vertices(d, node, ctx->sm_count, nullptr);
     cudaError_t e = cudaDeviceSynchronize();
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
         free_mesh(ctx, m);
-        return cuda_fail(ctx, e, "seed grid kernel");
+        return cuda_fail(ctx, e, "seed grid and vertex kernels");
     }
 
     cs_mesh_info &I = m->info;

@@ -653,7 +653,7 @@ __global__ void __launch_bounds__(kT) start_kernel(const DevMesh m, int64_t n,
             if (fallback) {
                 s = fallback[i];
             } else {
-                const int32_t e = m.node_elem[row0 + i];
+                const int32_t e = node_start(m.node_elem[row0 + i]);
                 s = e < 0 ? -1 : walk_uid<D>(m.recw, e);
             }
         }

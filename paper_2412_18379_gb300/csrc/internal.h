@@ -32,7 +32,7 @@ struct Server;   // serve.cpp
 // main: all but the struct's last 16 bytes, which are the tail. L1 busy 66% of a
 // plain 2-D step, 76% before: 81.1 -> 79.2 us on 1001^2 nodes, 3-D element-node
 // pairs 177 -> 174 us; a CNN-started 2-D step, whose walks take 1.7 steps, 66.7 ->
-// 66.9 us.
+// 66.9 us. An odd last record ends with its tail.
 //
 // The exact record holds v0 and M in FP64 (row k of M gives
 // lambda_{k+1} = M[k] . (x_p - v0)); it is read only when the FP32 filter
@@ -74,7 +74,14 @@ CS_HD inline int64_t walk_main(int dim, int64_t e) {
 CS_HD inline int64_t walk_tail(int dim, int64_t e) {
     return dim == 2 ? (e >> 1) * 96 + 32 + (e & 1) * 16 : (e >> 1) * 160 + 64 + (e & 1) * 16;
 }
-CS_HD inline int64_t walk_bytes(int dim, int64_t n_e) { return (n_e + 1) / 2 * (dim == 2 ? 96 : 160); }
+CS_HD inline int64_t walk_bytes(int dim, int64_t n_e) { return n_e * (dim == 2 ? 48 : 80); }
+
+// DevMesh::node_elem of a vertex: the internal id of its plain-SNS start e (the
+// incident element of the lowest user id), -1 without one, or -2 - e where that
+// element is also the host of every point within DevMesh::rest of the vertex on
+// each axis (3-D; search.cu)
+CS_HD inline int32_t node_start(int32_t s) { return s < -1 ? -2 - s : s; }
+CS_HD inline bool node_settled(int32_t s) { return s < -1; }
 
 // Everything a kernel needs to know about a resident mesh (passed by value).
 struct DevMesh {
@@ -85,11 +92,9 @@ struct DevMesh {
     const int32_t *conn;      // [n_e][dim+1] vertex ids, internal order
     const double *centroid;   // [n_e][dim], internal order
     const int32_t *iperm;     // user id -> internal id
-    const int32_t *node_elem; // [n_v] internal id of the plain-SNS start
+    const int32_t *node_elem; // [n_v] the plain-SNS start (node_start), and whether it
+                              // is the host of the points around (node_settled)
     const double *xyz;        // [n_v][dim] the uploaded vertices, user order
-    const int2 *vhost;        // [n_v] host (user id, or -1) of every point within (float
-                              // bits) .y of the vertex on each axis; .y < 0: unknown.
-                              // null: not resident (the walk searches instead)
     const int32_t *seed;      // [n_asg] internal id of the host of each cell centre, or -1
     const double *pool;       // [n_asg][dim] mean element centroid per ASG cell, NaN if none
     const float *pool_f;      // [n_asg][dim][2] the same as float hi + lo (NaN hi if none)
@@ -106,6 +111,7 @@ struct DevMesh {
     double margin;            // bucket boxes are grown by this much
     double lo_m[3], hi_m[3];  // lo - margin, hi + margin: no host beyond these
     double tau;               // canonicalisation threshold
+    double rest;              // half-width of the boxes of settled vertices
     int32_t cap;              // step cap
     int64_t n_asg, n_bucket;
     // predictor grid: cells of pstride^dim ASG cells (pstride odd), aligned at
@@ -238,7 +244,7 @@ struct HostMesh {
     double lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
     int32_t ga[3] = {1, 1, 1}, gb[3] = {1, 1, 1};
     double sa[3] = {1, 1, 1}, sb[3] = {1, 1, 1};
-    double margin = 0, tau = 0;
+    double margin = 0, tau = 0, rest = 0;
     int32_t cap = 0;
 };
 cs_status build_host_mesh(int dim, int64_t n_v, const double *xyz, int64_t n_e,
@@ -278,7 +284,8 @@ struct Profiler {
 int launch_track(const DevMesh &m, const TrackArgs &a, Scratch &s, int sm_count,
                  cudaStream_t st, Profiler *prof = nullptr);
 int launch_seed_grid(const DevMesh &m, int32_t *seed, int sm_count, cudaStream_t st);
-int launch_vertex_hosts(const DevMesh &m, int2 *vhost, int sm_count, cudaStream_t st);
+// marks the settled vertices in node_elem (3-D)
+int launch_settle_vertices(const DevMesh &m, int32_t *node_elem, int sm_count, cudaStream_t st);
 int launch_stats(int64_t n, const int32_t *path, const uint8_t *status, int64_t *out,
                  int sm_count, cudaStream_t st);
 int launch_error_stats(const DevMesh &m, int64_t n, const int32_t *start, const int32_t *host,

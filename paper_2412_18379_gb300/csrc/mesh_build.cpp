@@ -337,6 +337,9 @@ cs_status build_host_mesh(int dim, int64_t n_v, const double *xyz, int64_t n_e,
         hi = static_cast<float>(v);
         lo = static_cast<float>(v - static_cast<double>(hi));
     };
+    // how many elements have a sum |M| in each bucket of its exponent and three
+    // bits: what 99.9% of them stay below bounds the boxes of settled vertices
+    std::vector<int64_t> norms(dim == 3 ? size_t(1) << 14 : 0, 0);
     // a record into its two places of the paired layout
     auto put = [&](int64_t i, const void *w, size_t main) {
         std::memcpy(&H.recw[size_t(walk_main(dim, i))], w, main);
@@ -372,9 +375,25 @@ cs_status build_host_mesh(int dim, int64_t n_v, const double *xyz, int64_t n_e,
             w.uid = int32_t(l);
             put(i, &w, sizeof(w) - 16);
             std::memcpy(&H.recx[size_t(i) * xb], &x, xb);
+            double sum = 0;
+            for (int k = 0; k < 9; ++k) sum += std::fabs(x.m[k]);
+            uint64_t bits;
+            std::memcpy(&bits, &sum, sizeof(bits));
+            norms[size_t(bits >> 49) & 0x3fff] += 1;
         }
         for (int k = 0; k < nv; ++k) H.conn[i * nv + k] = conn_user[l * nv + k];
         for (int k = 0; k < dim; ++k) H.centroid[i * dim + k] = cent[l * dim + k];
+    }
+
+    if (dim == 3) {
+        // the upper bound of the bucket that the 99.9% end in
+        int64_t below = 0;
+        uint64_t b = 0;
+        while (b + 1 < norms.size() && (below += norms[b]) * 1000 < n_e * 999) ++b;
+        const uint64_t bits = (b + 1) << 49;
+        double top;
+        std::memcpy(&top, &bits, sizeof(top));
+        H.rest = 0.35 * CS_EPS / top;      // 0, or NaN (no vertex settles), if top is not finite
     }
 
     // ---- exact-search bucket index (internal ids) ----

@@ -39,8 +39,8 @@ __global__ void __launch_bounds__(256) seed_kernel(const DevMesh m, int32_t *see
     }
 }
 
-// The host of the points around every vertex. For vertex v with candidates e
-// (the elements of its bucket cell) and their FP64 coordinates at v:
+// The vertices whose surroundings have a host that is known (3-D). For vertex v
+// with candidates e (the elements of its bucket cell) and their FP64 coordinates at v:
 //   slack(e) = min_i lambda_i + eps      if e contains v (every lambda >= -eps)
 //            = max_i -eps - lambda_i     otherwise
 // is how far e's answer is from changing. Moving a point by at most r per axis
@@ -49,61 +49,61 @@ __global__ void __launch_bounds__(256) seed_kernel(const DevMesh m, int32_t *see
 // 1e-14 (1 + S), S = sum |M| |v - v0|. So no candidate's answer changes within
 //   r = min_e (slack / 2 - 1e-14 (1 + S)) / N, at most margin / 4:
 // every point there has v's containing elements, hence its host, the lowest
-// user id among them. (An element that is no candidate of v's cell has a box,
-// grown by margin, that misses v; it cannot contain a point within margin / 4 of
-// v either: containment to eps reaches eps times its extent past its box, far
-// below the margin.) r is rounded down to float; < 0 where some answer is too
-// close to call. Particles at rest at a node (no-slip walls, stagnation points)
-// end their walk at such a point.
-template <int D>
-__global__ void __launch_bounds__(256) vertex_host_kernel(const DevMesh m, int2 *vhost) {
+// user id among them. (An element that is no candidate of v's cell has its box, or
+// a face plane of it, clear of the cell grown by margin; it cannot contain a point
+// within margin / 4 of v either: containment to eps reaches eps times its extent
+// past its faces, far below the margin.)
+//
+// The vertex is settled where r is at least the mesh's `rest` and that host is
+// the vertex's plain-SNS start, the incident element of the lowest id, so that the
+// mark is a sign in an array the mesh holds anyway. (A host and radius of its own
+// per vertex answered no more of the particles at rest, whose distance is rounding:
+// 8 bytes a vertex for the same 58 us.) rest is what 99.9% of the elements allow: incident
+// ones have slack eps and S about 10, so r is about 0.39 eps / N.
+__global__ void __launch_bounds__(256) settle_kernel(const DevMesh m, int32_t *node_elem) {
+    constexpr int D = 3;
     using XR = typename Recs<D>::X;
     const int lane = threadIdx.x & 31;
     const int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
     for (int64_t v = warp; v < m.n_v; v += nwarps) {
+        const int32_t start = node_elem[v];
+        if (start < 0) continue;
         double x[D];
-        bool finite = true;
         #pragma unroll
-        for (int k = 0; k < D; ++k) {
-            x[k] = __ldg(m.xyz + v * D + k);
-            finite = finite && finite_bits(x[k]);
-        }
+        for (int k = 0; k < D; ++k) x[k] = __ldg(m.xyz + v * D + k);
         unsigned best = 0xffffffffu;
-        double r = finite ? m.margin * 0.25 : -1.0;
-        if (finite) {
-            const int64_t c = grid_cell<D>(x, m.lo, m.sb, m.gb);
-            const int32_t t1 = __ldg(m.bstart + c + 1);
-            for (int32_t t = __ldg(m.bstart + c) + lane; t < t1; t += 32) {
-                const int32_t e = __ldg(m.bitems + t);
-                const double *p = reinterpret_cast<const double *>(static_cast<const XR *>(m.recx) + e);
-                double lam[D + 1];
-                bary64(static_cast<const XR *>(m.recx), e, x, lam);
-                double lo = lam[0];
+        double r = m.margin * 0.25;
+        const int64_t c = grid_cell<D>(x, m.lo, m.sb, m.gb);
+        const int32_t t1 = __ldg(m.bstart + c + 1);
+        for (int32_t t = __ldg(m.bstart + c) + lane; t < t1; t += 32) {
+            const int32_t e = __ldg(m.bitems + t);
+            const double *p = reinterpret_cast<const double *>(static_cast<const XR *>(m.recx) + e);
+            double lam[D + 1];
+            bary64(static_cast<const XR *>(m.recx), e, x, lam);
+            double lo = lam[0];
+            #pragma unroll
+            for (int i = 1; i <= D; ++i) lo = fmin(lo, lam[i]);
+            double N = 0.0, S = 0.0;
+            #pragma unroll
+            for (int i = 0; i < D; ++i)
                 #pragma unroll
-                for (int i = 1; i <= D; ++i) lo = fmin(lo, lam[i]);
-                double N = 0.0, S = 0.0;
-                #pragma unroll
-                for (int i = 0; i < D; ++i)
-                    #pragma unroll
-                    for (int k = 0; k < D; ++k) {
-                        const double a = fabs(p[D + i * D + k]);
-                        N += a;
-                        S += a * fabs(x[k] - p[k]);
-                    }
-                const bool in = lo >= -CS_EPS;
-                const double slack = in ? lo + CS_EPS : -CS_EPS - lo;
-                r = fmin(r, (0.5 * slack - 1e-14 * (1.0 + S)) / N);
-                if (!(slack >= 0.0)) r = -1.0;     // NaN
-                if (in) best = min(best, unsigned(walk_uid<D>(m.recw, e)));
-            }
+                for (int k = 0; k < D; ++k) {
+                    const double a = fabs(p[D + i * D + k]);
+                    N += a;
+                    S += a * fabs(x[k] - p[k]);
+                }
+            const bool in = lo >= -CS_EPS;
+            const double slack = in ? lo + CS_EPS : -CS_EPS - lo;
+            const double re = (0.5 * slack - 1e-14 * (1.0 + S)) / N;
+            r = re >= 0.0 ? fmin(r, re) : -1.0;        // NaN too
+            if (in) best = min(best, unsigned(walk_uid<D>(m.recw, e)));
         }
         best = __reduce_min_sync(kFull, best);
         #pragma unroll
         for (int o = 16; o > 0; o >>= 1) r = fmin(r, __shfl_xor_sync(kFull, r, o));
-        if (lane == 0)
-            vhost[v] = make_int2(best == 0xffffffffu ? -1 : int32_t(best),
-                                 __float_as_int(r > 0.0 ? __double2float_rd(r) : -1.0f));
+        if (lane == 0 && r >= m.rest && best == unsigned(walk_uid<D>(m.recw, start)))
+            node_elem[v] = -2 - start;
     }
 }
 
@@ -241,9 +241,8 @@ int launch_seed_grid(const DevMesh &m, int32_t *seed, int sm_count, cudaStream_t
     return 1;
 }
 
-int launch_vertex_hosts(const DevMesh &m, int2 *vhost, int sm_count, cudaStream_t st) {
-    const int grid = sm_count * 8;
-    vertex_host_kernel<3><<<grid, 256, 0, st>>>(m, vhost);
+int launch_settle_vertices(const DevMesh &m, int32_t *node_elem, int sm_count, cudaStream_t st) {
+    settle_kernel<<<sm_count * 8, 256, 0, st>>>(m, node_elem);
     return 1;
 }
 

@@ -127,7 +127,7 @@ __device__ __forceinline__ void prepare(const DevMesh &m, const TrackArgs &a, in
             const int32_t su = kPrefetch<D> ? f.start[lane] : __ldg(a.start_user + pp);
             plain = (su >= 0 && su < m.n_e) ? __ldg(m.iperm + su) : -1;
         } else {
-            plain = kPrefetch<D> ? f.start[lane] : __ldg(m.node_elem + pp);
+            plain = node_start(kPrefetch<D> ? f.start[lane] : __ldg(m.node_elem + pp));
         }
         s = plain;
         int64_t c1 = -1;    // ASG cell whose seed starts the walk (ASG, CNN-SNS)
@@ -178,30 +178,26 @@ __device__ __forceinline__ void prepare(const DevMesh &m, const TrackArgs &a, in
     }
 }
 
-// The host of x_p when x_p lies so close to a vertex of element cur that the
-// mesh's table answers for it (search.cu); kNoVertex otherwise. Particles at
-// rest at a node (no-slip walls, stagnation points) end there, where many
-// elements meet. A line of wall nodes ends 32 walks of one warp so, each of
-// which took the whole warp through a search: on the 75^3 nodes of a cube, the
-// 884 on its edges alone took 243 us (58 now), and the CNN-SNS step 250 us
-// (116 now).
+// The host of x_p when x_p lies so close to vertex i of element cur, a settled
+// one, that it is the vertex's (search.cu); kNoVertex otherwise. Particles at rest
+// at a node (no-slip walls, stagnation points) end there, where many elements meet.
+// A line of wall nodes ends 32 walks of one warp so, each of which took the whole
+// warp through a search: on the 75^3 nodes of a cube, the 884 on its edges alone
+// took 243 us (58 now), and the CNN-SNS step 250 us (116 now). Bound by the
+// latency of its dependent loads: looking at all of the element's vertices, not
+// the one of the largest coordinate, took 5 us more.
 constexpr int32_t kNoVertex = INT32_MIN;
 template <int D>
-__device__ __forceinline__ int32_t vertex_host(const DevMesh &m, int32_t cur, const double *xp) {
-    int32_t host = kNoVertex;
-    if (!m.vhost) return host;
+__device__ __forceinline__ int32_t vertex_host(const DevMesh &m, int32_t cur, int i, const double *xp) {
+    const int32_t v = __ldg(m.conn + int64_t(cur) * (D + 1) + i);
+    const int32_t s = __ldg(m.node_elem + v);
+    double x[D];
     #pragma unroll
-    for (int i = 0; i <= D; ++i) {
-        const int32_t v = __ldg(m.conn + int64_t(cur) * (D + 1) + i);
-        const int2 h = __ldg(m.vhost + v);
-        const double r = double(__int_as_float(h.y));
-        bool close = true;
-        #pragma unroll
-        for (int k = 0; k < D; ++k)
-            close = close && fabs(__dsub_rn(xp[k], __ldg(m.xyz + int64_t(v) * D + k))) <= r;
-        if (close) host = h.x;
-    }
-    return host;
+    for (int k = 0; k < D; ++k) x[k] = __ldg(m.xyz + int64_t(v) * D + k);
+    bool close = node_settled(s);
+    #pragma unroll
+    for (int k = 0; k < D; ++k) close &= fabs(__dsub_rn(xp[k], x[k])) <= m.rest;
+    return close ? walk_uid<D>(m.recw, node_start(s)) : kNoVertex;
 }
 
 template <int D>
@@ -298,6 +294,7 @@ __global__ void __launch_bounds__(256, D == 2 ? 4 : 3) walk_kernel(const DevMesh
 
         // ---- one step of Algorithm 1 for every busy lane ----
         bool done = false, search = false, found = false;
+        int corner = 0;             // vertex of the largest coordinate
         if (p >= 0) {
             WalkE<D> e;
             load_walk(rw, cur, e);
@@ -384,6 +381,15 @@ __global__ void __launch_bounds__(256, D == 2 ? 4 : 3) walk_kernel(const DevMesh
                 a.status[p] = CS_FOUND;
                 done = found = true;
                 search = near;      // another element may contain x_p too
+                if (D == 3 && near) {
+                    float top = lf[0];
+                    #pragma unroll
+                    for (int i = 1; i <= D; ++i)
+                        if (lf[i] > top) {
+                            top = lf[i];
+                            corner = i;
+                        }
+                }
             } else if (next < 0 || it >= m.cap) {
                 a.path[p] = it;     // left the mesh or reached the step cap
                 done = true;
@@ -393,8 +399,8 @@ __global__ void __launch_bounds__(256, D == 2 ? 4 : 3) walk_kernel(const DevMesh
             }
         }
         if (D == 3 && search && found) {
-            // close to a vertex of the final element the mesh knows the host
-            const int32_t h = vertex_host<D>(m, cur, xp);
+            // close to a settled vertex of the final element the host is known
+            const int32_t h = vertex_host<D>(m, cur, corner, xp);
             if (h != kNoVertex) {
                 a.host[p] = h;
                 search = false;
