@@ -99,28 +99,44 @@ cs_status ensure_scratch(cs_ctx *ctx) {
 
 }  // namespace
 
-cs_status cs::dmalloc(cs_ctx *ctx, void **p, size_t bytes) {
-    *p = nullptr;
+namespace {
+
+// one attempt at a block; "" or why it failed
+std::string try_malloc(cs_ctx *ctx, void **p, size_t bytes) {
     {
         std::lock_guard<std::mutex> lock(ctx->hbm_mu);
         if (ctx->hbm_budget && ctx->hbm_used + bytes > ctx->hbm_budget)
-            return fail(ctx, CS_ENOMEM, "device allocation of " + std::to_string(bytes) +
-                                            " bytes would pass the context's HBM budget (" +
-                                            std::to_string(ctx->hbm_used) + " of " +
-                                            std::to_string(ctx->hbm_budget) + " bytes in use)");
+            return "device allocation of " + std::to_string(bytes) +
+                   " bytes would pass the context's HBM budget (" + std::to_string(ctx->hbm_used) +
+                   " of " + std::to_string(ctx->hbm_budget) + " bytes in use)";
         ctx->hbm_used += bytes;   // reserved while cudaMalloc runs
     }
     void *q = nullptr;
-    if (cudaMalloc(&q, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        std::lock_guard<std::mutex> lock(ctx->hbm_mu);
-        ctx->hbm_used -= bytes;
-        return fail(ctx, CS_ENOMEM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed");
-    }
+    const bool ok = cudaMalloc(&q, bytes) == cudaSuccess;
+    if (!ok) cudaGetLastError();
     std::lock_guard<std::mutex> lock(ctx->hbm_mu);
+    if (!ok) {
+        ctx->hbm_used -= bytes;
+        return "cudaMalloc of " + std::to_string(bytes) + " bytes failed";
+    }
     ctx->hbm_blocks[q] = bytes;
     *p = q;
-    return CS_OK;
+    return "";
+}
+
+}  // namespace
+
+thread_local uint32_t cs::workspace_use = 0;
+
+cs_status cs::dmalloc(cs_ctx *ctx, void **p, size_t bytes) {
+    *p = nullptr;
+    std::string why = try_malloc(ctx, p, bytes);
+    if (!why.empty()) {
+        // cudaFree waits for what still runs in a workspace
+        const bool a = cs::predictor_reclaim(ctx), b = cs::classifier_reclaim(ctx);
+        if (a || b) why = try_malloc(ctx, p, bytes);
+    }
+    return why.empty() ? CS_OK : fail(ctx, CS_ENOMEM, why);
 }
 
 void cs::dfree(cs_ctx *ctx, void *p) {

@@ -50,11 +50,11 @@ struct Classifier {
     int64_t n = 0;
     float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr, *loss = nullptr;
     int64_t t = 0;
-    // workspace: the fully connected layers' buffers for `cap` rows, the
-    // unfused module 1's for `cap_conv` rows and the backward pass's for
-    // `cap_grad` rows (0 until a path needs them): the fused inference path
-    // runs long chunks without growing the training path's im2col buffers
-    int64_t cap = 0, cap_conv = 0, cap_grad = 0;
+    // workspace of the layer-by-layer path: the fully connected layers' buffers for
+    // cap rows, the unfused module 1's for cap_conv rows, their backward passes' for
+    // cap_grad and cap_gconv rows (0 until a path needs them; a tiled step in 3-D
+    // takes module 1's alone)
+    int64_t cap = 0, cap_conv = 0, cap_grad = 0, cap_gconv = 0;
     std::vector<void *> ws;
     float *a0 = nullptr, *off = nullptr, *col1 = nullptr, *z1 = nullptr, *y1 = nullptr,
           *a1 = nullptr, *col2 = nullptr, *z2 = nullptr, *cat = nullptr, *h1 = nullptr,
@@ -127,7 +127,7 @@ void free_ws(cs_ctx *ctx, Classifier &C) {
     C.idx = nullptr;
     C.splitk = nullptr;
     C.splitk_n = 0;
-    C.cap = C.cap_conv = C.cap_grad = 0;
+    C.cap = C.cap_conv = C.cap_grad = C.cap_gconv = 0;
 }
 
 void free_list(cs_ctx *ctx, std::vector<void *> &v) {
@@ -143,6 +143,12 @@ void free_fc(cs_ctx *ctx, Classifier &C) {
     C.tidx = nullptr;
     C.fc_cap = 0;
     C.fc_grad = false;
+}
+
+void free_parts(cs_ctx *ctx, Classifier &C) {
+    dfree(ctx, C.parts);
+    C.parts = nullptr;
+    C.parts_cap = 0;
 }
 
 void free_tr(cs_ctx *ctx, Classifier &C) {
@@ -204,21 +210,13 @@ struct FcPlan {
     }
 };
 
-// buffers of the tiled fully connected layers for B rows
-cs_status ensure_fc(cs_ctx *ctx, Classifier &C, int64_t B, bool grad) {
-    cs_status rc = ensure_err(ctx);
-    if (rc) return rc;
-    const ClsShape S(C.dim);
-    if (!C.fcpack) {
-        if ((rc = dmalloc_n(ctx, &C.fcpack, size_t(FcPlan(S, 1, ctx->sm_count).bytes)))) return rc;
-        C.pack_bn[0] = 0;
-    }
-    if (C.fc_cap >= B && (!grad || C.fc_grad)) return CS_OK;
-    const int64_t cap = std::max(B, C.fc_cap);
-    const bool g = grad || C.fc_grad;
+// buffers of the tiled fully connected layers for `cap` rows, anew
+cs_status alloc_fc(cs_ctx *ctx, Classifier &C, int64_t cap, bool g) {
     free_fc(ctx, C);
+    const ClsShape S(C.dim);
     auto &v = C.fcws;
     const int np = fc_kp(S.n_cls);
+    cs_status rc;
     if ((rc = list_alloc(ctx, v, &C.tcat, fc_bytes(cap, S.ldc))) ||
         (rc = list_alloc(ctx, v, &C.tr1, fc_bytes(cap, kClsH1))) ||
         (rc = list_alloc(ctx, v, &C.tru, fc_bytes(cap, kClsH2))) ||
@@ -238,9 +236,23 @@ cs_status ensure_fc(cs_ctx *ctx, Classifier &C, int64_t B, bool grad) {
     return CS_OK;
 }
 
+cs_status ensure_fc(cs_ctx *ctx, Classifier &C, int64_t B, bool grad) {
+    cs_status rc = ensure_err(ctx);
+    if (rc) return rc;
+    use_workspace(C.dim, kUseFc);
+    const ClsShape S(C.dim);
+    if (!C.fcpack) {
+        if ((rc = dmalloc_n(ctx, &C.fcpack, size_t(FcPlan(S, 1, ctx->sm_count).bytes)))) return rc;
+        C.pack_bn[0] = 0;
+    }
+    if (C.fc_cap >= B && (!grad || C.fc_grad)) return CS_OK;
+    return alloc_fc(ctx, C, std::max(B, C.fc_cap), grad || C.fc_grad);
+}
+
 // buffers of module 1 of a 2-D training step
 cs_status ensure_tr(cs_ctx *ctx, Classifier &C, int64_t B) {
-    if (C.dim != 2 || C.tr_cap >= B) return CS_OK;
+    use_workspace(C.dim, kUseTrain);
+    if (C.tr_cap >= B) return CS_OK;
     free_tr(ctx, C);
     const ClsShape S(2);
     auto &v = C.trws;
@@ -263,61 +275,91 @@ cs_status ensure_tr(cs_ctx *ctx, Classifier &C, int64_t B) {
     return CS_OK;
 }
 
-// workspace for B rows of the fully connected layers; `conv` adds the
-// unfused module 1's buffers and the GEMMs' K splits (no product of the fully
-// connected layers alone splits its K off the tensor cores), `grad` the backward
-// pass's (which reuses module 1's, so it needs `conv` too). Growing any set
-// reallocates all of them, each at its own row count.
-cs_status ensure_ws(cs_ctx *ctx, Classifier &C, int64_t B, bool conv, bool grad) {
-    cs_status rc0 = ensure_err(ctx);
-    if (rc0) return rc0;
-    conv = conv || grad;
-    if (C.cap >= B && (!conv || C.cap_conv >= B) && (!grad || C.cap_grad >= B)) return CS_OK;
-    const int64_t rows = std::max(B, C.cap);
-    const int64_t rows_conv = conv ? std::max(B, C.cap_conv) : C.cap_conv;
-    const int64_t rows_grad = grad ? std::max(B, C.cap_grad) : C.cap_grad;
+// Workspace of the layer-by-layer path for B rows of the named parts: the fully
+// connected layers, module 1 (with the GEMMs' K splits; no product of the layers
+// alone splits its K off the tensor cores), and their backward passes (module 1's
+// reuses its forward buffers). Growing any part reallocates all of them, each at
+// its own row count.
+enum : unsigned { kWsFc = 1, kWsConv = 2, kWsFcGrad = 4, kWsConvGrad = 8 };
+constexpr unsigned kWsAll = kWsFc | kWsConv | kWsFcGrad | kWsConvGrad;
+
+// K splits of module 1's products alone: at most three of a forward product of
+// less than two waves of tiles, 128 x 32 floats each (the weight gradients', of at
+// most 32 x 864, take less)
+int64_t conv_splitk_floats(int sm_count) { return int64_t(3) * 2 * sm_count * 128 * kClsCh; }
+
+// the parts at rows[0..3] and a K-split workspace of sk floats, all anew
+cs_status alloc_ws(cs_ctx *ctx, Classifier &C, const int64_t (&rows)[4], int64_t sk) {
     free_ws(ctx, C);
     const ClsShape S(C.dim);
     const int64_t d = C.dim, K1 = d * S.taps, K2 = int64_t(kClsCh) * S.taps;
-    cs_status rc;
-    if ((rc = ws_alloc(ctx, C, &C.off, rows * d)) || (rc = ws_alloc(ctx, C, &C.cat, rows * S.ldc)) ||
-        (rc = ws_alloc(ctx, C, &C.h1, rows * kClsH1)) ||
-        (rc = ws_alloc(ctx, C, &C.r1, rows * kClsH1)) ||
-        (rc = ws_alloc(ctx, C, &C.h2, rows * kClsH1)) ||
-        (rc = ws_alloc(ctx, C, &C.u, rows * kClsH2)) ||
-        (rc = ws_alloc(ctx, C, &C.ru, rows * kClsH2)) ||
-        (rc = ws_alloc(ctx, C, &C.H, rows * S.n_cls))) {
+    const int64_t r = rows[0], rv = rows[1], rg = rows[2], rgv = rows[3];
+    cs_status rc = CS_OK;
+    if ((r > 0 && ((rc = ws_alloc(ctx, C, &C.off, r * d)) || (rc = ws_alloc(ctx, C, &C.cat, r * S.ldc)) ||
+                   (rc = ws_alloc(ctx, C, &C.h1, r * kClsH1)) ||
+                   (rc = ws_alloc(ctx, C, &C.r1, r * kClsH1)) ||
+                   (rc = ws_alloc(ctx, C, &C.h2, r * kClsH1)) ||
+                   (rc = ws_alloc(ctx, C, &C.u, r * kClsH2)) ||
+                   (rc = ws_alloc(ctx, C, &C.ru, r * kClsH2)) ||
+                   (rc = ws_alloc(ctx, C, &C.H, r * S.n_cls)))) ||
+        (sk > 0 && (rc = ws_alloc(ctx, C, &C.splitk, sk))) ||
+        (rv > 0 && ((rc = ws_alloc(ctx, C, &C.a0, rv * d * S.Pq)) ||
+                    (rc = ws_alloc(ctx, C, &C.col1, rv * S.P * K1)) ||
+                    (rc = ws_alloc(ctx, C, &C.z1, rv * S.P * kClsCh)) ||
+                    (rc = ws_alloc(ctx, C, &C.y1, rv * S.P * kClsCh)) ||
+                    (rc = ws_alloc(ctx, C, &C.a1, rv * S.Pq * kClsCh)) ||
+                    (rc = ws_alloc(ctx, C, &C.col2, rv * S.P * K2)) ||
+                    (rc = ws_alloc(ctx, C, &C.z2, rv * S.P * kClsCh)))) ||
+        (rg > 0 && ((rc = ws_alloc(ctx, C, &C.gH, rg * S.n_cls)) ||
+                    (rc = ws_alloc(ctx, C, &C.gu, rg * kClsH2)) ||
+                    (rc = ws_alloc(ctx, C, &C.gcat, rg * S.ldc)) ||
+                    (rc = ws_alloc(ctx, C, &C.gh2, rg * kClsH1)) ||
+                    (rc = ws_alloc(ctx, C, &C.gh1, rg * kClsH1)) || (rc = ws_alloc(ctx, C, &C.idx, rg)))) ||
+        (rgv > 0 && (rc = ws_alloc(ctx, C, &C.gz2, rgv * S.P * kClsCh)))) {
         free_ws(ctx, C);
         return rc;
     }
-    const int64_t rv = rows_conv;
-    if (rv > 0 &&
-        ((rc = ws_alloc(ctx, C, &C.splitk, tc_gemm_work_floats(ctx->sm_count))) ||
-         (rc = ws_alloc(ctx, C, &C.a0, rv * d * S.Pq)) ||
-         (rc = ws_alloc(ctx, C, &C.col1, rv * S.P * K1)) ||
-         (rc = ws_alloc(ctx, C, &C.z1, rv * S.P * kClsCh)) ||
-         (rc = ws_alloc(ctx, C, &C.y1, rv * S.P * kClsCh)) ||
-         (rc = ws_alloc(ctx, C, &C.a1, rv * S.Pq * kClsCh)) ||
-         (rc = ws_alloc(ctx, C, &C.col2, rv * S.P * K2)) ||
-         (rc = ws_alloc(ctx, C, &C.z2, rv * S.P * kClsCh)))) {
-        free_ws(ctx, C);
-        return rc;
-    }
-    const int64_t rg = rows_grad;
-    if (rg > 0 &&
-        ((rc = ws_alloc(ctx, C, &C.gH, rg * S.n_cls)) || (rc = ws_alloc(ctx, C, &C.gu, rg * kClsH2)) ||
-         (rc = ws_alloc(ctx, C, &C.gcat, rg * S.ldc)) ||
-         (rc = ws_alloc(ctx, C, &C.gh2, rg * kClsH1)) ||
-         (rc = ws_alloc(ctx, C, &C.gh1, rg * kClsH1)) ||
-         (rc = ws_alloc(ctx, C, &C.gz2, rg * S.P * kClsCh)) || (rc = ws_alloc(ctx, C, &C.idx, rg)))) {
-        free_ws(ctx, C);
-        return rc;
-    }
-    C.splitk_n = rv > 0 ? tc_gemm_work_floats(ctx->sm_count) : 0;
-    C.cap = rows;
-    C.cap_conv = rows_conv;
-    C.cap_grad = rows_grad;
+    C.splitk_n = sk;
+    C.cap = r;
+    C.cap_conv = rv;
+    C.cap_grad = rg;
+    C.cap_gconv = rgv;
     return CS_OK;
+}
+
+cs_status ensure_ws(cs_ctx *ctx, Classifier &C, int64_t B, unsigned what) {
+    cs_status rc = ensure_err(ctx);
+    if (rc) return rc;
+    use_workspace(C.dim, kUseWs);
+    const int64_t caps[4] = {C.cap, C.cap_conv, C.cap_grad, C.cap_gconv};
+    int64_t rows[4];
+    bool fits = true;
+    for (int i = 0; i < 4; ++i) {
+        rows[i] = (what >> i) & 1u ? std::max(B, caps[i]) : caps[i];
+        fits = fits && rows[i] == caps[i];
+    }
+    const int64_t sk = !(what & kWsConv) ? 0
+                       : what & kWsFc    ? tc_gemm_work_floats(ctx->sm_count)
+                                         : conv_splitk_floats(ctx->sm_count);
+    if (fits && C.splitk_n >= sk) return CS_OK;
+    return alloc_ws(ctx, C, rows, std::max(sk, C.splitk_n));
+}
+
+// need(): the workspaces of a call. Where memory has no room for them beside what
+// calls before left in the same sets (rows, gradients), they are made anew; a call
+// that is refused leaves none.
+template <class F>
+cs_status with_room(cs_ctx *ctx, Classifier &C, F need) {
+    const std::string message = ctx->err;
+    cs_status rc = need();
+    for (int i = 0; i < 2 && rc == CS_ENOMEM; ++i) {
+        free_ws(ctx, C);
+        free_fc(ctx, C);
+        free_tr(ctx, C);
+        free_parts(ctx, C);
+        if (i == 0 && (rc = need()) == CS_OK) ctx->err = message;
+    }
+    return rc;
 }
 
 int gemm(cs_ctx *ctx, Classifier &C, const float *A, const float *Bm, float *Cm, const float *bias,
@@ -463,13 +505,12 @@ int64_t train_parts(cs_ctx *ctx, const ClsShape &S, int64_t B) {
 
 cs_status ensure_train(cs_ctx *ctx, Classifier &C, int64_t B) {
     cs_status rc = ensure_fc(ctx, C, B, true);
-    if (rc == CS_OK) rc = C.dim == 2 ? ensure_tr(ctx, C, B) : CS_OK;
+    if (rc == CS_OK) rc = C.dim == 2 ? ensure_tr(ctx, C, B) : ensure_ws(ctx, C, B, kWsConv | kWsConvGrad);
     if (rc) return rc;
+    use_workspace(C.dim, kUseParts);
     const int64_t need = train_parts(ctx, ClsShape(C.dim), B);
     if (C.parts_cap >= need) return CS_OK;
-    dfree(ctx, C.parts);
-    C.parts = nullptr;
-    C.parts_cap = 0;
+    free_parts(ctx, C);
     if ((rc = dmalloc_n(ctx, &C.parts, size_t(need)))) return rc;
     C.parts_cap = need;
     return CS_OK;
@@ -699,12 +740,16 @@ template <class F>
 cs_status forward_chunks(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t n, const double *xp,
                          float *dst, cudaStream_t st, F each) {
     const bool fused = gemm_bf16();
+    WorkspaceScope use;
     const int ncls = cls_cells(C.dim);
     const int64_t R = std::min<int64_t>(n, chunk_rows(C.dim, fused));
-    cs_status rc = fused ? ensure_fc(ctx, C, R, false) : ensure_ws(ctx, C, R, true, false);
     // a chunk, the last one, of less than a tiled batch
     const int64_t rest = n % R > 0 ? n % R : R;
-    if (rc == CS_OK && fused && !tiled_batch(rest)) rc = ensure_ws(ctx, C, rest, false, false);
+    cs_status rc = with_room(ctx, C, [&] {
+        if (!fused) return ensure_ws(ctx, C, R, kWsFc | kWsConv);
+        const cs_status r = ensure_fc(ctx, C, R, false);
+        return r == CS_OK && !tiled_batch(rest) ? ensure_ws(ctx, C, rest, kWsFc) : r;
+    });
     if (rc) return rc;
     for (int64_t r0 = 0; r0 < n; r0 += R) {
         const int64_t B = std::min(R, n - r0);
@@ -725,6 +770,32 @@ cs_status forward_chunks(cs_ctx *ctx, Classifier &C, const DevMesh &m, int64_t n
 }  // namespace
 
 namespace cs {
+bool classifier_reclaim(cs_ctx *ctx) {
+    bool any = false;
+    for (Classifier *C : ctx->cls) {
+        if (!C) continue;
+        if (!in_use(C->dim, kUseWs) && !C->ws.empty()) {
+            free_ws(ctx, *C);
+            any = true;
+        }
+        if (!in_use(C->dim, kUseFc) && C->fcpack) {
+            free_fc(ctx, *C);
+            dfree(ctx, C->fcpack);
+            C->fcpack = nullptr;
+            any = true;
+        }
+        if (!in_use(C->dim, kUseTrain) && !C->trws.empty()) {
+            free_tr(ctx, *C);
+            any = true;
+        }
+        if (!in_use(C->dim, kUseParts) && C->parts) {
+            free_parts(ctx, *C);
+            any = true;
+        }
+    }
+    return any;
+}
+
 void classifier_release_all(cs_ctx *ctx) {
     for (auto &c : ctx->cls) {
         release(ctx, c);
@@ -899,8 +970,10 @@ cs_status cs_classifier_grad(cs_ctx *ctx, int32_t mesh_id, int64_t B, const doub
     if (!C) return fail(ctx, CS_ENOPRED, "cs_classifier_grad: no classifier loaded");
     CCHK(cudaSetDevice(ctx->device));
     const bool tiled = tiled_batch(B);
-    cs_status rc = tiled ? ensure_train(ctx, *C, B) : CS_OK;
-    if (rc == CS_OK && (!tiled || C->dim == 3)) rc = ensure_ws(ctx, *C, B, true, true);
+    WorkspaceScope use;
+    cs_status rc = with_room(ctx, *C, [&] {
+        return tiled ? ensure_train(ctx, *C, B) : ensure_ws(ctx, *C, B, kWsAll);
+    });
     if (rc) return rc;
     if (tiled) {
         ctx->launches += train_tiled(ctx, *C, m->d, B, xp, labels, nullptr, C->loss, nullptr);
@@ -933,8 +1006,10 @@ cs_status cs_classifier_train(cs_ctx *ctx, int32_t mesh_id, const double *xp,
     CCHK(cudaSetDevice(ctx->device));
     const int64_t B = std::min(batch, N);
     const bool tiled = tiled_batch(B);
-    cs_status rc = tiled ? ensure_train(ctx, *C, B) : CS_OK;
-    if (rc == CS_OK && (!tiled || C->dim == 3)) rc = ensure_ws(ctx, *C, B, true, true);
+    WorkspaceScope use;
+    cs_status rc = with_room(ctx, *C, [&] {
+        return tiled ? ensure_train(ctx, *C, B) : ensure_ws(ctx, *C, B, kWsAll);
+    });
     if (rc) return rc;
     float *losses = nullptr;
     if ((rc = dmalloc_n(ctx, &losses, size_t(std::max<int64_t>(steps, 1))))) return rc;

@@ -332,7 +332,9 @@ struct cs_ctx {
 
 namespace cs {
 // Device memory of a context (api.cpp). dmalloc fails with CS_ENOMEM when
-// cudaMalloc fails or the block would take the context past its HBM budget;
+// cudaMalloc fails or the block would take the context past its HBM budget, also
+// without the workspaces that no call in progress needs, which it then gives back
+// (a predictor has one for each of its paths, and keeps them from call to call);
 // dfree releases a block dmalloc returned (null is ignored).
 cs_status dmalloc(cs_ctx *ctx, void **p, size_t bytes);
 void dfree(cs_ctx *ctx, void *p);
@@ -359,6 +361,24 @@ cs_status cs_track_impl(cs_ctx *ctx, Mesh *m, int64_t n, const double *x, const 
                         int32_t *start_out, cudaStream_t stream);
 // predictor.cpp
 void predictor_release(cs_ctx *ctx, Predictor &P);
+// Workspaces that the call in progress on this thread uses: dmalloc may give back
+// the others. A bit per set of buffers and dimension.
+enum : uint32_t {
+    kUseIo = 1, kUseLayers = 2, kUseFused = 4, kUseTiles = 8,                        // Predictor
+    kUseWs = 1 << 8, kUseFc = 1 << 9, kUseTrain = 1 << 10, kUseParts = 1 << 11       // Classifier
+};
+extern thread_local uint32_t workspace_use;
+inline uint32_t use_bit(int dim, uint32_t set) { return dim == 2 ? set : set << 4; }
+inline void use_workspace(int dim, uint32_t set) { workspace_use |= use_bit(dim, set); }
+inline bool in_use(int dim, uint32_t set) { return (workspace_use & use_bit(dim, set)) != 0; }
+// the scope of a call: what it marks is in use until its end
+struct WorkspaceScope {
+    uint32_t outer = workspace_use;
+    ~WorkspaceScope() { workspace_use = outer; }
+};
+// free the predictors' (classifiers') workspaces that are not in use; true if any
+bool predictor_reclaim(cs_ctx *ctx);
+bool classifier_reclaim(cs_ctx *ctx);
 // prediction at every predictor cell of m from the grid velocity `grid`
 cs_status predict_grid(cs_ctx *ctx, Mesh *m, const float *grid, double dt, float *dhat,
                        cudaStream_t st);

@@ -103,6 +103,9 @@ void free_workspace(cs_ctx *ctx, Predictor &P) {
     P.splitk = nullptr;
     P.splitk_n = 0;
     P.cap = 0;
+}
+
+void free_tiles(cs_ctx *ctx, Predictor &P) {
     for (float *p : P.tiles) dfree(ctx, p);
     P.tiles.clear();
     P.tiles_cap.clear();
@@ -116,6 +119,7 @@ cs_status check_err(cs_ctx *ctx) { return err_raised(ctx) ? cs_device_status(ctx
 // the outputs and the batch of B rows
 cs_status ensure_io(cs_ctx *ctx, Predictor &P, int64_t B) {
     cs_status rc = ensure_err(ctx);
+    use_workspace(P.dim, kUseIo);
     if (rc || P.io_cap >= B) return rc;
     free_io(ctx, P);
     const NetShape S(P.dim);
@@ -155,6 +159,7 @@ struct FusedPack {
 cs_status ensure_fused(cs_ctx *ctx, Predictor &P, int64_t B, bool grad) {
     cs_status rc = ensure_err(ctx);
     if (rc) return rc;
+    use_workspace(P.dim, kUseFused);
     if (P.fcap >= B && (!grad || P.fpart)) return CS_OK;
     const int64_t cap = std::max(B, P.fcap);
     grad = grad || P.fpart;
@@ -186,22 +191,21 @@ cs_status ensure_fused(cs_ctx *ctx, Predictor &P, int64_t B, bool grad) {
 cs_status ensure_workspace(cs_ctx *ctx, Predictor &P, int64_t B) {
     cs_status rc0 = ensure_io(ctx, P, B);
     if (rc0) return rc0;
+    use_workspace(P.dim, kUseLayers);
     if (P.cap >= B) return CS_OK;
     free_workspace(ctx, P);
+    if (!in_use(P.dim, kUseTiles)) free_tiles(ctx, P);
     NetShape S(P.dim);
     int Si = S.S0, C = S.cin;
     int64_t max_col = 0, max_dy = 0;
     for (int l = 0; l < S.n_conv; ++l) {
         const int So = Si - 2;
         const int64_t Po = S.positions(So), K = int64_t(C) * S.taps();
-        float *col, *z, *y;
-        cs_status rc;
-        if ((rc = dalloc(ctx, &col, size_t(B * Po * K))) || (rc = dalloc(ctx, &z, size_t(B * Po * S.ch))) ||
-            (rc = dalloc(ctx, &y, size_t(B * Po * S.ch))))
-            return rc;
-        P.col.push_back(col);
-        P.z.push_back(z);
-        P.y.push_back(y);
+        for (auto &v : {std::make_pair(&P.col, K), {&P.z, int64_t(S.ch)}, {&P.y, int64_t(S.ch)}}) {
+            float *q = nullptr;
+            if (cs_status rc = dalloc(ctx, &q, size_t(B * Po * v.second))) return rc;
+            v.first->push_back(q);
+        }
         max_col = std::max(max_col, B * Po * K);
         if (l > 0) max_dy = std::max(max_dy, B * S.positions(Si) * S.ch);
         max_dy = std::max(max_dy, B * Po * S.ch);
@@ -370,18 +374,45 @@ int train_fused(cs_ctx *ctx, Predictor &P, int64_t B, const float *win, const fl
     return n + launch_reduce_parts(seg, ns, st);
 }
 
-// forward of B windows into P.out through whichever path takes the batch, and
-// the buffers of chunks of `rows` and a last one of `rest`
+// forward of B windows into P.out through whichever path takes the batch
 int forward_any(cs_ctx *ctx, Predictor &P, int64_t B, const float *win, cudaStream_t st) {
     return fused_batch(B) ? forward_fused(ctx, P, B, win, nullptr, st) : forward(ctx, P, B, win, st);
 }
 
-cs_status ensure_fwd(cs_ctx *ctx, Predictor &P, int64_t rows, int64_t rest) {
-    cs_status rc = CS_OK;
-    if (fused_batch(rows)) rc = ensure_fused(ctx, P, rows, false);
-    if (rc == CS_OK && !fused_batch(rows)) rc = ensure_workspace(ctx, P, rows);
-    if (rc == CS_OK && rest > 0 && !fused_batch(rest)) rc = ensure_workspace(ctx, P, rest);
+// need(): the workspaces of a call. Where memory has no room for them beside what
+// calls before left in the same sets (rows, gradients), they are made anew; a call
+// that is refused leaves none.
+template <class F>
+cs_status with_room(cs_ctx *ctx, Predictor &P, F need) {
+    const std::string message = ctx->err;
+    cs_status rc = need();
+    for (int i = 0; i < 2 && rc == CS_ENOMEM; ++i) {
+        free_io(ctx, P);
+        free_fused(ctx, P);
+        free_workspace(ctx, P);
+        if (i == 0 && (rc = need()) == CS_OK) ctx->err = message;
+    }
     return rc;
+}
+
+// the buffers of a forward pass in chunks of `rows` and a last one of `rest`
+cs_status ensure_fwd(cs_ctx *ctx, Predictor &P, int64_t rows, int64_t rest) {
+    return with_room(ctx, P, [&] {
+        cs_status rc = ensure_io(ctx, P, rows);
+        if (rc == CS_OK && fused_batch(rows)) rc = ensure_fused(ctx, P, rows, false);
+        if (rc == CS_OK && !fused_batch(rows)) rc = ensure_workspace(ctx, P, rows);
+        if (rc == CS_OK && rest > 0 && !fused_batch(rest)) rc = ensure_workspace(ctx, P, rest);
+        return rc;
+    });
+}
+
+// the buffers of a gradient or training call of B rows
+cs_status ensure_grad(cs_ctx *ctx, Predictor &P, int64_t B) {
+    return with_room(ctx, P, [&] {
+        cs_status rc = ensure_io(ctx, P, B);
+        if (rc) return rc;
+        return fused_batch(B) ? ensure_fused(ctx, P, B, true) : ensure_workspace(ctx, P, B);
+    });
 }
 
 Predictor *get_pred(cs_ctx *ctx, int dim) {
@@ -434,8 +465,33 @@ cs_status ensure_mesh_grid(cs_ctx *ctx, cs::Mesh *m) {
 
 namespace cs {
 
+bool predictor_reclaim(cs_ctx *ctx) {
+    bool any = false;
+    for (Predictor &P : ctx->pred) {
+        if (!in_use(P.dim, kUseLayers) && !P.col.empty()) {
+            free_workspace(ctx, P);
+            any = true;
+        }
+        if (!in_use(P.dim, kUseFused) && !P.fy.empty()) {
+            free_fused(ctx, P);
+            any = true;
+        }
+        if (!in_use(P.dim, kUseIo) && P.out) {
+            free_io(ctx, P);
+            any = true;
+        }
+        // serving predicts into the tiles
+        if (!in_use(P.dim, kUseTiles) && !ctx->server && !P.tiles.empty()) {
+            free_tiles(ctx, P);
+            any = true;
+        }
+    }
+    return any;
+}
+
 void predictor_release(cs_ctx *ctx, Predictor &P) {
     free_workspace(ctx, P);
+    free_tiles(ctx, P);
     free_io(ctx, P);
     free_fused(ctx, P);
     float **fs[] = {&P.w, &P.g, &P.m, &P.v, &P.loss};
@@ -496,6 +552,7 @@ TilePlan plan_tiles(const DevMesh &pv) {
 // Grow the tile workspace to hold plan t (buffers only grow, so a workspace
 // sized for every mesh of a serving run is never reallocated while in use).
 cs_status grow_tiles(cs_ctx *ctx, Predictor &P, const TilePlan &t) {
+    use_workspace(P.dim, kUseTiles);
     std::vector<int64_t> need(t.per.size());
     for (size_t i = 0; i < t.per.size(); ++i) need[i] = t.per[i] * t.Bt;
     bool fits = P.tiles.size() == need.size() && int64_t(P.tiles_cap.size()) == int64_t(need.size());
@@ -504,15 +561,12 @@ cs_status grow_tiles(cs_ctx *ctx, Predictor &P, const TilePlan &t) {
     std::vector<int64_t> cap(need.size());
     for (size_t i = 0; i < need.size(); ++i)
         cap[i] = std::max(need[i], i < P.tiles_cap.size() ? P.tiles_cap[i] : int64_t(0));
-    for (float *p : P.tiles) dfree(ctx, p);
-    P.tiles.clear();
-    P.tiles_cap.clear();
+    free_tiles(ctx, P);
     for (int64_t v : cap) {
         float *b = nullptr;
         cs_status rc = dalloc(ctx, &b, size_t(v));
         if (rc) {
-            for (float *p : P.tiles) dfree(ctx, p);
-            P.tiles.clear();
+            free_tiles(ctx, P);
             return rc;
         }
         P.tiles.push_back(b);
@@ -570,6 +624,7 @@ cs_status predict_grid_src(cs_ctx *ctx, cs::Mesh *m, const TcSource &src, double
                            cudaStream_t st) {
     Predictor *P = get_pred(ctx, m->d.dim);
     if (!P || !P->loaded) return fail(ctx, CS_ENOPRED, "no predictor loaded for this dimension");
+    WorkspaceScope use;
     const float *grid = src.U;
     if (!grid && !(src.node && ctx->engine == 1))
         return fail(ctx, CS_EINVAL, "the mesh has no grid velocity yet");
@@ -602,8 +657,7 @@ cs_status predict_grid_src(cs_ctx *ctx, cs::Mesh *m, const TcSource &src, double
     }
     if (m->d.dim == 3 && ctx->engine == 2) return predict_tiles(ctx, *P, m, grid, dt, dhat, st);
     const int64_t chunk = 8192;
-    cs_status rc = ensure_io(ctx, *P, chunk);
-    if (rc == CS_OK) rc = ensure_fwd(ctx, *P, chunk, m->d.n_pasg % chunk);
+    cs_status rc = ensure_fwd(ctx, *P, chunk, m->d.n_pasg % chunk);
     if (rc) return rc;
     const int D = m->d.dim;
     float scale[3] = {0, 0, 0};
@@ -641,6 +695,7 @@ bool serving_predictor_ready(cs_ctx *ctx, const cs::Mesh *m) {
 }
 
 cs_status prepare_serving(cs_ctx *ctx) {
+    WorkspaceScope use;
     for (int dim = 2; dim <= 3; ++dim) {
         Predictor &P = ctx->pred[dim - 2];
         if (!P.loaded || (ctx->engine != 1 && ctx->engine != 2)) continue;
@@ -940,10 +995,10 @@ cs_status cs_predictor_forward(cs_ctx *ctx, int dim, int64_t B, const float *win
         return fail(ctx, CS_EINVAL, "cs_predictor_forward: bad arguments");
     if (!P->loaded) return fail(ctx, CS_ENOPRED, "cs_predictor_forward: no predictor loaded");
     PCHK(cudaSetDevice(ctx->device));
+    WorkspaceScope use;
     const int64_t chunk = 8192;
     const int64_t rows = std::min<int64_t>(std::max<int64_t>(B, 1), chunk);
-    cs_status rc = ensure_io(ctx, *P, rows);
-    if (rc == CS_OK) rc = ensure_fwd(ctx, *P, rows, B % rows);
+    cs_status rc = ensure_fwd(ctx, *P, rows, B % rows);
     if (rc) return rc;
     NetShape S(dim);
     const int64_t row = int64_t(S.cin) * S.positions(S.S0);
@@ -981,10 +1036,10 @@ cs_status cs_predictor_train(cs_ctx *ctx, int dim, const float *windows, const f
         return fail(ctx, CS_EINVAL, "cs_predictor_train: bad arguments");
     if (!P->loaded) return fail(ctx, CS_ENOPRED, "cs_predictor_train: no predictor loaded");
     PCHK(cudaSetDevice(ctx->device));
+    WorkspaceScope use;
     const int64_t B = std::min(batch, N);
     const bool fused = fused_batch(B);
-    cs_status rc = ensure_io(ctx, *P, B);
-    if (rc == CS_OK) rc = fused ? ensure_fused(ctx, *P, B, true) : ensure_workspace(ctx, *P, B);
+    cs_status rc = ensure_grad(ctx, *P, B);
     if (rc) return rc;
     NetShape S(dim);
     const int64_t row = int64_t(S.cin) * S.positions(S.S0);
@@ -1066,9 +1121,9 @@ cs_status cs_predictor_grad(cs_ctx *ctx, int dim, int64_t B, const float *window
         return fail(ctx, CS_EINVAL, "cs_predictor_grad: bad arguments");
     if (!P->loaded) return fail(ctx, CS_ENOPRED, "cs_predictor_grad: no predictor loaded");
     PCHK(cudaSetDevice(ctx->device));
+    WorkspaceScope use;
     const bool fused = fused_batch(B);
-    cs_status rc = ensure_io(ctx, *P, B);
-    if (rc == CS_OK) rc = fused ? ensure_fused(ctx, *P, B, true) : ensure_workspace(ctx, *P, B);
+    cs_status rc = ensure_grad(ctx, *P, B);
     if (rc) return rc;
     if (fused) {
         ctx->launches += train_fused(ctx, *P, B, windows, targets, P->loss, nullptr);
