@@ -329,7 +329,8 @@ cs_status cs_predictor_save(cs_ctx *ctx, int dim, float *weights_out, int64_t n)
  * the start element is still looked up in the ASG seed grid. Default 1 (the
  * ASG grid itself). Drops the mesh's stored grid velocity and predictions.
  * Not while serving (CS_EBUSY). Errors: CS_EINVAL (even stride, or larger
- * than asg_grid on some axis), CS_ENOMESH, CS_ENOMEM.
+ * than asg_grid on some axis), CS_ENOMESH, CS_ENOMEM (the grid is then the
+ * ASG grid).
  */
 cs_status cs_predictor_grid(cs_ctx *ctx, int32_t mesh_id, int32_t stride);
 

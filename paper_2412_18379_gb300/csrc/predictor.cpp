@@ -434,13 +434,14 @@ cs::Mesh *find_mesh(cs_ctx *ctx, int32_t id) {
 
 // The static P1 interpolation table of the ASG cell centres (built once).
 cs_status ensure_interp(cs_ctx *ctx, cs::Mesh *m, cudaStream_t st) {
-    if (m->interp_node) return CS_OK;
+    if (m->interp_w) return CS_OK;       // allocated last: the table is whole
     const size_t n = size_t(pred_view(m->d).n_asg) * (m->d.dim + 1);
-    cs_status rc = dalloc(ctx, &m->interp_node, n);
-    if (rc) return rc;
-    m->allocs.push_back(m->interp_node);
-    rc = dalloc(ctx, &m->interp_w, n);
-    if (rc) return rc;
+    cs_status rc = CS_OK;
+    if (!m->interp_node) {
+        if ((rc = dalloc(ctx, &m->interp_node, n))) return rc;
+        m->allocs.push_back(m->interp_node);
+    }
+    if ((rc = dalloc(ctx, &m->interp_w, n))) return rc;
     m->allocs.push_back(m->interp_w);
     ctx->launches += launch_interp_table(pred_view(m->d), m->interp_node, m->interp_w, ctx->sm_count, st);
     return CS_OK;
@@ -689,7 +690,7 @@ cs_status reserve_tiles(cs_ctx *ctx, cs::Mesh *m) {
 
 bool serving_predictor_ready(cs_ctx *ctx, const cs::Mesh *m) {
     const Predictor &P = ctx->pred[m->d.dim - 2];
-    if (!P.loaded || !m->interp_node) return false;
+    if (!P.loaded || !m->interp_w) return false;
     if (ctx->engine == 1) return P.packed && !P.packed_dirty && ctx->dev_err;
     return ctx->engine == 2 && m->d.dim == 3 && !P.tiles.empty();
 }
@@ -939,8 +940,13 @@ cs_status cs_predictor_grid(cs_ctx *ctx, int32_t mesh_id, int32_t stride) {
         return CS_OK;
     }
     int32_t *ps = nullptr;
+    d.pseed = d.seed;        // the old grid's is gone
     cs_status rc = dalloc(ctx, &ps, size_t(n));
-    if (rc) return rc;
+    if (rc) {                // back to the ASG grid, which needs none
+        const std::string msg = ctx->err;
+        const cs_status back = cs_predictor_grid(ctx, mesh_id, 1);
+        return back ? back : fail(ctx, rc, msg);
+    }
     m->allocs.push_back(ps);
     d.pseed = ps;
     ctx->launches += launch_pred_seed(d, ps, ctx->sm_count, nullptr);

@@ -88,3 +88,57 @@ def test_an_exact_budget(cs):
         assert np.array_equal(out["host"].cpu().numpy(), want["host"]), delta
     assert ctx.memory_usage()[0] <= mesh_bytes + rest
     ctx.close()
+
+
+def test_a_refused_predictor_grid_or_table(cs):
+    """Each allocation of a coarser predictor grid, and of the table its grid
+    velocity is interpolated with, refused in turn: the mesh keeps a grid it can
+    use, and the call goes through once there is room. (Both had left a pointer
+    behind that the next call would have used: one to freed memory, one null.)"""
+    c = make_case("tg2d", n_side=41)
+    roomy = cs.Context(0)
+    mesh = roomy.upload_mesh(c.xyz, c.conn)
+    base = roomy.memory_usage()[0]
+    mesh.set_predictor_grid(3)
+    want = roomy.grid_velocity(mesh, _dev(c.u), out=_dev(np.zeros((np.prod(mesh.info()["pred_grid"]), 2),
+                                                                  np.float32))).cpu().numpy()
+    asg = int(np.prod(mesh.info()["asg_grid"]))
+    cells = int(np.prod(mesh.info()["pred_grid"]))
+    mesh.set_predictor_grid(1)
+    want1 = roomy.grid_velocity(mesh, _dev(c.u), out=_dev(np.zeros((asg, 2), np.float32))).cpu().numpy()
+    roomy.close()
+    table = 3 * 4 * cells            # node or weights
+    for room in (0, 4 * cells, 4 * cells + table):
+        ctx = cs.Context(0, hbm_budget=base + room)
+        mesh = ctx.upload_mesh(c.xyz, c.conn)
+        if room == 0:
+            for _ in range(2):
+                with pytest.raises(cs.CsError) as e:
+                    mesh.set_predictor_grid(3)
+                assert e.value.code == -2
+                assert mesh.info()["pred_stride"] == 1
+                assert list(mesh.info()["pred_grid"]) == list(mesh.info()["asg_grid"])
+        else:
+            mesh.set_predictor_grid(3)
+        n = asg if room == 0 else cells
+        out = _dev(np.zeros((n, 2), np.float32))
+        for _ in range(2):
+            with pytest.raises(cs.CsError) as e:
+                ctx.grid_velocity(mesh, _dev(c.u), out=out)
+            assert e.value.code == -2
+        ctx.close()
+    ctx = cs.Context(0, hbm_budget=base + 4 * cells + 2 * table)
+    mesh = ctx.upload_mesh(c.xyz, c.conn)
+    mesh.set_predictor_grid(3)
+    out = ctx.grid_velocity(mesh, _dev(c.u), out=_dev(np.zeros((cells, 2), np.float32)))
+    assert np.array_equal(out.cpu().numpy().view(np.uint32), want.view(np.uint32))
+    ctx.close()
+    # refused for the coarse grid's sake, then used with a released mesh's room
+    ctx = cs.Context(0, hbm_budget=2 * base)
+    other, mesh = ctx.upload_mesh(c.xyz, c.conn), ctx.upload_mesh(c.xyz, c.conn)
+    with pytest.raises(cs.CsError):
+        mesh.set_predictor_grid(3)
+    other.release()
+    out = ctx.grid_velocity(mesh, _dev(c.u), out=_dev(np.zeros((asg, 2), np.float32)))
+    assert np.array_equal(out.cpu().numpy().view(np.uint32), want1.view(np.uint32))
+    ctx.close()
