@@ -966,10 +966,10 @@ cs_status cs_grid_velocity(cs_ctx *ctx, int32_t mesh_id, const double *u_nodal, 
         cs_status rc = ensure_mesh_grid(ctx, m);
         if (rc) return rc;
         dst = m->grid_u;
-        m->grid_u_valid = true;
     }
     cs_status rc = ensure_interp(ctx, m, static_cast<cudaStream_t>(stream));
     if (rc) return rc;
+    if (dst == m->grid_u) m->grid_u_valid = true;
     ctx->launches += launch_resample(pred_view(m->d), m->interp_node, m->interp_w, u_nodal, dst,
                                      ctx->sm_count, static_cast<cudaStream_t>(stream));
     PCHK(cudaGetLastError());

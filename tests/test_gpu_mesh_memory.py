@@ -142,3 +142,22 @@ def test_a_refused_predictor_grid_or_table(cs):
     out = ctx.grid_velocity(mesh, _dev(c.u), out=_dev(np.zeros((asg, 2), np.float32)))
     assert np.array_equal(out.cpu().numpy().view(np.uint32), want1.view(np.uint32))
     ctx.close()
+
+
+def test_a_refused_grid_velocity_is_none(cs):
+    """The grid velocity's buffer fits, the table it is computed with does not:
+    the mesh has no grid velocity, and what reads it says so."""
+    c = make_case("tg2d", n_side=41)
+    probe = cs.Context(0)
+    mesh = probe.upload_mesh(c.xyz, c.conn)
+    base, asg = probe.memory_usage()[0], int(np.prod(mesh.info()["asg_grid"]))
+    probe.close()
+    ctx = cs.Context(0, hbm_budget=base + 2 * 8 * asg)       # velocity and prediction
+    mesh = ctx.upload_mesh(c.xyz, c.conn)
+    with pytest.raises(cs.CsError) as e:
+        ctx.grid_velocity(mesh, _dev(c.u))
+    assert e.value.code == -2
+    with pytest.raises(cs.CsError) as e:
+        ctx.windows(mesh, c.dt, B=4)
+    assert e.value.code == -1 and "no grid velocity" in str(e.value)
+    ctx.close()
