@@ -66,6 +66,7 @@
 #include <cstdint>
 
 #include "classifier.h"
+#include "launch_attr.h"
 #include "tc_common.cuh"
 
 namespace cs {
@@ -530,12 +531,8 @@ void launch_conv(const DevMesh &m, const float *pool_f, int64_t B, const double 
                  const uint8_t *packed, const FcMat &cat, float *off, int *err, int sm_count,
                  cudaStream_t st) {
     using G = ClsGeo<D, NP>;
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(cls_conv_tc_kernel<D, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             G::kSmTotal);
-        attr = true;
-    }
+    static std::atomic<uint64_t> done{0};
+    allow_smem(done, reinterpret_cast<const void *>(cls_conv_tc_kernel<D, NP>), G::kSmTotal);
     const int grid = int(std::min<int64_t>((B + NP - 1) / NP, int64_t(sm_count) * G::PerSm));
     cls_conv_tc_kernel<D, NP><<<grid, G::Threads, G::kSmTotal, st>>>(m, pool_f, B, xp, packed, cat,
                                                                     off, err);

@@ -45,6 +45,7 @@
 #include <cstdint>
 
 #include "cnn.h"
+#include "launch_attr.h"
 #include "tc_common.cuh"
 
 namespace cs {
@@ -432,12 +433,8 @@ int64_t cost3(const DevMesh &m, int sm_count) {
 template <int T>
 int launch3(const DevMesh &m, const TcSource &src, double dt, const uint8_t *packed, float *dhat,
             int *err, int sm_count, cudaStream_t st, TcHold hold) {
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(cnn3d_tc_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             Geo3<T>::kSmTotal);
-        attr = true;
-    }
+    static std::atomic<uint64_t> done{0};
+    allow_smem(done, reinterpret_cast<const void *>(cnn3d_tc_kernel<T>), Geo3<T>::kSmTotal);
     const int grid = int(std::min<int64_t>(tiles3<T>(m), sm_count));
     launch_pdl(cnn3d_tc_kernel<T>, dim3(grid), dim3(kThreads3), size_t(Geo3<T>::kSmTotal), st, m,
                src, float(dt / m.sa[0]), float(dt / m.sa[1]), float(dt / m.sa[2]), packed, dhat, err,

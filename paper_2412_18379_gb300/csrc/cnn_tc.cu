@@ -57,6 +57,7 @@
 #include <cstdint>
 
 #include "cnn.h"
+#include "launch_attr.h"
 #include "tc_common.cuh"
 
 namespace cs {
@@ -737,12 +738,8 @@ int64_t tile_cost(const DevMesh &m, int sm_count) {
 template <int TH>
 int launch_rows(const DevMesh &m, const TcSource &src, double dt, const uint8_t *packed,
                 float *dhat, int *err, int sm_count, cudaStream_t st, TcHold hold) {
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(cnn2d_tc_kernel<TH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             Geo<TH>::kSmTotal);
-        attr = true;
-    }
+    static std::atomic<uint64_t> done{0};
+    allow_smem(done, reinterpret_cast<const void *>(cnn2d_tc_kernel<TH>), Geo<TH>::kSmTotal);
     const int grid = std::min(tiles_of<TH>(m), sm_count);
     launch_pdl(cnn2d_tc_kernel<TH>, dim3(grid), dim3(kThreadsTC), size_t(Geo<TH>::kSmTotal), st, m,
                src, float(dt / m.sa[0]), float(dt / m.sa[1]), packed, dhat, err, hold);

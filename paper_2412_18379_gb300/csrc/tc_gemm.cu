@@ -26,6 +26,7 @@
 #include <cstdint>
 
 #include "cnn.h"
+#include "launch_attr.h"
 #include "tc_common.cuh"
 
 namespace cs {
@@ -323,11 +324,8 @@ void launch_bn(const TcGemm &g, int64_t splits, int *err, cudaStream_t st) {
     using G = GemmGeo<BN>;
     // at most two CTAs per SM, so their TMEM columns always fit the SM's 512
     constexpr int kSmem = G::kSmTotal < 80 * 1024 && G::kCols > 128 ? 80 * 1024 : G::kSmTotal;
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(tc_gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-        attr = true;
-    }
+    static std::atomic<uint64_t> done{0};
+    allow_smem(done, reinterpret_cast<const void *>(tc_gemm_kernel<BN>), kSmem);
     const dim3 grid(unsigned((g.M + kBM - 1) / kBM), unsigned((g.N + BN - 1) / BN), unsigned(splits));
     tc_gemm_kernel<BN><<<grid, kThreadsG, kSmem, st>>>(g, err);
 }
