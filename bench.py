@@ -16,7 +16,10 @@ of the same mesh (CFL 2-16).
   python bench.py [--gpus N] [--steps K] [--warmup W] [--cfl C] [--mode M]
   python bench.py --impl reference ...   # the CPU oracle, timed on host cores
 
-Prints one JSON line (rank 0).
+Prints one JSON line (rank 0): the workload's figure, how it was taken and its
+roofline, in under 2500 characters. Everything else that was measured (every
+mode, the CFL sweep, training, the classifier, serving, all rooflines) goes to
+stderr as one more JSON line, and to --details FILE if given.
 """
 
 import argparse
@@ -116,6 +119,39 @@ def ncu_traffic(profile, sources):
         return float(vals["dram_bytes_per_full_launch"])
     except (KeyError, ValueError):
         return None
+
+
+LINE_LIMIT = 2500      # characters of the printed line
+
+
+def _round6(v):
+    """Floats to six significant digits, everywhere in a JSON value."""
+    if isinstance(v, float):
+        return float("%.6g" % v)
+    if isinstance(v, dict):
+        return {k: _round6(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [_round6(x) for x in v]
+    return v
+
+
+def headline(full):
+    """The printed line of a run's full record: the keys that state the figure,
+    with the longer ones cut to their numbers, and each mode's time and mean walk."""
+    keys = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+            "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "config",
+            "mean_path_len", "max_path_len", "gpu_launches", "clocks")
+    line = {k: full[k] for k in keys if k in full}
+    parts = {"roofline": ("bound", "achieved", "peak", "unit", "frac", "kernel", "kernel_ms",
+                          "traffic"),
+             "cpu_baseline": ("value", "unit", "cores", "kind", "sample"),
+             "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "entry_point")}
+    for name, sub in parts.items():
+        if full.get(name) is not None:
+            line[name] = {k: full[name][k] for k in sub if k in full[name]}
+    line["modes"] = {m: {k: r[k] for k in ("ms_per_step", "mean_path_len") if k in r}
+                     for m, r in (full.get("modes") or {}).items()}
+    return _round6(line)
 
 
 def nvtx_push(name):
@@ -727,6 +763,8 @@ def main():
                     help="8-mode fields of training pairs (0: an untrained predictor)")
     ap.add_argument("--train-steps", type=int, default=1000)
     ap.add_argument("--train-batch", type=int, default=4096)
+    ap.add_argument("--details", metavar="FILE",
+                    help="write the full record (every mode, sweep, training, serving) there")
     ap.add_argument("--shard", action="store_true",
                     help="under torchrun: split one particle batch over the ranks "
                          "(shard_range; strong scaling) instead of one batch per rank")
@@ -976,7 +1014,14 @@ def main():
             "paper_context": "paper (4x Xeon 8269CY, CPU): 95.8% shorter paths, 97.0% less "
                              "time with CNN-SNS on the flow past a sphere (Table 2)",
         }
-        print(json.dumps(line))
+        text = json.dumps(headline(line))
+        assert len(text) < LINE_LIMIT, len(text)
+        if args.details:
+            with open(args.details, "w") as out:
+                json.dump(line, out, indent=1)
+        print(json.dumps(line), file=sys.stderr)
+        sys.stderr.flush()
+        print(text, flush=True)
     mesh.release()
     ctx.close()
     if dist is not None:
