@@ -20,8 +20,9 @@
 //          the ring and the rows past the window stay zero
 //   conv1  tcgen05.mma kind::f16, M = 128 rows, N = 32, K = 16 = two taps of
 //          8 channels: the A descriptor's leading byte offset is the row
-//          distance of the two taps (5 MMAs per M-tile in 2-D, 14 in 3-D; the
-//          last pair's first tap has zero weights)
+//          distance of the two taps (5 MMAs per M-tile in 2-D, 14 in 3-D). The
+//          odd last tap's partner is a block of zero rows with zero weights: rows
+//          of the window there would turn an infinite input into a NaN
 //   conv2  K = 32 channels of one tap in two K = 16 steps: 2 MMAs per tap
 //   act    [4 chunks][rows][8] BF16: ReLU(conv1 + b1), written at the window
 //          position of each valid output row (its padded layout is conv2's
@@ -109,7 +110,8 @@ struct ClsGeo {
     static constexpr int kB2 = kW2 + Taps * 2048;                    // f32 [32]
     static constexpr int kPacked = kB2 + 128;
     // shared memory
-    static constexpr int kSmIn = 0;
+    static constexpr int kSmZero = 0;                                // 128 zero rows
+    static constexpr int kSmIn = kSmZero + 128 * 16;
     static constexpr int kSmAct = kSmIn + NB * Rows * 16;
     static constexpr int kSmW = kSmAct + NB * 4 * Rows * 16;
     static constexpr int kSmStage = kSmW + kPacked;
@@ -121,7 +123,7 @@ struct ClsGeo {
     static constexpr int kSmTotal = kSmSlot + 16;
 
     static_assert(NeedCols <= int(Cols) && int(Cols) * PerSm <= 512, "TMEM columns");
-    static_assert(128 * MT + S < Rows, "operand reads in bounds (the zero tap included)");
+    static_assert(128 * MT + S < Rows, "operand reads in bounds");
     static_assert(Ro - 1 + Coff < Rows, "outputs land in the window");
     static_assert(kSmTotal <= (PerSm == 1 ? 232448 : PerSm == 2 ? 113 * 1024 : 75 * 1024), "shared memory of one CTA");
     static_assert(kSmW % 128 == 0 && kSmAct % 128 == 0, "operand alignment");
@@ -304,16 +306,19 @@ __global__ void __launch_bounds__(ClsGeo<D, NP>::Threads, ClsGeo<D, NP>::PerSm) 
         constexpr uint32_t id32 = idesc_bf16(128, 32);
         auto conv1 = [&](int k) {
             const uint64_t d_in = sdesc(smem_addr(in + (k % G::NB) * G::Rows * 16), 0, 128);
+            // the zero rows, and the distance to the buffer's last tap from there
+            const uint64_t d_zero = sdesc(smem_addr(smem + G::kSmZero),
+                                          G::kSmIn + (k % G::NB) * G::Rows * 16 + cls_shift<D>(G::Taps - 1) * 16, 128);
             #pragma unroll 1
             for (int mt = 0; mt < G::MT; ++mt) {
                 const uint32_t dcol = tmem + uint32_t(32 * mt);
                 #pragma unroll
                 for (int i = 0; i < G::Pairs; ++i) {
-                    // the last step's first tap has zero weights: it reads the
-                    // tap before, rows of the same particle
-                    const int t0 = min(2 * i, G::Taps - 2), t1 = t0 + 1;
-                    const int sh0 = cls_shift<D>(t0), sh1 = cls_shift<D>(t1);
-                    const uint64_t a = d_in + uint64_t(128 * mt + sh0) + (uint64_t(sh1 - sh0) << 16);
+                    const int sh0 = cls_shift<D>(2 * i);
+                    const int sh1 = cls_shift<D>(i + 1 < G::Pairs ? 2 * i + 1 : 2 * i);
+                    const uint64_t a = i + 1 < G::Pairs
+                                           ? d_in + uint64_t(128 * mt + sh0) + (uint64_t(sh1 - sh0) << 16)
+                                           : d_zero + (uint64_t(128 * mt) << 16);
                     mma_bf16(dcol, a, d_w1 + uint64_t(i * 64), id32, i > 0 ? 1u : 0u);
                 }
             }
@@ -510,7 +515,7 @@ __global__ void cls_pack_kernel(const float *__restrict__ w, int64_t off_w1, int
     __nv_bfloat16 *w1 = reinterpret_cast<__nv_bfloat16 *>(out + G::kW1);
     for (int e = tid; e < G::Pairs * 2 * 32 * 8; e += nth) {
         const int j = e % 8, o = (e / 8) % 32, h = (e / 256) % 2, p = e / 512;
-        // the odd last tap is the second of its step
+        // the odd last tap is the second of its step, behind the zero rows
         const int t = p < G::Pairs - 1 ? 2 * p + h : h == 1 ? G::Taps - 1 : -1;
         w1[e] = __float2bfloat16_rn(t >= 0 && j < D ? w[off_w1 + (o * D + j) * G::Taps + t] : 0.f);
     }
