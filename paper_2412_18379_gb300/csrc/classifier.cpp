@@ -1,9 +1,12 @@
 // The classifier start predictor (Sec. 2.3, Eq. 7-8) as a sequence of
-// kernels: pooled-centroid inputs, two zero-padded convolutions (im2col and
-// BF16-operand GEMMs with FP32 accumulation on the tensor cores), average
+// kernels: pooled-centroid inputs, two zero-padded convolutions, average
 // pooling, the offset branch, fusion, logits; the cross-entropy backward,
 // Adam on FP32 master parameters, the training loop, the start element of
 // the most probable class, and the C ABI entry points of the classifier.
+// Inference fuses inputs, convolutions and pooling (classifier_tc.cu); the
+// layers run on tiled BF16 operands (fc_tc.cu). A training step takes its 2-D
+// convolutions from train_tc.cu, its 3-D ones from im2col and the general GEMM.
+// FP32 operands and batches below 16 rows take im2col and that GEMM throughout.
 #include <cuda_runtime.h>
 
 #include <algorithm>

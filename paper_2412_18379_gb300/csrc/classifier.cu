@@ -1,8 +1,10 @@
 // The paper's classifier start predictor (Sec. 2.3, Eq. 7-8): the kernels
-// around its GEMMs. Inputs (pooled centroid windows and the offset of x_p),
-// the layout changes between layers (zero padding, average pooling,
-// concatenation), the softmax with its cross-entropy gradient, the labels
-// from plain SNS hosts and the start element K_p of the most probable class.
+// around its layers' products. Inputs (pooled centroid windows and the offset of
+// x_p), average pooling and its gradient, the softmax with its cross-entropy
+// gradient, each on the tiled BF16 layouts (fc_tc.h) and, for FP32 operands and
+// batches below 16 rows, on row-major FP32 with the zero padding and concatenation
+// that path needs; the labels from plain SNS hosts and the start element K_p of
+// the most probable class.
 //
 // Every FP64 step of the inputs, labels and starts is written with explicit
 // round-to-nearest intrinsics, so the integer decisions (cells, labels,
@@ -399,15 +401,14 @@ __global__ void __launch_bounds__(kT) pool_tiled_kernel(const float *__restrict_
     }
 }
 
-// a block takes whole rows: the row's pooled gradient goes through shared
+// 2-D. A block takes whole rows: the row's pooled gradient goes through shared
 // memory (read along the pooled positions, used along the channels); a thread
 // keeps one channel, whose column sum it carries
-template <int D>
 __global__ void __launch_bounds__(kT) pool_back_tiled_kernel(const float *__restrict__ dpool,
                                                              const float *__restrict__ z,
                                                              int64_t B, uint16_t *__restrict__ dz,
                                                              float *__restrict__ part) {
-    using G = Win<D>;
+    using G = Win<2>;
     constexpr int C = kClsCh, Ld = G::Pp | 1;      // odd stride: no bank conflicts
     __shared__ float sg[C * Ld];
     __shared__ float red[kT];
@@ -431,13 +432,9 @@ __global__ void __launch_bounds__(kT) pool_back_tiled_kernel(const float *__rest
         for (int j = 0; j < kZ; ++j) {
             const int p = threadIdx.x / C + j * (kT / C);
             if (p >= G::P) continue;
-            const int px = p % G::W, py = (p / G::W) % G::W, pz = D == 3 ? p / (G::W * G::W) : 0;
-            float g = 0.f;
-            if (px < 2 * G::Wp && py < 2 * G::Wp && (D == 2 || pz < 2 * G::Wp) && zv[j] > 0.f) {
-                const int pp = D == 2 ? (py / 2) * G::Wp + px / 2
-                                      : ((pz / 2) * G::Wp + py / 2) * G::Wp + px / 2;
-                g = sg[c * Ld + pp] / float(1 << D);
-            }
+            const int px = p % G::W, py = p / G::W;
+            const bool pooled = px < 2 * G::Wp && py < 2 * G::Wp && zv[j] > 0.f;
+            const float g = pooled ? sg[c * Ld + (py / 2) * G::Wp + px / 2] / 4.f : 0.f;
             sum += g;
             dz[(b * G::P + p) * C + c] = __bfloat16_as_ushort(__float2bfloat16_rn(g));
         }
@@ -751,7 +748,8 @@ int cls_pool_back_blocks(int64_t B, int sm_count) {
 
 void launch_cls_pool_back_tiled(const float *dpool, const float *z, int64_t B, uint16_t *dz,
                                 float *part, int sm_count, cudaStream_t st) {
-    launch_pdl(pool_back_tiled_kernel<2>, dim3(cls_pool_back_blocks(B, sm_count)), dim3(kT), 0, st, dpool, z, B, dz, part);
+    launch_pdl(pool_back_tiled_kernel, dim3(cls_pool_back_blocks(B, sm_count)), dim3(kT), 0, st, dpool,
+               z, B, dz, part);
 }
 
 int cls_softmax_blocks(int64_t B) { return int((B + 127) / 128 * (128 / kSmRows)); }

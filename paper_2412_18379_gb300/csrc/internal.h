@@ -30,9 +30,10 @@ struct Server;   // serve.cpp
 //   2-D, 96 bytes:  [main 0: 32][tail 0: 16][tail 1: 16][main 1: 32]
 //   3-D, 160 bytes: [main 0: 64][tail 0: 16][tail 1: 16][main 1: 64]
 // main: all but the struct's last 16 bytes, which are the tail. L1 busy 66% of a
-// plain 2-D step, 76% before: 81.1 -> 79.2 us on 1001^2 nodes, 3-D element-node
-// pairs 177 -> 174 us; a CNN-started 2-D step, whose walks take 1.7 steps, 66.7 ->
-// 66.9 us. An odd last record ends with its tail.
+// plain 2-D step, 76% before. Five runs of each in turn (each within 0.3%):
+// plain 2-D nodes 79.0 -> 77.1 us, 3-D element-node pairs 175.4 -> 172.9, 3-D
+// CNN-started 113.6 -> 112.9; a CNN-started 2-D step, whose walks take 1.7 steps,
+// 66.3 -> 66.5. An odd last record ends with its tail.
 //
 // The exact record holds v0 and M in FP64 (row k of M gives
 // lambda_{k+1} = M[k] . (x_p - v0)); it is read only when the FP32 filter

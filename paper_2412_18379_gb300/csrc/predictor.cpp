@@ -306,7 +306,8 @@ int backward(cs_ctx *ctx, Predictor &P, int64_t B, const float *tgt, float *loss
 }
 
 // The fused path's forward pass of B windows into P.out; train_fused adds the
-// gradients of the mean squared error into P.g, and *loss. Every sum over the batch is one of partials in a fixed order.
+// gradients of the mean squared error into P.g, and *loss. Every sum over the
+// batch is one of partials in a fixed order.
 int forward_fused(cs_ctx *ctx, Predictor &P, int64_t B, const float *win, const float *tgt,
                   cudaStream_t st) {
     const NetShape S(P.dim);
