@@ -30,10 +30,11 @@ struct Server;   // serve.cpp
 //   2-D, 96 bytes:  [main 0: 32][tail 0: 16][tail 1: 16][main 1: 32]
 //   3-D, 160 bytes: [main 0: 64][tail 0: 16][tail 1: 16][main 1: 64]
 // main: all but the struct's last 16 bytes, which are the tail. L1 busy 66% of a
-// plain 2-D step, 76% before. Five runs of each in turn (each within 0.3%):
-// plain 2-D nodes 79.0 -> 77.1 us, 3-D element-node pairs 175.4 -> 172.9, 3-D
+// plain 2-D step, 76% before. Four or five runs of each in turn (each within 0.3%):
+// plain 2-D nodes 78.8 -> 76.5 us, 3-D element-node pairs 175.4 -> 172.9, 3-D
 // CNN-started 113.6 -> 112.9; a CNN-started 2-D step, whose walks take 1.7 steps,
-// 66.3 -> 66.5. An odd last record ends with its tail.
+// 66.2 -> 66.4, and from cold caches on 1001^2 nodes 75.9 -> 76.1. An odd last
+// record ends with its tail.
 //
 // The exact record holds v0 and M in FP64 (row k of M gives
 // lambda_{k+1} = M[k] . (x_p - v0)); it is read only when the FP32 filter
@@ -63,17 +64,19 @@ static_assert(sizeof(WalkRec3) == 80, "WalkRec3 is 80 bytes");
 static_assert(sizeof(ExactRec2) == 48, "ExactRec2 is 48 bytes");
 static_assert(sizeof(ExactRec3) == 96, "ExactRec3 is 96 bytes");
 
-// byte offsets of record e's parts in the paired layout, and its size
+// byte offsets of record e's parts in the paired layout, and its size (one product
+// each: with the pair's and the half's apart the plain 2-D step took 77.2 us)
 #ifdef __CUDACC__
 #define CS_HD __host__ __device__
 #else
 #define CS_HD
 #endif
 CS_HD inline int64_t walk_main(int dim, int64_t e) {
-    return dim == 2 ? (e >> 1) * 96 + (e & 1) * 64 : (e >> 1) * 160 + (e & 1) * 96;
+    return e * (dim == 2 ? 48 : 80) + (e & 1) * 16;
 }
 CS_HD inline int64_t walk_tail(int dim, int64_t e) {
-    return dim == 2 ? (e >> 1) * 96 + 32 + (e & 1) * 16 : (e >> 1) * 160 + 64 + (e & 1) * 16;
+    const int main = dim == 2 ? 32 : 64;
+    return e * (main + 16) + main - (e & 1) * main;
 }
 CS_HD inline int64_t walk_bytes(int dim, int64_t n_e) { return n_e * (dim == 2 ? 48 : 80); }
 
