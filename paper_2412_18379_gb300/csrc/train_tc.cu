@@ -759,6 +759,20 @@ __device__ __forceinline__ bool handover(bool ok) {
     return r != 0;
 }
 
+// whether any thread of the epilogue warps has the flag (named barrier 2)
+__device__ __forceinline__ bool epi_or(bool flag) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 q, %1, 0;\n\t"
+        "barrier.cta.red.or.pred p, 2, %2, q;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(r)
+        : "r"(uint32_t(flag)), "n"(kBwdEpi * 32)
+        : "memory");
+    return r != 0;
+}
+
 // bounded wait for a phase that may be far away: sparse polls
 __device__ __forceinline__ bool idle_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
                                           int *err) {
@@ -829,13 +843,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
     pdl_wait();
     for (int i = tid; i < F::Kw * kTrainCh * 2 / 16; i += kBwdThreads) cp_async16(wop + 16 * i, a.w + 16 * i);
     cp_async_wait_all();
-    // weights that are not finite (each thread looks at those it copied)
-    uint32_t bad = 0;
-    for (int i = tid; i < F::Kw * kTrainCh * 2 / 16; i += kBwdThreads)
-        bad |= nonfinite8(reinterpret_cast<const uint4 *>(wop)[i]);
     fence_async_smem();
     fence_before();
-    const bool bad_w = __syncthreads_or(bad != 0) != 0;
+    __syncthreads();
     fence_after();
     const uint32_t tmem = *slot;
     const int n_mine = int((a.tiles - 1 - blockIdx.x) / gridDim.x + 1);
@@ -939,25 +949,25 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
                 for (int c = 0; c < 3; ++c)
                     *reinterpret_cast<uint4 *>(zb + ((4 * c + (i & 3)) * F::RowsZ + F::Front + q + c * N::Si) * 16) = vz[j];
             }
-            // the largest half (activations come from a ReLU: none is negative)
-            uint32_t top = 0;
+            auto put_act = [&](int j, const uint4 v) {
+                const int i = lt + j * kBwdLoad * 32, q = i >> 2;
+                if (i >= a.G * N::Pi * 4) return;
+                #pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    if (q >= c) *reinterpret_cast<uint4 *>(ab + ((4 * c + (i & 3)) * F::RowsA + q - c) * 16) = v;
+            };
+            uint32_t top = 0;     // the largest half: activations come from a ReLU, none is negative
             #pragma unroll
-            for (int j = 0; j < F::PieceA; ++j)
+            for (int j = 0; j < F::PieceA; ++j) {
+                put_act(j, va[j]);
                 top = __vmaxu2(top, __vmaxu2(__vmaxu2(va[j].x, va[j].y), __vmaxu2(va[j].z, va[j].w)));
+            }
             if (nonfinite2(top)) {
                 *bad_act = 1;
                 #pragma unroll
                 for (int j = 0; j < F::PieceA; ++j)
-                    va[j] = make_uint4(ones_for_nonfinite2(va[j].x), ones_for_nonfinite2(va[j].y),
-                                       ones_for_nonfinite2(va[j].z), ones_for_nonfinite2(va[j].w));
-            }
-            #pragma unroll
-            for (int j = 0; j < F::PieceA; ++j) {
-                const int i = lt + j * kBwdLoad * 32, q = i >> 2;
-                if (i >= a.G * N::Pi * 4) break;
-                #pragma unroll
-                for (int c = 0; c < 3; ++c)
-                    if (q >= c) *reinterpret_cast<uint4 *>(ab + ((4 * c + (i & 3)) * F::RowsA + q - c) * 16) = va[j];
+                    put_act(j, make_uint4(ones_for_nonfinite2(va[j].x), ones_for_nonfinite2(va[j].y),
+                                          ones_for_nonfinite2(va[j].z), ones_for_nonfinite2(va[j].w)));
             }
             fence_async_smem();
             __syncwarp();
@@ -970,6 +980,11 @@ __global__ void __launch_bounds__(kBwdThreads, 1) conv_bwd_kernel(const ConvArgs
         #pragma unroll
         for (int e = 0; e < 16; ++e) db[e] = 0.f;
         uint32_t ph = 0;                                 // phases of the parts' barriers
+        // weights that are not finite, while the first tile is on its way
+        uint32_t bad = 0;
+        for (int i = tid; i < F::Kw * kTrainCh * 2 / 16; i += kBwdEpi * 32)
+            bad |= nonfinite8(reinterpret_cast<const uint4 *>(wop)[i]);
+        const bool bad_w = epi_or(bad != 0);
         for (int k = 0; k < n_mine && ok; ++k) {
             const int64_t b0 = tile_b0(k);
             const int rows = tile_nb(k) * N::Pi, mts = (rows + 127) / 128;
