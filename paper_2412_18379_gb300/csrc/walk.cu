@@ -183,9 +183,11 @@ __device__ __forceinline__ void prepare(const DevMesh &m, const TrackArgs &a, in
 // at a node (no-slip walls, stagnation points) end there, where many elements meet.
 // A line of wall nodes ends 32 walks of one warp so, each of which took the whole
 // warp through a search: on the 75^3 nodes of a cube, the 884 on its edges alone
-// took 243 us (58 now), and the CNN-SNS step 250 us (116 now). Bound by the
-// latency of its dependent loads: looking at all of the element's vertices, not
-// the one of the largest coordinate, took 5 us more.
+// took 243 us (58 now), and the CNN-SNS step 250 us (107 now). Bound by the
+// latency of its three dependent loads, of which a walk from cold caches sees the
+// last: 101^3 nodes from the cell of x_p 109.1 us, 107.8 with the host beside the
+// mark, 8 bytes a vertex more. Looking at all of the element's vertices, not the
+// one of the largest coordinate, takes 8 us more on the CNN-SNS step.
 constexpr int32_t kNoVertex = INT32_MIN;
 template <int D>
 __device__ __forceinline__ int32_t vertex_host(const DevMesh &m, int32_t cur, int i, const double *xp) {
@@ -294,7 +296,6 @@ __global__ void __launch_bounds__(256, D == 2 ? 4 : 3) walk_kernel(const DevMesh
 
         // ---- one step of Algorithm 1 for every busy lane ----
         bool done = false, search = false, found = false;
-        int corner = 0;             // vertex of the largest coordinate
         if (p >= 0) {
             WalkE<D> e;
             load_walk(rw, cur, e);
@@ -376,12 +377,10 @@ __global__ void __launch_bounds__(256, D == 2 ? 4 : 3) walk_kernel(const DevMesh
                 }
             }
             if (inside) {
-                if (!near) a.host[p] = e.uid;
-                a.path[p] = it;
-                a.status[p] = CS_FOUND;
-                done = found = true;
-                search = near;      // another element may contain x_p too
+                int32_t host = e.uid;
                 if (D == 3 && near) {
+                    // close to a settled vertex the host is known
+                    int corner = 0;             // vertex of the largest coordinate
                     float top = lf[0];
                     #pragma unroll
                     for (int i = 1; i <= D; ++i)
@@ -389,21 +388,21 @@ __global__ void __launch_bounds__(256, D == 2 ? 4 : 3) walk_kernel(const DevMesh
                             top = lf[i];
                             corner = i;
                         }
+                    const int32_t h = vertex_host<D>(m, cur, corner, xp);
+                    near = h == kNoVertex;
+                    host = h;
                 }
+                if (!near) a.host[p] = host;
+                a.path[p] = it;
+                a.status[p] = CS_FOUND;
+                done = found = true;
+                search = near;      // another element may contain x_p too
             } else if (next < 0 || it >= m.cap) {
                 a.path[p] = it;     // left the mesh or reached the step cap
                 done = true;
                 search = true;
             } else {
                 cur = next;
-            }
-        }
-        if (D == 3 && search && found) {
-            // close to a settled vertex of the final element the host is known
-            const int32_t h = vertex_host<D>(m, cur, corner, xp);
-            if (h != kNoVertex) {
-                a.host[p] = h;
-                search = false;
             }
         }
         for (unsigned want = __ballot_sync(kFull, search); want; want &= want - 1) {
