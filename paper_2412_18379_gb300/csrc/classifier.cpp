@@ -714,8 +714,8 @@ uint64_t splitmix(uint64_t &s) {
 }
 
 // rows per forward chunk. The fused path needs only the fully connected
-// layers' buffers (about 10 KB a row in 2-D, 13 KB in 3-D): chunks of this
-// size give those GEMMs enough tiles to fill the GPU without splitting K.
+// layers' buffers (about 3.4 KB a row in 2-D, 5.2 KB in 3-D): chunks of this
+// size give those products enough tiles to fill the GPU without splitting K.
 // The unfused path's im2col buffers take about 1 GB at its smaller chunks.
 int64_t chunk_rows(int dim, bool fused) {
     if (fused) return dim == 2 ? 32768 : 16384;
