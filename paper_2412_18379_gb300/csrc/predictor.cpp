@@ -194,7 +194,7 @@ cs_status ensure_workspace(cs_ctx *ctx, Predictor &P, int64_t B) {
     use_workspace(P.dim, kUseLayers);
     if (P.cap >= B) return CS_OK;
     free_workspace(ctx, P);
-    if (!in_use(P.dim, kUseTiles)) free_tiles(ctx, P);
+    if (!ctx->server) free_tiles(ctx, P);     // serving predicts into them
     NetShape S(P.dim);
     int Si = S.S0, C = S.cin;
     int64_t max_col = 0, max_dy = 0;

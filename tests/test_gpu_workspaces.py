@@ -112,3 +112,33 @@ def test_other_allocations_take_idle_workspaces(cs):
     assert e.value.code == -2
     assert np.array_equal(tight.grad(4096), want)
     tight.ctx.close()
+
+
+def test_a_layers_call_leaves_the_serving_tiles(cs):
+    """With the CUDA-core engine, serving predicts in 3-D into a workspace that a
+    layer-by-layer call (fewer than 16 rows) had freed as it grew its own."""
+    import torch
+    c = make_case("abc3d", n_side=13)
+    ctx = cs.Context(0)
+    ctx.load_predictor(3, init_weights(3, 1))
+    ctx.predictor_engine("tiles")
+    mesh = ctx.upload_mesh(c.xyz, c.conn)
+    field = ctx.upload_field(mesh, c.u)
+    x, u = (torch.from_numpy(np.ascontiguousarray(a)).pin_memory() for a in (c.x, c.u))
+    start = torch.from_numpy(mesh.node_start_elements()).pin_memory()
+    win = torch.randn((8, 3, 7, 7, 7), device="cuda")
+    tgt = torch.randn((8, 3), device="cuda")
+    torch.cuda.synchronize()
+    ctx.serve_start(slots=2, arena_bytes=64 << 20)
+    try:
+        results = []
+        for _ in range(2):
+            ticket, out = ctx.submit(mesh, x, u, c.dt, start=start, mode="cnn", field=field)
+            assert ctx.wait(ticket) == 1              # started by the predictor
+            results.append({k: v.clone() for k, v in out.items()})
+            ctx.predictor_grad(3, win, tgt)
+        for k in results[0]:
+            assert torch.equal(results[0][k], results[1][k]), k
+    finally:
+        ctx.serve_stop()
+    ctx.close()
